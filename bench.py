@@ -5,9 +5,11 @@ One step = one HMC-style forward + gradient of the 100-layer emission model:
 layer temperatures, both species' line-sum cross-sections, optical depth,
 emission solve, Gaussian log-likelihood, and the adjoints of all of them, in the
 mixed precision form (FP32 Voigt and compensated sums, FP64 offsets and
-strengths, FP64 radiative transfer).  The metric counts Voigt evaluations: every
-in-cut (line, grid point, layer) triple is evaluated once in the forward line sum
-and once in its adjoint.
+strengths, FP64 radiative transfer).  The metric counts the Voigt evaluations that the
+sum stands for: every in-cut (line, grid point, layer) triple once in the forward line
+sum and once in its adjoint.  Triples far from the line are summed through
+interpolation nodes (to below FP32 rounding, csrc/xs_linesum.cu), so they cost less
+than an evaluation each.
 
 The headline workload is the precision form at scale: 10,000,000 water-like +
 200,000 CO-like lines, a 100,000-point log grid over 4340-4390 cm^-1, 100 layers
@@ -49,8 +51,7 @@ FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM on sm_103a (one FFMA = 2 flops)
 # instruction counts of one ncu capture per workload (FFMA 2, FADD/FMUL 1, packed
 # FFMA2 4, FADD2/FMUL2 2 flops per thread instruction; MUFU reciprocals not
 # counted), divided by the launch's in-cut triples.  Valid only for the kernel
-# sources they were taken on (the hash); otherwise the bench falls back to the
-# cheapest-form lower bound and says so.
+# sources they were taken on (the hash); otherwise the bench reports no rate and says so.
 FLOPS_PER_TRIPLE = {
     "sources_sha256": "bcfd701beb7a1f40c608e700fbcde5e1301ffb6eae228c6aed4523b1b23de8d7",
     "scale": {"fwd": 9.00, "adj": 13.21,
@@ -60,7 +61,6 @@ FLOPS_PER_TRIPLE = {
                  "capture": "both species' launches of a 20-layer slice of the emission workload (200,000 + 20,000 "
                             "lines, 20,000 points): 6.05e11 and 8.84e11 FP32 flops over 6.60e10 triples"},
 }
-FLOPS_LOWER_BOUND = {"fwd": 8, "adj": 12}  # cheapest packed wing forms, RCP counted as 1 flop
 
 # DRAM bytes (read + write) per layer of one launch of each line-sum kernel, averaged
 # over the two species' launches, from one ncu capture of the same reduced-layer
@@ -422,8 +422,8 @@ def roofline(res, atm, workload, steps, n_sm, clk):
     per_launch = res["triples"] / len(atm.species)  # one launch per species and step, averaged over species
     fl = FLOPS_PER_TRIPLE.get(workload)
     measured = bool(fl) and FLOPS_PER_TRIPLE["sources_sha256"] == kernel_sources_sha256()
-    fpt = fl[kind] if measured else FLOPS_LOWER_BOUND[kind]
-    achieved = per_launch * fpt / (k_ms / 1000.0) / 1e12
+    fpt = fl[kind] if measured else None
+    achieved = per_launch * fpt / (k_ms / 1000.0) / 1e12 if measured else None
     peaks = read_peaks()
     sm_max = float(clk.get("sm_max_mhz") or peaks.get("sm_max_mhz") or 2070.0)
     peak_max = n_sm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
@@ -439,15 +439,17 @@ def roofline(res, atm, workload, steps, n_sm, clk):
     nl_avg = sum(sp.n for sp in atm.species) / len(atm.species)
     rec = 48 if kind == "adj" else 40
     algo_bytes = nl_avg * (rec * L + 16) + L * N * (8 + (0 if kind == "adj" else 4))
-    name = "linesum_adjoint_kernel<float>" if kind == "adj" else "linesum_kernel<float>"
-    return {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "TFLOP/s", "frac": achieved / peak_max,
+    name = ("up_kernel + far_adjoint_kernel + leaf_adjoint_f32" if kind == "adj" else
+            "far_sum_kernel + down_kernel + leaf_kernel_f32")
+    return {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "TFLOP/s",
+            "frac": achieved / peak_max if measured else None,
             "traffic": traffic, "kernel": name, "kernel_ms_per_launch": k_ms, "triples_per_launch": per_launch,
             "flops_per_triple": fpt,
             "flops_basis": (f"ncu SASS FP32 instruction counts ({fl['capture']})" if measured else
-                            "lower bound: cheapest packed wing form, ncu counts not taken on these sources"),
+                            "ncu counts not taken on these sources"),
             "peak_note": f"FP32 pipe: {n_sm} SMs (device) x {FP32_LANES_PER_SM} lanes x 2 flop x {sm_max:.0f} MHz "
                          "(max SM clock); derived, not measured",
-            "frac_at_sampled_clock": achieved / peak_med, "sampled_sm_mhz": sm_med,
+            "frac_at_sampled_clock": achieved / peak_med if measured else None, "sampled_sm_mhz": sm_med,
             "algorithmic_bytes": algo_bytes,
             "traffic_note": TRAFFIC["capture"] if traffic else "no ncu DRAM capture on these sources"}
 
