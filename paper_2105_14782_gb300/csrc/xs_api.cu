@@ -306,7 +306,7 @@ int layer_temperatures(double T0, double alpha, const double* P_bar, int32_t L, 
 {
     XS_NVTX("layer_temperatures");
     if (!P_bar || !T || L <= 0 || !(T0 > 0.0) || !std::isfinite(alpha)) return XS_EINVAL;
-    return xsi::rt_temperatures(T0, alpha, P_bar, L, T, S(stream));
+    return xsi::rt_atmosphere(T0, alpha, P_bar, L, T, 0, nullptr, nullptr, S(stream));
 }
 
 } // extern "C"
@@ -400,14 +400,10 @@ int model_forward_impl(const xs_model* m, const double* theta, double* F0out, ch
     char* sig = ws + p.sigma;
     double* dtau = (double*)(ws + p.dtau);
     int r;
-    if (T_given) {
-        if (cudaMemcpyAsync(T, T_given, sizeof(double) * m->L, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-            return XS_ECUDA;
-    } else {
-        r = xsi::rt_temperatures(theta[0], theta[1], m->P_bar, m->L, T, st);
-        if (r) return r;
-    }
-    r = xsi::rt_fill_vmr(nullptr, Sp, m->L, theta + 2, vmr, st);
+    if (T_given &&
+        cudaMemcpyAsync(T, T_given, sizeof(double) * m->L, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        return XS_ECUDA;
+    r = xsi::rt_atmosphere(theta[0], theta[1], m->P_bar, m->L, T_given ? nullptr : T, Sp, theta + 2, vmr, st);
     if (r) return r;
     const void* sp[XS_MAX_SPECIES];
     for (int s = 0; s < Sp; ++s) {
@@ -500,9 +496,10 @@ int model_adjoint_impl(const xs_model* m, const double* theta, const double* gF,
         else
             r = xsi::xs_run(&m->species[s], m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec,
                             nullptr, ws + p.xsws_sp[s], p.xsws_sp_bytes[s], true, gsp[s], gTtmp, gb + s, st,
-                            xsi::XS_RUN_REUSE);
+                            xsi::XS_RUN_REUSE, gT);
         if (r) return r;
-        if ((r = xsi::rt_accumulate(gT, gTtmp, m->L, 0, st))) return r;
+        // a species without lines has no kernel that adds its (zero) gradient
+        if (m->method == XS_METHOD_MODIT && (r = xsi::rt_accumulate(gT, gTtmp, m->L, 0, st))) return r;
     }
     if (per_layer) return xsi::rt_layer_grad(Sp, m->L, theta + 2, gT, gvmr, gb, out, st);
     return xsi::rt_theta_grad(Sp, m->L, theta[0], theta[1], theta + 2, theta[2 + Sp], T, m->P_bar, gT, gvmr, gb, out,

@@ -45,6 +45,38 @@ constexpr double SQRT2 = 1.41421356237309504880;
 constexpr double MIXED_SCALE = 1208925819614629174706176.0; // 2^80
 constexpr double MIXED_UNSCALE = 8.27180612553027674871e-25; // 2^-80
 
+// cos x at compile time, 0 <= x <= pi/2 (Taylor series)
+constexpr double cos_quadrant(double x)
+{
+    double s = 0.0;
+    for (int k = 14; k >= 1; --k) s = -(1.0 + s) * x * x / ((2.0 * k - 1.0) * (2.0 * k));
+    return 1.0 + s;
+}
+
+// Chebyshev nodes t_m = cos((2m + 1) pi/(2n)) and T_k(t_m) = cos(k (2m + 1) pi/(2n)),
+// built at compile time.
+template <int n>
+struct ChebTable {
+    double T[n][n]; // [k][m]; T[1] are the nodes
+};
+template <int n>
+constexpr ChebTable<n> make_cheb()
+{
+    ChebTable<n> c{};
+    for (int k = 0; k < n; ++k)
+        for (int m = 0; m < n; ++m) {
+            int j = (k * (2 * m + 1)) % (4 * n); // angle j pi/(2n), one period
+            double s = 1.0;
+            if (j > 2 * n) j = 4 * n - j;
+            if (j > n) {
+                j = 2 * n - j;
+                s = -1.0;
+            }
+            c.T[k][m] = (j == n) ? 0.0 : s * cos_quadrant(PI * j / (2.0 * n));
+        }
+    return c;
+}
+
 template <class R> struct vec4;
 template <> struct vec4<float> { using type = float4; };
 template <> struct vec4<double> { using type = double4_32a; };

@@ -42,11 +42,11 @@ int check_lines(const xs_lines* ln);
 int check_common(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L,
                  double sb, double W, int prec);
 
-// line-sum forward (adjoint == false: writes sigma) or adjoint (writes g_T, g_b);
-// flags as above (0 for a self-contained call)
+// line-sum forward (adjoint == false: writes sigma) or adjoint (writes g_T, g_b, and adds
+// g_T to g_T_sum where that is given); flags as above (0 for a self-contained call)
 int xs_run(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
            double W, int prec, void* sigma, void* ws, size_t ws_bytes, bool adjoint, const double* g_sigma,
-           double* g_T, double* g_b, cudaStream_t st, int flags = 0);
+           double* g_T, double* g_b, cudaStream_t st, int flags = 0, double* g_T_sum = nullptr);
 
 // checks ascending (grid == false: non-decreasing centres; grid == true: strictly
 // increasing grid) on the device; blocks on `st`; flag_dev is one device int
@@ -64,9 +64,9 @@ int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T,
                         int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st);
 int rt_loglike(const double* F, const double* d, const double* s, int64_t N, double* logL, double* g_F,
                cudaStream_t st);
-int rt_temperatures(double T0, double alpha, const double* P, int32_t L, double* T, cudaStream_t st);
-int rt_fill_vmr(const double* theta_dev_unused, int32_t S, int32_t L, const double* log10_vmr_host, double* vmr,
-                cudaStream_t st);
+// layer temperatures (T may be null) and mixing ratios (vmr may be null)
+int rt_atmosphere(double T0, double alpha, const double* P, int32_t L, double* T, int32_t S,
+                  const double* log10_vmr_host, double* vmr, cudaStream_t st);
 int rt_theta_grad(int32_t S, int32_t L, double T0, double alpha, const double* log10_vmr_host, double sb,
                   const double* T, const double* P, const double* g_T, const double* g_vmr, const double* g_b,
                   double* out, cudaStream_t st);

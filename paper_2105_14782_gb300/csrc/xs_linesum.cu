@@ -66,35 +66,6 @@ template <> struct Far<double> {
     static constexpr double kappa = 5.0, Z0 = 8.0;
 };
 
-// Chebyshev nodes t_m = cos((2m + 1) pi/(2n)) and T_k(t_m) = cos(k (2m + 1) pi/(2n)),
-// built at compile time from the Taylor series of the cosine on the first quadrant.
-template <int n>
-struct ChebTable {
-    double T[n][n]; // [k][m]; T[1] are the nodes
-};
-constexpr double cos_quadrant(double x)
-{
-    double s = 0.0;
-    for (int k = 14; k >= 1; --k) s = -(1.0 + s) * x * x / ((2.0 * k - 1.0) * (2.0 * k));
-    return 1.0 + s;
-}
-template <int n>
-constexpr ChebTable<n> make_cheb()
-{
-    ChebTable<n> c{};
-    for (int k = 0; k < n; ++k)
-        for (int m = 0; m < n; ++m) {
-            int j = (k * (2 * m + 1)) % (4 * n); // angle j pi/(2n), one period
-            double s = 1.0;
-            if (j > 2 * n) j = 4 * n - j;
-            if (j > n) {
-                j = 2 * n - j;
-                s = -1.0;
-            }
-            c.T[k][m] = (j == n) ? 0.0 : s * cos_quadrant(PI * j / (2.0 * n));
-        }
-    return c;
-}
 __device__ const ChebTable<10> CHEB10 = make_cheb<10>();
 __device__ const ChebTable<18> CHEB18 = make_cheb<18>();
 template <int n> __device__ __forceinline__ double cheb(int k, int m) { return (n == 10) ? CHEB10.T[k][m] : CHEB18.T[k][m]; }
@@ -1676,14 +1647,17 @@ __global__ void adjoint_reduce_kernel(const double* __restrict__ part, int per_l
     }
 }
 
-// g_b = sum over layers of gbl (in layer order) / s_b
-__global__ void broad_sum_kernel(const double* __restrict__ gbl, int L, double inv_sb, double* __restrict__ g_b)
+// g_b = sum over layers of gbl / s_b (one warp, fixed order); g_T_sum += g_T where given
+__global__ void broad_sum_kernel(const double* __restrict__ gbl, int L, double inv_sb, double* __restrict__ g_b,
+                                 const double* __restrict__ g_T, double* __restrict__ g_T_sum)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int n = 0; n < L; ++n) s += gbl[n];
-        g_b[0] = s * inv_sb;
+    double s = 0.0;
+    for (int n = threadIdx.x; n < L; n += 32) {
+        s += gbl[n];
+        if (g_T_sum) g_T_sum[n] += g_T[n];
     }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) g_b[0] = s * inv_sb;
 }
 
 } // namespace xsd
@@ -1832,7 +1806,7 @@ static unsigned blocks_of(int64_t n, int threads) { return (unsigned)((n + threa
 template <class R>
 static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L,
                   double sb, double W, void* sigma, char* ws, const XsPlan& p, bool adjoint,
-                  const double* g_sigma, double* g_T, double* g_b, cudaStream_t st, int flags)
+                  const double* g_sigma, double* g_T, double* g_b, cudaStream_t st, int flags, double* g_T_sum)
 {
     // flags: XS_RUN_KEEP_ADJ  (forward) also write the adjoint's per-line records
     //        XS_RUN_REUSE     (adjoint) the records and ranges of an immediately preceding
@@ -1934,7 +1908,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
     }
     if (adjoint) {
         adjoint_reduce_kernel<<<L, 256, 0, st>>>(leaf, p.leaf_blocks, tr.on ? slots : nullptr, p.fw.slots, g_T, gbl);
-        broad_sum_kernel<<<1, 32, 0, st>>>(gbl, L, 1.0 / sb, g_b);
+        broad_sum_kernel<<<1, 32, 0, st>>>(gbl, L, 1.0 / sb, g_b, g_T, g_T_sum);
         count_launch(2);
     }
     return (cudaGetLastError() == cudaSuccess) ? XS_OK : XS_ECUDA;
@@ -1942,13 +1916,15 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
 
 int xs_run(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
            double W, int prec, void* sigma, void* ws, size_t ws_bytes, bool adjoint, const double* g_sigma,
-           double* g_T, double* g_b, cudaStream_t st, int flags)
+           double* g_T, double* g_b, cudaStream_t st, int flags, double* g_T_sum)
 {
     XsPlan p;
     if (pick_plan(ln->n, N, L, prec, ws_bytes, &p) != XS_OK) return XS_EINVAL;
     if (prec == XS_PREC_FP64)
-        return run_xs<double>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags);
-    return run_xs<float>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags);
+        return run_xs<double>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags,
+                              g_T_sum);
+    return run_xs<float>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags,
+                              g_T_sum);
 }
 
 int check_sorted(const double* nu_hat, int64_t n, cudaStream_t st, int* flag_dev, bool grid)
