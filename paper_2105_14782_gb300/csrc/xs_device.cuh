@@ -285,82 +285,125 @@ __device__ __forceinline__ void w_series(R xh, R xl, R a, R Kc, R* wr, R* wi)
     *wi = ex * (-Kc * s2 + hpi * s2_a) + hpi * ss;
 }
 
-// Per-line table for w_series_tab (near kernels, |z| < 6 so n0 = round(x/h) <= 9):
-// d[n + SER_OFF] = 1/(n^2 h^2 + a^2) for n = 1 .. SER_TAB - 1 - SER_OFF, and 0 for
-// n <= 0 (terms that do not exist).
-constexpr int SER_OFF = 6;  // n0 - 6 >= -6
-constexpr int SER_TAB = 22; // n up to 9 + 6 = 15
+// Per-line table for w_series_tab: d[n + SER_OFF] = 1/(n^2 h^2 + a^2) for n != 0 and 0
+// for n = 0, n = -SER_OFF .. SER_TAB - 1 - SER_OFF.  The odd row length keeps the lanes
+// that fill 32 rows on different banks.
+constexpr int SER_OFF = 6;   // terms on each side of the peak
+constexpr int SER_N0 = 16;   // largest peak index: x <= SER_X
+constexpr int SER_TAB = SER_N0 + 2 * SER_OFF + 1; // 29
+constexpr float SER_X = 11.5f;
 
 __device__ __forceinline__ void series_table(float a, float* d)
 {
     const float h = Tier<float>::h;
     const float a2 = a * a;
-#pragma unroll 2
-    for (int i = 0; i < SER_TAB; ++i) {
-        const int n = i - SER_OFF;
+    d[SER_OFF] = 0.0f;
+#pragma unroll 4
+    for (int n = 1; n < SER_TAB - SER_OFF; ++n) {
         const float nh = (float)n * h;
-        d[i] = (n >= 1) ? rcp_fast(fmaf(nh, nh, a2)) : 0.0f;
+        const float v = rcp_fast(fmaf(nh, nh, a2));
+        d[SER_OFF + n] = v;
+        if (n <= SER_OFF) d[SER_OFF - n] = v;
     }
 }
 
-// FP32 small-|z| series (near kernels, 0 <= x < 6.3) with the E_n^- taken by a
-// two-way recurrence from the term nearest the peak, n0 = round(x/h), where
-// t = n0 h - x = delta is small:
+__device__ __forceinline__ float exp2_fast(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// sin r for |r| <= pi/2 and, if want_c, cos r: Taylor series (next terms below 7e-10)
+__device__ __forceinline__ void sincos_half(float r, bool want_c, float* s, float* c)
+{
+    const float t = r * r;
+    float p = 1.0f / 6227020800.0f;
+    p = fmaf(p, t, -1.0f / 39916800.0f);
+    p = fmaf(p, t, 1.0f / 362880.0f);
+    p = fmaf(p, t, -1.0f / 5040.0f);
+    p = fmaf(p, t, 1.0f / 120.0f);
+    p = fmaf(p, t, -1.0f / 6.0f);
+    *s = fmaf(p * t, r, r);
+    if (want_c) {
+        float q = -1.0f / 87178291200.0f;
+        q = fmaf(q, t, 1.0f / 479001600.0f);
+        q = fmaf(q, t, -1.0f / 3628800.0f);
+        q = fmaf(q, t, 1.0f / 40320.0f);
+        q = fmaf(q, t, -1.0f / 720.0f);
+        q = fmaf(q, t, 1.0f / 24.0f);
+        q = fmaf(q, t, -0.5f);
+        *c = fmaf(q, t, 1.0f);
+    }
+}
+
+// FP32 small-|z| series, 0 <= x <= SER_X, written as one sum over all integers n != 0 of
+// exp(-(nh - x)^2) d_|n| (the E_n^+ of the head of this file are its negative n).  The
+// exponentials come by a two-way recurrence from the term nearest the peak,
+// n0 = round(x/h), where t = n0 h - x = delta is small:
 //   E_{n0+k} = E_{n0+k-1} e^{-2h delta} q^{2k-1},  E_{n0-k} = E_{n0-k+1} e^{+2h delta} q^{2k-1},
 //   q = e^{-h^2};
-// every factor has a small exponent, so no digits are lost to e^{-x^2} e^{2nhx}.
-// E_n^+ = E_n^- e^{-4nhx} rides along.  Terms with |k| > 6 are below 1e-9 of the
-// peak term.  The terms above and below the peak go as packed pairs, with the
-// line's table of 1/(n^2 h^2 + a^2) (series_table).
-__device__ __forceinline__ void w_series_tab(float xh, float xl, float a, float Kc, const float* dt, float* wr,
-                                             float* wi)
+// every factor has a small exponent, so no digits are lost to e^{-x^2} e^{2nhx}.  Terms
+// with |k| > 6 are below 1e-9 of the peak term.  The terms above and below the peak go as
+// packed pairs, with the line's table d (series_table).  sin and cos of ax enter as
+// sin^2 and sin cos only, so ax is reduced modulo pi and its sign dropped.  inv_a = 1/a.
+template <bool WANT_WI>
+__device__ __forceinline__ void w_series_tab(float xh, float xl, float a, float inv_a, float Kc, const float* dt,
+                                             float* wr, float* wi)
 {
     const float h = Tier<float>::h;
-    // q^(2k-1), q = exp(-h^2) with h = 0.7f
-    const float Q[6] = {0.61262643f, 0.22992550f, 0.08629359f, 0.03238694f, 0.012155180f, 0.0045619742f};
+    constexpr float L2E = 1.44269504f, MAGIC = 12582912.0f; // 1.5 2^23: rounds to an integer
+    constexpr float h2L = 0.7f * 0.7f * L2E;
+    const float q2 = 0.375311099f; // e^{-2 h^2}
     const float x = xh;
-    const int n0 = __float2int_rn(x * (1.0f / h));
-    const float n0h = (float)n0 * h;
-    const float delta = (n0h - xh) - xl;
-    const float E0 = __expf(-delta * delta);
-    const float2 f = make_float2(__expf(-2.0f * h * delta), __expf(2.0f * h * delta));
-    const float R4 = __expf(-4.0f * h * x);
-    const float2 g = make_float2(R4, rcp_fast(R4));
-    const float Rn = __expf(-4.0f * h * x * (float)n0);
-    if (!XS_CHECK(n0 >= 0 && n0 + 2 * SER_OFF < SER_TAB)) { // |z| < 6 keeps n0 <= 9
+    const float tm = fmaf(x, 1.0f / h, MAGIC);
+    const float n0f = tm - MAGIC;
+    const int n0 = __float_as_int(tm) & 31;
+    if (!XS_CHECK(n0 <= SER_N0)) {
         *wr = 0.0f;
         *wi = 0.0f;
         return;
     }
+    const float n0h = n0f * h;
+    const float delta = (n0h - xh) - xl;
+    const float E0 = exp2_fast(-L2E * delta * delta);
+    const float u = 2.0f * h * L2E * delta;
+    float2 r = make_float2(exp2_fast(-u - h2L), exp2_fast(u - h2L));
     const float* d0 = dt + (n0 + SER_OFF);
-    // centre term (d0[0] = 0 when n0 = 0)
-    const float ep0 = E0 * Rn;
-    const float dc = d0[0];
-    float2 sc = make_float2(dc * (E0 + ep0), 0.0f);
-    float2 ss = make_float2(n0h * dc * (E0 - ep0), 0.0f);
-    float2 E = make_float2(E0, E0), R = make_float2(Rn, Rn), nh = make_float2(n0h, n0h);
+    float2 E = make_float2(E0, E0);
+    const float e0 = d0[0] * E0;
+    float2 sc = make_float2(e0, 0.0f), ss = make_float2(n0h * e0, 0.0f);
+    float2 nh = make_float2(n0h, n0h);
     const float2 hstep = make_float2(h, -h);
 #pragma unroll
-    for (int k = 1; k <= 6; ++k) {
-        E = __fmul2_rn(__fmul2_rn(E, f), make_float2(Q[k - 1], Q[k - 1])); // (E_{n0+k}, E_{n0-k})
-        R = __fmul2_rn(R, g);
-        nh = __fadd2_rn(nh, hstep);
-        const float2 ep = __fmul2_rn(E, R);
+    for (int k = 1; k <= SER_OFF; ++k) {
+        E = __fmul2_rn(E, r); // (E_{n0+k}, E_{n0-k})
+        if (k < SER_OFF) r = __fmul2_rn(r, make_float2(q2, q2));
         const float2 dd = make_float2(d0[k], d0[-k]);
-        sc = __ffma2_rn(dd, __fadd2_rn(E, ep), sc);
-        ss = __ffma2_rn(__fmul2_rn(nh, dd), __fadd2_rn(E, make_float2(-ep.x, -ep.y)), ss);
+        if (WANT_WI) {
+            const float2 e = __fmul2_rn(E, dd);
+            nh = __fadd2_rn(nh, hstep);
+            sc = __fadd2_rn(sc, e);
+            ss = __ffma2_rn(nh, e, ss);
+        } else {
+            sc = __ffma2_rn(E, dd, sc);
+        }
     }
     const float scs = sc.x + sc.y, sss = ss.x + ss.y;
     const float ex = exp_negsq(xh) * (1.0f - 2.0f * xh * xl);
+    const float ax = a * x;
+    const float km = fmaf(ax, (float)(1.0 / PI), MAGIC) - MAGIC;
+    const float rr = fmaf(-km, (float)(PI - (double)(float)PI), fmaf(-km, (float)PI, ax));
     float sax, cax;
-    sincosf(a * x, &sax, &cax);
-    const float c2v = 1.0f - 2.0f * sax * sax; // cos 2ax
-    const float s2 = 2.0f * sax * cax;         // sin 2ax
-    const float sax_a = (a > 0.0f) ? sax * rcp_fast(a) : x;
-    const float s2_a = 2.0f * sax_a * cax;
+    sincos_half(rr, WANT_WI, &sax, &cax);
+    const float c2v = fmaf(-2.0f * sax, sax, 1.0f); // cos 2ax
     const float hpi = h * (float)(1.0 / PI);
-    *wr = ex * (Kc * c2v + 2.0f * hpi * sax * sax_a) + a * hpi * scs;
-    *wi = ex * (-Kc * s2 + hpi * s2_a) + hpi * sss;
+    *wr = ex * fmaf(2.0f * hpi * inv_a * sax, sax, Kc * c2v) + a * hpi * scs;
+    if (WANT_WI) {
+        const float s2 = 2.0f * sax * cax; // sin 2ax
+        const float s2_a = a > 0.0f ? s2 * inv_a : 2.0f * x;
+        *wi = ex * (-Kc * s2 + hpi * s2_a) + hpi * sss;
+    }
 }
 
 template <class R>

@@ -1097,8 +1097,7 @@ struct LeafScratch {
 };
 struct NearTile {
     LeafScratch<10> fs;
-    float2 nb[32]; // middle of the leaf - centre, hi and lo
-    float clo[32];
+    float4 nb[32]; // middle of the leaf - centre (hi, lo), the part of c that r2.x misses, 1/a
     float4 r2[32]; // c, a, Av, Kc
     int2 jr[32];
     float4 hc[32][4];      // Av C'_0 .. Av C'_12 of the wing polynomial (6 <= |z|), or the wing form's constants
@@ -1107,8 +1106,7 @@ struct NearTile {
 struct NearAdjTile {
     LeafScratch<10> fs;
     float lam[10];
-    float2 nb[32];
-    float clo[32];
+    float4 nb[32];
     float4 r2[32];
     int2 jr[32];
     float aS[32], nn[32];
@@ -1297,9 +1295,8 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
                 }
             } else {
                 if (have) {
-                    tl.nb[lane] = make_float2(nb, nbl);
+                    tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
                     tl.r2[lane] = p2;
-                    tl.clo[lane] = ln.clo[l];
                     float C[ASY_N];
                     asy_coeffs(p2.y, p2.z, C);
                     store16(tl.hc[lane], C, ASY_N);
@@ -1312,23 +1309,23 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
                     // x to FP32 accuracy suffices for the polynomial (a rational
                     // function of x); the series takes the exact pair
                     const float4 c4 = tl.r2[q];
-                    const float2 b = tl.nb[q];
+                    const float4 b = tl.nb[q];
                     const float dh = ohi + b.x, dl = olo + b.y;
                     const float xq = c4.x * (dh + dl);
                     const float zz = fmaf(xq, xq, c4.y * c4.y);
-                    const bool ser = in && zz < NEAR_POLY_Z2;
-                    if (!__any_sync(0xffffffffu, ser)) {
+                    if (!__any_sync(0xffffffffu, in && zz < NEAR_POLY_Z2)) {
                         // no lane in the series zone: the polynomial, branch-free
                         const float hv = horner13(tl.hc[q], rcp_fast(zz));
                         acc += in ? hv : 0.0f;
                     } else if (in) {
-                        if (!ser) {
+                        // the series also serves the lanes just outside its zone
+                        if (!(fabsf(xq) <= SER_X)) {
                             acc += horner13(tl.hc[q], rcp_fast(zz));
                         } else {
                             float x, xl;
-                            scaled_pair(dh, dl, c4.x, tl.clo[q], &x, &xl);
+                            scaled_pair(dh, dl, c4.x, b.z, &x, &xl);
                             float wr, wi;
-                            w_series_tab(x, xl, c4.y, c4.w, tl.sd[q], &wr, &wi);
+                            w_series_tab<false>(x, xl, c4.y, b.w, c4.w, tl.sd[q], &wr, &wi);
                             acc = fmaf(c4.z, wr, acc);
                         }
                     }
@@ -1499,10 +1496,9 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
                     }
                 } else {
                     if (have) {
-                        tl.nb[lane] = make_float2(nb, nbl);
+                        tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
                         tl.r2[lane] = p2;
-                        tl.clo[lane] = ln.clo[l];
-                        tl.aS[lane] = p3.x;
+                            tl.aS[lane] = p3.x;
                         tl.nn[lane] = p3.y;
                         float F[ASY_N + 1], G[ASY_N + 1];
                         asy_coeffs_adj(p2.y, p2.z, p3.x, hT, p3.y, F, G);
@@ -1516,10 +1512,11 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
                         // x to FP32 accuracy suffices for the polynomial (a rational
                         // function of x); the series takes the exact pair
                         const float4 c4 = tl.r2[q];
-                        const float2 b = tl.nb[q];
+                        const float4 b = tl.nb[q];
                         const float dh = ohi + b.x, dl = olo + b.y;
                         const float xq = c4.x * (dh + dl);
                         const float zz = fmaf(xq, xq, c4.y * c4.y);
+                        // (the series loses 2|z|^2 in w', so it stops at its zone's edge)
                         const bool ser = in && zz < NEAR_POLY_Z2;
                         if (!__any_sync(0xffffffffu, ser)) {
                             // no lane in the series zone: the polynomials, branch-free
@@ -1534,10 +1531,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
                                 aB += horner14(tl.hg[q], u);
                             } else {
                                 float x, xl;
-                                scaled_pair(dh, dl, c4.x, tl.clo[q], &x, &xl);
+                                scaled_pair(dh, dl, c4.x, b.z, &x, &xl);
                                 const float a = c4.y;
                                 float wr, wi;
-                                w_series_tab(x, xl, a, c4.w, tl.sd[q], &wr, &wi);
+                                w_series_tab<true>(x, xl, a, b.w, c4.w, tl.sd[q], &wr, &wi);
                                 // w' = -2 z w + 2i/sqrt(pi);  H_x = Re w', H_a = -Im w'
                                 const float dr = -2.0f * (x * wr - a * wi);
                                 const float di = -2.0f * (x * wi + a * wr) + (float)(2.0 * INV_SQRTPI);
