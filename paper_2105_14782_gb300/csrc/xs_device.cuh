@@ -152,14 +152,12 @@ __device__ __forceinline__ void scaled_pair(float dh, float dl, float ch, float 
 {
     // renormalise d = dh + dl first (Fast2Sum, |dl| << |dh| or both tiny) so that
     // xh, which the asymptotic tiers use alone, carries all of d's leading bits
-    float d = dh + dl;
-    float e = (dh - d) + dl;
-    float sgn = (d < 0.0f) ? -1.0f : 1.0f;
-    d *= sgn;
-    e *= sgn;
-    float p = d * ch;
-    *xh = p;
-    *xl = fmaf(d, ch, -p) + fmaf(d, cl, e * ch);
+    const float d = dh + dl;
+    const float e = (dh - d) + dl;
+    const float p = d * ch;
+    const float r = fmaf(d, ch, -p) + fmaf(d, cl, e * ch);
+    *xh = fabsf(p);
+    *xl = __int_as_float(__float_as_int(r) ^ (__float_as_int(d) & 0x80000000)); // r with d's sign taken out
 }
 __device__ __forceinline__ void scaled_pair(double dh, double, double ch, double, double* xh, double* xl)
 {
@@ -182,11 +180,11 @@ __device__ __forceinline__ float sin_r(float v) { return sinf(v); }
 __device__ __forceinline__ double sin_r(double v) { return sin(v); }
 
 // exp(-x^2) with x^2 split into hi + lo so the rounding of x*x does not enter.
-__device__ __forceinline__ float exp_negsq(float x)
+__device__ __forceinline__ float exp_negsq(float x, float xl) // x + xl, |xl| << |x|
 {
     float hi = x * x;
-    float lo = fmaf(x, x, -hi);
-    return expf(-hi) * (1.0f - lo);
+    float lo = fmaf(2.0f * x, xl, fmaf(x, x, -hi));
+    return fmaf(expf(-hi), -lo, expf(-hi));
 }
 __device__ __forceinline__ double exp_negsq(double x)
 {
@@ -338,23 +336,20 @@ __device__ __forceinline__ void sincos_half(float r, bool want_c, float* s, floa
 }
 
 // FP32 small-|z| series, 0 <= x <= SER_X, written as one sum over all integers n != 0 of
-// exp(-(nh - x)^2) d_|n| (the E_n^+ of the head of this file are its negative n).  The
-// exponentials come by a two-way recurrence from the term nearest the peak,
-// n0 = round(x/h), where t = n0 h - x = delta is small:
-//   E_{n0+k} = E_{n0+k-1} e^{-2h delta} q^{2k-1},  E_{n0-k} = E_{n0-k+1} e^{+2h delta} q^{2k-1},
-//   q = e^{-h^2};
-// every factor has a small exponent, so no digits are lost to e^{-x^2} e^{2nhx}.  Terms
-// with |k| > 6 are below 1e-9 of the peak term.  The terms above and below the peak go as
-// packed pairs, with the line's table d (series_table).  sin and cos of ax enter as
-// sin^2 and sin cos only, so ax is reduced modulo pi and its sign dropped.  inv_a = 1/a.
+// exp(-(nh - x)^2) d_|n| (the E_n^+ of the head of this file are its negative n).  From
+// the term nearest the peak, n0 = round(x/h), where n0 h - x = delta is small,
+//   exp(-((n0 +- k)h - x)^2) = e^{-delta^2} Q_k e^{-+2kh delta},  Q_k = e^{-(kh)^2},
+// so each side is a polynomial in e^{-+2h delta}: no digits are lost to e^{-x^2} e^{2nhx}.
+// Terms with |k| > 6 are below 1e-9 of the peak term.  The two sides go as packed pairs,
+// with the line's table d (series_table).  sin and cos of ax enter as sin^2 and sin cos
+// only, so ax is reduced modulo pi and its sign dropped.  inv_a = 1/a.  Issue-bound:
+// about 100 instructions a pair of line and point (150 for w) with its loop.
 template <bool WANT_WI>
 __device__ __forceinline__ void w_series_tab(float xh, float xl, float a, float inv_a, float Kc, const float* dt,
                                              float* wr, float* wi)
 {
     const float h = Tier<float>::h;
     constexpr float L2E = 1.44269504f, MAGIC = 12582912.0f; // 1.5 2^23: rounds to an integer
-    constexpr float h2L = 0.7f * 0.7f * L2E;
-    const float q2 = 0.375311099f; // e^{-2 h^2}
     const float x = xh;
     const float tm = fmaf(x, 1.0f / h, MAGIC);
     const float n0f = tm - MAGIC;
@@ -368,29 +363,24 @@ __device__ __forceinline__ void w_series_tab(float xh, float xl, float a, float 
     const float delta = (n0h - xh) - xl;
     const float E0 = exp2_fast(-L2E * delta * delta);
     const float u = 2.0f * h * L2E * delta;
-    float2 r = make_float2(exp2_fast(-u - h2L), exp2_fast(u - h2L));
+    const float2 f = make_float2(exp2_fast(-u), exp2_fast(u)); // e^{-2h delta}, e^{2h delta}
     const float* d0 = dt + (n0 + SER_OFF);
-    float2 E = make_float2(E0, E0);
-    const float e0 = d0[0] * E0;
-    float2 sc = make_float2(e0, 0.0f), ss = make_float2(n0h * e0, 0.0f);
-    float2 nh = make_float2(n0h, n0h);
-    const float2 hstep = make_float2(h, -h);
+    // sums over k of Q_k d_{n0 +- k} f^k by Horner, Q_k = e^{-(kh)^2}; the sums with a
+    // factor k, for Im w, are f times the derivative in f
+    const float Q[SER_OFF + 1] = {1.0f, 0.612626433f, 0.140858427f, 0.0121551799f, 0.00039366915f, 4.78511947e-06f,
+                                  2.18295906e-08f};
+    float2 s = __fmul2_rn(make_float2(d0[SER_OFF], d0[-SER_OFF]), make_float2(Q[SER_OFF], Q[SER_OFF]));
+    float2 ds = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int k = 1; k <= SER_OFF; ++k) {
-        E = __fmul2_rn(E, r); // (E_{n0+k}, E_{n0-k})
-        if (k < SER_OFF) r = __fmul2_rn(r, make_float2(q2, q2));
-        const float2 dd = make_float2(d0[k], d0[-k]);
-        if (WANT_WI) {
-            const float2 e = __fmul2_rn(E, dd);
-            nh = __fadd2_rn(nh, hstep);
-            sc = __fadd2_rn(sc, e);
-            ss = __ffma2_rn(nh, e, ss);
-        } else {
-            sc = __ffma2_rn(E, dd, sc);
-        }
+    for (int k = SER_OFF - 1; k >= 0; --k) {
+        if (WANT_WI) ds = __ffma2_rn(ds, f, s);
+        // the centre term, k = 0, belongs to the first of the pair
+        const float2 w = k ? __fmul2_rn(make_float2(d0[k], d0[-k]), make_float2(Q[k], Q[k])) : make_float2(d0[0], 0.0f);
+        s = __ffma2_rn(s, f, w);
     }
-    const float scs = sc.x + sc.y, sss = ss.x + ss.y;
-    const float ex = exp_negsq(xh) * (1.0f - 2.0f * xh * xl);
+    const float scs = E0 * (s.x + s.y);
+    const float sss = WANT_WI ? fmaf(n0h, scs, h * E0 * (f.x * ds.x - f.y * ds.y)) : 0.0f;
+    const float ex = exp_negsq(xh, xl);
     const float ax = a * x;
     const float km = fmaf(ax, (float)(1.0 / PI), MAGIC) - MAGIC;
     const float rr = fmaf(-km, (float)(PI - (double)(float)PI), fmaf(-km, (float)PI, ax));

@@ -12,10 +12,9 @@
 // edge inside it, is summed point by point.  Lines are sorted, so all of these sets
 // are index ranges and every in-cut (line, point) pair belongs to exactly one.
 //
-//   far_sum_kernel    node sums of the 128-, 512- and 2,048-point intervals
-//   down_kernel       node sums -> polynomials, from the larger intervals into the smaller
-//   leaf_kernel       per leaf: its own far lines at its nodes, its near lines at its
-//                     points, plus the polynomials; writes sigma
+//   far_sum_kernel    node sums of the leaves and of the intervals above
+//   down_kernel       node sums -> polynomials, from the larger intervals into the leaves
+//   leaf_kernel       per leaf: its near lines at its points plus its polynomial; writes sigma
 // and for the adjoint, where sum_j lambda_j f(nu_j) = sum_m Lambda_m f(node_m) for every
 // polynomial f of the degree kept:
 //   up_kernel         lambda -> the intervals' node weights Lambda
@@ -797,7 +796,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
     }
 }
 
-// ------------------------------------------------------------------ intervals above the leaves
+// ------------------------------------------------------------------ far kernels
 
 // Work of the far kernels: blocks of FAR_WARPS neighbouring intervals of a level and
 // one part of their lists, largest intervals (longest lists) first.
@@ -809,7 +808,7 @@ struct FarWork {
 
 __device__ __forceinline__ bool far_task(const Tree& tr, const FarWork& fw, int* level, int* i, int* part)
 {
-    int k = 1;
+    int k = 0;
     while (k < LEVELS - 1 && (int)blockIdx.x < fw.block0[k]) ++k;
     const int r = blockIdx.x - fw.block0[k];
     *level = k;
@@ -880,7 +879,7 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(
     if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
     double sT = 0.0, sB = 0.0;
     far_adjoint_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * layer],
-                    weights + ((size_t)nloc * (tr.total - tr.cnt[0]) + (tr.off[k] - tr.cnt[0]) + i) * n,
+                    weights + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
                     (R)(0.5 / T[layer]), sT, sB);
     for (int o = 16; o > 0; o >>= 1) {
         sT += __shfl_xor_sync(0xffffffffu, sT, o);
@@ -921,39 +920,44 @@ __device__ __forceinline__ R clenshaw(const R* c, R x)
     return x * b1 + (c[0] - b2);
 }
 
-// Polynomials of the 128-point intervals: per layer and top interval, the node sums of
-// each level plus the polynomial of the interval above.  coef[layer][interval][n].
+// Polynomials of the leaves: per layer and top interval, the node sums of each level
+// plus the polynomial of the interval above.  coef[layer][leaf][n].
+constexpr int DOWN_ROWS = 16; // intervals of a level that a block takes at a time
 template <class R>
-__global__ void __launch_bounds__(16 * Far<R>::n) down_kernel(const __grid_constant__ Tree tr, const __grid_constant__ FarWork fw, int Lc,
-                                                              const double* __restrict__ sums,
-                                                              double* __restrict__ coef)
+__global__ void __launch_bounds__(DOWN_ROWS * Far<R>::n) down_kernel(const __grid_constant__ Tree tr,
+                                                                     const __grid_constant__ FarWork fw, int Lc,
+                                                                     const double* __restrict__ sums,
+                                                                     double* __restrict__ coef)
 {
-    constexpr int n = Far<R>::n;
-    __shared__ double v[16][n], c[16][n];
-    const int t = threadIdx.x, m = t % n, q = t / n;
+    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
+    __shared__ double v[DOWN_ROWS][n], c[2][TOP][n];
+    const int m = threadIdx.x % n, row = threadIdx.x / n;
     const int nloc = blockIdx.y, top = blockIdx.x;
-    for (int k = LEVELS - 1; k >= 1; --k) {
+    for (int k = LEVELS - 1; k >= 0; --k) {
         const int many = 1 << (2 * (LEVELS - 1 - k)); // intervals of this level under the top one
-        const int i = top * many + q;
-        const bool mine = q < many && i < tr.cnt[k];
-        double s = 0.0;
-        if (mine) {
-            for (int p = 0; p < fw.parts[k]; ++p)
-                s += sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
-            if (k < LEVELS - 1) {
-                const double2 g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
-                s += clenshaw<n, double>(c[q >> 2], in_span(fma(g.y, cheb<n>(1, m), g.x), gp));
+        for (int q0 = 0; q0 < many; q0 += DOWN_ROWS) {
+            const int q = q0 + row, i = top * many + q;
+            const bool mine = q < many && i < tr.cnt[k];
+            if (mine) {
+                double s = 0.0;
+                for (int p = 0; p < fw.parts[k]; ++p)
+                    s += sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
+                if (k < LEVELS - 1) {
+                    const double2 g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
+                    s += clenshaw<n, double>(c[(k + 1) & 1][q >> 2], in_span(fma(g.y, cheb<n>(1, m), g.x), gp));
+                }
+                v[row][m] = s;
             }
+            __syncthreads();
+            if (mine) {
+                const double ck = cheb_coeff<n>(v[row], m);
+                if (k > 0)
+                    c[k & 1][q][m] = ck;
+                else
+                    coef[((size_t)nloc * tr.cnt[0] + i) * n + m] = ck;
+            }
+            __syncthreads();
         }
-        __syncthreads(); // c of the level above is read
-        if (mine) v[q][m] = s;
-        __syncthreads();
-        if (mine) {
-            const double ck = cheb_coeff<n>(v[q], m);
-            c[q][m] = ck;
-            if (k == 1) coef[((size_t)nloc * tr.cnt[1] + i) * n + m] = ck;
-        }
-        __syncthreads();
     }
 }
 
@@ -984,53 +988,53 @@ __device__ __forceinline__ double node_weight(const double* M, int m)
     return s * (2.0 / n);
 }
 
-// Node weights of the intervals above the leaves: per layer and top interval, one warp
-// per 128-point interval takes its points, then the larger intervals take the nodes of
-// the four below (their weights reproduce every polynomial of the degree kept).
-// weights[layer][interval above the leaves][n].
+// Node weights of all intervals: per layer and top interval, one warp per leaf takes its
+// points, then the larger intervals take the nodes of the four below (whose weights
+// reproduce every polynomial of the degree kept).  weights[layer][interval][n].
+constexpr int UP_WARPS = 16;
 template <class R>
-__global__ void __launch_bounds__(512) up_kernel(const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N, int layer0,
-                                                 const double* __restrict__ g_sigma, double lam_scale,
-                                                 R* __restrict__ weights)
+__global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant__ Tree tr,
+                                                           const double* __restrict__ nu, int64_t N, int layer0,
+                                                           const double* __restrict__ g_sigma, double lam_scale,
+                                                           R* __restrict__ weights)
 {
-    constexpr int n = Far<R>::n;
-    __shared__ double M[16][n], w[2][16][n];
-    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
+    __shared__ double M[UP_WARPS][n], w[2][TOP][n];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int nloc = blockIdx.y, top = blockIdx.x;
     const double* g = g_sigma + (size_t)(layer0 + nloc) * N;
-    for (int k = 1; k < LEVELS; ++k) {
+    for (int k = 0; k < LEVELS; ++k) {
         const int many = 1 << (2 * (LEVELS - 1 - k));
-        const int i = top * many + q;
-        const bool mine = q < many && i < tr.cnt[k];
-        if (mine) {
+        for (int q = row; q < many; q += UP_WARPS) {
+            const int i = top * many + q;
+            if (i >= tr.cnt[k]) break;
             const double2 sp = tr.geo[tr.off[k] + i];
             double s[n];
 #pragma unroll
             for (int m = 0; m < n; ++m) s[m] = 0.0;
-            if (k == 1) {
-#pragma unroll 1
-                for (int r = 0; r < 4; ++r) {
-                    const int64_t j = (int64_t)i * (4 * LEAF) + r * LEAF + lane;
-                    if (j < N) add_moments<n>(g[j] * lam_scale, in_span(nu[j], sp), s);
-                }
+            if (k == 0) {
+                const int64_t j = (int64_t)i * LEAF + lane;
+                if (j < N) add_moments<n>(g[j] * lam_scale, in_span(nu[j], sp), s);
             } else {
 #pragma unroll 1
                 for (int r = lane; r < 4 * n; r += 32) {
                     const int ch = 4 * i + r / n, m = r % n; // child interval and its node
                     if (ch >= tr.cnt[k - 1]) break;
                     const double2 gc = tr.geo[tr.off[k - 1] + ch];
-                    add_moments<n>(w[k & 1][ch - top * 4 * many][m], in_span(fma(gc.y, cheb<n>(1, m), gc.x), sp), s);
+                    add_moments<n>(w[(k - 1) & 1][4 * q + r / n][m], in_span(fma(gc.y, cheb<n>(1, m), gc.x), sp), s);
                 }
             }
+            __syncwarp();
             int idx;
             const double v = warp_reduce_scatter<n>(s, idx);
-            if (idx >= 0) M[q][idx] = v;
+            if (idx >= 0) M[row][idx] = v;
             __syncwarp();
             if (lane < n) {
-                const double x = node_weight<n>(M[q], lane);
-                w[(k + 1) & 1][q][lane] = x;
-                weights[((size_t)nloc * (tr.total - tr.cnt[0]) + (tr.off[k] - tr.cnt[0]) + i) * n + lane] = (R)x;
+                const double x = node_weight<n>(M[row], lane);
+                w[k & 1][q][lane] = x;
+                weights[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = (R)x;
             }
+            __syncwarp();
         }
         __syncthreads();
     }
@@ -1091,12 +1095,7 @@ __device__ __forceinline__ void store16(float4* dst, const float* v, int n)
 // Near-line tiles of a leaf's warp: 32 lines staged for its 32 points, offsets to the
 // leaf's middle as hi + lo floats (their sum keeps the relative accuracy of a small
 // distance in a wide leaf).
-template <int n>
-struct LeafScratch {
-    double v[n], c[2][n]; // node sums or moments; coefficients
-};
 struct NearTile {
-    LeafScratch<10> fs;
     float4 nb[32]; // middle of the leaf - centre (hi, lo), the part of c that r2.x misses, 1/a
     float4 r2[32]; // c, a, Av, Kc
     int2 jr[32];
@@ -1104,8 +1103,6 @@ struct NearTile {
     float sd[32][SER_TAB]; // series table (|z| < 6, lines with a < 6)
 };
 struct NearAdjTile {
-    LeafScratch<10> fs;
-    float lam[10];
     float4 nb[32];
     float4 r2[32];
     int2 jr[32];
@@ -1114,8 +1111,6 @@ struct NearAdjTile {
     float sd[32][SER_TAB];
 };
 struct NearTile64 {
-    LeafScratch<18> fs;
-    double lam[18];
     double cen[32];
     double4_32a r2[32];
     double aS[32], nn[32];
@@ -1128,15 +1123,14 @@ constexpr float NEAR_POLY_Z2 = 36.0f;
 
 __device__ __forceinline__ bool in_range(int j, int2 r) { return j >= r.x && j <= r.y; }
 
-// A leaf: its points, its near lines as up to three ranges (the middle one inside every
-// line's cut, the outer ones masked per point) and its far set.
+// A leaf: its points and its near lines as up to three ranges (the middle one inside
+// every line's cut, the outer ones masked per point).
 template <class R>
 struct Leaf {
     int64_t jb, jl;
     int lane, i;
     bool live;
     int s[3], e[3];
-    FarSet fs;
     double2 g;
 
     __device__ bool init(const Tree& tr, const double* nu_hat, int64_t nl, const double* nu, int64_t N, double W,
@@ -1150,7 +1144,7 @@ struct Leaf {
         live = jb + lane <= jl;
         if (tr.on) {
             g = tr.geo[i];
-            fs = far_set(tr, 0, i, nloc);
+            const FarSet fs = far_set(tr, 0, i, nloc);
             const int2 w = tr.win[i];
             s[0] = w.x;
             e[0] = fs.a;
@@ -1174,64 +1168,28 @@ struct Leaf {
     }
 };
 
-// The far lines' part of sigma at a leaf's point: the leaf's own far lines through its
-// nodes plus the polynomial of the interval above.
-template <class R, class Tile>
-__device__ __forceinline__ double leaf_far(Tile& tl, const Leaf<R>& lf, const Lines<R>& ln, const Tree& tr,
-                                           const double* nu, double nuj, float cmin, int nloc, const double* coef)
+// The far lines' part of sigma at a leaf's point.  FP32: the constant term, which
+// dominates, in FP64, the rest in FP32.
+template <class R>
+__device__ __forceinline__ double leaf_far(const Leaf<R>& lf, const Tree& tr, double nuj, int nloc, const double* coef)
 {
     constexpr int n = Far<R>::n;
-    double v[n];
+    const double* cg = coef + ((size_t)nloc * tr.cnt[0] + lf.i) * n;
+    R c[n];
 #pragma unroll
-    for (int m = 0; m < n; ++m) v[m] = 0.0;
-    const FarList fl(lf.fs);
-    far_sum(ln, fl, 0, fl.total, Span(lf.g, nu[0]), cmin, v);
-    int idx;
-    const double s = warp_reduce_scatter<n>(v, idx);
-    if (idx >= 0) tl.fs.v[idx] = s;
-    __syncwarp();
-    if (lf.lane < n) {
-        tl.fs.c[0][lf.lane] = cheb_coeff<n>(tl.fs.v, lf.lane);
-        tl.fs.c[1][lf.lane] = coef[((size_t)nloc * tr.cnt[1] + (lf.i >> 2)) * n + lf.lane];
-    }
-    __syncwarp();
-    const double x0 = in_span(nuj, lf.g), x1 = in_span(nuj, tr.geo[tr.off[1] + (lf.i >> 2)]);
+    for (int k = 0; k < n; ++k) c[k] = (R)cg[k];
+    const R x = (R)in_span(nuj, lf.g);
     if constexpr (std::is_same<R, double>::value) {
-        return clenshaw<n, double>(tl.fs.c[0], x0) + clenshaw<n, double>(tl.fs.c[1], x1);
+        return clenshaw<n, double>(c, x);
     } else {
-        // the constant terms, which dominate, in FP64; the rest in FP32
-        float c0[n], c1[n];
-#pragma unroll
-        for (int k = 1; k < n; ++k) {
-            c0[k] = (float)tl.fs.c[0][k];
-            c1[k] = (float)tl.fs.c[1][k];
-        }
-        c0[0] = c1[0] = 0.0f;
-        return (tl.fs.c[0][0] + tl.fs.c[1][0]) +
-               (double)(clenshaw<n, float>(c0, (float)x0) + clenshaw<n, float>(c1, (float)x1));
+        c[0] = 0.0f;
+        return cg[0] + (double)clenshaw<n, float>(c, x);
     }
-}
-
-// Node weights of the leaf's own far lines.
-template <class R, class Tile>
-__device__ __forceinline__ void leaf_weights(Tile& tl, const Leaf<R>& lf, double lam, double nuj)
-{
-    constexpr int n = Far<R>::n;
-    double s[n];
-#pragma unroll
-    for (int m = 0; m < n; ++m) s[m] = 0.0;
-    add_moments<n>(lam, in_span(nuj, lf.g), s);
-    int idx;
-    const double v = warp_reduce_scatter<n>(s, idx);
-    if (idx >= 0) tl.fs.v[idx] = v;
-    __syncwarp();
-    if (lf.lane < n) tl.lam[lf.lane] = (R)node_weight<n>(tl.fs.v, lf.lane);
-    __syncwarp();
 }
 
 // sigma of one leaf: FP32
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
-    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const float* __restrict__ agg, const double* __restrict__ nu, int64_t N,
+    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ coef, double unscale, float* __restrict__ sigma)
 {
     __shared__ NearTile tiles[LeafWarps<float>::v];
@@ -1243,8 +1201,6 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
-    double far = 0.0;
-    if (tr.on) far = leaf_far<float>(tl, lf, ln, tr, nu, nuj, agg[4 * layer], nloc, coef);
     const double oj = nuj - lf.g.x;
     const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.y;
     float shi = 0.0f, slo = 0.0f;
@@ -1334,12 +1290,13 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
             two_sum(shi, slo, acc); // the chunk's FP32 partial into the compensated sum
         }
     }
+    const double far = tr.on ? leaf_far<float>(lf, tr, nuj, nloc, coef) : 0.0;
     if (lf.live) sigma[(size_t)layer * N + j] = (float)((far + ((double)shi + (double)slo)) * unscale);
 }
 
 // sigma of one leaf: FP64
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
-    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const float* __restrict__ agg, const double* __restrict__ nu, int64_t N,
+    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ coef, double unscale, double* __restrict__ sigma)
 {
     __shared__ NearTile64 tiles[LeafWarps<double>::v];
@@ -1374,8 +1331,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
             }
         }
     }
-    __syncwarp();
-    if (tr.on) acc += leaf_far<double>(tl, lf, ln, tr, nu, nuj, agg[4 * layer], nloc, coef);
+    if (tr.on) acc += leaf_far<double>(lf, tr, nuj, nloc, coef);
     if (lf.live) sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
@@ -1405,7 +1361,7 @@ __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
 }
 
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
-    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const float* __restrict__ agg, const double* __restrict__ nu, int64_t N,
+    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
     double* __restrict__ part)
 {
@@ -1421,11 +1377,6 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
         const double nuj = nu[j];
         const double lamd = lf.live ? g_sigma[(size_t)layer * N + j] * lam_scale : 0.0;
         const float hT = (float)(0.5 / T[layer]);
-        if (tr.on) {
-            leaf_weights<float>(tl, lf, lamd, nuj);
-            const FarList fl(lf.fs);
-            far_adjoint_sum(ln, fl, 0, fl.total, Span(lf.g, nu[0]), agg[4 * layer], tl.lam, hT, sT, sB);
-        }
         const float lam = (float)lamd;
         const double oj = nuj - lf.g.x;
         const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.y;
@@ -1557,7 +1508,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
 }
 
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
-    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const float* __restrict__ agg, const double* __restrict__ nu, int64_t N,
+    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
     double* __restrict__ part)
 {
@@ -1598,12 +1549,6 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
                     }
                 }
             }
-        }
-        __syncwarp();
-        if (tr.on) {
-            leaf_weights<double>(tl, lf, lam, nuj);
-            const FarList fl(lf.fs);
-            far_adjoint_sum(ln, fl, 0, fl.total, Span(lf.g, nu[0]), agg[4 * layer], tl.lam, hT, sT, sB);
         }
     }
     block_pair<LeafWarps<double>::v>(sT, sB, part + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
@@ -1676,6 +1621,7 @@ struct XsPlan {
     Tree tree; // counts and offsets; pointers set at run time
     FarWork fw;
     int far_blocks;
+    size_t rows; // node-sum rows of all levels and parts
     size_t off_jr, off_nuf, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq, off_fwd,
         off_coef, off_wts, off_slots, off_leaf, off_gbl, total;
 };
@@ -1690,7 +1636,7 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
     int block = 0;
     size_t row = 0;
     p->fw.slots = 0;
-    for (int k = LEVELS - 1; k >= 1; --k) {
+    for (int k = LEVELS - 1; k >= 0; --k) {
         const double share = std::min(1.0, 16.0 * (double)(LEAF << (2 * k)) / (double)N);
         const int64_t est = (k == LEVELS - 1) ? nl : (int64_t)(share * (double)nl);
         const int64_t want = (warps + (int64_t)Lc * p->tree.cnt[k] - 1) / ((int64_t)Lc * p->tree.cnt[k]);
@@ -1703,11 +1649,8 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
         row += (size_t)parts * Lc * p->tree.cnt[k];
         p->fw.slots += parts * p->tree.cnt[k];
     }
-    p->fw.parts[0] = 0;
-    p->fw.block0[0] = block;
-    p->fw.out0[0] = row;
-    p->fw.slot0[0] = p->fw.slots;
     p->far_blocks = block;
+    p->rows = row;
 }
 
 XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
@@ -1752,13 +1695,13 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     // the forward's node sums and polynomials; the adjoint's weights and partials reuse the space
     const size_t base = off;
     if (tree) {
-        p.off_fwd = take(sizeof(double) * n * p.fw.out0[0]);
-        p.off_coef = take(sizeof(double) * n * (size_t)Lc * p.tree.cnt[1]);
+        p.off_fwd = take(sizeof(double) * n * p.rows);
+        p.off_coef = take(sizeof(double) * n * (size_t)Lc * p.tree.cnt[0]);
     }
     const size_t fwd_end = off;
     off = base;
     if (tree) {
-        p.off_wts = take(rs * n * (size_t)Lc * (p.tree.total - p.tree.cnt[0]));
+        p.off_wts = take(rs * n * (size_t)Lc * p.tree.total);
         p.off_slots = take(sizeof(double) * 2 * (size_t)L * p.fw.slots);
     }
     p.off_leaf = take(sizeof(double) * 2 * (size_t)L * p.leaf_blocks);
@@ -1877,27 +1820,28 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
         if (!adjoint) {
             if (tr.on) {
                 far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, sums);
-                down_kernel<R><<<dim3(tops, (unsigned)lc), 16 * Far<R>::n, 0, st>>>(tr, p.fw, lc, sums, coef);
+                down_kernel<R><<<dim3(tops, (unsigned)lc), DOWN_ROWS * Far<R>::n, 0, st>>>(tr, p.fw, lc,
+                                                                                       sums, coef);
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, agg, nu, N, W, l0, coef, unscale,
+                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
                                                             (float*)sigma);
             else
-                leaf_kernel_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, agg, nu, N, W, l0, coef, unscale,
+                leaf_kernel_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
                                                             (double*)sigma);
         } else {
             if (tr.on) {
-                up_kernel<R><<<dim3(tops, (unsigned)lc), 512, 0, st>>>(tr, nu, N, l0, g_sigma, unscale, wts);
+                up_kernel<R><<<dim3(tops, (unsigned)lc), 32 * UP_WARPS, 0, st>>>(tr, nu, N, l0, g_sigma, unscale, wts);
                 far_adjoint_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, T, wts,
                                                                         slots);
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, agg, nu, N, W, l0, T, g_sigma, unscale,
+                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
                                                              leaf);
             else
-                leaf_adjoint_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, agg, nu, N, W, l0, T, g_sigma, unscale,
+                leaf_adjoint_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
                                                              leaf);
         }
         prof_end(adjoint ? 1 : 0, st);
