@@ -42,6 +42,7 @@ constexpr double SQRT2 = 1.41421356237309504880;
 
 // Scale applied to line strengths in the FP32 path so that partial sums of the
 // cross-section (1e-35 .. 1e-12 cm^2) sit well inside the normal float range.
+constexpr int MIXED_SCALE_LOG2 = 80;
 constexpr double MIXED_SCALE = 1208925819614629174706176.0; // 2^80
 constexpr double MIXED_UNSCALE = 8.27180612553027674871e-25; // 2^-80
 

@@ -123,7 +123,8 @@ __device__ __forceinline__ int first_line(const double* nu_hat, int64_t nl, doub
 // relative to the first grid point as float pairs, the intervals' line ranges (four
 // each) and geometry, and the start values of the per-layer minima.
 __global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, const double* __restrict__ nu, int64_t N,
-                             double W, int2* __restrict__ jr, float2* __restrict__ nuf, float* __restrict__ agg,
+                             double W, int2* __restrict__ jr, float2* __restrict__ nuf,
+                             double* __restrict__ inv_nu, float* __restrict__ agg,
                              int n_agg, const __grid_constant__ Tree tr, double2* __restrict__ geo, int2* __restrict__ cov,
                              int2* __restrict__ win)
 {
@@ -133,6 +134,7 @@ __global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, cons
         const int upper = (int)(t & 1);
         const double c = nu_hat[l];
         ((int*)jr)[t] = cut_index(nu, N, c, W, upper);
+        if (!upper) inv_nu[l] = 1.0 / c;
         if (nuf && upper) {
             const double o = c - nu[0];
             const float h = (float)o;
@@ -214,47 +216,127 @@ __device__ __forceinline__ double series_K(double a)
     return erfcx(a) - 2.0 * a * h / PI * s1;
 }
 
+// Layer constants of the line parameters.
+struct LayerConst {
+    double kE, kq, kc, kg, k2E, kqT; // exponent slopes, c nu_hat, pressure factor, dlnS slopes
+    double lnTr, T;
+};
+
+__device__ __forceinline__ LayerConst layer_const(double Tn, double Pn, double mass, double qexp, double sb)
+{
+    LayerConst k;
+    const double lnTr = log(Tn / Tref), iT = 1.0 / Tn;
+    k.kE = c2 * (iT - 1.0 / Tref);
+    k.kq = qexp * lnTr;
+    k.kc = cL / (SQRT2 * sqrt(kB * Tn / (mass * amu)));
+    k.kg = sb * (Pn / bar_per_atm);
+    k.k2E = c2 * iT * iT;
+    k.kqT = qexp * iT;
+    k.lnTr = lnTr;
+    k.T = Tn;
+    return k;
+}
+
+// 2^(i/64) as hi + lo floats
+struct Exp2Table {
+    float hi[64], lo[64];
+};
+constexpr double LN2 = 0.69314718055994530942;
+constexpr Exp2Table make_exp2_table()
+{
+    Exp2Table t{};
+    for (int i = 0; i < 64; ++i) {
+        const double x = i * LN2 / 64;
+        double s = 1.0;
+        for (int k = 20; k >= 1; --k) s = 1.0 + s * x / k;
+        t.hi[i] = (float)s;
+        t.lo[i] = (float)(s - (double)t.hi[i]);
+    }
+    return t;
+}
+__device__ const Exp2Table EXP2 = make_exp2_table();
+
+// e^v = 2^e (hi + lo), 1 <= hi < 2, to about 1e-10, table-driven (Tang 1989): the argument
+// is reduced in FP64 (three operations), the rest is FP32.
+__device__ __forceinline__ void exp_pair(double v, const float* tab, int* e, float* hi, float* lo)
+{
+    const int top = __double2hiint(v) & 0x7fffffff;
+    if (top >= 0x40900000 && top <= 0x7ff00000 && v == v) v = v < 0.0 ? -1000.0 : 1000.0; // beyond FP32 either way
+    const double magic = 6755399441055744.0; // 1.5 2^52: rounds to an integer
+    const double t = fma(v, 64.0 / LN2, magic);
+    const int k = __double2loint(t);
+    const float r = (float)fma(t - magic, -LN2 / 64, v);
+    const float h = tab[k & 63];
+    *e = k >> 6;
+    *hi = h;
+    *lo = fmaf(h, fmaf(r * r, fmaf(r, 1.0f / 6.0f, 0.5f), r), tab[64 + (k & 63)]);
+}
+
 // Per (layer, line), rounded once to R:
 //   rec1 = {G = gamma^2, Al = s gamma/pi, F1 = 1.5 B Al, F2 = -2 G B Al}   (B = 2 beta^2)
 //   rec2 = {c = 1/(sqrt2 beta), a = gamma c, Av = s c / sqrt(pi), Kc = K(a)}
 //   clo  = c - (R)c,  rec3 = {dlnS/dT, -n/T} (adjoint only)
 // s = S(T) * scale.  The Boltzmann exponent of S (Eq. Slog) and c are formed in
-// FP64 in both paths; in the FP32 path the factors that only need ~1e-7
-// (stimulated emission, the width's temperature power, K(a)) use FP32.
-// Per layer: agg[4n .. 4n+2] = min c, min a, min gamma.
+// FP64 in both paths; in the FP32 path the strength is carried as hi + lo floats and
+// the factors that only need ~1e-7 (stimulated emission, the width's temperature power,
+// K(a)) use FP32.  Per layer: agg[4n .. 4n+2] = min c, min a, min gamma.
+//
+// Bound by FP64 operations (2 lanes a clock and SM): what depends on the layer alone is
+// formed once a block, 1/nu_hat once a call, and the exponential and the products of the
+// FP32 path run in FP32: about 20 FP64 operations and conversions a line instead of about
+// 200 (220,000 lines x 100 layers: 6.9 ms before).
 template <class R>
-__global__ void line_params_kernel(const double* __restrict__ nu_hat, const double* __restrict__ ln_S0,
-                                   const double* __restrict__ elower, const double* __restrict__ gamma_ref,
-                                   const double* __restrict__ n_temp, int64_t nl, double mass, double qexp,
-                                   const double* __restrict__ T, const double* __restrict__ P_bar, int layer0,
-                                   double sb, double scale, typename vec4<R>::type* __restrict__ rec1,
-                                   typename vec4<R>::type* __restrict__ rec2, R* __restrict__ clo,
-                                   R* __restrict__ rec3, float* __restrict__ agg)
+__global__ void __launch_bounds__(256) line_params_kernel(
+    const double* __restrict__ nu_hat, const double* __restrict__ inv_nu, const double* __restrict__ ln_S0,
+    const double* __restrict__ elower, const double* __restrict__ gamma_ref, const double* __restrict__ n_temp,
+    int64_t nl, double mass, double qexp, const double* __restrict__ T, const double* __restrict__ P_bar, int layer0,
+    double sb, typename vec4<R>::type* __restrict__ rec1, typename vec4<R>::type* __restrict__ rec2,
+    R* __restrict__ clo, R* __restrict__ rec3, float* __restrict__ agg)
 {
-    int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int n = blockIdx.y;
+    constexpr bool FAST = std::is_same<R, float>::value;
+    __shared__ LayerConst lc;
+    __shared__ float tab[128];
+    const int n = blockIdx.y;
+    if (threadIdx.x == 0) lc = layer_const(T[layer0 + n], P_bar[layer0 + n], mass, qexp, sb);
+    if (FAST && threadIdx.x >= 128) {
+        const int i = threadIdx.x - 128;
+        tab[i] = i < 64 ? EXP2.hi[i] : EXP2.lo[i - 64];
+    }
+    __syncthreads();
+    const LayerConst k = lc;
+    const float lnTr = (float)k.lnTr, Tf = (float)k.T;
     float cmin = __int_as_float(0x7f800000), amin = cmin, gmin = cmin;
-    if (l < nl) {
-        const double Tn = T[layer0 + n], Pn = P_bar[layer0 + n];
-        const double nuh = nu_hat[l];
-        const double lnTr = log(Tn / Tref);
-        const double boltz = exp(ln_S0[l] - c2 * elower[l] * (1.0 / Tn - 1.0 / Tref) - qexp * lnTr);
-        const double beta = sqrt(kB * Tn / (mass * amu)) * nuh / cL;
-        const double c = 1.0 / (SQRT2 * beta);
-        R stim, gam;
-        if (std::is_same<R, float>::value) {
-            const float u = (float)(c2 * nuh);
-            stim = (R)(expm1f(-u / (float)Tn) / expm1f(-u / (float)Tref));
-            gam = (R)((float)(sb * gamma_ref[l] * (Pn / bar_per_atm)) * expf(-(float)n_temp[l] * (float)lnTr));
-        } else {
-            stim = (R)(expm1(-c2 * nuh / Tn) / expm1(-c2 * nuh / Tref));
-            gam = (R)(sb * gamma_ref[l] * exp(-n_temp[l] * lnTr) * (Pn / bar_per_atm));
-        }
-        const double s = boltz * scale * (double)stim;
+    for (int64_t l = (int64_t)blockIdx.x * 256 + threadIdx.x; l < nl; l += (int64_t)gridDim.x * 256) {
+        const double nuh = nu_hat[l], E = elower[l];
+        const double v = fma(-E, k.kE, ln_S0[l]) - k.kq;
+        const double c = k.kc * inv_nu[l];
         const R cr = (R)c;
+        R gam, Al, Av;
+        float u = 0.0f;
+        if constexpr (FAST) {
+            const float cu = (float)(c2 * nuh);
+            u = cu / Tf;
+            const float stim = expm1f(-u) / expm1f(-cu / (float)Tref);
+            gam = (float)(k.kg * gamma_ref[l]) * expf(-(float)n_temp[l] * lnTr);
+            int e;
+            float hi, lo;
+            exp_pair(v, tab, &e, &hi, &lo);
+            // s = 2^e (hi + lo) stim 2^80, products in FP32 with the low part carried
+            const float s = hi * stim, sl = fmaf(hi, stim, -s) + lo * stim;
+            const float g = gam * (float)(1.0 / PI), ci = cr * (float)INV_SQRTPI;
+            constexpr float gl0 = (float)(1.0 / PI - (double)(float)(1.0 / PI));
+            constexpr float cl0 = (float)(INV_SQRTPI - (double)(float)INV_SQRTPI);
+            const float gl = fmaf(gam, (float)(1.0 / PI), -g) + gam * gl0;
+            const float cl = fmaf(cr, (float)INV_SQRTPI, -ci) + cr * cl0;
+            Al = ldexpf(fmaf(s, g, fmaf(s, gl, sl * g)), e + MIXED_SCALE_LOG2);
+            Av = ldexpf(fmaf(s, ci, fmaf(s, cl, sl * ci)), e + MIXED_SCALE_LOG2);
+        } else {
+            const double s = exp(v) * (expm1(-c2 * nuh / k.T) / expm1(-c2 * nuh / Tref));
+            gam = k.kg * gamma_ref[l] * exp(-n_temp[l] * k.lnTr);
+            Al = s * gam / PI;
+            Av = s * c * INV_SQRTPI;
+        }
         const R a = gam * cr;
-        const R Al = (R)(s * (double)gam / PI);
-        const R Av = (R)(s * c * INV_SQRTPI);
         const R B = R(1) / (cr * cr);
         const R G = gam * gam;
         const R Kc = (a * a < (R)Tier<R>::z2_series) ? series_K(a) : R(0);
@@ -270,19 +352,22 @@ __global__ void line_params_kernel(const double* __restrict__ nu_hat, const doub
         v2.w = Kc;
         rec1[idx] = v1;
         rec2[idx] = v2;
-        if (clo) clo[idx] = (R)(c - (double)cr); // the part of c the rounded value misses (FP32 path)
+        if (FAST) clo[idx] = (R)(c - (double)cr); // the part of c the rounded value misses
         if (rec3) {
-            const R Tr = (R)Tn;
-            const R u = (R)(c2 * nuh) / Tr;
-            const R dlnS = (R)(c2 * elower[l] / (Tn * Tn) - qexp / Tn) - (u / Tr) / (R)expm1((double)u);
-            rec3[2 * idx] = dlnS;
-            rec3[2 * idx + 1] = (R)(-n_temp[l]) / Tr;
+            if constexpr (FAST) {
+                const float aS = (float)fma(k.k2E, E, -k.kqT) - (u / Tf) / expm1f(u);
+                ((float2*)rec3)[idx] = make_float2(aS, -(float)n_temp[l] / Tf);
+            } else {
+                const double ud = c2 * nuh / k.T;
+                rec3[2 * idx] = fma(k.k2E, E, -k.kqT) - (ud / k.T) / expm1(ud);
+                rec3[2 * idx + 1] = -n_temp[l] / k.T;
+            }
         }
-        cmin = (float)cr * (1.0f - 1e-6f);
-        amin = (float)a * (1.0f - 1e-6f);
-        gmin = (float)gam * (1.0f - 1e-6f);
+        cmin = fminf(cmin, (float)cr * (1.0f - 1e-6f));
+        amin = fminf(amin, (float)a * (1.0f - 1e-6f));
+        gmin = fminf(gmin, (float)gam * (1.0f - 1e-6f));
     }
-    // block min then one atomic per block (positive floats order like their bits)
+    // warp min then one atomic per warp (positive floats order like their bits)
     for (int o = 16; o > 0; o >>= 1) {
         cmin = fminf(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
         amin = fminf(amin, __shfl_xor_sync(0xffffffffu, amin, o));
@@ -1622,7 +1707,7 @@ struct XsPlan {
     FarWork fw;
     int far_blocks;
     size_t rows; // node-sum rows of all levels and parts
-    size_t off_jr, off_nuf, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq, off_fwd,
+    size_t off_jr, off_nuf, off_inv, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq, off_fwd,
         off_coef, off_wts, off_slots, off_leaf, off_gbl, total;
 };
 
@@ -1672,6 +1757,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     p.leaf_blocks = (int)((N + per_block - 1) / per_block);
     p.off_jr = take(sizeof(int2) * n1);
     p.off_nuf = take(mixed ? sizeof(float2) * n1 : 0);
+    p.off_inv = take(sizeof(double) * n1);
     p.off_agg = take(sizeof(float) * 4 * (size_t)L);
     p.off_rec1 = take(4 * rs * n1 * Lc);
     p.off_rec2 = take(4 * rs * n1 * Lc);
@@ -1756,7 +1842,6 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
     const bool want_rec3 = adjoint || (flags & XS_RUN_KEEP_ADJ);
     using R4 = typename vec4<R>::type;
     const int64_t nl = ln->n;
-    const double scale = FAST ? MIXED_SCALE : 1.0;
     const double unscale = FAST ? MIXED_UNSCALE : 1.0;
     if (nl == 0) {
         if (adjoint) {
@@ -1770,6 +1855,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
     }
     int2* jr = (int2*)(ws + p.off_jr);
     float2* nuf = FAST ? (float2*)(ws + p.off_nuf) : nullptr;
+    double* inv_nu = (double*)(ws + p.off_inv);
     float* agg = (float*)(ws + p.off_agg);
     R4* rec1 = (R4*)(ws + p.off_rec1);
     R4* rec2 = (R4*)(ws + p.off_rec2);
@@ -1795,17 +1881,18 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
 
     if (!reuse) {
         setup_kernel<<<blocks_of(2 * nl + 4 * (int64_t)L + 4 * (int64_t)tr.total, 256), 256, 0, st>>>(
-            ln->nu_hat, nl, nu, N, W, jr, nuf, agg, 4 * L, tr, geo, cov, win);
+            ln->nu_hat, nl, nu, N, W, jr, nuf, inv_nu, agg, 4 * L, tr, geo, cov, win);
         count_launch();
     }
     for (int c = 0; c < p.nchunks; ++c) {
         const int l0 = c * p.Lc;
         const int lc = std::min(p.Lc, L - l0);
         if (!reuse) {
-            dim3 pg(blocks_of(nl, 256), (unsigned)lc);
-            line_params_kernel<R><<<pg, 256, 0, st>>>(ln->nu_hat, ln->ln_S0, ln->elower, ln->gamma_ref, ln->n_temp,
-                                                       nl, ln->mass_amu, ln->q_exponent, T, P, l0, sb, scale, rec1,
-                                                       rec2, clo, want_rec3 ? rec3 : nullptr, agg);
+            // four lines a thread where that leaves enough blocks: the layer's constants are formed per block
+            const dim3 pg(nl >= 65536 ? blocks_of(nl, 1024) : blocks_of(nl, 256), (unsigned)lc);
+            line_params_kernel<R><<<pg, 256, 0, st>>>(ln->nu_hat, inv_nu, ln->ln_S0, ln->elower, ln->gamma_ref,
+                                                      ln->n_temp, nl, ln->mass_amu, ln->q_exponent, T, P, l0, sb, rec1,
+                                                      rec2, clo, want_rec3 ? rec3 : nullptr, agg);
             count_launch();
             if (tr.on) {
                 near_range_kernel<R><<<dim3(blocks_of(2 * (int64_t)tr.total, 256), (unsigned)lc), 256, 0, st>>>(
