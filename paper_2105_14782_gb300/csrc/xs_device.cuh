@@ -313,9 +313,13 @@ __device__ __forceinline__ float exp2_fast(float x)
     return r;
 }
 
-// sin r for |r| <= pi/2 and, if want_c, cos r: Taylor series (next terms below 7e-10)
-__device__ __forceinline__ void sincos_half(float r, bool want_c, float* s, float* c)
+// sin v and, if want_c, cos v, both up to the sign (-1)^k of the multiple of pi taken out:
+// Taylor series on |r| <= pi/2 (next terms below 7e-10)
+__device__ __forceinline__ void sin_cos_mod_pi(float v, bool want_c, float* s, float* c)
 {
+    constexpr float MAGIC = 12582912.0f;
+    const float k = fmaf(v, (float)(1.0 / PI), MAGIC) - MAGIC;
+    const float r = fmaf(-k, (float)(PI - (double)(float)PI), fmaf(-k, (float)PI, v));
     const float t = r * r;
     float p = 1.0f / 6227020800.0f;
     p = fmaf(p, t, -1.0f / 39916800.0f);
@@ -344,57 +348,90 @@ __device__ __forceinline__ void sincos_half(float r, bool want_c, float* s, floa
 // Terms with |k| > 6 are below 1e-9 of the peak term.  The two sides go as packed pairs,
 // with the line's table d (series_table).  sin and cos of ax enter as sin^2 and sin cos
 // only, so ax is reduced modulo pi and its sign dropped.  inv_a = 1/a.  Issue-bound:
-// about 100 instructions a pair of line and point (150 for w) with its loop.
-template <bool WANT_WI>
-__device__ __forceinline__ void w_series_tab(float xh, float xl, float a, float inv_a, float Kc, const float* dt,
-                                             float* wr, float* wi)
+// about 100 instructions a pair of line and point with its loop.
+//
+// Derivatives (DERIV): w' = -2 z w + 2i/sqrt(pi) loses 2|z|^2 of its accuracy when it is
+// taken from w.  With 1/sqrt(pi) = (h/pi) sum_n E_n the sums cancel term by term instead:
+//   Re w' = -2 Re(z g) + (2 a h/pi) S1,   Im w' = -2 Im(z g) + (2h/pi)(e^{-x^2} + x S1 + S2),
+//   S_i = sum_{n != 0} E_n d_n (nh - x)^i,
+// g the part of w with e^{-x^2}; S1 and S2 come from the first and second derivatives of
+// the Horner polynomials.
+struct SeriesSums {
+    float s0, s1, s2;
+};
+
+template <bool DERIV>
+__device__ __forceinline__ SeriesSums series_sums(float xh, float xl, const float* dt)
 {
     const float h = Tier<float>::h;
     constexpr float L2E = 1.44269504f, MAGIC = 12582912.0f; // 1.5 2^23: rounds to an integer
-    const float x = xh;
-    const float tm = fmaf(x, 1.0f / h, MAGIC);
+    const float tm = fmaf(xh, 1.0f / h, MAGIC);
     const float n0f = tm - MAGIC;
     const int n0 = __float_as_int(tm) & 31;
-    if (!XS_CHECK(n0 <= SER_N0)) {
-        *wr = 0.0f;
-        *wi = 0.0f;
-        return;
-    }
-    const float n0h = n0f * h;
-    const float delta = (n0h - xh) - xl;
+    if (!XS_CHECK(n0 <= SER_N0)) return {0.0f, 0.0f, 0.0f};
+    const float delta = (n0f * h - xh) - xl;
     const float E0 = exp2_fast(-L2E * delta * delta);
     const float u = 2.0f * h * L2E * delta;
     const float2 f = make_float2(exp2_fast(-u), exp2_fast(u)); // e^{-2h delta}, e^{2h delta}
     const float* d0 = dt + (n0 + SER_OFF);
-    // sums over k of Q_k d_{n0 +- k} f^k by Horner, Q_k = e^{-(kh)^2}; the sums with a
-    // factor k, for Im w, are f times the derivative in f
     const float Q[SER_OFF + 1] = {1.0f, 0.612626433f, 0.140858427f, 0.0121551799f, 0.00039366915f, 4.78511947e-06f,
                                   2.18295906e-08f};
-    float2 s = __fmul2_rn(make_float2(d0[SER_OFF], d0[-SER_OFF]), make_float2(Q[SER_OFF], Q[SER_OFF]));
-    float2 ds = make_float2(0.0f, 0.0f);
+    // p = sum_k w_k f^k and, for the factors k and k^2, p' and p''/2
+    float2 p = __fmul2_rn(make_float2(d0[SER_OFF], d0[-SER_OFF]), make_float2(Q[SER_OFF], Q[SER_OFF]));
+    float2 p1 = make_float2(0.0f, 0.0f), p2 = p1;
 #pragma unroll
     for (int k = SER_OFF - 1; k >= 0; --k) {
-        if (WANT_WI) ds = __ffma2_rn(ds, f, s);
+        if (DERIV) {
+            p2 = __ffma2_rn(p2, f, p1);
+            p1 = __ffma2_rn(p1, f, p);
+        }
         // the centre term, k = 0, belongs to the first of the pair
         const float2 w = k ? __fmul2_rn(make_float2(d0[k], d0[-k]), make_float2(Q[k], Q[k])) : make_float2(d0[0], 0.0f);
-        s = __ffma2_rn(s, f, w);
+        p = __ffma2_rn(p, f, w);
     }
-    const float scs = E0 * (s.x + s.y);
-    const float sss = WANT_WI ? fmaf(n0h, scs, h * E0 * (f.x * ds.x - f.y * ds.y)) : 0.0f;
+    SeriesSums r;
+    const float s0 = p.x + p.y;
+    r.s0 = E0 * s0;
+    r.s1 = r.s2 = 0.0f;
+    if (DERIV) {
+        const float2 k1 = __fmul2_rn(p1, f);                                         // sum k w f^k
+        const float2 k2 = __ffma2_rn(__fmul2_rn(p2, f), make_float2(2.0f * f.x, 2.0f * f.y), k1); // sum k^2 w f^k
+        const float m1 = h * (k1.x - k1.y), m2 = h * h * (k2.x + k2.y); // sums of kh and (kh)^2, sides signed
+        r.s1 = E0 * fmaf(delta, s0, m1);
+        r.s2 = E0 * fmaf(delta, fmaf(delta, s0, 2.0f * m1), m2);
+    }
+    return r;
+}
+
+// Re w
+__device__ __forceinline__ float w_series_re(float xh, float xl, float a, float inv_a, float Kc, const float* dt)
+{
+    const SeriesSums q = series_sums<false>(xh, xl, dt);
     const float ex = exp_negsq(xh, xl);
-    const float ax = a * x;
-    const float km = fmaf(ax, (float)(1.0 / PI), MAGIC) - MAGIC;
-    const float rr = fmaf(-km, (float)(PI - (double)(float)PI), fmaf(-km, (float)PI, ax));
     float sax, cax;
-    sincos_half(rr, WANT_WI, &sax, &cax);
+    sin_cos_mod_pi(a * xh, false, &sax, &cax);
     const float c2v = fmaf(-2.0f * sax, sax, 1.0f); // cos 2ax
-    const float hpi = h * (float)(1.0 / PI);
-    *wr = ex * fmaf(2.0f * hpi * inv_a * sax, sax, Kc * c2v) + a * hpi * scs;
-    if (WANT_WI) {
-        const float s2 = 2.0f * sax * cax; // sin 2ax
-        const float s2_a = a > 0.0f ? s2 * inv_a : 2.0f * x;
-        *wi = ex * (-Kc * s2 + hpi * s2_a) + hpi * sss;
-    }
+    const float hpi = Tier<float>::h * (float)(1.0 / PI);
+    return ex * fmaf(2.0f * hpi * inv_a * sax, sax, Kc * c2v) + a * hpi * q.s0;
+}
+
+// Re w, Re w' and Im w'
+__device__ __forceinline__ void w_series_deriv(float xh, float xl, float a, float inv_a, float Kc, const float* dt,
+                                               float* wr, float* dr, float* di)
+{
+    const SeriesSums q = series_sums<true>(xh, xl, dt);
+    const float x = xh, ex = exp_negsq(xh, xl);
+    float sax, cax;
+    sin_cos_mod_pi(a * x, true, &sax, &cax);
+    const float c2v = fmaf(-2.0f * sax, sax, 1.0f), s2 = 2.0f * sax * cax;
+    const float hpi = Tier<float>::h * (float)(1.0 / PI);
+    const float s2_a = a > 0.0f ? s2 * inv_a : 2.0f * x;
+    const float gr = ex * fmaf(2.0f * hpi * inv_a * sax, sax, Kc * c2v);
+    const float gi = ex * fmaf(hpi, s2_a, -Kc * s2);
+    const float ah = a * hpi;
+    *wr = fmaf(ah, q.s0, gr);
+    *dr = 2.0f * fmaf(ah, q.s1, a * gi - x * gr);
+    *di = 2.0f * fmaf(hpi, ex + fmaf(x, q.s1, q.s2), -fmaf(x, gi, a * gr));
 }
 
 template <class R>

@@ -81,9 +81,14 @@ constexpr NodeTable<n> make_nodes()
     return r;
 }
 
+// Middle, half-width and its reciprocal (0 in an interval of one point).
+struct Geo {
+    double mid, h, inv;
+};
+
 // Intervals of the grid, all levels, leaves first.
 struct Tree {
-    const double2* geo; // middle and half-width
+    const Geo* geo;
     const int2* cov;    // lines [x, y) that cover the interval with their cut
     const int2* win;    // lines [x, y) with an in-cut point in it (leaves only)
     const int2* pq;     // per layer: lines [x, y) too near for the far form
@@ -125,7 +130,7 @@ __device__ __forceinline__ int first_line(const double* nu_hat, int64_t nl, doub
 __global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, const double* __restrict__ nu, int64_t N,
                              double W, int2* __restrict__ jr, float2* __restrict__ nuf,
                              double* __restrict__ inv_nu, float* __restrict__ agg,
-                             int n_agg, const __grid_constant__ Tree tr, double2* __restrict__ geo, int2* __restrict__ cov,
+                             int n_agg, const __grid_constant__ Tree tr, Geo* __restrict__ geo, int2* __restrict__ cov,
                              int2* __restrict__ win)
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -156,7 +161,8 @@ __global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, cons
     const int64_t j1 = min64(N, j0 + (LEAF << (2 * k))) - 1;
     const double v0 = nu[j0], v1 = nu[j1];
     if (which == 0) {
-        geo[q] = make_double2(0.5 * (v0 + v1), 0.5 * (v1 - v0));
+        const double h = 0.5 * (v1 - v0);
+        geo[q] = {0.5 * (v0 + v1), h, h > 0.0 ? 1.0 / h : 0.0};
         cov[q].x = first_line(nu_hat, nl, v1, W, 1); // covers v1 from its lower side on
     } else if (which == 1) {
         cov[q].y = first_line(nu_hat, nl, v0, W, 0); // first that no longer reaches v0
@@ -219,7 +225,7 @@ __device__ __forceinline__ double series_K(double a)
 // Layer constants of the line parameters.
 struct LayerConst {
     double kE, kq, kc, kg, k2E, kqT; // exponent slopes, c nu_hat, pressure factor, dlnS slopes
-    double lnTr, T;
+    double lnTr, T, bk; // ln(T/296), T, beta cL/nu_hat
 };
 
 __device__ __forceinline__ LayerConst layer_const(double Tn, double Pn, double mass, double qexp, double sb)
@@ -228,7 +234,8 @@ __device__ __forceinline__ LayerConst layer_const(double Tn, double Pn, double m
     const double lnTr = log(Tn / Tref), iT = 1.0 / Tn;
     k.kE = c2 * (iT - 1.0 / Tref);
     k.kq = qexp * lnTr;
-    k.kc = cL / (SQRT2 * sqrt(kB * Tn / (mass * amu)));
+    k.bk = sqrt(kB * Tn / (mass * amu));
+    k.kc = cL / (SQRT2 * k.bk);
     k.kg = sb * (Pn / bar_per_atm);
     k.k2E = c2 * iT * iT;
     k.kqT = qexp * iT;
@@ -309,7 +316,7 @@ __global__ void __launch_bounds__(256) line_params_kernel(
     for (int64_t l = (int64_t)blockIdx.x * 256 + threadIdx.x; l < nl; l += (int64_t)gridDim.x * 256) {
         const double nuh = nu_hat[l], E = elower[l];
         const double v = fma(-E, k.kE, ln_S0[l]) - k.kq;
-        const double c = k.kc * inv_nu[l];
+        const double c = FAST ? k.kc * inv_nu[l] : 1.0 / (SQRT2 * (k.bk * nuh / cL));
         const R cr = (R)c;
         R gam, Al, Av;
         float u = 0.0f;
@@ -402,10 +409,10 @@ __global__ void near_range_kernel(const double* __restrict__ nu_hat, int64_t nl,
     if (t >= 2 * (int64_t)tr.total) return;
     const int q = (int)(t >> 1), n = blockIdx.y;
     const bool upper = t & 1;
-    const double2 g = tr.geo[q];
+    const Geo g = tr.geo[q];
     const float* ag = agg + 4 * (layer0 + n);
-    const double r = far_radius<R>(g.y, ag[0], ag[1], ag[2]);
-    const double v = upper ? g.x + r : g.x - r;
+    const double r = far_radius<R>(g.h, ag[0], ag[1], ag[2]);
+    const double v = upper ? g.mid + r : g.mid - r;
     int64_t lo = 0, hi = nl; // first line with centre >= v (upper) or > v
     while (lo < hi) {
         const int64_t m = (lo + hi) >> 1;
@@ -493,21 +500,41 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float v)
     hi = s;
 }
 
+// A sum carried as hi + lo floats, and its addition (TwoSum): eight FP32 operations where
+// an FP64 addition takes the FP64 pipe for 16 clocks.
+struct Pair {
+    float hi, lo;
+};
+__device__ __forceinline__ Pair add(const Pair& a, const Pair& b)
+{
+    const float s = a.hi + b.hi, bb = s - a.hi;
+    return {s, (a.lo + b.lo) + ((a.hi - (s - bb)) + (b.hi - bb))};
+}
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ Pair shfl_xor(const Pair& v, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double to_double(const Pair& v) { return (double)v.hi + (double)v.lo; }
+
 // Sums v[0 .. n-1] over the warp, each sum ending in one lane: halving exchanges, so
 // about n adds a lane instead of 5 n.  Returns the lane's sum; idx its index or -1.
-template <int n, int o>
-__device__ __forceinline__ double reduce_scatter_step(double (&v)[n], int base, int cnt, int& idx)
+template <int n, int o, class V>
+__device__ __forceinline__ V reduce_scatter_step(V (&v)[n], int base, int cnt, int& idx)
 {
     constexpr int h = (n + 1) / 2;
     const bool up = (threadIdx.x & o) != 0;
-    double w[h];
+    V w[h];
     if constexpr (n == 1) {
-        w[0] = v[0] + __shfl_xor_sync(0xffffffffu, v[0], o);
+        w[0] = add(v[0], shfl_xor(v[0], o));
     } else {
 #pragma unroll
         for (int i = 0; i < h; ++i) {
-            const double a = v[i], b = (i + h < n) ? v[i + h] : 0.0;
-            w[i] = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, o);
+            const V a = v[i], b = (i + h < n) ? v[i + h] : V{};
+            w[i] = add(up ? b : a, shfl_xor(up ? a : b, o));
         }
         base += up ? h : 0;
         cnt = up ? max(cnt - h, 0) : min(cnt, h);
@@ -516,13 +543,19 @@ __device__ __forceinline__ double reduce_scatter_step(double (&v)[n], int base, 
         idx = cnt > 0 ? base : -1;
         return w[0];
     } else {
-        return reduce_scatter_step<h, o / 2>(w, base, cnt, idx);
+        return reduce_scatter_step<h, o / 2, V>(w, base, cnt, idx);
     }
 }
-template <int n>
-__device__ __forceinline__ double warp_reduce_scatter(double (&v)[n], int& idx)
+template <int n, class V>
+__device__ __forceinline__ V warp_reduce_scatter(V (&v)[n], int& idx)
 {
-    return reduce_scatter_step<n, 16>(v, 0, n, idx);
+    return reduce_scatter_step<n, 16, V>(v, 0, n, idx);
+}
+template <class V>
+__device__ __forceinline__ V warp_sum(V v)
+{
+    for (int o = 16; o > 0; o >>= 1) v = add(v, shfl_xor(v, o));
+    return v;
 }
 
 // ------------------------------------------------------------------ far lines, FP32
@@ -572,7 +605,7 @@ struct Lines {
 struct Span {
     double mid, h;
     float rh, rl; // mid - nu[0] as hi + lo floats
-    __device__ __forceinline__ Span(double2 g, double nu0) : mid(g.x), h(g.y)
+    __device__ __forceinline__ Span(const Geo& g, double nu0) : mid(g.mid), h(g.h)
     {
         const double o = mid - nu0;
         rh = (float)o;
@@ -582,11 +615,11 @@ struct Span {
 
 constexpr int FAR_FOLD = 16; // lines of a lane between two foldings of its FP32 partial sums
 
-// out[m] += sum over the lines t0 .. t1 - 1 of a list (this warp's lanes take 32 at a
-// time) of Av H at node m.  Lanes hold lines, the nodes are in registers: a line is read
-// once for all nodes, with no staging.
-__device__ __forceinline__ void far_sum(const Lines<float>& ln, const FarList& fl, int t0, int t1, const Span& sp,
-                                        float cmin, double (&out)[Far<float>::n])
+// Sums over the lines t0 .. t1 - 1 of a list of Av H at the nodes: returns the sum at node
+// idx (-1: none in this lane).  Lanes hold lines, 32 at a time, the nodes are in registers:
+// a line is read once for all nodes, with no staging.
+__device__ __forceinline__ double far_sum(const Lines<float>& ln, const FarList& fl, int t0, int t1, const Span& sp,
+                                          float cmin, int& idx)
 {
     constexpr int H = Far<float>::n / 2;
     constexpr NodeTable<Far<float>::n> nt = make_nodes<Far<float>::n>();
@@ -673,12 +706,14 @@ __device__ __forceinline__ void far_sum(const Lines<float>& ln, const FarList& f
             }
         }
     }
+    Pair v[2 * H];
 #pragma unroll
     for (int p = 0; p < H; ++p) {
         two_sum2(hi[p], lo[p], acc[p]);
-        out[2 * p] += (double)hi[p].x + (double)lo[p].x;
-        out[2 * p + 1] += (double)hi[p].y + (double)lo[p].y;
+        v[2 * p] = {hi[p].x, lo[p].x};
+        v[2 * p + 1] = {hi[p].y, lo[p].y};
     }
+    return to_double(warp_reduce_scatter(v, idx));
 }
 
 // Adjoint: per evaluation
@@ -718,7 +753,7 @@ __device__ __forceinline__ void rho_moments(const float2 (&o2)[Far<float>::n / 2
     for (int k = 0; k < K; ++k) r[k] = s[k].x + s[k].y;
 }
 
-// (sT, sB) += sum over the lines of sum_m Lambda_m (f_T, f_b)(node m)
+// (sT, sB) = sum over the lines of sum_m Lambda_m (f_T, f_b)(node m), in every lane
 __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const FarList& fl, int t0, int t1,
                                                 const Span& sp, float cmin, const float* lam, float hT, double& sT,
                                                 double& sB)
@@ -820,29 +855,33 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
         two_sum(Th, Tl, aS * V0 + hT * Db + nn * Dg);
         two_sum(Bh, Bl, Dg);
     }
-    sT += (double)Th + (double)Tl;
-    sB += (double)Bh + (double)Bl;
+    sT = to_double(warp_sum(Pair{Th, Tl}));
+    sB = to_double(warp_sum(Pair{Bh, Bl}));
 }
 
 // ------------------------------------------------------------------ far lines, FP64
 
 // One line at the nodes, the double-precision tiers of xs_device.cuh.
-__device__ __forceinline__ void far_sum(const Lines<double>& ln, const FarList& fl, int t0, int t1, const Span& sp,
-                                        float, double (&out)[Far<double>::n])
+__device__ __forceinline__ double far_sum(const Lines<double>& ln, const FarList& fl, int t0, int t1, const Span& sp,
+                                          float, int& idx)
 {
     constexpr int n = Far<double>::n;
     const int lane = threadIdx.x & 31;
-    for (int t = t0; t < t1; t += 32) {
-        if (t + lane >= t1) break;
-        const int l = fl.line(t + lane);
+    double v[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) v[m] = 0.0;
+    for (int t = t0 + lane; t < t1; t += 32) {
+        const int l = fl.line(t);
         const double nb = sp.mid - ln.nu_hat[l];
         const double4_32a p2 = ln.r2[l];
 #pragma unroll
         for (int m = 0; m < n; ++m) {
             const double x = fabs(fma(sp.h, cheb<n>(1, m), nb)) * p2.x;
-            out[m] = fma(p2.z, voigt_H<double>(x, 0.0, p2.y, p2.w, nullptr), out[m]);
+            v[m] = fma(p2.z, voigt_H<double>(x, 0.0, p2.y, p2.w, nullptr), v[m]);
         }
     }
+    __syncwarp();
+    return warp_reduce_scatter(v, idx);
 }
 
 __device__ __forceinline__ void adjoint_terms(double x, const double4_32a& p2, double aS, double hT, double nn,
@@ -865,9 +904,9 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
 {
     constexpr int n = Far<double>::n;
     const int lane = threadIdx.x & 31;
-    for (int t = t0; t < t1; t += 32) {
-        if (t + lane >= t1) break;
-        const int l = fl.line(t + lane);
+    sT = sB = 0.0;
+    for (int t = t0 + lane; t < t1; t += 32) {
+        const int l = fl.line(t);
         const double nb = sp.mid - ln.nu_hat[l];
         const double4_32a p2 = ln.r2[l];
         const double aS = ln.r3[2 * (size_t)l], nn = ln.r3[2 * (size_t)l + 1];
@@ -879,6 +918,9 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
             sB = fma(lam[m], fb, sB);
         }
     }
+    __syncwarp();
+    sT = warp_sum(sT);
+    sB = warp_sum(sB);
 }
 
 // ------------------------------------------------------------------ far kernels
@@ -937,12 +979,8 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(Lines<R> lines,
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
     if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
-    double v[n];
-#pragma unroll
-    for (int m = 0; m < n; ++m) v[m] = 0.0;
-    far_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * (layer0 + nloc)], v);
     int idx;
-    const double s = warp_reduce_scatter<n>(v, idx);
+    const double s = far_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * (layer0 + nloc)], idx);
     const size_t row = fw.out0[k] + ((size_t)part * gridDim.y + nloc) * tr.cnt[k] + i;
     if (idx >= 0) sums[row * n + idx] = s;
 }
@@ -962,14 +1000,10 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
     if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
-    double sT = 0.0, sB = 0.0;
+    double sT, sB;
     far_adjoint_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * layer],
                     weights + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
                     (R)(0.5 / T[layer]), sT, sB);
-    for (int o = 16; o > 0; o >>= 1) {
-        sT += __shfl_xor_sync(0xffffffffu, sT, o);
-        sB += __shfl_xor_sync(0xffffffffu, sB, o);
-    }
     if ((threadIdx.x & 31) == 0) {
         const size_t o = (size_t)layer * fw.slots + fw.slot0[k] + (size_t)part * tr.cnt[k] + i;
         part_out[2 * o] = sT;
@@ -977,8 +1011,8 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(
     }
 }
 
-// x of a position in an interval, -1 .. 1 (0 in an interval of one point)
-__device__ __forceinline__ double in_span(double v, double2 g) { return g.y > 0.0 ? (v - g.x) / g.y : 0.0; }
+// x of a position in an interval, -1 .. 1
+__device__ __forceinline__ double in_span(double v, const Geo& g) { return (v - g.mid) * g.inv; }
 
 // coefficient k of the polynomial through the node values v
 template <int n>
@@ -1005,17 +1039,49 @@ __device__ __forceinline__ R clenshaw(const R* c, R x)
     return x * b1 + (c[0] - b2);
 }
 
+// A leaf's polynomial: n doubles, or in the FP32 path the constant term, which dominates,
+// in FP64 and the others in FP32, in half the space.
+template <class R>
+struct LeafPoly {
+    static constexpr int n = Far<R>::n, stride = n;
+    __device__ static void store(double* coef, size_t leaf, int k, double c) { coef[leaf * stride + k] = c; }
+    __device__ static double eval(const double* coef, size_t leaf, double x)
+    {
+        return clenshaw<n, double>(coef + leaf * stride, x);
+    }
+};
+template <>
+struct LeafPoly<float> {
+    static constexpr int n = Far<float>::n, stride = 1 + n / 2;
+    __device__ static void store(double* coef, size_t leaf, int k, double c)
+    {
+        double* p = coef + leaf * stride;
+        if (k == 0) p[0] = c;
+        else ((float*)(p + 1))[k] = (float)c;
+    }
+    __device__ static double eval(const double* coef, size_t leaf, double x)
+    {
+        const double* p = coef + leaf * stride;
+        float c[n];
+        c[0] = 0.0f;
+#pragma unroll
+        for (int k = 1; k < n; ++k) c[k] = ((const float*)(p + 1))[k];
+        return p[0] + (double)clenshaw<n, float>(c, (float)x);
+    }
+};
+
 // Polynomials of the leaves: per layer and top interval, the node sums of each level
 // plus the polynomial of the interval above.  coef[layer][leaf][n].
-constexpr int DOWN_ROWS = 16; // intervals of a level that a block takes at a time
+template <class R> struct DownRows { static constexpr int v = 64; }; // intervals of a level that a block takes at a time
+template <> struct DownRows<double> { static constexpr int v = 32; };
 template <class R>
-__global__ void __launch_bounds__(DOWN_ROWS * Far<R>::n) down_kernel(const __grid_constant__ Tree tr,
+__global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const __grid_constant__ Tree tr,
                                                                      const __grid_constant__ FarWork fw, int Lc,
                                                                      const double* __restrict__ sums,
                                                                      double* __restrict__ coef)
 {
-    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
-    __shared__ double v[DOWN_ROWS][n], c[2][TOP][n];
+    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1)), DOWN_ROWS = DownRows<R>::v;
+    __shared__ double v[DOWN_ROWS][n], c[2][TOP / 4][n];
     const int m = threadIdx.x % n, row = threadIdx.x / n;
     const int nloc = blockIdx.y, top = blockIdx.x;
     for (int k = LEVELS - 1; k >= 0; --k) {
@@ -1028,8 +1094,8 @@ __global__ void __launch_bounds__(DOWN_ROWS * Far<R>::n) down_kernel(const __gri
                 for (int p = 0; p < fw.parts[k]; ++p)
                     s += sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
                 if (k < LEVELS - 1) {
-                    const double2 g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
-                    s += clenshaw<n, double>(c[(k + 1) & 1][q >> 2], in_span(fma(g.y, cheb<n>(1, m), g.x), gp));
+                    const Geo g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
+                    s += clenshaw<n, double>(c[(k + 1) & 1][q >> 2], in_span(fma(g.h, cheb<n>(1, m), g.mid), gp));
                 }
                 v[row][m] = s;
             }
@@ -1039,7 +1105,7 @@ __global__ void __launch_bounds__(DOWN_ROWS * Far<R>::n) down_kernel(const __gri
                 if (k > 0)
                     c[k & 1][q][m] = ck;
                 else
-                    coef[((size_t)nloc * tr.cnt[0] + i) * n + m] = ck;
+                    LeafPoly<R>::store(coef, (size_t)nloc * tr.cnt[0] + i, m, ck);
             }
             __syncthreads();
         }
@@ -1047,16 +1113,16 @@ __global__ void __launch_bounds__(DOWN_ROWS * Far<R>::n) down_kernel(const __gri
 }
 
 // moments sum w T_k(x) of a weight at x, added to s
-template <int n>
-__device__ __forceinline__ void add_moments(double w, double x, double (&s)[n])
+template <int n, class R>
+__device__ __forceinline__ void add_moments(R w, R x, R (&s)[n])
 {
-    double a = w, b = w * x;
-    const double x2 = x + x;
+    R a = w, b = w * x;
+    const R x2 = x + x;
     s[0] += a;
     s[1] += b;
 #pragma unroll
     for (int k = 2; k < n; ++k) {
-        const double t = fma(x2, b, -a);
+        const R t = x2 * b - a;
         s[k] += t;
         a = b;
         b = t;
@@ -1064,18 +1130,20 @@ __device__ __forceinline__ void add_moments(double w, double x, double (&s)[n])
 }
 
 // node weight m from the moments M: sum_k (1 or 2)/n M_k T_k(t_m)
-template <int n>
-__device__ __forceinline__ double node_weight(const double* M, int m)
+template <int n, class R>
+__device__ __forceinline__ R node_weight(const R* M, int m)
 {
-    double s = 0.5 * M[0];
+    R s = R(0.5) * M[0];
 #pragma unroll
-    for (int k = 1; k < n; ++k) s = fma(M[k], cheb<n>(k, m), s);
-    return s * (2.0 / n);
+    for (int k = 1; k < n; ++k) s += M[k] * (R)cheb<n>(k, m);
+    return s * R(2.0 / n);
 }
 
 // Node weights of all intervals: per layer and top interval, one warp per leaf takes its
 // points, then the larger intervals take the nodes of the four below (whose weights
-// reproduce every polynomial of the degree kept).  weights[layer][interval][n].
+// reproduce every polynomial of the degree kept).  In the FP32 path in FP32, as lambda
+// itself: the rounding of one leaf's weights is independent of the next one's.
+// weights[layer][interval][n].
 constexpr int UP_WARPS = 16;
 template <class R>
 __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant__ Tree tr,
@@ -1084,7 +1152,7 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
                                                            R* __restrict__ weights)
 {
     constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
-    __shared__ double M[UP_WARPS][n], w[2][TOP][n];
+    __shared__ R M[UP_WARPS][n], w[2][TOP][n];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int nloc = blockIdx.y, top = blockIdx.x;
     const double* g = g_sigma + (size_t)(layer0 + nloc) * N;
@@ -1093,31 +1161,32 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
         for (int q = row; q < many; q += UP_WARPS) {
             const int i = top * many + q;
             if (i >= tr.cnt[k]) break;
-            const double2 sp = tr.geo[tr.off[k] + i];
-            double s[n];
+            const Geo sp = tr.geo[tr.off[k] + i];
+            R s[n];
 #pragma unroll
-            for (int m = 0; m < n; ++m) s[m] = 0.0;
+            for (int m = 0; m < n; ++m) s[m] = R(0);
             if (k == 0) {
                 const int64_t j = (int64_t)i * LEAF + lane;
-                if (j < N) add_moments<n>(g[j] * lam_scale, in_span(nu[j], sp), s);
+                if (j < N) add_moments<n, R>((R)(g[j] * lam_scale), (R)in_span(nu[j], sp), s);
             } else {
 #pragma unroll 1
                 for (int r = lane; r < 4 * n; r += 32) {
                     const int ch = 4 * i + r / n, m = r % n; // child interval and its node
                     if (ch >= tr.cnt[k - 1]) break;
-                    const double2 gc = tr.geo[tr.off[k - 1] + ch];
-                    add_moments<n>(w[(k - 1) & 1][4 * q + r / n][m], in_span(fma(gc.y, cheb<n>(1, m), gc.x), sp), s);
+                    const Geo gc = tr.geo[tr.off[k - 1] + ch];
+                    const R x = (R)in_span(fma(gc.h, cheb<n>(1, m), gc.mid), sp);
+                    add_moments<n, R>(w[(k - 1) & 1][4 * q + r / n][m], x, s);
                 }
             }
             __syncwarp();
             int idx;
-            const double v = warp_reduce_scatter<n>(s, idx);
+            const R v = warp_reduce_scatter(s, idx);
             if (idx >= 0) M[row][idx] = v;
             __syncwarp();
             if (lane < n) {
-                const double x = node_weight<n>(M[row], lane);
+                const R x = node_weight<n, R>(M[row], lane);
                 w[k & 1][q][lane] = x;
-                weights[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = (R)x;
+                weights[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = x;
             }
             __syncwarp();
         }
@@ -1216,7 +1285,7 @@ struct Leaf {
     int lane, i;
     bool live;
     int s[3], e[3];
-    double2 g;
+    Geo g;
 
     __device__ bool init(const Tree& tr, const double* nu_hat, int64_t nl, const double* nu, int64_t N, double W,
                          int nloc)
@@ -1244,7 +1313,7 @@ struct Leaf {
             s[0] = __shfl_sync(0xffffffffu, v, 0);
             e[0] = __shfl_sync(0xffffffffu, v, 1);
             s[1] = e[1] = s[2] = e[2] = 0;
-            g = make_double2(0.5 * (nu[jb] + nu[jl]), 0.5 * (nu[jl] - nu[jb]));
+            g = {0.5 * (nu[jb] + nu[jl]), 0.5 * (nu[jl] - nu[jb]), 0.0};
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k)
@@ -1252,25 +1321,6 @@ struct Leaf {
         return true;
     }
 };
-
-// The far lines' part of sigma at a leaf's point.  FP32: the constant term, which
-// dominates, in FP64, the rest in FP32.
-template <class R>
-__device__ __forceinline__ double leaf_far(const Leaf<R>& lf, const Tree& tr, double nuj, int nloc, const double* coef)
-{
-    constexpr int n = Far<R>::n;
-    const double* cg = coef + ((size_t)nloc * tr.cnt[0] + lf.i) * n;
-    R c[n];
-#pragma unroll
-    for (int k = 0; k < n; ++k) c[k] = (R)cg[k];
-    const R x = (R)in_span(nuj, lf.g);
-    if constexpr (std::is_same<R, double>::value) {
-        return clenshaw<n, double>(c, x);
-    } else {
-        c[0] = 0.0f;
-        return cg[0] + (double)clenshaw<n, float>(c, x);
-    }
-}
 
 // sigma of one leaf: FP32
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
@@ -1286,8 +1336,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
-    const double oj = nuj - lf.g.x;
-    const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.y;
+    const Span sp(lf.g, nu[0]);
+    const float rh = sp.rh, rl = sp.rl;
+    const double oj = nuj - lf.g.mid;
+    const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
     float shi = 0.0f, slo = 0.0f;
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
@@ -1300,9 +1352,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
             float nb = 0.0f, nbl = 0.0f, z2 = 1e30f;
             float4 p2 = make_float4(1.f, 1.f, 0.f, 0.f);
             if (have) {
-                const double o = lf.g.x - ln.nu_hat[l];
-                nb = (float)o;
-                nbl = (float)(o - (double)nb);
+                const float2 nf = ln.nuf[l];
+                nb = rh - nf.x; // (nb, nbl) = middle - centre, TwoSum of the high parts
+                const float bb = nb - rh;
+                nbl = ((rh - (nb - bb)) - (nf.x + bb)) + (rl - nf.y);
                 p2 = ln.r2[l];
                 const float x = fmaxf(fabsf(nb) - h, 0.0f) * p2.x;
                 z2 = fmaf(x, x, p2.y * p2.y);
@@ -1365,9 +1418,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
                         } else {
                             float x, xl;
                             scaled_pair(dh, dl, c4.x, b.z, &x, &xl);
-                            float wr, wi;
-                            w_series_tab<false>(x, xl, c4.y, b.w, c4.w, tl.sd[q], &wr, &wi);
-                            acc = fmaf(c4.z, wr, acc);
+                            acc = fmaf(c4.z, w_series_re(x, xl, c4.y, b.w, c4.w, tl.sd[q]), acc);
                         }
                     }
                 }
@@ -1375,7 +1426,9 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
             two_sum(shi, slo, acc); // the chunk's FP32 partial into the compensated sum
         }
     }
-    const double far = tr.on ? leaf_far<float>(lf, tr, nuj, nloc, coef) : 0.0;
+    // the far lines' part
+    const double far =
+        tr.on ? LeafPoly<float>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
     if (lf.live) sigma[(size_t)layer * N + j] = (float)((far + ((double)shi + (double)slo)) * unscale);
 }
 
@@ -1416,7 +1469,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
             }
         }
     }
-    if (tr.on) acc += leaf_far<double>(lf, tr, nuj, nloc, coef);
+    if (tr.on) acc += LeafPoly<double>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
     if (lf.live) sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
@@ -1463,8 +1516,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
         const double lamd = lf.live ? g_sigma[(size_t)layer * N + j] * lam_scale : 0.0;
         const float hT = (float)(0.5 / T[layer]);
         const float lam = (float)lamd;
-        const double oj = nuj - lf.g.x;
-        const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.y;
+        const Span sp(lf.g, nu[0]);
+        const float rh = sp.rh, rl = sp.rl;
+        const double oj = nuj - lf.g.mid;
+        const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
 #pragma unroll 1
         for (int k = 0; k < 3; ++k) {
             const bool masked = k != 1;
@@ -1477,9 +1532,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
                 float4 p2 = make_float4(1.f, 1.f, 0.f, 0.f);
                 float2 p3 = make_float2(0.f, 0.f);
                 if (have) {
-                    const double o = lf.g.x - ln.nu_hat[l];
-                    nb = (float)o;
-                    nbl = (float)(o - (double)nb);
+                    const float2 nf = ln.nuf[l];
+                    nb = rh - nf.x; // (nb, nbl) = middle - centre, TwoSum of the high parts
+                    const float bb = nb - rh;
+                    nbl = ((rh - (nb - bb)) - (nf.x + bb)) + (rl - nf.y);
                     p2 = ln.r2[l];
                     p3 = ((const float2*)ln.r3)[l];
                     const float x = fmaxf(fabsf(nb) - h, 0.0f) * p2.x;
@@ -1552,32 +1608,26 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
                         const float dh = ohi + b.x, dl = olo + b.y;
                         const float xq = c4.x * (dh + dl);
                         const float zz = fmaf(xq, xq, c4.y * c4.y);
-                        // (the series loses 2|z|^2 in w', so it stops at its zone's edge)
-                        const bool ser = in && zz < NEAR_POLY_Z2;
-                        if (!__any_sync(0xffffffffu, ser)) {
+                        if (!__any_sync(0xffffffffu, in && zz < NEAR_POLY_Z2)) {
                             // no lane in the series zone: the polynomials, branch-free
                             const float u = rcp_fast(zz);
                             const float ft = horner14(tl.hf[q], u), fb = horner14(tl.hg[q], u);
                             aT += in ? ft : 0.0f;
                             aB += in ? fb : 0.0f;
                         } else if (in) {
-                            if (!ser) {
+                            // the series also serves the lanes just outside its zone
+                            if (!(fabsf(xq) <= SER_X)) {
                                 const float u = rcp_fast(zz);
                                 aT += horner14(tl.hf[q], u);
                                 aB += horner14(tl.hg[q], u);
                             } else {
                                 float x, xl;
                                 scaled_pair(dh, dl, c4.x, b.z, &x, &xl);
-                                const float a = c4.y;
-                                float wr, wi;
-                                w_series_tab<true>(x, xl, a, b.w, c4.w, tl.sd[q], &wr, &wi);
-                                // w' = -2 z w + 2i/sqrt(pi);  H_x = Re w', H_a = -Im w'
-                                const float dr = -2.0f * (x * wr - a * wi);
-                                const float di = -2.0f * (x * wi + a * wr) + (float)(2.0 * INV_SQRTPI);
+                                float wr, dr, di; // H_x = dr, H_a = -di
+                                w_series_deriv(x, xl, c4.y, b.w, c4.w, tl.sd[q], &wr, &dr, &di);
                                 const float V0 = c4.z * wr;
-                                const float V1 = c4.z * x * dr;
-                                const float V2 = -c4.z * a * di;
-                                const float Db = -(V0 + V1 + V2);
+                                const float V2 = -c4.z * c4.y * di;
+                                const float Db = -(V0 + c4.z * x * dr + V2);
                                 aT += tl.aS[q] * V0 + hT * Db + tl.nn[q] * V2;
                                 aB += V2;
                             }
@@ -1717,7 +1767,7 @@ struct XsPlan {
 // its own far radius and its parent's, about 16 interval lengths.
 void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
 {
-    const int64_t warps = mixed ? 20000 : 8000, min_lines = mixed ? 1024 : 128;
+    const int64_t warps = mixed ? 10000 : 8000, min_lines = mixed ? 1024 : 128;
     int block = 0;
     size_t row = 0;
     p->fw.slots = 0;
@@ -1773,7 +1823,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
             p.tree.total += p.tree.cnt[k];
         }
         split_far(&p, nl, N, Lc, mixed);
-        p.off_geo = take(sizeof(double2) * (size_t)p.tree.total);
+        p.off_geo = take(sizeof(Geo) * (size_t)p.tree.total);
         p.off_cov = take(sizeof(int2) * (size_t)p.tree.total);
         p.off_win = take(sizeof(int2) * (size_t)p.tree.cnt[0]);
         p.off_pq = take(sizeof(int2) * (size_t)p.tree.total * Lc);
@@ -1782,7 +1832,8 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     const size_t base = off;
     if (tree) {
         p.off_fwd = take(sizeof(double) * n * p.rows);
-        p.off_coef = take(sizeof(double) * n * (size_t)Lc * p.tree.cnt[0]);
+        p.off_coef = take(sizeof(double) * (mixed ? LeafPoly<float>::stride : LeafPoly<double>::stride) * (size_t)Lc *
+                          p.tree.cnt[0]);
     }
     const size_t fwd_end = off;
     off = base;
@@ -1861,7 +1912,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
     R4* rec2 = (R4*)(ws + p.off_rec2);
     R* rec3 = (R*)(ws + p.off_rec3);
     R* clo = FAST ? (R*)(ws + p.off_clo) : nullptr;
-    double2* geo = (double2*)(ws + p.off_geo);
+    Geo* geo = (Geo*)(ws + p.off_geo);
     int2* cov = (int2*)(ws + p.off_cov);
     int2* win = (int2*)(ws + p.off_win);
     int2* pq = (int2*)(ws + p.off_pq);
@@ -1907,7 +1958,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
         if (!adjoint) {
             if (tr.on) {
                 far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, sums);
-                down_kernel<R><<<dim3(tops, (unsigned)lc), DOWN_ROWS * Far<R>::n, 0, st>>>(tr, p.fw, lc,
+                down_kernel<R><<<dim3(tops, (unsigned)lc), DownRows<R>::v * Far<R>::n, 0, st>>>(tr, p.fw, lc,
                                                                                        sums, coef);
                 count_launch(2);
             }
