@@ -409,9 +409,9 @@ int model_forward_impl(const xs_model* m, const double* theta, double* F0out, ch
     for (int s = 0; s < Sp; ++s) {
         sp[s] = sig + es * LN * s;
         if (m->method == XS_METHOD_MODIT)
-            r = modit_compute(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
-                              m->n_gamma, m->n_fft[s], m->prec, (void*)sp[s], ws + p.xsws_sp[s], p.xsws_sp_bytes[s],
-                              st);
+            r = xsi::modit_forward(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
+                                   m->n_gamma, m->n_fft[s], m->prec, (void*)sp[s], ws + p.xsws_sp[s],
+                                   p.xsws_sp_bytes[s], st, xs_flags);
         else
             r = xsi::xs_run(&m->species[s], m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec,
                             (void*)sp[s], ws + p.xsws_sp[s], p.xsws_sp_bytes[s], false, nullptr, nullptr, nullptr, st,
@@ -490,9 +490,9 @@ int model_adjoint_impl(const xs_model* m, const double* theta, const double* gF,
         return r;
     for (int s = 0; s < Sp; ++s) {
         if (m->method == XS_METHOD_MODIT)
-            r = modit_compute_adjoint(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
-                                      m->n_gamma, m->n_fft[s], m->prec, gsp[s], gTtmp, gb + s, ws + p.xsws_sp[s],
-                                      p.xsws_sp_bytes[s], st);
+            r = xsi::modit_adjoint(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
+                                   m->n_gamma, m->n_fft[s], m->prec, gsp[s], gTtmp, gb + s, ws + p.xsws_sp[s],
+                                   p.xsws_sp_bytes[s], st, xsi::XS_RUN_REUSE);
         else
             r = xsi::xs_run(&m->species[s], m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec,
                             nullptr, ws + p.xsws_sp[s], p.xsws_sp_bytes[s], true, gsp[s], gTtmp, gb + s, st,

@@ -48,6 +48,14 @@ int xs_run(const xs_lines* ln, const double* nu, int64_t N, const double* T, con
            double W, int prec, void* sigma, void* ws, size_t ws_bytes, bool adjoint, const double* g_sigma,
            double* g_T, double* g_b, cudaStream_t st, int flags = 0, double* g_T_sum = nullptr);
 
+// MODIT forward and adjoint with the composite model's flags (KEEP_ADJ, REUSE as above)
+int modit_forward(const xs_lines* lines, double nu_min, double nu_max, int64_t N, const double* T, const double* P_bar,
+                  int32_t L, double broad_scale, int32_t n_gamma, int64_t n_fft, int prec, void* sigma,
+                  void* workspace, size_t workspace_bytes, cudaStream_t st, int flags);
+int modit_adjoint(const xs_lines* lines, double nu_min, double nu_max, int64_t N, const double* T, const double* P_bar,
+                  int32_t L, double broad_scale, int32_t n_gamma, int64_t n_fft, int prec, const double* g_sigma,
+                  double* g_T, double* g_broad, void* workspace, size_t workspace_bytes, cudaStream_t st, int flags);
+
 // checks ascending (grid == false: non-decreasing centres; grid == true: strictly
 // increasing grid) on the device; blocks on `st`; flag_dev is one device int
 int check_sorted(const double* v, int64_t n, cudaStream_t st, int* flag_dev, bool grid);
