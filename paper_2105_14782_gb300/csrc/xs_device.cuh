@@ -17,9 +17,8 @@
 //       Im w = e^{-x^2} [-K(a) sin 2ax + (h/pi) sin(2ax)/a]       + (h/pi) Ss
 //       Sc = sum_n (E_n^- + E_n^+)/(n^2h^2 + a^2),  Ss = sum_n nh (E_n^- - E_n^+)/(n^2h^2 + a^2)
 //       K(a) = erfcx(a) - (2ah/pi) sum_n e^{-n^2h^2}/(n^2h^2 + a^2)   (per line, precomputed)
-//     Every E_n is taken directly from its own small exponent (no recurrence
-//     through e^{-x^2} e^{2nhx}, which would lose digits); only the n near x/h
-//     (and, for small x, the first E_n^+) are summed.
+//     Every E_n is a product of factors with small exponents about the term nearest
+//     the peak (nothing passes through e^{-x^2} e^{2nhx}, which would lose digits).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -92,16 +91,10 @@ template <> struct Tier<float> {
     static constexpr float h = 0.7f;           // series step (error ~1e-8 relative)
 };
 template <> struct Tier<double> {
-    static constexpr double z2_fast = 1e300;   // no truncated fast form in double precision
-    static constexpr double z2_fast_adj = 1e300;
     static constexpr double z2_far = 22500.0;  // |z| >= 150: K = 3
-    static constexpr double z2_mid1 = 1600.0;  // |z| >= 40 : K = 5
-    static constexpr double z2_mid2 = 100.0;   // |z| >= 10 : K = 12, below: series
-    static constexpr double z2_series = 100.0;
-    static constexpr int K1 = 3, K2 = 5, K3 = 12;
+    static constexpr double z2_mid = 1600.0;   // |z| >= 40 : K = 5
+    static constexpr double z2_series = 100.0; // |z| >= 10 : K = 12, below: series
     static constexpr double h = 0.5;           // series step (error ~1e-17)
-    static constexpr int nwin = 13;
-    static constexpr double tcut = 6.5;
 };
 
 // Bounds-checked build (nvcc -DXS_CHECKED): index checks guard the kernels'
@@ -145,7 +138,6 @@ __device__ __forceinline__ float rcp_fast(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double rcp_fast(double x) { return 1.0 / x; }
 
 // x = |d| c with d = dh + dl and c = ch + cl as unevaluated float pairs:
 // returns x as a pair (xh, xl), xh = fl(|dh| ch).
@@ -160,25 +152,55 @@ __device__ __forceinline__ void scaled_pair(float dh, float dl, float ch, float 
     *xh = fabsf(p);
     *xl = __int_as_float(__float_as_int(r) ^ (__float_as_int(d) & 0x80000000)); // r with d's sign taken out
 }
-__device__ __forceinline__ void scaled_pair(double dh, double, double ch, double, double* xh, double* xl)
-{
-    *xh = fabs(dh) * ch;
-    *xl = 0.0;
-}
-
 __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 
-__device__ __forceinline__ int round_int(float v) { return __float2int_rn(v); }
-__device__ __forceinline__ int round_int(double v) { return __double2int_rn(v); }
+// e^v in FP64, table-driven (Tang 1989): 2^(i/64) from a table, the rest (|r| <= ln2/128)
+// by the series to r^5 (next term 4e-17): half the operations of exp.  Beyond +-700 exp.
+struct Exp2Table64 {
+    double t[64];
+};
+constexpr Exp2Table64 make_exp2_table64()
+{
+    Exp2Table64 r{};
+    const double ln2 = 0.69314718055994530942;
+    for (int i = 0; i < 64; ++i) {
+        // series of e^(i ln2/64) about the nearer end
+        const double x = (i <= 32 ? i : i - 64) * ln2 / 64;
+        double s = 1.0;
+        for (int k = 22; k >= 1; --k) s = 1.0 + s * x / k;
+        r.t[i] = i <= 32 ? s : 2.0 * s;
+    }
+    return r;
+}
+__device__ const Exp2Table64 EXP2_64 = make_exp2_table64();
 
-// accurate expf (a few ulp): the small-|z| tier is rare, and its exponent can reach ~40
-__device__ __forceinline__ float exp_neg(float t2) { return expf(-t2); }
-__device__ __forceinline__ double exp_neg(double t2) { return exp(-t2); }
+__device__ __forceinline__ double exp_tab(double v)
+{
+    if ((__double2hiint(v) & 0x7fffffff) >= 0x4085e000) return exp(v); // |v| >= 700, infinities, NaN
+    const double magic = 6755399441055744.0; // 1.5 2^52
+    // ln 2 = its float value (products with k are exact) + the rest
+    const double ln2_hi = (double)0.693147182f, ln2_lo = -1.904654299957767878541823e-9;
+    const double t = fma(v, 64.0 / 0.69314718055994530942, magic), kd = t - magic;
+    const int k = __double2loint(t);
+    const double r = fma(kd, -ln2_lo / 64, fma(kd, -ln2_hi / 64, v));
+    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(r, p, 1.0 / 6.0);
+    p = fma(r, p, 0.5);
+    p = fma(r * r, p, r);
+    const double h = EXP2_64.t[k & 63];
+    const double s = fma(h, p, h);
+    return __hiloint2double(__double2hiint(s) + ((k >> 6) << 20), __double2loint(s));
+}
 
-__device__ __forceinline__ void sincos_r(float v, float* s, float* c) { sincosf(v, s, c); }
-__device__ __forceinline__ void sincos_r(double v, double* s, double* c) { sincos(v, s, c); }
-__device__ __forceinline__ float sin_r(float v) { return sinf(v); }
-__device__ __forceinline__ double sin_r(double v) { return sin(v); }
+// 1/x in FP64 to about an ulp, x normal: the hardware's approximation and two steps of
+// Newton's iteration, five operations
+__device__ __forceinline__ double rcp64(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
 
 // exp(-x^2) with x^2 split into hi + lo so the rounding of x*x does not enter.
 __device__ __forceinline__ float exp_negsq(float x, float xl) // x + xl, |xl| << |x|
@@ -191,97 +213,8 @@ __device__ __forceinline__ double exp_negsq(double x)
 {
     double hi = x * x;
     double lo = fma(x, x, -hi);
-    return exp(-hi) * (1.0 - lo);
-}
-
-// Asymptotic series (Eq. asywofz) with K correction terms; x >= 0, a >= 0,
-// r = 1/(x^2 + a^2).  Returns w.
-template <class R, int K>
-__device__ __forceinline__ void w_asym(R x, R a, R r, R* wr, R* wi)
-{
-    // u = 1/(2 z^2) = conj(z)^2 r^2 / 2
-    R hr2 = R(0.5) * r * r;
-    R ur = (x - a) * (x + a) * hr2;
-    R ui = R(-2) * a * x * hr2;
-    R pr = R(1), pi = R(0);
-#pragma unroll
-    for (int k = K; k >= 1; --k) {
-        R c = R(2 * k - 1);
-        R tr = ur * pr - ui * pi;
-        R ti = ur * pi + ui * pr;
-        pr = R(1) + c * tr;
-        pi = c * ti;
-    }
-    R s = r * R(INV_SQRTPI);
-    *wr = (a * pr - x * pi) * s;
-    *wi = (x * pr + a * pi) * s;
-}
-
-// Asymptotic series of w'(z) = dw/dz:  w' ~ -(2 i u / sqrt(pi)) (1 + sum_k (2k+1)!! u^k).
-template <class R, int K>
-__device__ __forceinline__ void dw_asym(R x, R a, R r, R* dr, R* di)
-{
-    R hr2 = R(0.5) * r * r;
-    R ur = (x - a) * (x + a) * hr2;
-    R ui = R(-2) * a * x * hr2;
-    R pr = R(1), pi = R(0);
-#pragma unroll
-    for (int k = K; k >= 1; --k) {
-        R c = R(2 * k + 1);
-        R tr = ur * pr - ui * pi;
-        R ti = ur * pi + ui * pr;
-        pr = R(1) + c * tr;
-        pi = c * ti;
-    }
-    // q = u p ; w' = -(2i/sqrt(pi)) q = (2/sqrt(pi)) (Im q - i Re q)
-    R qr = ur * pr - ui * pi;
-    R qi = ur * pi + ui * pr;
-    *dr = R(2 * INV_SQRTPI) * qi;
-    *di = R(-2 * INV_SQRTPI) * qr;
-}
-
-// Small-|z| series; x = xh + xl >= 0 (xl a small correction carrying the bits
-// of x a single float cannot: exp(-x^2) has condition number 2x^2 in x),
-// a >= 0, Kc = K(a) for this precision's step h.
-template <class R>
-__device__ __forceinline__ void w_series(R xh, R xl, R a, R Kc, R* wr, R* wi)
-{
-    const R x = xh;
-    const R h = Tier<R>::h;
-    const int nwin = Tier<R>::nwin;
-    R sc = R(0), ss = R(0);
-    int n0 = round_int(x / h);
-    R a2 = a * a;
-#pragma unroll 1
-    for (int k = -nwin; k <= nwin; ++k) {
-        int n = n0 + k;
-        if (n < 1) continue;
-        R nh = R(n) * h;
-        R t = (nh - xh) - xl;
-        R e = exp_neg(t * t);
-        R d = rcp_fast(fma(nh, nh, a2));
-        sc = fma(d, e, sc);
-        ss = fma(nh * d, e, ss);
-    }
-#pragma unroll 1
-    for (int n = 1; n <= 64; ++n) { // bounded even for non-finite x
-        R nh = R(n) * h;
-        R t = (nh + xh) + xl;
-        if (!(t < Tier<R>::tcut)) break;
-        R e = exp_neg(t * t);
-        R d = rcp_fast(fma(nh, nh, a2));
-        sc = fma(d, e, sc);
-        ss = fma(-nh * d, e, ss);
-    }
-    R ex = exp_negsq(xh) * (R(1) - R(2) * xh * xl);
-    R s2, c2v;
-    sincos_r(R(2) * a * x, &s2, &c2v);
-    R sax = sin_r(a * x);
-    R sax_a = (a > R(0)) ? sax / a : x;
-    R s2_a = (a > R(0)) ? s2 / a : R(2) * x;
-    const R hpi = h * R(1.0 / PI);
-    *wr = ex * (Kc * c2v + R(2) * hpi * sax * sax_a) + a * hpi * sc;
-    *wi = ex * (-Kc * s2 + hpi * s2_a) + hpi * ss;
+    const double e = exp_tab(-hi);
+    return fma(e, -lo, e);
 }
 
 // Per-line table for w_series_tab: d[n + SER_OFF] = 1/(n^2 h^2 + a^2) for n != 0 and 0
@@ -434,53 +367,91 @@ __device__ __forceinline__ void w_series_deriv(float xh, float xl, float a, floa
     *di = 2.0f * fmaf(hpi, ex + fmaf(x, q.s1, q.s2), -fmaf(x, gi, a * gr));
 }
 
-template <class R>
-__device__ __forceinline__ void w_small(R x, R xl, R a, R Kc, const R*, R* wr, R* wi)
-{
-    w_series<R>(x, xl, a, Kc, wr, wi);
-}
+// The same in FP64, h = 1/2 and 13 terms on each side (the next are below 1e-19 of the
+// peak): n0 = round(x/h) <= SER64_N0 for x <= 10.  (A loop of an exponential a term
+// before, 27 and more of them; some 150 operations now, 220 with derivatives.)
+constexpr int SER64_OFF = 13, SER64_N0 = 20, SER64_TAB = SER64_N0 + 2 * SER64_OFF + 1; // 47
+// e^{-(k h)^2}, k = 1 .. 13
+__device__ const double KC_E64[SER64_OFF] = {0.77880078307140488, 0.36787944117144233, 0.10539922456186433,
+                                             0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956,
+                                             4.7851173921290088e-06, 1.1253517471925912e-07, 1.6052280551856116e-09,
+                                             1.3887943864964021e-11, 7.2877240958196922e-14, 2.3195228302435691e-16,
+                                             4.4777324417183015e-19};
 
-// w(x + ia) for any tier (the FP64 path); x = x + xl >= 0; dtab is not used.
-template <class R>
-__device__ __forceinline__ void faddeeva(R x, R xl, R a, R Kc, R* wr, R* wi, const R* dtab = nullptr)
+__device__ __forceinline__ void series_table64(double a, double* d)
 {
-    R z2 = fma(x, x, a * a);
-    if (z2 >= Tier<R>::z2_mid2) {
-        R r = rcp_fast(z2);
-        if (z2 >= Tier<R>::z2_far)
-            w_asym<R, Tier<R>::K1>(x, a, r, wr, wi);
-        else if (z2 >= Tier<R>::z2_mid1)
-            w_asym<R, Tier<R>::K2>(x, a, r, wr, wi);
-        else
-            w_asym<R, Tier<R>::K3>(x, a, r, wr, wi);
-    } else {
-        w_small<R>(x, xl, a, Kc, dtab, wr, wi);
+    const double a2 = a * a;
+    d[SER64_OFF] = 0.0;
+#pragma unroll 1
+    for (int n = 1; n < SER64_TAB - SER64_OFF; ++n) {
+        const double v = rcp64(fma(0.25 * n, (double)n, a2));
+        d[SER64_OFF + n] = v;
+        if (n <= SER64_OFF) d[SER64_OFF - n] = v;
     }
 }
 
-// w and w' for any tier; x = x + xl >= 0.
-template <class R>
-__device__ __forceinline__ void faddeeva_d(R x, R xl, R a, R Kc, R* wr, R* wi, R* dr, R* di, const R* dtab = nullptr)
+struct SeriesSums64 {
+    double s0, s1, s2;
+};
+template <bool DERIV>
+__device__ __forceinline__ SeriesSums64 series_sums64(double x, const double* dt)
 {
-    R z2 = fma(x, x, a * a);
-    if (z2 >= Tier<R>::z2_mid2) {
-        R r = rcp_fast(z2);
-        if (z2 >= Tier<R>::z2_far) {
-            w_asym<R, Tier<R>::K1>(x, a, r, wr, wi);
-            dw_asym<R, Tier<R>::K1>(x, a, r, dr, di);
-        } else if (z2 >= Tier<R>::z2_mid1) {
-            w_asym<R, Tier<R>::K2>(x, a, r, wr, wi);
-            dw_asym<R, Tier<R>::K2>(x, a, r, dr, di);
-        } else {
-            w_asym<R, Tier<R>::K3>(x, a, r, wr, wi);
-            dw_asym<R, Tier<R>::K3>(x, a, r, dr, di);
+    const int n0 = __double2int_rn(2.0 * x);
+    if (!XS_CHECK(n0 >= 0 && n0 <= SER64_N0)) return {0.0, 0.0, 0.0};
+    const double delta = 0.5 * n0 - x; // exact
+    const double E0 = exp_tab(-delta * delta);
+    const double f = exp_tab(-delta), g = rcp64(f); // e^{-2h delta}, e^{2h delta}
+    const double* d0 = dt + (n0 + SER64_OFF);
+    double p = KC_E64[SER64_OFF - 1] * d0[SER64_OFF], q = KC_E64[SER64_OFF - 1] * d0[-SER64_OFF];
+    double p1 = 0.0, p2 = 0.0, q1 = 0.0, q2 = 0.0;
+#pragma unroll
+    for (int k = SER64_OFF - 1; k >= 0; --k) {
+        if (DERIV) {
+            p2 = fma(p2, f, p1);
+            p1 = fma(p1, f, p);
+            q2 = fma(q2, g, q1);
+            q1 = fma(q1, g, q);
         }
-    } else {
-        w_small<R>(x, xl, a, Kc, dtab, wr, wi);
-        // w' = -2 z w + 2i/sqrt(pi)
-        *dr = R(-2) * (x * *wr - a * *wi);
-        *di = R(-2) * (x * *wi + a * *wr) + R(2 * INV_SQRTPI);
+        p = fma(p, f, k ? KC_E64[k ? k - 1 : 0] * d0[k] : d0[0]);
+        q = k ? fma(q, g, KC_E64[k ? k - 1 : 0] * d0[-k]) : q * g; // the centre term belongs to the first
     }
+    SeriesSums64 r;
+    const double s0 = p + q;
+    r.s0 = E0 * s0;
+    r.s1 = r.s2 = 0.0;
+    if (DERIV) {
+        const double k1 = p1 * f, l1 = q1 * g;                          // sums of k w f^k
+        const double k2 = fma(p2 * f, 2.0 * f, k1), l2 = fma(q2 * g, 2.0 * g, l1); // of k^2 w f^k
+        const double m1 = 0.5 * (k1 - l1), m2 = 0.25 * (k2 + l2);
+        r.s1 = E0 * fma(delta, s0, m1);
+        r.s2 = E0 * fma(delta, fma(delta, s0, 2.0 * m1), m2);
+    }
+    return r;
+}
+
+__device__ __forceinline__ double w_series_re(double x, double a, double inv_a, double Kc, const double* dt)
+{
+    const SeriesSums64 q = series_sums64<false>(x, dt);
+    const double sax = sin(a * x);
+    const double hpi = 0.5 / PI;
+    return exp_negsq(x) * fma(2.0 * hpi * inv_a * sax, sax, Kc * fma(-2.0 * sax, sax, 1.0)) + a * hpi * q.s0;
+}
+
+__device__ __forceinline__ void w_series_deriv(double x, double a, double inv_a, double Kc, const double* dt, double* wr,
+                                               double* dr, double* di)
+{
+    const SeriesSums64 q = series_sums64<true>(x, dt);
+    double sax, cax;
+    sincos(a * x, &sax, &cax);
+    const double ex = exp_negsq(x), hpi = 0.5 / PI;
+    const double c2v = fma(-2.0 * sax, sax, 1.0), s2 = 2.0 * sax * cax;
+    const double s2_a = a > 0.0 ? s2 * inv_a : 2.0 * x;
+    const double gr = ex * fma(2.0 * hpi * inv_a * sax, sax, Kc * c2v);
+    const double gi = ex * fma(hpi, s2_a, -Kc * s2);
+    const double ah = a * hpi;
+    *wr = fma(ah, q.s0, gr);
+    *dr = 2.0 * fma(ah, q.s1, a * gi - x * gr);
+    *di = 2.0 * fma(hpi, ex + fma(x, q.s1, q.s2), -fma(x, gi, a * gr));
 }
 
 // ------------------------------------------------------------------ wing polynomials
@@ -599,17 +570,81 @@ __device__ __forceinline__ void asy_coeffs_adj(float a, float amp, float aS, flo
     }
 }
 
-template <class R>
-__device__ __noinline__ R voigt_H(R x, R xl, R a, R Kc, const R* dtab)
+// The FP64 path: the same polynomials in u, unscaled, truncated after K = 3, 5 or 12
+// correction terms (2K + 1 coefficients) by |z| (Tier<double>).
+constexpr int ASY64_K = 12;
+struct AsyTable64 {
+    double cq[ASY64_K + 1][ASY64_K + 1]; // c_k q_kj (j <= k)
+};
+constexpr AsyTable64 make_asy_table64()
 {
-    R wr, wi;
-    faddeeva<R>(x, xl, a, Kc, &wr, &wi, dtab);
-    return wr;
+    long long b[ASY64_K + 2] = {}, c[ASY64_K + 2] = {}; // as make_asy_table
+    b[0] = 1;
+    c[0] = 1;
+    AsyTable64 t{};
+    double ck = 1.0;
+    for (int k = 0; k <= ASY64_K; ++k) {
+        if (k > 0) {
+            long long nb[ASY64_K + 2] = {}, nc[ASY64_K + 2] = {};
+            for (int s = 0; s <= k; ++s) {
+                const long long bs1 = s > 0 ? b[s - 1] : 0, cs1 = s > 0 ? c[s - 1] : 0;
+                nc[s] = cs1 - 2 * c[s] - 2 * b[s];
+                nb[s] = bs1 - 2 * b[s] + 2 * cs1 - 2 * c[s];
+            }
+            for (int s = 0; s <= k; ++s) {
+                b[s] = nb[s];
+                c[s] = nc[s];
+            }
+            ck *= (2.0 * k - 1.0) / 2.0;
+        }
+        for (int j = 0; j <= k; ++j) t.cq[k][j] = ck * (double)b[k - j];
+    }
+    return t;
 }
-template <class R>
-__device__ __noinline__ void voigt_w_dw(R x, R xl, R a, R Kc, R* w4, const R* dtab)
+__constant__ const AsyTable64 ASY64 = make_asy_table64();
+
+// C_n (n = 0 .. 2K) of H = u sum_n C_n u^n, times amp
+template <int K>
+__device__ __forceinline__ void asy64_coeffs(double a, double amp, double (&C)[2 * K + 1])
 {
-    faddeeva_d<R>(x, xl, a, Kc, &w4[0], &w4[1], &w4[2], &w4[3], dtab);
+    const double a2 = a * a;
+    double ap = amp * a * INV_SQRTPI;
+#pragma unroll
+    for (int n = 0; n <= 2 * K; ++n) C[n] = 0.0;
+#pragma unroll
+    for (int j = 0; j <= K; ++j) {
+#pragma unroll
+        for (int k = j; k <= K; ++k) C[k + j] = fma(ASY64.cq[k][j], ap, C[k + j]);
+        ap *= a2;
+    }
+}
+
+// From the moments r_n = sum lambda u^(n+1) (n = 0 .. 2K + 1) of a line: the sums of
+// lambda V0, lambda D_beta and lambda D_gamma (see asy_coeffs_adj).
+template <int K>
+__device__ __forceinline__ void asy64_adjoint(double a, double amp, const double (&r)[2 * K + 2], double* V0, double* Db,
+                                              double* Dg)
+{
+    const double a2 = a * a;
+    double ap = amp * a * INV_SQRTPI, v0 = 0.0, db = 0.0, dg = 0.0;
+#pragma unroll
+    for (int j = 0; j <= K; ++j) {
+        double s = 0.0, sk = 0.0, sn = 0.0; // over k of c q r_n, k c q r_n, (n + 1) c q r_{n+1}
+#pragma unroll
+        for (int k = j; k <= K; ++k) {
+            const double v = ASY64.cq[k][j] * r[k + j];
+            s += v;
+            sk = fma((double)k, v, sk);
+            sn = fma(ASY64.cq[k][j] * (double)(k + j + 1), r[k + j + 1], sn);
+        }
+        v0 = fma(ap, s, v0);
+        db = fma(ap, 2.0 * sk, db);
+        dg = fma(ap, fma((double)(2 * j + 1), s, -2.0 * a2 * sn), dg);
+        ap *= a2;
+    }
+    *V0 = v0;
+    *Db = db;
+    *Dg = dg;
 }
 
 } // namespace xsd

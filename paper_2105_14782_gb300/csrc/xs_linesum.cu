@@ -25,7 +25,7 @@
 // away), and |z| >= Z0 at every point of the interval.  Measured over a in 1e-4 .. 100
 // and half-widths of 0.01 .. 300 Doppler units against wofz, the interpolation error is
 // below 1.5e-8 of the profile with 10 nodes, kappa = 4.5, Z0 = 6 (FP32) and below 2e-16
-// with 18 nodes, kappa = 5, Z0 = 8 (FP64): under the rounding of the evaluations.
+// with 18 nodes, kappa = 5, Z0 >= 8 (FP64, where the forms need |z| >= 10): under the rounding of the evaluations.
 //
 // What it saves: of the in-cut pairs of 220,000 lines on a 20,000-point grid about 4% are
 // evaluated at a point and the rest at 10 nodes per interval.  The 100-layer forward +
@@ -62,7 +62,7 @@ template <> struct Far<float> {
 };
 template <> struct Far<double> {
     static constexpr int n = 18;
-    static constexpr double kappa = 5.0, Z0 = 8.0;
+    static constexpr double kappa = 5.0, Z0 = 10.0;
 };
 
 __device__ const ChebTable<10> CHEB10 = make_cheb<10>();
@@ -192,12 +192,6 @@ __global__ void grid_check_kernel(const double* __restrict__ nu, int64_t N, int*
 __device__ const float KC_E32[10] = {0.612626433f, 0.140858427f, 0.0121551799f, 0.00039366915f, 4.78511947e-06f,
                                      2.18295906e-08f, 3.73757449e-11f, 2.40173736e-14f, 5.79232066e-18f,
                                      5.24289428e-22f};
-__device__ const double KC_E64[13] = {0.77880078307140488, 0.36787944117144233, 0.10539922456186433,
-                                      0.018315638888734179, 0.0019304541362277093, 0.00012340980408667956,
-                                      4.7851173921290088e-06, 1.1253517471925912e-07, 1.6052280551856116e-09,
-                                      1.3887943864964021e-11, 7.2877240958196922e-14, 2.3195228302435691e-16,
-                                      4.4777324417183015e-19};
-
 // K(a) = erfcx(a) - (2 a h/pi) sum_k e^{-(kh)^2} / ((kh)^2 + a^2), the per-line constant
 // of the small-|z| series (see xs_device.cuh)
 __device__ __forceinline__ float series_K(float a)
@@ -225,18 +219,20 @@ __device__ __forceinline__ double series_K(double a)
 // Layer constants of the line parameters.
 struct LayerConst {
     double kE, kq, kc, kg, k2E, kqT; // exponent slopes, c nu_hat, pressure factor, dlnS slopes
-    double lnTr, T, bk; // ln(T/296), T, beta cL/nu_hat
+    double lnTr, T, bk, bT, Patm; // ln(T/296), T, beta cL/nu_hat, 1/T - 1/296, P/atm
 };
 
 __device__ __forceinline__ LayerConst layer_const(double Tn, double Pn, double mass, double qexp, double sb)
 {
     LayerConst k;
     const double lnTr = log(Tn / Tref), iT = 1.0 / Tn;
-    k.kE = c2 * (iT - 1.0 / Tref);
+    k.bT = iT - 1.0 / Tref;
+    k.kE = c2 * k.bT;
+    k.Patm = Pn / bar_per_atm;
     k.kq = qexp * lnTr;
     k.bk = sqrt(kB * Tn / (mass * amu));
     k.kc = cL / (SQRT2 * k.bk);
-    k.kg = sb * (Pn / bar_per_atm);
+    k.kg = sb * k.Patm;
     k.k2E = c2 * iT * iT;
     k.kqT = qexp * iT;
     k.lnTr = lnTr;
@@ -315,7 +311,6 @@ __global__ void __launch_bounds__(256) line_params_kernel(
     float cmin = __int_as_float(0x7f800000), amin = cmin, gmin = cmin;
     for (int64_t l = (int64_t)blockIdx.x * 256 + threadIdx.x; l < nl; l += (int64_t)gridDim.x * 256) {
         const double nuh = nu_hat[l], E = elower[l];
-        const double v = fma(-E, k.kE, ln_S0[l]) - k.kq;
         const double c = FAST ? k.kc * inv_nu[l] : 1.0 / (SQRT2 * (k.bk * nuh / cL));
         const R cr = (R)c;
         R gam, Al, Av;
@@ -327,7 +322,7 @@ __global__ void __launch_bounds__(256) line_params_kernel(
             gam = (float)(k.kg * gamma_ref[l]) * expf(-(float)n_temp[l] * lnTr);
             int e;
             float hi, lo;
-            exp_pair(v, tab, &e, &hi, &lo);
+            exp_pair(fma(-E, k.kE, ln_S0[l]) - k.kq, tab, &e, &hi, &lo);
             // s = 2^e (hi + lo) stim 2^80, products in FP32 with the low part carried
             const float s = hi * stim, sl = fmaf(hi, stim, -s) + lo * stim;
             const float g = gam * (float)(1.0 / PI), ci = cr * (float)INV_SQRTPI;
@@ -338,8 +333,9 @@ __global__ void __launch_bounds__(256) line_params_kernel(
             Al = ldexpf(fmaf(s, g, fmaf(s, gl, sl * g)), e + MIXED_SCALE_LOG2);
             Av = ldexpf(fmaf(s, ci, fmaf(s, cl, sl * ci)), e + MIXED_SCALE_LOG2);
         } else {
-            const double s = exp(v) * (expm1(-c2 * nuh / k.T) / expm1(-c2 * nuh / Tref));
-            gam = k.kg * gamma_ref[l] * exp(-n_temp[l] * k.lnTr);
+            // the checking path keeps the plain expressions, operation by operation
+            const double s = exp(ln_S0[l] - c2 * E * k.bT - k.kq) * (expm1(-c2 * nuh / k.T) / expm1(-c2 * nuh / Tref));
+            gam = sb * gamma_ref[l] * exp(-n_temp[l] * k.lnTr) * k.Patm;
             Al = s * gam / PI;
             Av = s * c * INV_SQRTPI;
         }
@@ -366,7 +362,7 @@ __global__ void __launch_bounds__(256) line_params_kernel(
                 ((float2*)rec3)[idx] = make_float2(aS, -(float)n_temp[l] / Tf);
             } else {
                 const double ud = c2 * nuh / k.T;
-                rec3[2 * idx] = fma(k.k2E, E, -k.kqT) - (ud / k.T) / expm1(ud);
+                rec3[2 * idx] = (c2 * E / (k.T * k.T) - qexp / k.T) - (ud / k.T) / expm1(ud);
                 rec3[2 * idx + 1] = -n_temp[l] / k.T;
             }
         }
@@ -861,7 +857,35 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
 
 // ------------------------------------------------------------------ far lines, FP64
 
-// One line at the nodes, the double-precision tiers of xs_device.cuh.
+// The wing polynomials in u = 1/|z|^2 (asy64_coeffs) with the fewest terms that all 32
+// lines of a warp allow: about 20 operations a line and node at |z| >= 150 (the generic
+// tiers with their divisions took 60 and more).
+
+template <int K>
+__device__ __forceinline__ void far_nodes64(double nb, double h, const double4_32a& p2, double amp,
+                                            double (&v)[Far<double>::n])
+{
+    double C[2 * K + 1];
+    asy64_coeffs<K>(p2.y, amp, C);
+    const double a2 = p2.y * p2.y;
+#pragma unroll
+    for (int m = 0; m < Far<double>::n; ++m) {
+        const double x = fma(h, cheb<Far<double>::n>(1, m), nb) * p2.x;
+        const double u = rcp64(fma(x, x, a2));
+        double p = C[2 * K];
+#pragma unroll
+        for (int n = 2 * K - 1; n >= 0; --n) p = fma(p, u, C[n]);
+        v[m] = fma(p, u, v[m]);
+    }
+}
+
+// |z|^2 of a line's nearest point of an interval
+__device__ __forceinline__ double nearest_z2(double nb, double h, const double4_32a& p2)
+{
+    const double x = fmax(fabs(nb) - h, 0.0) * p2.x;
+    return fma(x, x, p2.y * p2.y);
+}
+
 __device__ __forceinline__ double far_sum(const Lines<double>& ln, const FarList& fl, int t0, int t1, const Span& sp,
                                           float, int& idx)
 {
@@ -870,55 +894,72 @@ __device__ __forceinline__ double far_sum(const Lines<double>& ln, const FarList
     double v[n];
 #pragma unroll
     for (int m = 0; m < n; ++m) v[m] = 0.0;
-    for (int t = t0 + lane; t < t1; t += 32) {
-        const int l = fl.line(t);
+    for (int t = t0; t < t1; t += 32) {
+        const int l = fl.line(min(t + lane, t1 - 1));
         const double nb = sp.mid - ln.nu_hat[l];
         const double4_32a p2 = ln.r2[l];
-#pragma unroll
-        for (int m = 0; m < n; ++m) {
-            const double x = fabs(fma(sp.h, cheb<n>(1, m), nb)) * p2.x;
-            v[m] = fma(p2.z, voigt_H<double>(x, 0.0, p2.y, p2.w, nullptr), v[m]);
-        }
+        const double amp = t + lane < t1 ? p2.z : 0.0, z2 = nearest_z2(nb, sp.h, p2);
+        if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far))
+            far_nodes64<3>(nb, sp.h, p2, amp, v);
+        else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid))
+            far_nodes64<5>(nb, sp.h, p2, amp, v);
+        else
+            far_nodes64<12>(nb, sp.h, p2, amp, v);
     }
-    __syncwarp();
     return warp_reduce_scatter(v, idx);
 }
 
-__device__ __forceinline__ void adjoint_terms(double x, const double4_32a& p2, double aS, double hT, double nn,
-                                              double* ft, double* fb)
+// f_T and f_b from a line's V0, D_beta and D_gamma sums
+__device__ __forceinline__ void add_adjoint(double V0, double Db, double Dg, double aS, double hT, double nn, double& sT,
+                                            double& sB)
 {
-    double w4[4];
-    voigt_w_dw<double>(x, 0.0, p2.y, p2.w, w4, nullptr);
-    // H_x = Re w', H_a = -Im w'
-    const double V0 = p2.z * w4[0];
-    const double V1 = p2.z * x * w4[2];
-    const double V2 = -p2.z * p2.y * w4[3];
-    const double Db = -(V0 + V1 + V2);
-    *ft = aS * V0 + hT * Db + nn * V2;
-    *fb = V2;
+    sT += fma(aS, V0, fma(hT, Db, nn * Dg));
+    sB += Dg;
+}
+
+template <int K>
+__device__ __forceinline__ void far_adjoint64(double nb, double h, const double4_32a& p2, double amp, const double* lam,
+                                              double aS, double hT, double nn, double& sT, double& sB)
+{
+    double r[2 * K + 2];
+#pragma unroll
+    for (int k = 0; k < 2 * K + 2; ++k) r[k] = 0.0;
+    const double a2 = p2.y * p2.y;
+#pragma unroll 2
+    for (int m = 0; m < Far<double>::n; ++m) {
+        const double x = fma(h, cheb<Far<double>::n>(1, m), nb) * p2.x;
+        const double u = rcp64(fma(x, x, a2));
+        double q = lam[m] * u;
+#pragma unroll
+        for (int k = 0; k < 2 * K + 2; ++k) {
+            r[k] += q;
+            q *= u;
+        }
+    }
+    double V0, Db, Dg;
+    asy64_adjoint<K>(p2.y, amp, r, &V0, &Db, &Dg);
+    add_adjoint(V0, Db, Dg, aS, hT, nn, sT, sB);
 }
 
 __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const FarList& fl, int t0, int t1,
                                                 const Span& sp, float, const double* lam, double hT, double& sT,
                                                 double& sB)
 {
-    constexpr int n = Far<double>::n;
     const int lane = threadIdx.x & 31;
     sT = sB = 0.0;
-    for (int t = t0 + lane; t < t1; t += 32) {
-        const int l = fl.line(t);
+    for (int t = t0; t < t1; t += 32) {
+        const int l = fl.line(min(t + lane, t1 - 1));
         const double nb = sp.mid - ln.nu_hat[l];
         const double4_32a p2 = ln.r2[l];
         const double aS = ln.r3[2 * (size_t)l], nn = ln.r3[2 * (size_t)l + 1];
-#pragma unroll 1
-        for (int m = 0; m < n; ++m) {
-            double ft, fb;
-            adjoint_terms(fabs(fma(sp.h, cheb<n>(1, m), nb)) * p2.x, p2, aS, hT, nn, &ft, &fb);
-            sT = fma(lam[m], ft, sT);
-            sB = fma(lam[m], fb, sB);
-        }
+        const double amp = t + lane < t1 ? p2.z : 0.0, z2 = nearest_z2(nb, sp.h, p2);
+        if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far))
+            far_adjoint64<3>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
+        else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid))
+            far_adjoint64<5>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
+        else
+            far_adjoint64<12>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
     }
-    __syncwarp();
     sT = warp_sum(sT);
     sB = warp_sum(sB);
 }
@@ -1264,11 +1305,23 @@ struct NearAdjTile {
     float4 hf[32][4], hg[32][4]; // f_T and f_b wing polynomials (6 <= |z|)
     float sd[32][SER_TAB];
 };
+// FP64: 16 lines at a time.
+constexpr int NEAR64 = 16;
 struct NearTile64 {
-    double cen[32];
-    double4_32a r2[32];
-    double aS[32], nn[32];
-    int2 jr[32];
+    double cen[NEAR64];
+    double4_32a r2[NEAR64]; // c, a, Av, Kc
+    double ia[NEAR64];      // 1/a
+    int2 jr[NEAR64];
+    double C[NEAR64][2 * ASY64_K + 1];
+    double sd[NEAR64][SER64_TAB];
+};
+struct NearAdjTile64 {
+    double pos[LEAF], lam[LEAF]; // the leaf's points
+    double cen[NEAR64];
+    double4_32a r2[NEAR64];
+    double ia[NEAR64], aS[NEAR64], nn[NEAR64];
+    int2 jr[NEAR64];
+    double sd[NEAR64][SER64_TAB];
 };
 
 // |z|^2 from which the near lines take the wing polynomial in u = 1/|z|^2;
@@ -1432,13 +1485,48 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     if (lf.live) sigma[(size_t)layer * N + j] = (float)((far + ((double)shi + (double)slo)) * unscale);
 }
 
-// sigma of one leaf: FP64
+template <int K>
+__device__ __forceinline__ void stage_poly64(double a, double amp, double* dst)
+{
+    double C[2 * K + 1];
+    asy64_coeffs<K>(a, amp, C);
+#pragma unroll
+    for (int n = 0; n < 2 * K + 1; ++n) dst[n] = C[n];
+}
+template <int K>
+__device__ __forceinline__ double poly64(const double* C, double z2)
+{
+    const double u = rcp64(z2);
+    double p = C[2 * K];
+#pragma unroll
+    for (int n = 2 * K - 1; n >= 0; --n) p = fma(p, u, C[n]);
+    return p * u;
+}
+
+// sum over the staged lines at one point, wing polynomials of one length
+template <int K>
+__device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, double nuj, int j, bool masked)
+{
+    double acc = 0.0;
+    for (int q = 0; q < cnt; ++q) {
+        const double4_32a p2 = tl.r2[q];
+        const double x = (nuj - tl.cen[q]) * p2.x;
+        const double v = poly64<K>(tl.C[q], fma(x, x, p2.y * p2.y));
+        acc += (!masked || in_range(j, tl.jr[q])) ? v : 0.0;
+    }
+    return acc;
+}
+
+// sigma of one leaf: FP64.  Bound by FP64 operations: a chunk of 16 lines takes the
+// shortest wing polynomial that all of them allow, and the series only its own lanes.
+// (2,000 lines, 4,096 points, one layer: this kernel 3.1 ms with the generic tiers and one
+// exponential a term of the series.)
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
     Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ coef, double unscale, double* __restrict__ sigma)
 {
-    __shared__ NearTile64 tiles[LeafWarps<double>::v];
-    NearTile64& tl = tiles[threadIdx.x >> 5];
+    extern __shared__ __align__(32) unsigned char smem64[];
+    NearTile64& tl = ((NearTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<double> lf;
     if (!lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc)) return;
@@ -1449,22 +1537,48 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
     double acc = 0.0;
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
+        const bool masked = k != 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k]; t0 < ce; t0 += 32) {
+        for (int t0 = lf.s[k]; t0 < ce; t0 += NEAR64) {
             const int l = t0 + lane;
+            const bool have = lane < NEAR64 && l < ce;
             __syncwarp();
-            if (l < ce) {
-                tl.cen[lane] = ln.nu_hat[l];
-                tl.r2[lane] = ln.r2[l];
-                tl.jr[lane] = ln.jr[l];
+            double z2 = 1e300;
+            double4_32a p2{};
+            if (have) {
+                const double c = ln.nu_hat[l];
+                p2 = ln.r2[l];
+                z2 = nearest_z2(lf.g.mid - c, lf.g.h, p2);
+                tl.cen[lane] = c;
+                tl.r2[lane] = p2;
+                if (masked) tl.jr[lane] = ln.jr[l];
             }
-            __syncwarp();
-            const int cnt = min(32, ce - t0);
-            for (int q = 0; q < cnt; ++q) {
-                if (lf.live && in_range((int)j, tl.jr[q])) {
-                    const double4_32a p2 = tl.r2[q];
-                    const double x = fabs(nuj - tl.cen[q]) * p2.x;
-                    acc = fma(p2.z, voigt_H<double>(x, 0.0, p2.y, p2.w, nullptr), acc);
+            const int cnt = min(NEAR64, ce - t0);
+            if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far)) {
+                if (have) stage_poly64<3>(p2.y, p2.z, tl.C[lane]);
+                __syncwarp();
+                acc += near_poly64<3>(tl, cnt, nuj, (int)j, masked);
+            } else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid)) {
+                if (have) stage_poly64<5>(p2.y, p2.z, tl.C[lane]);
+                __syncwarp();
+                acc += near_poly64<5>(tl, cnt, nuj, (int)j, masked);
+            } else {
+                if (have) stage_poly64<ASY64_K>(p2.y, p2.z, tl.C[lane]);
+                if (have && z2 < Tier<double>::z2_series) {
+                    tl.ia[lane] = p2.y > 0.0 ? 1.0 / p2.y : 0.0;
+                    series_table64(p2.y, tl.sd[lane]);
+                }
+                __syncwarp();
+                for (int q = 0; q < cnt; ++q) {
+                    const bool in = lf.live && (!masked || in_range((int)j, tl.jr[q]));
+                    const double4_32a c4 = tl.r2[q];
+                    const double x = fabs(nuj - tl.cen[q]) * c4.x, zz = fma(x, x, c4.y * c4.y);
+                    if (in) {
+                        if (zz < Tier<double>::z2_series)
+                            acc = fma(c4.z, w_series_re(x, c4.y, tl.ia[q], c4.w, tl.sd[q]), acc);
+                        else
+                            acc += poly64<ASY64_K>(tl.C[q], zz);
+                    }
                 }
             }
         }
@@ -1642,13 +1756,44 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
     block_pair<LeafWarps<float>::v>(sT, sB, part + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
 }
 
+// Moments over half of the leaf's points (the lane's half) of lambda u^(n+1) for the lane's
+// line, where the point is inside the cut and at |z| >= 10, and the line's terms.
+template <int K>
+__device__ __forceinline__ void near_adjoint64(const NearAdjTile64& tl, int q, int half, double amp, bool masked, int jb,
+                                               double hT, double& sT, double& sB)
+{
+    double r[2 * K + 2];
+#pragma unroll
+    for (int k = 0; k < 2 * K + 2; ++k) r[k] = 0.0;
+    const double4_32a p2 = tl.r2[q];
+    const double c = tl.cen[q], a2 = p2.y * p2.y;
+    const int2 jr = tl.jr[q];
+    for (int i = half * (LEAF / 2); i < (half + 1) * (LEAF / 2); ++i) {
+        const double x = (tl.pos[i] - c) * p2.x, zz = fma(x, x, a2);
+        const bool in = (!masked || in_range(jb + i, jr)) && zz >= Tier<double>::z2_series;
+        const double u = rcp64(in ? zz : 1.0);
+        double s = in ? tl.lam[i] * u : 0.0;
+#pragma unroll
+        for (int k = 0; k < 2 * K + 2; ++k) {
+            r[k] += s;
+            s *= u;
+        }
+    }
+    double V0, Db, Dg;
+    asy64_adjoint<K>(p2.y, amp, r, &V0, &Db, &Dg);
+    add_adjoint(V0, Db, Dg, tl.aS[q], hT, tl.nn[q], sT, sB);
+}
+
+// FP64 adjoint of a leaf: the wing polynomials with a line (and half of the points) a
+// lane, so that a line's coefficients are applied once to its moments; the series with a
+// point a lane.
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
     Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
     double* __restrict__ part)
 {
-    __shared__ NearTile64 tiles[LeafWarps<double>::v];
-    NearTile64& tl = tiles[threadIdx.x >> 5];
+    extern __shared__ __align__(32) unsigned char smem64[];
+    NearAdjTile64& tl = ((NearAdjTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<double> lf;
@@ -1659,28 +1804,56 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
         const double nuj = nu[j];
         const double lam = lf.live ? g_sigma[(size_t)layer * N + j] * lam_scale : 0.0;
         const double hT = 0.5 / T[layer];
+        tl.pos[lane] = nuj;
+        tl.lam[lane] = lam;
 #pragma unroll 1
         for (int k = 0; k < 3; ++k) {
+            const bool masked = k != 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k]; t0 < ce; t0 += 32) {
+            for (int t0 = lf.s[k]; t0 < ce; t0 += NEAR64) {
                 const int l = t0 + lane;
+                const bool have = lane < NEAR64 && l < ce;
+                const int cnt = min(NEAR64, ce - t0);
                 __syncwarp();
-                if (l < ce) {
-                    tl.cen[lane] = ln.nu_hat[l];
-                    tl.r2[lane] = ln.r2[l];
-                    tl.jr[lane] = ln.jr[l];
+                double z2 = 1e300;
+                if (have) {
+                    const double c = ln.nu_hat[l];
+                    const double4_32a p2 = ln.r2[l];
+                    z2 = nearest_z2(lf.g.mid - c, lf.g.h, p2);
+                    tl.cen[lane] = c;
+                    tl.r2[lane] = p2;
                     tl.aS[lane] = ln.r3[2 * (size_t)l];
                     tl.nn[lane] = ln.r3[2 * (size_t)l + 1];
+                    if (masked) tl.jr[lane] = ln.jr[l];
+                    if (z2 < Tier<double>::z2_series) {
+                        tl.ia[lane] = p2.y > 0.0 ? 1.0 / p2.y : 0.0;
+                        series_table64(p2.y, tl.sd[lane]);
+                    }
                 }
+                unsigned near = __ballot_sync(0xffffffffu, z2 < Tier<double>::z2_series); // lines with series points
+                const bool far = __all_sync(0xffffffffu, z2 >= Tier<double>::z2_far);
+                const bool mid = __all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid);
                 __syncwarp();
-                const int cnt = min(32, ce - t0);
-                for (int q = 0; q < cnt; ++q) {
-                    if (lf.live && in_range((int)j, tl.jr[q])) {
-                        const double4_32a p2 = tl.r2[q];
-                        double ft, fb;
-                        adjoint_terms(fabs(nuj - tl.cen[q]) * p2.x, p2, tl.aS[q], hT, tl.nn[q], &ft, &fb);
-                        sT = fma(lam, ft, sT);
-                        sB = fma(lam, fb, sB);
+                const int q = min(lane % NEAR64, cnt - 1), half = lane / NEAR64;
+                const double amp = lane % NEAR64 < cnt ? tl.r2[q].z : 0.0;
+                if (far)
+                    near_adjoint64<3>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
+                else if (mid)
+                    near_adjoint64<5>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
+                else
+                    near_adjoint64<ASY64_K>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
+                while (near) {
+                    const int i = __ffs(near) - 1;
+                    near &= near - 1;
+                    const double4_32a c4 = tl.r2[i];
+                    const double x = fabs(nuj - tl.cen[i]) * c4.x, zz = fma(x, x, c4.y * c4.y);
+                    if (lf.live && zz < Tier<double>::z2_series && (!masked || in_range((int)j, tl.jr[i]))) {
+                        double wr, dr, di; // H_x = dr, H_a = -di
+                        w_series_deriv(x, c4.y, tl.ia[i], c4.w, tl.sd[i], &wr, &dr, &di);
+                        const double V0 = c4.z * wr, V2 = -c4.z * c4.y * di;
+                        const double Db = -(V0 + c4.z * x * dr + V2);
+                        sT = fma(lam, fma(tl.aS[i], V0, fma(hT, Db, tl.nn[i] * V2)), sT);
+                        sB = fma(lam, V2, sB);
                     }
                 }
             }
@@ -1954,6 +2127,14 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
         const dim3 lgrid((unsigned)p.leaf_blocks, (unsigned)lc);
         const dim3 fgrid((unsigned)p.far_blocks, (unsigned)lc);
         constexpr int lthreads = 32 * LeafWarps<R>::v;
+        if constexpr (!FAST) {
+            // beyond 48 KB of shared memory a block has to ask (cheap; per device)
+            if (cudaFuncSetAttribute(leaf_kernel_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(LeafWarps<double>::v * sizeof(NearTile64))) != cudaSuccess ||
+                cudaFuncSetAttribute(leaf_adjoint_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(LeafWarps<double>::v * sizeof(NearAdjTile64))) != cudaSuccess)
+                return XS_ECUDA;
+        }
         prof_begin(adjoint ? 1 : 0, st);
         if (!adjoint) {
             if (tr.on) {
@@ -1966,7 +2147,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
                 leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
                                                             (float*)sigma);
             else
-                leaf_kernel_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
+                leaf_kernel_f64<<<lgrid, lthreads, LeafWarps<double>::v * sizeof(NearTile64), st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
                                                             (double*)sigma);
         } else {
             if (tr.on) {
@@ -1979,7 +2160,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
                 leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
                                                              leaf);
             else
-                leaf_adjoint_f64<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
+                leaf_adjoint_f64<<<lgrid, lthreads, LeafWarps<double>::v * sizeof(NearAdjTile64), st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
                                                              leaf);
         }
         prof_end(adjoint ? 1 : 0, st);

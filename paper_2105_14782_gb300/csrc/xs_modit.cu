@@ -154,44 +154,6 @@ __global__ void modit_layer_kernel(int ng, double mass, double R0, const double*
     }
 }
 
-// e^v in FP64, table-driven (Tang 1989): 2^(i/64) from a table, the rest (|r| <= ln2/128)
-// by the series to r^5 (next term 4e-17): half the operations of exp.  Beyond +-700 exp.
-struct Exp2Table64 {
-    double t[64];
-};
-constexpr Exp2Table64 make_exp2_table64()
-{
-    Exp2Table64 r{};
-    const double ln2 = 0.69314718055994530942;
-    for (int i = 0; i < 64; ++i) {
-        // series of e^(i ln2/64) about the nearer end
-        const double x = (i <= 32 ? i : i - 64) * ln2 / 64;
-        double s = 1.0;
-        for (int k = 22; k >= 1; --k) s = 1.0 + s * x / k;
-        r.t[i] = i <= 32 ? s : 2.0 * s;
-    }
-    return r;
-}
-__device__ const Exp2Table64 EXP2_64 = make_exp2_table64();
-
-__device__ __forceinline__ double exp_tab(double v)
-{
-    if ((__double2hiint(v) & 0x7fffffff) >= 0x4085e000) return exp(v); // |v| >= 700, infinities, NaN
-    const double magic = 6755399441055744.0; // 1.5 2^52
-    // ln 2 = its float value (products with k are exact) + the rest
-    const double ln2_hi = (double)0.693147182f, ln2_lo = -1.904654299957767878541823e-9;
-    const double t = fma(v, 64.0 / 0.69314718055994530942, magic), kd = t - magic;
-    const int k = __double2loint(t);
-    const double r = fma(kd, -ln2_lo / 64, fma(kd, -ln2_hi / 64, v));
-    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    p = fma(r, p, 1.0 / 6.0);
-    p = fma(r, p, 0.5);
-    p = fma(r * r, p, r);
-    const double h = EXP2_64.t[k & 63];
-    const double s = fma(h, p, h);
-    return __hiloint2double(__double2hiint(s) + ((k >> 6) << 20), __double2loint(s));
-}
-
 // 1 - e^-u, u >= 0, given e = e^-u
 __device__ __forceinline__ double one_minus(double u, double e) { return u < 0.5 ? -expm1(-u) : 1.0 - e; }
 
