@@ -501,9 +501,8 @@ int model_adjoint_impl(const xs_model* m, const double* theta, const double* gF,
         // a species without lines has no kernel that adds its (zero) gradient
         if (m->method == XS_METHOD_MODIT && (r = xsi::rt_accumulate(gT, gTtmp, m->L, 0, st))) return r;
     }
-    if (per_layer) return xsi::rt_layer_grad(Sp, m->L, theta + 2, gT, gvmr, gb, out, st);
-    return xsi::rt_theta_grad(Sp, m->L, theta[0], theta[1], theta + 2, theta[2 + Sp], T, m->P_bar, gT, gvmr, gb, out,
-                              st);
+    if (per_layer) return xsi::rt_layer_grad(Sp, m->L, vmr, gT, gvmr, gb, out, st);
+    return xsi::rt_theta_grad(Sp, m->L, theta[0], vmr, T, m->P_bar, gT, gvmr, gb, out, st);
 }
 
 int model_args(const xs_model* m, const double* theta, void* workspace, size_t workspace_bytes, ModelPlan* p)

@@ -75,17 +75,17 @@ int rt_loglike(const double* F, const double* d, const double* s, int64_t N, dou
 // layer temperatures (T may be null) and mixing ratios (vmr may be null)
 int rt_atmosphere(double T0, double alpha, const double* P, int32_t L, double* T, int32_t S,
                   const double* log10_vmr_host, double* vmr, cudaStream_t st);
-int rt_theta_grad(int32_t S, int32_t L, double T0, double alpha, const double* log10_vmr_host, double sb,
-                  const double* T, const double* P, const double* g_T, const double* g_vmr, const double* g_b,
-                  double* out, cudaStream_t st);
+// vmr: the [S][L] mixing ratios of rt_atmosphere
+int rt_theta_grad(int32_t S, int32_t L, double T0, const double* vmr, const double* T, const double* P,
+                  const double* g_T, const double* g_vmr, const double* g_b, double* out, cudaStream_t st);
 int rt_tau_cia(const double* alpha, const double* Tg, int32_t nT, const double* T, const double* P, const double* dP,
                int32_t L, int64_t N, double vmr1, double vmr2, double g, double mu, int accumulate, double* dtau,
                cudaStream_t st);
 int rt_tau_cia_adjoint(const double* g_dtau, const double* alpha, const double* Tg, int32_t nT, const double* T,
                        const double* P, const double* dP, int32_t L, int64_t N, double vmr1, double vmr2, double g,
                        double mu, double* g_T, cudaStream_t st);
-int rt_layer_grad(int32_t S, int32_t L, const double* log10_vmr_host, const double* g_T, const double* g_vmr,
-                  const double* g_b, double* out, cudaStream_t st);
+int rt_layer_grad(int32_t S, int32_t L, const double* vmr, const double* g_T, const double* g_vmr, const double* g_b,
+                  double* out, cudaStream_t st);
 int rt_accumulate(double* dst, const double* src, int64_t n, int first, cudaStream_t st);
 
 } // namespace xsi

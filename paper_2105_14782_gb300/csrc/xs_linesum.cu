@@ -50,7 +50,7 @@ constexpr int LEAF = 32;       // grid points of a leaf: one per lane
 constexpr int LEVELS = 4;      // leaves and the intervals of 4, 16, 64 leaves
 constexpr int FAR_WARPS = 4;   // neighbouring intervals of one block share most lines
 
-// leaves per block of the leaf kernels
+// most warps of a leaf kernel's block (choose_leaf_blocks)
 template <class R> struct LeafWarps { static constexpr int v = 4; };
 template <> struct LeafWarps<double> { static constexpr int v = 8; };
 
@@ -68,6 +68,21 @@ template <> struct Far<double> {
 __device__ const ChebTable<10> CHEB10 = make_cheb<10>();
 __device__ const ChebTable<18> CHEB18 = make_cheb<18>();
 template <int n> __device__ __forceinline__ double cheb(int k, int m) { return (n == 10) ? CHEB10.T[k][m] : CHEB18.T[k][m]; }
+struct ChebTableF {
+    float T[10][10];
+};
+constexpr ChebTableF make_cheb_f()
+{
+    ChebTableF r{};
+    const ChebTable<10> c = make_cheb<10>();
+    for (int k = 0; k < 10; ++k)
+        for (int m = 0; m < 10; ++m) r.T[k][m] = (float)c.T[k][m];
+    return r;
+}
+__device__ const ChebTableF CHEB10F = make_cheb_f();
+// in the type of the path
+__device__ __forceinline__ float cheb_r(float, int k, int m) { return CHEB10F.T[k][m]; }
+__device__ __forceinline__ double cheb_r(double, int k, int m) { return CHEB18.T[k][m]; }
 // the nodes as literals for unrolled loops
 template <int n> struct NodeTable {
     float t[n];
@@ -1111,24 +1126,28 @@ struct LeafPoly<float> {
     }
 };
 
-// Polynomials of the leaves: per layer and top interval, the node sums of each level
-// plus the polynomial of the interval above.  coef[layer][leaf][n].
+// Polynomials of the leaves: the node sums of each level plus the polynomial of the
+// interval above, from the top interval down.  A block takes the leaves under one interval
+// of level `root` and repeats the chain of intervals above it: root = 3 (64 leaves, nothing
+// repeated) where that makes enough blocks to fill the chip, smaller subtrees otherwise.
 template <class R> struct DownRows { static constexpr int v = 64; }; // intervals of a level that a block takes at a time
 template <> struct DownRows<double> { static constexpr int v = 32; };
 template <class R>
 __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const __grid_constant__ Tree tr,
                                                                      const __grid_constant__ FarWork fw, int Lc,
-                                                                     const double* __restrict__ sums,
+                                                                     int root, const double* __restrict__ sums,
                                                                      double* __restrict__ coef)
 {
-    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1)), DOWN_ROWS = DownRows<R>::v;
-    __shared__ double v[DOWN_ROWS][n], c[2][TOP / 4][n];
-    const int m = threadIdx.x % n, row = threadIdx.x / n;
-    const int nloc = blockIdx.y, top = blockIdx.x;
+    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
+    __shared__ double v[DownRows<R>::v][n], c[2][TOP / 4][n];
+    const int m = threadIdx.x % n, row = threadIdx.x / n, rows = blockDim.x / n;
+    const int nloc = blockIdx.y;
     for (int k = LEVELS - 1; k >= 0; --k) {
-        const int many = 1 << (2 * (LEVELS - 1 - k)); // intervals of this level under the top one
-        for (int q0 = 0; q0 < many; q0 += DOWN_ROWS) {
-            const int q = q0 + row, i = top * many + q;
+        const int below = max(root - k, 0);
+        const int many = 1 << (2 * below);                                   // intervals of this level
+        const int first = k >= root ? blockIdx.x >> (2 * (k - root)) : blockIdx.x * many;
+        for (int q0 = 0; q0 < many; q0 += rows) {
+            const int q = q0 + row, i = first + q;
             const bool mine = q < many && i < tr.cnt[k];
             if (mine) {
                 double s = 0.0;
@@ -1176,7 +1195,7 @@ __device__ __forceinline__ R node_weight(const R* M, int m)
 {
     R s = R(0.5) * M[0];
 #pragma unroll
-    for (int k = 1; k < n; ++k) s += M[k] * (R)cheb<n>(k, m);
+    for (int k = 1; k < n; ++k) s += M[k] * cheb_r(R(0), k, m);
     return s * R(2.0 / n);
 }
 
@@ -1330,25 +1349,32 @@ constexpr float NEAR_POLY_Z2 = 36.0f;
 
 __device__ __forceinline__ bool in_range(int j, int2 r) { return j >= r.x && j <= r.y; }
 
-// A leaf: its points and its near lines as up to three ranges (the middle one inside
-// every line's cut, the outer ones masked per point).
+// A warp's leaf: its points and its near lines as up to three ranges (the middle one
+// inside every line's cut, the outer ones masked per point).  `split` neighbouring warps
+// of the block share a leaf and take every split-th chunk of its lines.
 template <class R>
 struct Leaf {
     int64_t jb, jl;
-    int lane, i;
-    bool live;
+    int lane, i, sub;
+    bool any, live; // the leaf has points; the lane has one
     int s[3], e[3];
     Geo g;
 
-    __device__ bool init(const Tree& tr, const double* nu_hat, int64_t nl, const double* nu, int64_t N, double W,
-                         int nloc)
+    __device__ void init(const Tree& tr, const double* nu_hat, int64_t nl, const double* nu, int64_t N, double W,
+                         int nloc, int split)
     {
+        const int w = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
-        i = blockIdx.x * LeafWarps<R>::v + (threadIdx.x >> 5);
+        i = (blockIdx.x * (blockDim.x >> 5) + w) / split;
+        sub = w % split;
         jb = (int64_t)i * LEAF;
-        if (jb >= N) return false;
         jl = min64(N - 1, jb + LEAF - 1);
-        live = jb + lane <= jl;
+        any = jb < N;
+        g = {0.0, 0.0, 0.0};
+        live = any && jb + lane <= jl;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] = e[k] = 0;
+        if (!any) return;
         if (tr.on) {
             g = tr.geo[i];
             const FarSet fs = far_set(tr, 0, i, nloc);
@@ -1365,31 +1391,44 @@ struct Leaf {
             if (lane == 1) v = first_line(nu_hat, nl, nu[jl], W, 0);
             s[0] = __shfl_sync(0xffffffffu, v, 0);
             e[0] = __shfl_sync(0xffffffffu, v, 1);
-            s[1] = e[1] = s[2] = e[2] = 0;
             g = {0.5 * (nu[jb] + nu[jl]), 0.5 * (nu[jl] - nu[jb]), 0.0};
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             if (!XS_CHECK(s[k] >= 0 && e[k] <= nl)) e[k] = s[k];
-        return true;
     }
 };
+
+// sum of v over the warps that share a leaf, valid in the first of them (fixed order)
+template <int warps>
+__device__ __forceinline__ double split_sum(double v, int split)
+{
+    __shared__ double part[warps][LEAF];
+    if (split == 1) return v;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    part[w][lane] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (w % split == 0)
+        for (int q = 0; q < split; ++q) s += part[w + q][lane];
+    return s;
+}
 
 // sigma of one leaf: FP32
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ coef, double unscale, float* __restrict__ sigma)
+    double W, int layer0, const double* __restrict__ coef, double unscale, int split, float* __restrict__ sigma)
 {
     __shared__ NearTile tiles[LeafWarps<float>::v];
     NearTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<float> lf;
-    if (!lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc)) return;
+    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
     const Lines<float> ln = layer_lines(lines, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
-    const Span sp(lf.g, nu[0]);
+    const Span sp(lf.g, nu[0]); // (a leaf without points has no lines either)
     const float rh = sp.rh, rl = sp.rl;
     const double oj = nuj - lf.g.mid;
     const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
@@ -1398,7 +1437,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     for (int k = 0; k < 3; ++k) {
         const bool masked = k != 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k]; t0 < ce; t0 += 32) {
+        for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
             const int l = t0 + lane;
             const bool have = l < ce;
             __syncwarp();
@@ -1479,10 +1518,12 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
             two_sum(shi, slo, acc); // the chunk's FP32 partial into the compensated sum
         }
     }
+    const double near = split_sum<LeafWarps<float>::v>((double)shi + (double)slo, split);
+    if (!lf.live || lf.sub) return;
     // the far lines' part
     const double far =
         tr.on ? LeafPoly<float>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
-    if (lf.live) sigma[(size_t)layer * N + j] = (float)((far + ((double)shi + (double)slo)) * unscale);
+    sigma[(size_t)layer * N + j] = (float)((far + near) * unscale);
 }
 
 template <int K>
@@ -1523,13 +1564,13 @@ __device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, dou
 // exponential a term of the series.)
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
     Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ coef, double unscale, double* __restrict__ sigma)
+    double W, int layer0, const double* __restrict__ coef, double unscale, int split, double* __restrict__ sigma)
 {
     extern __shared__ __align__(32) unsigned char smem64[];
     NearTile64& tl = ((NearTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<double> lf;
-    if (!lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc)) return;
+    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
     const Lines<double> ln = layer_lines(lines, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1539,7 +1580,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
     for (int k = 0; k < 3; ++k) {
         const bool masked = k != 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k]; t0 < ce; t0 += NEAR64) {
+        for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
             const int l = t0 + lane;
             const bool have = lane < NEAR64 && l < ce;
             __syncwarp();
@@ -1583,8 +1624,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
             }
         }
     }
+    acc = split_sum<LeafWarps<double>::v>(acc, split);
+    if (!lf.live || lf.sub) return;
     if (tr.on) acc += LeafPoly<double>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
-    if (lf.live) sigma[(size_t)layer * N + j] = acc * unscale;
+    sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
 // a block's sums of the leaves' (f_T, f_b) to part[layer][block], fixed order
@@ -1603,7 +1646,7 @@ __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
-        for (int i = 0; i < warps; ++i) {
+        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
             a += red[0][i];
             b += red[1][i];
         }
@@ -1615,14 +1658,15 @@ __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
     Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
-    double* __restrict__ part)
+    int split, double* __restrict__ part)
 {
     __shared__ NearAdjTile tiles[LeafWarps<float>::v];
     NearAdjTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<float> lf;
-    if (lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc)) {
+    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
+    if (lf.any) {
         const Lines<float> ln = layer_lines(lines, nl, nloc);
         const int lane = lf.lane;
         const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1638,7 +1682,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
         for (int k = 0; k < 3; ++k) {
             const bool masked = k != 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k]; t0 < ce; t0 += 32) {
+            for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
                 const int l = t0 + lane;
                 const bool have = l < ce;
                 __syncwarp();
@@ -1790,14 +1834,15 @@ __device__ __forceinline__ void near_adjoint64(const NearAdjTile64& tl, int q, i
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
     Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
     double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
-    double* __restrict__ part)
+    int split, double* __restrict__ part)
 {
     extern __shared__ __align__(32) unsigned char smem64[];
     NearAdjTile64& tl = ((NearAdjTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<double> lf;
-    if (lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc)) {
+    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
+    if (lf.any) {
         const Lines<double> ln = layer_lines(lines, nl, nloc);
         const int lane = lf.lane;
         const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1810,7 +1855,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
         for (int k = 0; k < 3; ++k) {
             const bool masked = k != 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k]; t0 < ce; t0 += NEAR64) {
+            for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
                 const int l = t0 + lane;
                 const bool have = lane < NEAR64 && l < ce;
                 const int cnt = min(NEAR64, ce - t0);
@@ -1925,7 +1970,7 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 constexpr int64_t TREE_MIN_LINES = 256;
 
 struct XsPlan {
-    int prec, Lc, nchunks, leaf_blocks;
+    int prec, Lc, nchunks, leaf_blocks, leaf_warps, leaf_split;
     Tree tree; // counts and offsets; pointers set at run time
     FarWork fw;
     int far_blocks;
@@ -1940,7 +1985,7 @@ struct XsPlan {
 // its own far radius and its parent's, about 16 interval lengths.
 void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
 {
-    const int64_t warps = mixed ? 10000 : 8000, min_lines = mixed ? 1024 : 128;
+    const int64_t warps = mixed ? 10000 : 8000, min_lines = mixed ? 1024 : 64;
     int block = 0;
     size_t row = 0;
     p->fw.slots = 0;
@@ -1961,6 +2006,26 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
     p->rows = row;
 }
 
+// Blocks of the leaf kernels.  With enough leaves, a warp each and full blocks; fewer
+// leaves than fill the chip share each leaf's lines between up to a block's warps and use
+// smaller blocks, so that the work reaches more SMs (one layer of 4,096 points has 128
+// leaves: in FP64, 16 blocks of 8 leaves took 616 us, 128 blocks with 8 warps on a leaf
+// 125 us; FP32, 32 blocks of 4 leaves 22 us, 128 blocks of one 14 us).
+void choose_leaf_blocks(XsPlan* p, int64_t N, int Lc, bool mixed, bool small)
+{
+    const int most = mixed ? LeafWarps<float>::v : LeafWarps<double>::v;
+    const int64_t leaves = (N + LEAF - 1) / LEAF, all = leaves * Lc;
+    const int64_t want = mixed ? 152 * 16 : 152 * 8; // warps
+    int split = 1;
+    while (!small && split < most && all * split < want) split *= 2;
+    int warps = most;
+    while (!small && warps > split && all * split / warps < 2 * 152) warps /= 2;
+    p->leaf_split = split;
+    p->leaf_warps = warps;
+    const int per = warps / split;
+    p->leaf_blocks = (int)((leaves + per - 1) / per);
+}
+
 XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
 {
     XsPlan p{};
@@ -1969,7 +2034,6 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     const bool mixed = (prec == XS_PREC_MIXED);
     const size_t rs = mixed ? sizeof(float) : sizeof(double);
     const int n = mixed ? Far<float>::n : Far<double>::n;
-    const int per_block = LEAF * (mixed ? LeafWarps<float>::v : LeafWarps<double>::v);
     const size_t n1 = (size_t)std::max<int64_t>(nl, 1);
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -1977,7 +2041,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
         off += align256(bytes);
         return o;
     };
-    p.leaf_blocks = (int)((N + per_block - 1) / per_block);
+    choose_leaf_blocks(&p, N, Lc, mixed, !tree); // the smallest workspaces hold one partial per full block
     p.off_jr = take(sizeof(int2) * n1);
     p.off_nuf = take(mixed ? sizeof(float2) * n1 : 0);
     p.off_inv = take(sizeof(double) * n1);
@@ -2126,7 +2190,7 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
         }
         const dim3 lgrid((unsigned)p.leaf_blocks, (unsigned)lc);
         const dim3 fgrid((unsigned)p.far_blocks, (unsigned)lc);
-        constexpr int lthreads = 32 * LeafWarps<R>::v;
+        const int lthreads = 32 * p.leaf_warps;
         if constexpr (!FAST) {
             // beyond 48 KB of shared memory a block has to ask (cheap; per device)
             if (cudaFuncSetAttribute(leaf_kernel_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2139,16 +2203,19 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
         if (!adjoint) {
             if (tr.on) {
                 far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, sums);
-                down_kernel<R><<<dim3(tops, (unsigned)lc), DownRows<R>::v * Far<R>::n, 0, st>>>(tr, p.fw, lc,
-                                                                                       sums, coef);
+                int root = LEVELS - 1;
+                while (root > 1 && (int64_t)tr.cnt[root] * lc < 2 * 152) --root;
+                const int rows = std::min(DownRows<R>::v, 1 << (2 * root));
+                down_kernel<R><<<dim3((unsigned)tr.cnt[root], (unsigned)lc), rows * Far<R>::n, 0, st>>>(
+                    tr, p.fw, lc, root, sums, coef);
                 count_launch(2);
             }
             if constexpr (FAST)
                 leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
-                                                            (float*)sigma);
+                                                            p.leaf_split, (float*)sigma);
             else
-                leaf_kernel_f64<<<lgrid, lthreads, LeafWarps<double>::v * sizeof(NearTile64), st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
-                                                            (double*)sigma);
+                leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
+                                                            p.leaf_split, (double*)sigma);
         } else {
             if (tr.on) {
                 up_kernel<R><<<dim3(tops, (unsigned)lc), 32 * UP_WARPS, 0, st>>>(tr, nu, N, l0, g_sigma, unscale, wts);
@@ -2158,10 +2225,10 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
             }
             if constexpr (FAST)
                 leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
-                                                             leaf);
+                                                             p.leaf_split, leaf);
             else
-                leaf_adjoint_f64<<<lgrid, lthreads, LeafWarps<double>::v * sizeof(NearAdjTile64), st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
-                                                             leaf);
+                leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
+                                                             p.leaf_split, leaf);
         }
         prof_end(adjoint ? 1 : 0, st);
         count_launch();

@@ -119,20 +119,27 @@ struct GSigPtrs {
     double* p[XS_MAX_SPECIES];
 };
 
+// A row of a layer per block row: the layer's factors are formed once a block (a division
+// for them and one of the index an element before: 101 x 49,999, two species, 236 us).
 __global__ void tau_kernel(SigPtrs sig, int S, const double* __restrict__ vmr, const double* __restrict__ P,
                            const double* __restrict__ dP, int L, int64_t N, double g, double mu, double kappa,
                            int is_float, double* __restrict__ dtau)
 {
-    int64_t total = (int64_t)L * N;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int n = (int)(i / N);
-        double col = dP[n] * 1e6 / (mu * amu * g);
-        double s = 0.0;
-        for (int m = 0; m < S; ++m) {
-            double v = is_float ? (double)((const float*)sig.p[m])[i] : ((const double*)sig.p[m])[i];
-            s += vmr[(size_t)m * L + n] * v;
+    __shared__ double f[XS_MAX_SPECIES + 1];
+    for (int64_t n = blockIdx.y; n < L; n += gridDim.y) {
+        __syncthreads();
+        if (threadIdx.x <= S) {
+            const int m = threadIdx.x;
+            f[m] = m < S ? dP[n] * 1e6 / (mu * amu * g) * vmr[(size_t)m * L + n] : kappa * P[n] * dP[n] * 1e6 / g;
         }
-        dtau[i] = col * s + kappa * P[n] * dP[n] * 1e6 / g;
+        __syncthreads();
+        for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
+            const size_t i = (size_t)n * N + j;
+            double s = f[S];
+            for (int m = 0; m < S; ++m)
+                s = fma(f[m], is_float ? (double)((const float*)sig.p[m])[i] : ((const double*)sig.p[m])[i], s);
+            dtau[i] = s;
+        }
     }
 }
 
@@ -392,7 +399,7 @@ __device__ __forceinline__ double warp_sum(double v)
 //   log10 vmr_m: ln10 sum_n g_vmr[m][n] vmr_m
 //   broadening scale: sum_m g_b[m]
 // (100 layers: 200 us when one thread did it.)
-__global__ void theta_grad_kernel(int S, int L, double T0, VmrArgs a, const double* __restrict__ T,
+__global__ void theta_grad_kernel(int S, int L, double T0, const double* __restrict__ vmr, const double* __restrict__ T,
                                   const double* __restrict__ P, const double* __restrict__ g_T,
                                   const double* __restrict__ g_vmr, const double* __restrict__ g_b,
                                   double* __restrict__ out)
@@ -411,7 +418,7 @@ __global__ void theta_grad_kernel(int S, int L, double T0, VmrArgs a, const doub
         double s = 0.0;
         for (int n = lane; n < L; n += 32) s += g_vmr[(size_t)m * L + n];
         s = warp_sum(s);
-        if (lane == 0) out[3 + m] = 2.30258509299404568402 * pow(10.0, a.lg[m]) * s;
+        if (lane == 0) out[3 + m] = 2.30258509299404568402 * vmr[(size_t)m * L] * s;
         gb += g_b[m];
     }
     if (lane == 0) {
@@ -498,7 +505,7 @@ __global__ void tau_cia_adjoint_kernel(const double* __restrict__ g_dtau, const 
 
 // Gradient for per-layer temperatures: out[1 + n] = dlogL/dT_n, then
 // dlogL/dlog10 vmr_m and dlogL/ds_b (out[0], logL, is left as it is).
-__global__ void layer_grad_kernel(int S, int L, VmrArgs a, const double* __restrict__ g_T,
+__global__ void layer_grad_kernel(int S, int L, const double* __restrict__ vmr, const double* __restrict__ g_T,
                                   const double* __restrict__ g_vmr, const double* __restrict__ g_b,
                                   double* __restrict__ out)
 {
@@ -509,7 +516,7 @@ __global__ void layer_grad_kernel(int S, int L, VmrArgs a, const double* __restr
         double s = 0.0;
         for (int n = lane; n < L; n += 32) s += g_vmr[(size_t)m * L + n];
         s = warp_sum(s);
-        if (lane == 0) out[1 + L + m] = 2.30258509299404568402 * pow(10.0, a.lg[m]) * s;
+        if (lane == 0) out[1 + L + m] = 2.30258509299404568402 * vmr[(size_t)m * L] * s;
         gb += g_b[m];
     }
     if (lane == 0) out[1 + L + S] = gb;
@@ -534,18 +541,13 @@ static inline int launched(int n)
     return last_status();
 }
 
-static unsigned grid_for(int64_t total)
-{
-    int64_t b = (total + RT_THREADS - 1) / RT_THREADS;
-    return (unsigned)std::min<int64_t>(std::max<int64_t>(b, 1), 152 * 32);
-}
-
 int rt_tau(const void* const* sigma, int32_t S, const double* vmr, const double* P, const double* dP, int32_t L,
            int64_t N, double g, double mu, double kappa, int prec, double* dtau, cudaStream_t st)
 {
     SigPtrs sp{};
     for (int m = 0; m < S; ++m) sp.p[m] = sigma[m];
-    tau_kernel<<<grid_for((int64_t)L * N), RT_THREADS, 0, st>>>(sp, S, vmr, P, dP, L, N, g, mu, kappa,
+    const unsigned gx = (unsigned)std::min<int64_t>((N + 4 * RT_THREADS - 1) / (4 * RT_THREADS), 1024);
+    tau_kernel<<<dim3(gx, (unsigned)std::min(L, 65535)), RT_THREADS, 0, st>>>(sp, S, vmr, P, dP, L, N, g, mu, kappa,
                                                                  prec == XS_PREC_MIXED, dtau);
     return launched(1);
 }
@@ -614,15 +616,10 @@ int rt_atmosphere(double T0, double alpha, const double* P, int32_t L, double* T
     return launched(1);
 }
 
-int rt_theta_grad(int32_t S, int32_t L, double T0, double alpha, const double* lg, double sb, const double* T,
-                  const double* P, const double* g_T, const double* g_vmr, const double* g_b, double* out,
-                  cudaStream_t st)
+int rt_theta_grad(int32_t S, int32_t L, double T0, const double* vmr, const double* T, const double* P,
+                  const double* g_T, const double* g_vmr, const double* g_b, double* out, cudaStream_t st)
 {
-    (void)alpha;
-    (void)sb;
-    VmrArgs a{};
-    for (int m = 0; m < S; ++m) a.lg[m] = lg[m];
-    theta_grad_kernel<<<1, 32, 0, st>>>(S, L, T0, a, T, P, g_T, g_vmr, g_b, out);
+    theta_grad_kernel<<<1, 32, 0, st>>>(S, L, T0, vmr, T, P, g_T, g_vmr, g_b, out);
     return launched(1);
 }
 
@@ -650,12 +647,10 @@ int rt_tau_cia_adjoint(const double* g_dtau, const double* alpha, const double* 
     return launched(1);
 }
 
-int rt_layer_grad(int32_t S, int32_t L, const double* lg, const double* g_T, const double* g_vmr, const double* g_b,
+int rt_layer_grad(int32_t S, int32_t L, const double* vmr, const double* g_T, const double* g_vmr, const double* g_b,
                   double* out, cudaStream_t st)
 {
-    VmrArgs a{};
-    for (int m = 0; m < S; ++m) a.lg[m] = lg[m];
-    layer_grad_kernel<<<1, 32, 0, st>>>(S, L, a, g_T, g_vmr, g_b, out);
+    layer_grad_kernel<<<1, 32, 0, st>>>(S, L, vmr, g_T, g_vmr, g_b, out);
     return launched(1);
 }
 
