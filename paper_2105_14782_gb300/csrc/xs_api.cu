@@ -202,8 +202,8 @@ int xs_compute(const xs_lines* lines, const double* nu, int64_t N, const double*
     if (r) return r;
     if (!sigma || !workspace) return XS_EINVAL;
     if (workspace_bytes < xs_workspace_min_bytes(lines->n, N, L, prec)) return XS_EINVAL;
-    return xsi::xs_run(lines, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, sigma, workspace, workspace_bytes,
-                       false, nullptr, nullptr, nullptr, S(stream));
+    const xsi::XsJob job{lines, workspace, workspace_bytes, sigma, nullptr, nullptr, nullptr};
+    return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, false, S(stream));
 }
 
 int xs_compute_adjoint(const xs_lines* lines, const double* nu, int64_t N, const double* T, const double* P_bar,
@@ -215,8 +215,8 @@ int xs_compute_adjoint(const xs_lines* lines, const double* nu, int64_t N, const
     if (r) return r;
     if (!g_sigma || !g_T || !g_broad || !workspace) return XS_EINVAL;
     if (workspace_bytes < xs_workspace_min_bytes(lines->n, N, L, prec)) return XS_EINVAL;
-    return xsi::xs_run(lines, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, nullptr, workspace, workspace_bytes,
-                       true, g_sigma, g_T, g_broad, S(stream));
+    const xsi::XsJob job{lines, workspace, workspace_bytes, nullptr, g_sigma, g_T, g_broad};
+    return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, true, S(stream));
 }
 
 int tau_layers(const void* const* sigma, int32_t nsp, const double* vmr, const double* P_bar, const double* dP_bar,
@@ -367,7 +367,7 @@ ModelPlan plan_model(const xs_model* m)
     p.gsig = take(sizeof(double) * LN * Sp);
     p.gvmr = take(sizeof(double) * Sp * m->L);
     p.gT = take(sizeof(double) * m->L);
-    p.gTtmp = take(sizeof(double) * m->L);
+    p.gTtmp = take(sizeof(double) * Sp * m->L);
     p.gb = take(sizeof(double) * Sp);
     // one full workspace per species, so the forward's line records stay valid
     // for the adjoint of the same call
@@ -406,18 +406,20 @@ int model_forward_impl(const xs_model* m, const double* theta, double* F0out, ch
     r = xsi::rt_atmosphere(theta[0], theta[1], m->P_bar, m->L, T_given ? nullptr : T, Sp, theta + 2, vmr, st);
     if (r) return r;
     const void* sp[XS_MAX_SPECIES];
+    xsi::XsJob job[XS_MAX_SPECIES];
     for (int s = 0; s < Sp; ++s) {
         sp[s] = sig + es * LN * s;
-        if (m->method == XS_METHOD_MODIT)
-            r = xsi::modit_forward(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
-                                   m->n_gamma, m->n_fft[s], m->prec, (void*)sp[s], ws + p.xsws_sp[s],
-                                   p.xsws_sp_bytes[s], st, xs_flags);
-        else
-            r = xsi::xs_run(&m->species[s], m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec,
-                            (void*)sp[s], ws + p.xsws_sp[s], p.xsws_sp_bytes[s], false, nullptr, nullptr, nullptr, st,
-                            xs_flags);
-        if (r) return r;
+        job[s] = {&m->species[s], ws + p.xsws_sp[s], p.xsws_sp_bytes[s], sig + es * LN * s, nullptr, nullptr, nullptr};
+        if (m->method == XS_METHOD_MODIT &&
+            (r = xsi::modit_forward(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
+                                    m->n_gamma, m->n_fft[s], m->prec, (void*)sp[s], ws + p.xsws_sp[s],
+                                    p.xsws_sp_bytes[s], st, xs_flags)))
+            return r;
     }
+    if (m->method != XS_METHOD_MODIT &&
+        (r = xsi::xs_run(Sp, job, m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec, false, st,
+                         xs_flags)))
+        return r;
     r = xsi::rt_tau(sp, Sp, vmr, m->P_bar, m->dP_bar, m->L, m->N, m->gravity, m->mu, m->kappa_coef, m->prec, dtau, st);
     if (r) return r;
     if (m->cia_alpha) {
@@ -488,19 +490,21 @@ int model_adjoint_impl(const xs_model* m, const double* theta, const double* gF,
     if ((r = xsi::rt_tau_adjoint(sp, Sp, vmr, m->P_bar, m->dP_bar, m->L, m->N, m->gravity, m->mu, m->prec, gdtau, gsp,
                                  gvmr, st)))
         return r;
+    xsi::XsJob job[XS_MAX_SPECIES];
     for (int s = 0; s < Sp; ++s) {
-        if (m->method == XS_METHOD_MODIT)
-            r = xsi::modit_adjoint(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
-                                   m->n_gamma, m->n_fft[s], m->prec, gsp[s], gTtmp, gb + s, ws + p.xsws_sp[s],
-                                   p.xsws_sp_bytes[s], st, xsi::XS_RUN_REUSE);
-        else
-            r = xsi::xs_run(&m->species[s], m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec,
-                            nullptr, ws + p.xsws_sp[s], p.xsws_sp_bytes[s], true, gsp[s], gTtmp, gb + s, st,
-                            xsi::XS_RUN_REUSE, gT);
-        if (r) return r;
-        // a species without lines has no kernel that adds its (zero) gradient
-        if (m->method == XS_METHOD_MODIT && (r = xsi::rt_accumulate(gT, gTtmp, m->L, 0, st))) return r;
+        double* gTs = gTtmp + (size_t)s * m->L;
+        job[s] = {&m->species[s], ws + p.xsws_sp[s], p.xsws_sp_bytes[s], nullptr, gsp[s], gTs, gb + s};
+        if (m->method == XS_METHOD_MODIT &&
+            ((r = xsi::modit_adjoint(&m->species[s], m->nu_min, m->nu_max, m->N, T, m->P_bar, m->L, theta[2 + Sp],
+                                     m->n_gamma, m->n_fft[s], m->prec, gsp[s], gTs, gb + s, ws + p.xsws_sp[s],
+                                     p.xsws_sp_bytes[s], st, xsi::XS_RUN_REUSE)) ||
+             (r = xsi::rt_accumulate(gT, gTs, m->L, 0, st))))
+            return r;
     }
+    if (m->method != XS_METHOD_MODIT &&
+        (r = xsi::xs_run(Sp, job, m->nu, m->N, T, m->P_bar, m->L, theta[2 + Sp], m->wing_cut, m->prec, true, st,
+                         xsi::XS_RUN_REUSE, gT)))
+        return r;
     if (per_layer) return xsi::rt_layer_grad(Sp, m->L, vmr, gT, gvmr, gb, out, st);
     return xsi::rt_theta_grad(Sp, m->L, theta[0], vmr, T, m->P_bar, gT, gvmr, gb, out, st);
 }

@@ -42,11 +42,21 @@ int check_lines(const xs_lines* ln);
 int check_common(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L,
                  double sb, double W, int prec);
 
-// line-sum forward (adjoint == false: writes sigma) or adjoint (writes g_T, g_b, and adds
-// g_T to g_T_sum where that is given); flags as above (0 for a self-contained call)
-int xs_run(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
-           double W, int prec, void* sigma, void* ws, size_t ws_bytes, bool adjoint, const double* g_sigma,
-           double* g_T, double* g_b, cudaStream_t st, int flags = 0, double* g_T_sum = nullptr);
+// One species of a line-sum call.
+struct XsJob {
+    const xs_lines* lines;
+    void* ws;
+    size_t ws_bytes;
+    void* sigma;           // forward: output
+    const double* g_sigma; // adjoint: input,
+    double *g_T, *g_b;     // and outputs [L] and [1]
+};
+
+// line sums of n species (adjoint == false: writes sigma) or their adjoints (writes g_T
+// and g_b, and adds every g_T to g_T_sum where that is given); flags as above (0 for a
+// self-contained call)
+int xs_run(int n, const XsJob* job, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
+           double W, int prec, bool adjoint, cudaStream_t st, int flags = 0, double* g_T_sum = nullptr);
 
 // MODIT forward and adjoint with the composite model's flags (KEEP_ADJ, REUSE as above)
 int modit_forward(const xs_lines* lines, double nu_min, double nu_max, int64_t N, const double* T, const double* P_bar,

@@ -111,6 +111,62 @@ struct Tree {
     int on;             // 0: no intervals (small workspaces): every line is near
 };
 
+// Line arrays of one layer.
+template <class R>
+struct Lines {
+    using R4 = typename vec4<R>::type;
+    const double* nu_hat;
+    const float2* nuf; // centre - nu[0] as hi + lo floats (FP32)
+    const int2* jr;
+    const R4 *r1, *r2;
+    const R* r3;
+    const R* clo;
+};
+
+// Work of the far kernels: blocks of FAR_WARPS neighbouring intervals of a level and
+// one part of their lists, largest intervals (longest lists) first.
+struct FarWork {
+    int parts[LEVELS], block0[LEVELS]; // block0: first block of the level
+    size_t out0[LEVELS];               // first node-sum row of the level (in rows of n)
+    int slot0[LEVELS], slots;          // first adjoint slot of the level, slots per layer
+};
+
+// One species of a launch: its lists, workspace arrays and plan.  The line sums of a
+// model's species are independent of one another and run in the same launches
+// (blockIdx.z), which halves the launches of a two-species step and fills the chip with
+// the blocks of both.
+template <class R>
+struct Species {
+    using R4 = typename vec4<R>::type;
+    Lines<R> ln;
+    const double *inv_nu, *ln_S0, *elower, *gamma_ref, *n_temp;
+    double mass, qexp;
+    int64_t nl;
+    Tree tree;
+    FarWork fw;
+    int setup_blocks, param_blocks, far_blocks;
+    // per-call arrays (the same memory as the const pointers above)
+    int2* jr;
+    float2* nuf;
+    double* w_inv_nu;
+    float* agg;
+    R4 *rec1, *rec2;
+    R *rec3, *clo;
+    Geo* geo;
+    int2 *cov, *win, *pq;
+    double *sums, *coef; // forward: node sums, leaf polynomials
+    R* wts;              // adjoint: node weights,
+    double *slots, *leaf, *gbl; // and the partials of the far, the leaf and the reduction kernel
+    void* sigma;
+    const double* g_sigma;
+    double *g_T, *g_b;
+};
+template <class R>
+struct Batch {
+    Species<R> s[XS_MAX_SPECIES];
+    int n;
+};
+
 // ------------------------------------------------------------------ setup
 
 // lo if upper == 0: first grid index with nu_j - c >= -W; else the last with nu_j - c <= W
@@ -142,29 +198,31 @@ __device__ __forceinline__ int first_line(const double* nu_hat, int64_t nl, doub
 // One thread per search: cut ranges of the lines (two each) and their centres
 // relative to the first grid point as float pairs, the intervals' line ranges (four
 // each) and geometry, and the start values of the per-layer minima.
-__global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, const double* __restrict__ nu, int64_t N,
-                             double W, int2* __restrict__ jr, float2* __restrict__ nuf,
-                             double* __restrict__ inv_nu, float* __restrict__ agg,
-                             int n_agg, const __grid_constant__ Tree tr, Geo* __restrict__ geo, int2* __restrict__ cov,
-                             int2* __restrict__ win)
+template <class R>
+__global__ void setup_kernel(const __grid_constant__ Batch<R> batch, const double* __restrict__ nu, int64_t N, double W,
+                             int n_agg)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    const double* __restrict__ nu_hat = sp.ln.nu_hat;
+    const int64_t nl = sp.nl;
+    const Tree& tr = sp.tree;
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < 2 * nl) {
         const int64_t l = t >> 1;
         const int upper = (int)(t & 1);
         const double c = nu_hat[l];
-        ((int*)jr)[t] = cut_index(nu, N, c, W, upper);
-        if (!upper) inv_nu[l] = 1.0 / c;
-        if (nuf && upper) {
+        ((int*)sp.jr)[t] = cut_index(nu, N, c, W, upper);
+        if (!upper) sp.w_inv_nu[l] = 1.0 / c;
+        if (sp.nuf && upper) {
             const double o = c - nu[0];
             const float h = (float)o;
-            nuf[l] = make_float2(h, (float)(o - (double)h));
+            sp.nuf[l] = make_float2(h, (float)(o - (double)h));
         }
         return;
     }
     t -= 2 * nl;
     if (t < n_agg) {
-        agg[t] = __int_as_float(0x7f800000); // +inf: minima
+        sp.agg[t] = __int_as_float(0x7f800000); // +inf: minima
         return;
     }
     t -= n_agg;
@@ -177,15 +235,15 @@ __global__ void setup_kernel(const double* __restrict__ nu_hat, int64_t nl, cons
     const double v0 = nu[j0], v1 = nu[j1];
     if (which == 0) {
         const double h = 0.5 * (v1 - v0);
-        geo[q] = {0.5 * (v0 + v1), h, h > 0.0 ? 1.0 / h : 0.0};
-        cov[q].x = first_line(nu_hat, nl, v1, W, 1); // covers v1 from its lower side on
+        sp.geo[q] = {0.5 * (v0 + v1), h, h > 0.0 ? 1.0 / h : 0.0};
+        sp.cov[q].x = first_line(nu_hat, nl, v1, W, 1); // covers v1 from its lower side on
     } else if (which == 1) {
-        cov[q].y = first_line(nu_hat, nl, v0, W, 0); // first that no longer reaches v0
+        sp.cov[q].y = first_line(nu_hat, nl, v0, W, 0); // first that no longer reaches v0
     } else if (k == 0) {
         if (which == 2)
-            win[q].x = first_line(nu_hat, nl, v0, W, 1);
+            sp.win[q].x = first_line(nu_hat, nl, v0, W, 1);
         else
-            win[q].y = first_line(nu_hat, nl, v1, W, 0);
+            sp.win[q].y = first_line(nu_hat, nl, v1, W, 0);
     }
 }
 
@@ -304,13 +362,26 @@ __device__ __forceinline__ void exp_pair(double v, const float* tab, int* e, flo
 // FP32 path run in FP32: about 20 FP64 operations and conversions a line instead of about
 // 200 (220,000 lines x 100 layers: 6.9 ms before).
 template <class R>
-__global__ void __launch_bounds__(256) line_params_kernel(
-    const double* __restrict__ nu_hat, const double* __restrict__ inv_nu, const double* __restrict__ ln_S0,
-    const double* __restrict__ elower, const double* __restrict__ gamma_ref, const double* __restrict__ n_temp,
-    int64_t nl, double mass, double qexp, const double* __restrict__ T, const double* __restrict__ P_bar, int layer0,
-    double sb, typename vec4<R>::type* __restrict__ rec1, typename vec4<R>::type* __restrict__ rec2,
-    R* __restrict__ clo, R* __restrict__ rec3, float* __restrict__ agg)
+__global__ void __launch_bounds__(256) line_params_kernel(const __grid_constant__ Batch<R> batch,
+                                                          const double* __restrict__ T,
+                                                          const double* __restrict__ P_bar, int layer0, double sb,
+                                                          bool want_rec3)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    if ((int)blockIdx.x >= sp.param_blocks) return;
+    const double* __restrict__ nu_hat = sp.ln.nu_hat;
+    const double* __restrict__ inv_nu = sp.inv_nu;
+    const double* __restrict__ ln_S0 = sp.ln_S0;
+    const double* __restrict__ elower = sp.elower;
+    const double* __restrict__ gamma_ref = sp.gamma_ref;
+    const double* __restrict__ n_temp = sp.n_temp;
+    const int64_t nl = sp.nl;
+    const double mass = sp.mass, qexp = sp.qexp;
+    auto* __restrict__ rec1 = sp.rec1;
+    auto* __restrict__ rec2 = sp.rec2;
+    R* __restrict__ clo = sp.clo;
+    R* __restrict__ rec3 = want_rec3 ? sp.rec3 : nullptr;
+    float* __restrict__ agg = sp.agg;
     constexpr bool FAST = std::is_same<R, float>::value;
     __shared__ LayerConst lc;
     __shared__ float tab[128];
@@ -324,7 +395,7 @@ __global__ void __launch_bounds__(256) line_params_kernel(
     const LayerConst k = lc;
     const float lnTr = (float)k.lnTr, Tf = (float)k.T;
     float cmin = __int_as_float(0x7f800000), amin = cmin, gmin = cmin;
-    for (int64_t l = (int64_t)blockIdx.x * 256 + threadIdx.x; l < nl; l += (int64_t)gridDim.x * 256) {
+    for (int64_t l = (int64_t)blockIdx.x * 256 + threadIdx.x; l < nl; l += (int64_t)sp.param_blocks * 256) {
         const double nuh = nu_hat[l], E = elower[l];
         const double c = FAST ? k.kc * inv_nu[l] : 1.0 / (SQRT2 * (k.bk * nuh / cL));
         const R cr = (R)c;
@@ -413,15 +484,18 @@ __device__ __forceinline__ double far_radius(double h, double cmin, double amin,
 
 // pq[layer][interval]: lines with |centre - middle| below the far radius
 template <class R>
-__global__ void near_range_kernel(const double* __restrict__ nu_hat, int64_t nl, const __grid_constant__ Tree tr, const float* __restrict__ agg,
-                                  int layer0, int2* __restrict__ pq)
+__global__ void near_range_kernel(const __grid_constant__ Batch<R> batch, int layer0)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    const double* __restrict__ nu_hat = sp.ln.nu_hat;
+    const int64_t nl = sp.nl;
+    const Tree& tr = sp.tree;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 2 * (int64_t)tr.total) return;
     const int q = (int)(t >> 1), n = blockIdx.y;
     const bool upper = t & 1;
     const Geo g = tr.geo[q];
-    const float* ag = agg + 4 * (layer0 + n);
+    const float* ag = sp.agg + 4 * (layer0 + n);
     const double r = far_radius<R>(g.h, ag[0], ag[1], ag[2]);
     const double v = upper ? g.mid + r : g.mid - r;
     int64_t lo = 0, hi = nl; // first line with centre >= v (upper) or > v
@@ -429,7 +503,7 @@ __global__ void near_range_kernel(const double* __restrict__ nu_hat, int64_t nl,
         const int64_t m = (lo + hi) >> 1;
         if (upper ? nu_hat[m] >= v : nu_hat[m] > v) hi = m; else lo = m + 1;
     }
-    ((int*)pq)[2 * (size_t)tr.total * n + t] = (int)lo;
+    ((int*)sp.pq)[2 * (size_t)tr.total * n + t] = (int)lo;
 }
 
 // Far lines of an interval: [a, p) and [q, b); its parent's, [A, P) and [Q, B), are
@@ -599,18 +673,6 @@ __device__ __forceinline__ float2 horner13_2(const float (&C)[ASY_N], float2 u)
     for (int n = ASY_N - 2; n >= 0; --n) p = __ffma2_rn(p, v, dup(C[n]));
     return __fmul2_rn(p, u);
 }
-
-// Line arrays of one layer.
-template <class R>
-struct Lines {
-    using R4 = typename vec4<R>::type;
-    const double* nu_hat;
-    const float2* nuf; // centre - nu[0] as hi + lo floats (FP32)
-    const int2* jr;
-    const R4 *r1, *r2;
-    const R* r3;
-    const R* clo;
-};
 
 // An interval as the warps see it.
 struct Span {
@@ -981,14 +1043,6 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
 
 // ------------------------------------------------------------------ far kernels
 
-// Work of the far kernels: blocks of FAR_WARPS neighbouring intervals of a level and
-// one part of their lists, largest intervals (longest lists) first.
-struct FarWork {
-    int parts[LEVELS], block0[LEVELS]; // block0: first block of the level
-    size_t out0[LEVELS];               // first node-sum row of the level (in rows of n)
-    int slot0[LEVELS], slots;          // first adjoint slot of the level, slots per layer
-};
-
 __device__ __forceinline__ bool far_task(const Tree& tr, const FarWork& fw, int* level, int* i, int* part)
 {
     int k = 0;
@@ -1020,50 +1074,59 @@ __device__ __forceinline__ Lines<R> layer_lines(Lines<R> ln, int64_t nl, int nlo
 }
 
 template <class R>
-__global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(Lines<R> lines, int64_t nl, const __grid_constant__ Tree tr, const __grid_constant__ FarWork fw,
-                                                                 const float* __restrict__ agg,
-                                                                 const double* __restrict__ nu, int layer0,
-                                                                 double* __restrict__ sums)
+__global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(const __grid_constant__ Batch<R> batch,
+                                                                 const double* __restrict__ nu, int layer0)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    if ((int)blockIdx.x >= sp.far_blocks) return;
+    const Tree& tr = sp.tree;
+    const FarWork& fw = sp.fw;
+    const int64_t nl = sp.nl;
     constexpr int n = Far<R>::n;
     int k, i, part;
     if (!far_task(tr, fw, &k, &i, &part)) return;
     const int nloc = blockIdx.y;
-    const Lines<R> ln = layer_lines(lines, nl, nloc);
+    const Lines<R> ln = layer_lines(sp.ln, nl, nloc);
     const FarSet fs = far_set(tr, k, i, nloc);
     const FarList fl(fs);
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
     if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
     int idx;
-    const double s = far_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * (layer0 + nloc)], idx);
+    const double s = far_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), sp.agg[4 * (layer0 + nloc)],
+                             idx);
     const size_t row = fw.out0[k] + ((size_t)part * gridDim.y + nloc) * tr.cnt[k] + i;
-    if (idx >= 0) sums[row * n + idx] = s;
+    if (idx >= 0) sp.sums[row * n + idx] = s;
 }
 
 template <class R>
-__global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(
-    Lines<R> lines, int64_t nl, const __grid_constant__ Tree tr, const __grid_constant__ FarWork fw, const float* __restrict__ agg, const double* __restrict__ nu,
-    int layer0, const double* __restrict__ T, const R* __restrict__ weights, double* __restrict__ part_out)
+__global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(const __grid_constant__ Batch<R> batch,
+                                                                     const double* __restrict__ nu, int layer0,
+                                                                     const double* __restrict__ T)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    if ((int)blockIdx.x >= sp.far_blocks) return;
+    const Tree& tr = sp.tree;
+    const FarWork& fw = sp.fw;
+    const int64_t nl = sp.nl;
     constexpr int n = Far<R>::n;
     int k, i, part;
     if (!far_task(tr, fw, &k, &i, &part)) return;
     const int nloc = blockIdx.y, layer = layer0 + nloc;
-    const Lines<R> ln = layer_lines(lines, nl, nloc);
+    const Lines<R> ln = layer_lines(sp.ln, nl, nloc);
     const FarSet fs = far_set(tr, k, i, nloc);
     const FarList fl(fs);
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
     if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
     double sT, sB;
-    far_adjoint_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), agg[4 * layer],
-                    weights + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
+    far_adjoint_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), sp.agg[4 * layer],
+                    sp.wts + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
                     (R)(0.5 / T[layer]), sT, sB);
     if ((threadIdx.x & 31) == 0) {
         const size_t o = (size_t)layer * fw.slots + fw.slot0[k] + (size_t)part * tr.cnt[k] + i;
-        part_out[2 * o] = sT;
-        part_out[2 * o + 1] = sB;
+        sp.slots[2 * o] = sT;
+        sp.slots[2 * o + 1] = sB;
     }
 }
 
@@ -1133,11 +1196,12 @@ struct LeafPoly<float> {
 template <class R> struct DownRows { static constexpr int v = 64; }; // intervals of a level that a block takes at a time
 template <> struct DownRows<double> { static constexpr int v = 32; };
 template <class R>
-__global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const __grid_constant__ Tree tr,
-                                                                     const __grid_constant__ FarWork fw, int Lc,
-                                                                     int root, const double* __restrict__ sums,
-                                                                     double* __restrict__ coef)
+__global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const __grid_constant__ Batch<R> batch, int Lc,
+                                                                     int root)
 {
+    const Species<R>& sp = batch.s[blockIdx.z];
+    const Tree& tr = sp.tree;
+    const FarWork& fw = sp.fw;
     constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
     __shared__ double v[DownRows<R>::v][n], c[2][TOP / 4][n];
     const int m = threadIdx.x % n, row = threadIdx.x / n, rows = blockDim.x / n;
@@ -1152,7 +1216,7 @@ __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const 
             if (mine) {
                 double s = 0.0;
                 for (int p = 0; p < fw.parts[k]; ++p)
-                    s += sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
+                    s += sp.sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
                 if (k < LEVELS - 1) {
                     const Geo g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
                     s += clenshaw<n, double>(c[(k + 1) & 1][q >> 2], in_span(fma(g.h, cheb<n>(1, m), g.mid), gp));
@@ -1165,7 +1229,7 @@ __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const 
                 if (k > 0)
                     c[k & 1][q][m] = ck;
                 else
-                    LeafPoly<R>::store(coef, (size_t)nloc * tr.cnt[0] + i, m, ck);
+                    LeafPoly<R>::store(sp.coef, (size_t)nloc * tr.cnt[0] + i, m, ck);
             }
             __syncthreads();
         }
@@ -1206,16 +1270,17 @@ __device__ __forceinline__ R node_weight(const R* M, int m)
 // weights[layer][interval][n].
 constexpr int UP_WARPS = 16;
 template <class R>
-__global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant__ Tree tr,
+__global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant__ Batch<R> batch,
                                                            const double* __restrict__ nu, int64_t N, int layer0,
-                                                           const double* __restrict__ g_sigma, double lam_scale,
-                                                           R* __restrict__ weights)
+                                                           double lam_scale)
 {
+    const Species<R>& spc = batch.s[blockIdx.z];
+    const Tree& tr = spc.tree;
     constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
     __shared__ R M[UP_WARPS][n], w[2][TOP][n];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int nloc = blockIdx.y, top = blockIdx.x;
-    const double* g = g_sigma + (size_t)(layer0 + nloc) * N;
+    const double* g = spc.g_sigma + (size_t)(layer0 + nloc) * N;
     for (int k = 0; k < LEVELS; ++k) {
         const int many = 1 << (2 * (LEVELS - 1 - k));
         for (int q = row; q < many; q += UP_WARPS) {
@@ -1246,7 +1311,7 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
             if (lane < n) {
                 const R x = node_weight<n, R>(M[row], lane);
                 w[k & 1][q][lane] = x;
-                weights[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = x;
+                spc.wts[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = x;
             }
             __syncwarp();
         }
@@ -1415,21 +1480,26 @@ __device__ __forceinline__ double split_sum(double v, int split)
 }
 
 // sigma of one leaf: FP32
-__global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
-    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ coef, double unscale, int split, float* __restrict__ sigma)
+__global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(const __grid_constant__ Batch<float> batch,
+                                                                           const double* __restrict__ nu, int64_t N,
+                                                                           double W, int layer0, double unscale,
+                                                                           int split)
 {
+    const Species<float>& sp = batch.s[blockIdx.z];
+    const Tree& tr = sp.tree;
+    const int64_t nl = sp.nl;
+    float* __restrict__ sigma = (float*)sp.sigma;
     __shared__ NearTile tiles[LeafWarps<float>::v];
     NearTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<float> lf;
-    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
-    const Lines<float> ln = layer_lines(lines, nl, nloc);
+    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
-    const Span sp(lf.g, nu[0]); // (a leaf without points has no lines either)
-    const float rh = sp.rh, rl = sp.rl;
+    const Span span(lf.g, nu[0]);
+    const float rh = span.rh, rl = span.rl;
     const double oj = nuj - lf.g.mid;
     const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
     float shi = 0.0f, slo = 0.0f;
@@ -1522,7 +1592,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(
     if (!lf.live || lf.sub) return;
     // the far lines' part
     const double far =
-        tr.on ? LeafPoly<float>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
+        tr.on ? LeafPoly<float>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
     sigma[(size_t)layer * N + j] = (float)((far + near) * unscale);
 }
 
@@ -1562,16 +1632,21 @@ __device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, dou
 // shortest wing polynomial that all of them allow, and the series only its own lanes.
 // (2,000 lines, 4,096 points, one layer: this kernel 3.1 ms with the generic tiers and one
 // exponential a term of the series.)
-__global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
-    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ coef, double unscale, int split, double* __restrict__ sigma)
+__global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(const __grid_constant__ Batch<double> batch,
+                                                                           const double* __restrict__ nu, int64_t N,
+                                                                           double W, int layer0, double unscale,
+                                                                           int split)
 {
+    const Species<double>& sp = batch.s[blockIdx.z];
+    const Tree& tr = sp.tree;
+    const int64_t nl = sp.nl;
+    double* __restrict__ sigma = (double*)sp.sigma;
     extern __shared__ __align__(32) unsigned char smem64[];
     NearTile64& tl = ((NearTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<double> lf;
-    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
-    const Lines<double> ln = layer_lines(lines, nl, nloc);
+    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
@@ -1626,7 +1701,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(
     }
     acc = split_sum<LeafWarps<double>::v>(acc, split);
     if (!lf.live || lf.sub) return;
-    if (tr.on) acc += LeafPoly<double>::eval(coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
+    if (tr.on) acc += LeafPoly<double>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
     sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
@@ -1655,27 +1730,32 @@ __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
     }
 }
 
-__global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
-    Lines<float> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
-    int split, double* __restrict__ part)
+__global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(const __grid_constant__ Batch<float> batch,
+                                                                            const double* __restrict__ nu, int64_t N,
+                                                                            double W, int layer0,
+                                                                            const double* __restrict__ T,
+                                                                            double lam_scale, int split)
 {
+    const Species<float>& sp = batch.s[blockIdx.z];
+    const Tree& tr = sp.tree;
+    const int64_t nl = sp.nl;
+    const double* __restrict__ g_sigma = sp.g_sigma;
     __shared__ NearAdjTile tiles[LeafWarps<float>::v];
     NearAdjTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<float> lf;
-    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
     if (lf.any) {
-        const Lines<float> ln = layer_lines(lines, nl, nloc);
+        const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
         const int64_t j = min64(lf.jb + lane, N - 1);
         const double nuj = nu[j];
         const double lamd = lf.live ? g_sigma[(size_t)layer * N + j] * lam_scale : 0.0;
         const float hT = (float)(0.5 / T[layer]);
         const float lam = (float)lamd;
-        const Span sp(lf.g, nu[0]);
-        const float rh = sp.rh, rl = sp.rl;
+        const Span span(lf.g, nu[0]);
+        const float rh = span.rh, rl = span.rl;
         const double oj = nuj - lf.g.mid;
         const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
 #pragma unroll 1
@@ -1797,7 +1877,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(
             }
         }
     }
-    block_pair<LeafWarps<float>::v>(sT, sB, part + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
+    block_pair<LeafWarps<float>::v>(sT, sB, sp.leaf + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
 }
 
 // Moments over half of the leaf's points (the lane's half) of lambda u^(n+1) for the lane's
@@ -1831,19 +1911,24 @@ __device__ __forceinline__ void near_adjoint64(const NearAdjTile64& tl, int q, i
 // FP64 adjoint of a leaf: the wing polynomials with a line (and half of the points) a
 // lane, so that a line's coefficients are applied once to its moments; the series with a
 // point a lane.
-__global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
-    Lines<double> lines, int64_t nl, const __grid_constant__ Tree tr, const double* __restrict__ nu, int64_t N,
-    double W, int layer0, const double* __restrict__ T, const double* __restrict__ g_sigma, double lam_scale,
-    int split, double* __restrict__ part)
+__global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(const __grid_constant__ Batch<double> batch,
+                                                                            const double* __restrict__ nu, int64_t N,
+                                                                            double W, int layer0,
+                                                                            const double* __restrict__ T,
+                                                                            double lam_scale, int split)
 {
+    const Species<double>& sp = batch.s[blockIdx.z];
+    const Tree& tr = sp.tree;
+    const int64_t nl = sp.nl;
+    const double* __restrict__ g_sigma = sp.g_sigma;
     extern __shared__ __align__(32) unsigned char smem64[];
     NearAdjTile64& tl = ((NearAdjTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<double> lf;
-    lf.init(tr, lines.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
     if (lf.any) {
-        const Lines<double> ln = layer_lines(lines, nl, nloc);
+        const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
         const int64_t j = min64(lf.jb + lane, N - 1);
         const double nuj = nu[j];
@@ -1904,28 +1989,28 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(
             }
         }
     }
-    block_pair<LeafWarps<double>::v>(sT, sB, part + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
+    block_pair<LeafWarps<double>::v>(sT, sB, sp.leaf + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
 }
 
 // g_T[n] = sum over the leaf blocks' and the far kernel's partials of layer n (one
-// block per layer, fixed order);
-// gbl[n] the same for the broadening term.
-__global__ void adjoint_reduce_kernel(const double* __restrict__ part, int per_layer,
-                                      const double* __restrict__ part_far, int per_layer_far,
-                                      double* __restrict__ g_T, double* __restrict__ gbl)
+// block per layer, fixed order); gbl[n] the same for the broadening term.
+template <class R>
+__global__ void __launch_bounds__(256) adjoint_reduce_kernel(const __grid_constant__ Batch<R> batch, int leaf_blocks)
 {
     __shared__ double red[2][256];
-    const int n = blockIdx.x;
+    const Species<R>& sp = batch.s[blockIdx.z];
+    const int n = blockIdx.x, slots = sp.tree.on ? sp.fw.slots : 0;
+    const double* __restrict__ leaf = sp.leaf + 2 * (size_t)n * leaf_blocks;
+    const double* __restrict__ far = sp.slots + 2 * (size_t)n * slots;
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < per_layer; i += blockDim.x) {
-        a += part[2 * ((size_t)n * per_layer + i)];
-        b += part[2 * ((size_t)n * per_layer + i) + 1];
+    for (int i = threadIdx.x; i < leaf_blocks; i += blockDim.x) {
+        a += leaf[2 * (size_t)i];
+        b += leaf[2 * (size_t)i + 1];
     }
-    if (part_far)
-        for (int i = threadIdx.x; i < per_layer_far; i += blockDim.x) {
-            a += part_far[2 * ((size_t)n * per_layer_far + i)];
-            b += part_far[2 * ((size_t)n * per_layer_far + i) + 1];
-        }
+    for (int i = threadIdx.x; i < slots; i += blockDim.x) {
+        a += far[2 * (size_t)i];
+        b += far[2 * (size_t)i + 1];
+    }
     red[0][threadIdx.x] = a;
     red[1][threadIdx.x] = b;
     __syncthreads();
@@ -1937,22 +2022,27 @@ __global__ void adjoint_reduce_kernel(const double* __restrict__ part, int per_l
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        g_T[n] = red[0][0];
-        gbl[n] = red[1][0];
+        sp.g_T[n] = red[0][0];
+        sp.gbl[n] = red[1][0];
     }
 }
 
-// g_b = sum over layers of gbl / s_b (one warp, fixed order); g_T_sum += g_T where given
-__global__ void broad_sum_kernel(const double* __restrict__ gbl, int L, double inv_sb, double* __restrict__ g_b,
-                                 const double* __restrict__ g_T, double* __restrict__ g_T_sum)
+// g_b = sum over layers of gbl / s_b per species (one warp, fixed order); g_T_sum += the
+// species' g_T where given
+template <class R>
+__global__ void broad_sum_kernel(const __grid_constant__ Batch<R> batch, int L, double inv_sb,
+                                 double* __restrict__ g_T_sum)
 {
-    double s = 0.0;
-    for (int n = threadIdx.x; n < L; n += 32) {
-        s += gbl[n];
-        if (g_T_sum) g_T_sum[n] += g_T[n];
+    for (int m = 0; m < batch.n; ++m) {
+        const Species<R>& sp = batch.s[m];
+        double s = 0.0;
+        for (int n = threadIdx.x; n < L; n += 32) {
+            s += sp.gbl[n];
+            if (g_T_sum) g_T_sum[n] += sp.g_T[n];
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) sp.g_b[0] = s * inv_sb;
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) g_b[0] = s * inv_sb;
 }
 
 } // namespace xsd
@@ -2117,10 +2207,59 @@ static int pick_plan(int64_t nl, int64_t N, int32_t L, int prec, size_t ws_bytes
 
 static unsigned blocks_of(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
+// A species' arrays in its workspace.
 template <class R>
-static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L,
-                  double sb, double W, void* sigma, char* ws, const XsPlan& p, bool adjoint,
-                  const double* g_sigma, double* g_T, double* g_b, cudaStream_t st, int flags, double* g_T_sum)
+static Species<R> make_species(const xs_lines* ln, const XsPlan& p, char* ws, int32_t L)
+{
+    constexpr bool FAST = std::is_same<R, float>::value;
+    using R4 = typename vec4<R>::type;
+    const int64_t nl = ln->n;
+    Species<R> s{};
+    s.ln_S0 = ln->ln_S0;
+    s.elower = ln->elower;
+    s.gamma_ref = ln->gamma_ref;
+    s.n_temp = ln->n_temp;
+    s.mass = ln->mass_amu;
+    s.qexp = ln->q_exponent;
+    s.nl = nl;
+    s.fw = p.fw;
+    s.setup_blocks = (int)blocks_of(2 * nl + 4 * (int64_t)L + 4 * (int64_t)p.tree.total, 256);
+    // four lines a thread where that leaves enough blocks: the layer's constants are formed per block
+    s.param_blocks = (int)(nl >= 65536 ? blocks_of(nl, 1024) : blocks_of(nl, 256));
+    s.far_blocks = p.far_blocks;
+    s.jr = (int2*)(ws + p.off_jr);
+    s.nuf = FAST ? (float2*)(ws + p.off_nuf) : nullptr;
+    s.w_inv_nu = (double*)(ws + p.off_inv);
+    s.agg = (float*)(ws + p.off_agg);
+    s.rec1 = (R4*)(ws + p.off_rec1);
+    s.rec2 = (R4*)(ws + p.off_rec2);
+    s.rec3 = (R*)(ws + p.off_rec3);
+    s.clo = FAST ? (R*)(ws + p.off_clo) : nullptr;
+    s.geo = (Geo*)(ws + p.off_geo);
+    s.cov = (int2*)(ws + p.off_cov);
+    s.win = (int2*)(ws + p.off_win);
+    s.pq = (int2*)(ws + p.off_pq);
+    s.sums = (double*)(ws + p.off_fwd);
+    s.coef = (double*)(ws + p.off_coef);
+    s.wts = (R*)(ws + p.off_wts);
+    s.slots = (double*)(ws + p.off_slots);
+    s.leaf = (double*)(ws + p.off_leaf);
+    s.gbl = (double*)(ws + p.off_gbl);
+    s.inv_nu = s.w_inv_nu;
+    s.tree = p.tree;
+    s.tree.geo = s.geo;
+    s.tree.cov = s.cov;
+    s.tree.win = s.win;
+    s.tree.pq = s.pq;
+    s.ln = Lines<R>{ln->nu_hat, s.nuf, s.jr, s.rec1, s.rec2, s.rec3, s.clo};
+    return s;
+}
+
+// The line sums (or their adjoints) of a batch of species with plans of the same shape
+// (same chunks of layers, same use of the intervals); p: the first one's.
+template <class R>
+static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64_t N, const double* T, const double* P,
+                     int32_t L, double sb, double W, bool adjoint, cudaStream_t st, int flags, double* g_T_sum)
 {
     // flags: XS_RUN_KEEP_ADJ  (forward) also write the adjoint's per-line records
     //        XS_RUN_REUSE     (adjoint) the records and ranges of an immediately preceding
@@ -2128,130 +2267,126 @@ static int run_xs(const xs_lines* ln, const double* nu, int64_t N, const double*
     constexpr bool FAST = std::is_same<R, float>::value;
     const bool reuse = adjoint && (flags & XS_RUN_REUSE) && p.nchunks == 1;
     const bool want_rec3 = adjoint || (flags & XS_RUN_KEEP_ADJ);
-    using R4 = typename vec4<R>::type;
-    const int64_t nl = ln->n;
     const double unscale = FAST ? MIXED_UNSCALE : 1.0;
-    if (nl == 0) {
-        if (adjoint) {
-            if (cudaMemsetAsync(g_T, 0, sizeof(double) * L, st) != cudaSuccess) return XS_ECUDA;
-            if (cudaMemsetAsync(g_b, 0, sizeof(double), st) != cudaSuccess) return XS_ECUDA;
-        } else {
-            size_t es = FAST ? sizeof(float) : sizeof(double);
-            if (cudaMemsetAsync(sigma, 0, es * (size_t)L * N, st) != cudaSuccess) return XS_ECUDA;
-        }
-        return XS_OK;
+    const unsigned nz = (unsigned)b.n;
+    const Tree& tr = p.tree;
+    int setup_blocks = 0, param_blocks = 0, far_blocks = 0;
+    for (int m = 0; m < b.n; ++m) {
+        setup_blocks = std::max(setup_blocks, b.s[m].setup_blocks);
+        param_blocks = std::max(param_blocks, b.s[m].param_blocks);
+        far_blocks = std::max(far_blocks, b.s[m].far_blocks);
     }
-    int2* jr = (int2*)(ws + p.off_jr);
-    float2* nuf = FAST ? (float2*)(ws + p.off_nuf) : nullptr;
-    double* inv_nu = (double*)(ws + p.off_inv);
-    float* agg = (float*)(ws + p.off_agg);
-    R4* rec1 = (R4*)(ws + p.off_rec1);
-    R4* rec2 = (R4*)(ws + p.off_rec2);
-    R* rec3 = (R*)(ws + p.off_rec3);
-    R* clo = FAST ? (R*)(ws + p.off_clo) : nullptr;
-    Geo* geo = (Geo*)(ws + p.off_geo);
-    int2* cov = (int2*)(ws + p.off_cov);
-    int2* win = (int2*)(ws + p.off_win);
-    int2* pq = (int2*)(ws + p.off_pq);
-    double* sums = (double*)(ws + p.off_fwd);
-    double* coef = (double*)(ws + p.off_coef);
-    R* wts = (R*)(ws + p.off_wts);
-    double* slots = (double*)(ws + p.off_slots);
-    double* leaf = (double*)(ws + p.off_leaf);
-    double* gbl = (double*)(ws + p.off_gbl);
-    Tree tr = p.tree;
-    tr.geo = geo;
-    tr.cov = cov;
-    tr.win = win;
-    tr.pq = pq;
-    const Lines<R> lines{ln->nu_hat, nuf, jr, rec1, rec2, rec3, clo};
-    const unsigned tops = tr.on ? (unsigned)tr.cnt[LEVELS - 1] : 0;
-
+    if constexpr (!FAST) {
+        // beyond 48 KB of shared memory a block has to ask (cheap; per device)
+        if (cudaFuncSetAttribute(leaf_kernel_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(LeafWarps<double>::v * sizeof(NearTile64))) != cudaSuccess ||
+            cudaFuncSetAttribute(leaf_adjoint_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(LeafWarps<double>::v * sizeof(NearAdjTile64))) != cudaSuccess)
+            return XS_ECUDA;
+    }
     if (!reuse) {
-        setup_kernel<<<blocks_of(2 * nl + 4 * (int64_t)L + 4 * (int64_t)tr.total, 256), 256, 0, st>>>(
-            ln->nu_hat, nl, nu, N, W, jr, nuf, inv_nu, agg, 4 * L, tr, geo, cov, win);
+        setup_kernel<R><<<dim3((unsigned)setup_blocks, 1, nz), 256, 0, st>>>(b, nu, N, W, 4 * L);
         count_launch();
     }
     for (int c = 0; c < p.nchunks; ++c) {
         const int l0 = c * p.Lc;
         const int lc = std::min(p.Lc, L - l0);
         if (!reuse) {
-            // four lines a thread where that leaves enough blocks: the layer's constants are formed per block
-            const dim3 pg(nl >= 65536 ? blocks_of(nl, 1024) : blocks_of(nl, 256), (unsigned)lc);
-            line_params_kernel<R><<<pg, 256, 0, st>>>(ln->nu_hat, inv_nu, ln->ln_S0, ln->elower, ln->gamma_ref,
-                                                      ln->n_temp, nl, ln->mass_amu, ln->q_exponent, T, P, l0, sb, rec1,
-                                                      rec2, clo, want_rec3 ? rec3 : nullptr, agg);
+            line_params_kernel<R>
+                <<<dim3((unsigned)param_blocks, (unsigned)lc, nz), 256, 0, st>>>(b, T, P, l0, sb, want_rec3);
             count_launch();
             if (tr.on) {
-                near_range_kernel<R><<<dim3(blocks_of(2 * (int64_t)tr.total, 256), (unsigned)lc), 256, 0, st>>>(
-                    ln->nu_hat, nl, tr, agg, l0, pq);
+                near_range_kernel<R>
+                    <<<dim3(blocks_of(2 * (int64_t)tr.total, 256), (unsigned)lc, nz), 256, 0, st>>>(b, l0);
                 count_launch();
             }
         }
-        const dim3 lgrid((unsigned)p.leaf_blocks, (unsigned)lc);
-        const dim3 fgrid((unsigned)p.far_blocks, (unsigned)lc);
+        const dim3 lgrid((unsigned)p.leaf_blocks, (unsigned)lc, nz);
+        const dim3 fgrid((unsigned)far_blocks, (unsigned)lc, nz);
         const int lthreads = 32 * p.leaf_warps;
-        if constexpr (!FAST) {
-            // beyond 48 KB of shared memory a block has to ask (cheap; per device)
-            if (cudaFuncSetAttribute(leaf_kernel_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(LeafWarps<double>::v * sizeof(NearTile64))) != cudaSuccess ||
-                cudaFuncSetAttribute(leaf_adjoint_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(LeafWarps<double>::v * sizeof(NearAdjTile64))) != cudaSuccess)
-                return XS_ECUDA;
-        }
         prof_begin(adjoint ? 1 : 0, st);
         if (!adjoint) {
             if (tr.on) {
-                far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, sums);
+                far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(b, nu, l0);
                 int root = LEVELS - 1;
-                while (root > 1 && (int64_t)tr.cnt[root] * lc < 2 * 152) --root;
+                while (root > 1 && (int64_t)tr.cnt[root] * lc * b.n < 2 * 152) --root;
                 const int rows = std::min(DownRows<R>::v, 1 << (2 * root));
-                down_kernel<R><<<dim3((unsigned)tr.cnt[root], (unsigned)lc), rows * Far<R>::n, 0, st>>>(
-                    tr, p.fw, lc, root, sums, coef);
+                down_kernel<R><<<dim3((unsigned)tr.cnt[root], (unsigned)lc, nz), rows * Far<R>::n, 0, st>>>(b, lc, root);
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
-                                                            p.leaf_split, (float*)sigma);
+                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, W, l0, unscale, p.leaf_split);
             else
-                leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(lines, nl, tr, nu, N, W, l0, coef, unscale,
-                                                            p.leaf_split, (double*)sigma);
+                leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(b, nu, N, W, l0, unscale,
+                                                                                           p.leaf_split);
         } else {
             if (tr.on) {
-                up_kernel<R><<<dim3(tops, (unsigned)lc), 32 * UP_WARPS, 0, st>>>(tr, nu, N, l0, g_sigma, unscale, wts);
-                far_adjoint_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(lines, nl, tr, p.fw, agg, nu, l0, T, wts,
-                                                                        slots);
+                up_kernel<R><<<dim3((unsigned)tr.cnt[LEVELS - 1], (unsigned)lc, nz), 32 * UP_WARPS, 0, st>>>(b, nu, N, l0,
+                                                                                                            unscale);
+                far_adjoint_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(b, nu, l0, T);
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
-                                                             p.leaf_split, leaf);
+                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, W, l0, T, unscale, p.leaf_split);
             else
-                leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(lines, nl, tr, nu, N, W, l0, T, g_sigma, unscale,
-                                                             p.leaf_split, leaf);
+                leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(b, nu, N, W, l0, T,
+                                                                                              unscale, p.leaf_split);
         }
         prof_end(adjoint ? 1 : 0, st);
         count_launch();
     }
     if (adjoint) {
-        adjoint_reduce_kernel<<<L, 256, 0, st>>>(leaf, p.leaf_blocks, tr.on ? slots : nullptr, p.fw.slots, g_T, gbl);
-        broad_sum_kernel<<<1, 32, 0, st>>>(gbl, L, 1.0 / sb, g_b, g_T, g_T_sum);
+        adjoint_reduce_kernel<R><<<dim3((unsigned)L, 1, nz), 256, 0, st>>>(b, p.leaf_blocks);
+        broad_sum_kernel<R><<<1, 32, 0, st>>>(b, L, 1.0 / sb, g_T_sum);
         count_launch(2);
     }
     return (cudaGetLastError() == cudaSuccess) ? XS_OK : XS_ECUDA;
 }
 
-int xs_run(const xs_lines* ln, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
-           double W, int prec, void* sigma, void* ws, size_t ws_bytes, bool adjoint, const double* g_sigma,
-           double* g_T, double* g_b, cudaStream_t st, int flags, double* g_T_sum)
+// Species with lines and plans of one shape run together, the others by themselves, in order.
+template <class R>
+static int run_species(int n, const XsJob* job, const XsPlan* plan, const double* nu, int64_t N, const double* T,
+                       const double* P, int32_t L, double sb, double W, bool adjoint, cudaStream_t st, int flags,
+                       double* g_T_sum)
 {
-    XsPlan p;
-    if (pick_plan(ln->n, N, L, prec, ws_bytes, &p) != XS_OK) return XS_EINVAL;
+    int m = 0;
+    while (m < n) {
+        if (job[m].lines->n == 0) {
+            if (adjoint) {
+                if (cudaMemsetAsync(job[m].g_T, 0, sizeof(double) * L, st) != cudaSuccess) return XS_ECUDA;
+                if (cudaMemsetAsync(job[m].g_b, 0, sizeof(double), st) != cudaSuccess) return XS_ECUDA;
+            } else if (cudaMemsetAsync(job[m].sigma, 0, sizeof(R) * (size_t)L * N, st) != cudaSuccess) {
+                return XS_ECUDA;
+            }
+            ++m;
+            continue;
+        }
+        const int first = m;
+        Batch<R> b{};
+        while (m < n && job[m].lines->n > 0 && plan[m].tree.on == plan[first].tree.on && plan[m].Lc == plan[first].Lc) {
+            Species<R>& s = b.s[b.n++];
+            s = make_species<R>(job[m].lines, plan[m], (char*)job[m].ws, L);
+            s.sigma = job[m].sigma;
+            s.g_sigma = job[m].g_sigma;
+            s.g_T = job[m].g_T;
+            s.g_b = job[m].g_b;
+            ++m;
+        }
+        const int r = run_batch<R>(b, plan[first], nu, N, T, P, L, sb, W, adjoint, st, flags, g_T_sum);
+        if (r != XS_OK) return r;
+    }
+    return XS_OK;
+}
+
+int xs_run(int n, const XsJob* job, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
+           double W, int prec, bool adjoint, cudaStream_t st, int flags, double* g_T_sum)
+{
+    XsPlan plan[XS_MAX_SPECIES];
+    for (int m = 0; m < n; ++m)
+        if (pick_plan(job[m].lines->n, N, L, prec, job[m].ws_bytes, &plan[m]) != XS_OK) return XS_EINVAL;
     if (prec == XS_PREC_FP64)
-        return run_xs<double>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags,
-                              g_T_sum);
-    return run_xs<float>(ln, nu, N, T, P, L, sb, W, sigma, (char*)ws, p, adjoint, g_sigma, g_T, g_b, st, flags,
-                              g_T_sum);
+        return run_species<double>(n, job, plan, nu, N, T, P, L, sb, W, adjoint, st, flags, g_T_sum);
+    return run_species<float>(n, job, plan, nu, N, T, P, L, sb, W, adjoint, st, flags, g_T_sum);
 }
 
 int check_sorted(const double* nu_hat, int64_t n, cudaStream_t st, int* flag_dev, bool grid)

@@ -62,6 +62,6 @@ extern "C" int xs_compute_noalloc(const xs_lines* lines, const double* nu, int64
     // Every scratch region the forward pass reads is written earlier in the same
     // call (cut ranges, per-layer minima, line records, split-K partials), so the
     // previous call's contents never need clearing.
-    return xsi::xs_run(lines, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, sigma, scratch,
-                       XS_NOALLOC_SCRATCH_BYTES, false, nullptr, nullptr, nullptr, (cudaStream_t)stream);
+    const xsi::XsJob job{lines, scratch, XS_NOALLOC_SCRATCH_BYTES, sigma, nullptr, nullptr, nullptr};
+    return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, false, (cudaStream_t)stream);
 }
