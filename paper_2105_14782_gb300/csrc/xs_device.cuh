@@ -154,32 +154,52 @@ __device__ __forceinline__ void scaled_pair(float dh, float dl, float ch, float 
 }
 __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 
-// e^v in FP64, table-driven (Tang 1989): 2^(i/64) from a table, the rest (|r| <= ln2/128)
-// by the series to r^5 (next term 4e-17): half the operations of exp.  Beyond +-700 exp.
-struct Exp2Table64 {
-    double t[64];
+// e^v in FP64, table-driven (Tang 1989): 2^(i/64) as hi + lo from a table, the rest
+// (|r| <= ln2/128) by the series to r^5 (next term 4e-17): 12 operations, within 0.52 ulp
+// of the exact value.  Beyond +-700 exp.
+struct Exp2Entry {
+    double hi, lo;
 };
-constexpr Exp2Table64 make_exp2_table64()
-{
-    Exp2Table64 r{};
-    const double ln2 = 0.69314718055994530942;
-    for (int i = 0; i < 64; ++i) {
-        // series of e^(i ln2/64) about the nearer end
-        const double x = (i <= 32 ? i : i - 64) * ln2 / 64;
-        double s = 1.0;
-        for (int k = 22; k >= 1; --k) s = 1.0 + s * x / k;
-        r.t[i] = i <= 32 ? s : 2.0 * s;
-    }
-    return r;
-}
-__device__ const Exp2Table64 EXP2_64 = make_exp2_table64();
+__device__ const Exp2Entry EXP2_64[64] = {
+    {1.0, 0.0}, {1.0108892860517005, -1.5234778603368577e-17},
+    {1.0218971486541166, 5.109225028973444e-17}, {1.0330248790212284, 7.600838874027088e-18},
+    {1.0442737824274138, 8.551889705537965e-17}, {1.0556451783605572, 1.759325738772092e-18},
+    {1.0671404006768237, -7.899853966841582e-17}, {1.0787607977571199, -6.656660436056593e-17},
+    {1.0905077326652577, -3.046782079812471e-17}, {1.102382583307841, 5.2660368715706944e-17},
+    {1.1143867425958924, 1.0410278456845571e-16}, {1.1265216186082418, 5.165856758795457e-17},
+    {1.1387886347566916, 8.912812676025408e-17}, {1.1511892299529827, 3.250710218863827e-17},
+    {1.1637248587775775, 3.8292048369240935e-17}, {1.1763969916502812, 5.554203254218079e-17},
+    {1.189207115002721, 3.982015231465646e-17}, {1.202156731452703, 6.644981499252301e-17},
+    {1.215247359980469, -7.712630692681488e-17}, {1.22848053610687, -1.89878163130253e-17},
+    {1.241857812073484, 4.658027591836937e-17}, {1.255380757024691, -6.7113898212968784e-18},
+    {1.2690509571917332, 2.667932131342186e-18}, {1.2828700160787783, 1.713594918243561e-17},
+    {1.2968395546510096, 2.5382502794888315e-17}, {1.3109612115247644, -7.181536135519454e-17},
+    {1.3252366431597413, -2.8587312100388614e-17}, {1.339667524053303, 8.927282594831732e-17},
+    {1.3542555469368927, 7.70094837980299e-17}, {1.3690024229745905, 9.593797919118849e-17},
+    {1.383909881963832, -6.770511658794786e-17}, {1.3989796725383112, -9.614213209051323e-17},
+    {1.4142135623730951, -9.667293313452913e-17}, {1.42961333839197, -1.2031642489053655e-17},
+    {1.4451808069770467, -3.0237581349939873e-17}, {1.460917794180647, -5.600377186075216e-17},
+    {1.4768261459394993, -3.483994556892796e-17}, {1.4929077282912648, 1.4192920154284036e-17},
+    {1.5091644275934228, -1.016455327754295e-16}, {1.5255981507445384, -1.1024941712342561e-16},
+    {1.5422108254079407, 7.949834809697621e-17}, {1.559004400237837, 3.7812070533575275e-17},
+    {1.5759808451078865, -1.0136916471278304e-17}, {1.593142151342267, -1.0094406542311964e-16},
+    {1.6104903319492543, 2.4707192569797888e-17}, {1.6280274218573478, -6.712955084707084e-17},
+    {1.645755478153965, -1.0125679913674773e-16}, {1.6636765803267364, 5.8909926967131e-17},
+    {1.681792830507429, 8.199010020581497e-17}, {1.7001063537185235, -8.0237193703977e-18},
+    {1.718619298122478, -1.851380418263111e-17}, {1.7373338352737062, 3.164389299292957e-17},
+    {1.7562521603732995, 2.960140695448873e-17}, {1.7753764925265212, 6.429731796556572e-17},
+    {1.7947090750031072, 1.8227458427912087e-17}, {1.8142521755003989, -9.969531538920349e-17},
+    {1.8340080864093424, 3.283107224245627e-17}, {1.8539791250833855, 9.761887490727594e-17},
+    {1.8741676341103, -6.122763413004143e-17}, {1.8945759815869656, 3.4034035352165297e-17},
+    {1.9152065613971474, -1.0619946056195963e-16}, {1.9360617934922943, 1.0332385960676326e-16},
+    {1.9571441241754002, 8.960767791036668e-17}, {1.978456026387951, 4.0388753109278167e-17}};
 
 __device__ __forceinline__ double exp_tab(double v)
 {
     if ((__double2hiint(v) & 0x7fffffff) >= 0x4085e000) return exp(v); // |v| >= 700, infinities, NaN
     const double magic = 6755399441055744.0; // 1.5 2^52
     // ln 2 = its float value (products with k are exact) + the rest
-    const double ln2_hi = (double)0.693147182f, ln2_lo = -1.904654299957767878541823e-9;
+    const double ln2_hi = (double)0.693147182f, ln2_lo = -0.000000001904654299957767878541823;
     const double t = fma(v, 64.0 / 0.69314718055994530942, magic), kd = t - magic;
     const int k = __double2loint(t);
     const double r = fma(kd, -ln2_lo / 64, fma(kd, -ln2_hi / 64, v));
@@ -187,8 +207,8 @@ __device__ __forceinline__ double exp_tab(double v)
     p = fma(r, p, 1.0 / 6.0);
     p = fma(r, p, 0.5);
     p = fma(r * r, p, r);
-    const double h = EXP2_64.t[k & 63];
-    const double s = fma(h, p, h);
+    const Exp2Entry h = EXP2_64[k & 63];
+    const double s = h.hi + fma(h.hi, p, h.lo);
     return __hiloint2double(__double2hiint(s) + ((k >> 6) << 20), __double2loint(s));
 }
 
@@ -200,6 +220,13 @@ __device__ __forceinline__ double rcp64(double x)
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     y = fma(y, fma(-x, y, 1.0), y);
     return fma(y, fma(-x, y, 1.0), y);
+}
+
+// the same for any x: 0, infinities and what overflows as a division gives them
+__device__ __forceinline__ double rcp64_any(double x)
+{
+    const int e = __double2hiint(x) & 0x7ff00000;
+    return (e < 0x00200000 || e >= 0x7fd00000) ? 1.0 / x : rcp64(x);
 }
 
 // exp(-x^2) with x^2 split into hi + lo so the rounding of x*x does not enter.

@@ -76,7 +76,7 @@ __device__ const ExpIntTable EXPINT = make_exp_int_table();
 
 __device__ __forceinline__ void exp_int23(double x, double* E2, double* E3)
 {
-    const double ex = exp(-x);
+    const double ex = exp_tab(-x);
     double e2;
     if (x <= 1.5) {
         if (x == 0.0) {
@@ -105,11 +105,21 @@ __device__ __forceinline__ void exp_int23(double x, double* E2, double* E3)
     *E3 = 0.5 * (ex - x * e2);
 }
 
+// a/(e^u - 1), u > 0: from e^-u where that loses nothing, the quotient corrected by its
+// residual
+__device__ __forceinline__ double bose(double a, double u)
+{
+    if (!(u >= 0.5)) return a / expm1(u);
+    const double e = exp_tab(-u), d = 1.0 - e, y = rcp64(d), n = a * e;
+    const double q = n * y;
+    return fma(fma(-q, d, n), y, q);
+}
+
 // pi B(nu, T) = planck_c nu^3/(e^u - 1), u = c2 nu/T
 constexpr double PLANCK_C = PI * 2.0 * hP * cL * cL;
 __device__ __forceinline__ double planck_pi(double nu, double T)
 {
-    return PLANCK_C * nu * nu * nu / expm1(c2 * nu / T);
+    return bose(PLANCK_C * nu * nu * nu, c2 * nu / T);
 }
 
 struct SigPtrs {
@@ -203,39 +213,40 @@ __global__ void __cluster_dims__(RT_CLUSTER, 1, 1)
 
 // Emission solve (Sec. 2.3):  F0 = sum_n Phi_n (1 - T_n) S_n + Phi_L S_B, with
 // Phi_n = prod_{k<n} T_k, T_n = 2 E3(dtau_n), S_n = pi B(nu, T_n), S_B = pi B(nu, T_{L-1}).
-// A block takes 32 grid points (lane = point, coalesced rows of dtau) and its
-// RT_SEG warps take contiguous segments of the layers: each warp reduces its
-// segment to (prod T, local sum), and the segments are chained in order.
-constexpr int RT_SEG = 8;
-
-__device__ __forceinline__ void seg_range(int L, int w, int* n0, int* n1)
+// A block takes PTS grid points (neighbouring lanes, so rows of dtau are read in whole
+// sectors) and its RT_THREADS/PTS groups of lanes take contiguous segments of the layers:
+// each reduces its segment to (prod T, local sum), and the segments are chained in
+// order.  Bound by FP64 operations (about 70 a point and layer) on the SMs that have
+// blocks: 32 points a block from 608 blocks (four a SM) on, fewer points and shorter
+// segments below (a served request of 20 layers x 2,003 points ran on 63 SMs).
+__device__ __forceinline__ void seg_range(int L, int w, int segs, int* n0, int* n1)
 {
-    *n0 = (int)(((int64_t)L * w) / RT_SEG);
-    *n1 = (int)(((int64_t)L * (w + 1)) / RT_SEG);
+    *n0 = (int)(((int64_t)L * w) / segs);
+    *n1 = (int)(((int64_t)L * (w + 1)) / segs);
 }
 
-__global__ void __launch_bounds__(32 * RT_SEG) emission_kernel(const double* __restrict__ dtau,
-                                                               const double* __restrict__ T,
-                                                               const double* __restrict__ nu, int L, int64_t N,
-                                                               double* __restrict__ F0)
+template <int PTS>
+__global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __restrict__ dtau,
+                                                              const double* __restrict__ T,
+                                                              const double* __restrict__ nu, int L, int64_t N,
+                                                              double* __restrict__ F0)
 {
-    __shared__ double segP[RT_SEG][32], segF[RT_SEG][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
+    constexpr int SEG = RT_THREADS / PTS;
+    __shared__ double segP[SEG][PTS], segF[SEG][PTS];
+    const int lane = threadIdx.x % PTS, w = threadIdx.x / PTS;
+    const int64_t j = (int64_t)blockIdx.x * PTS + lane;
     const bool valid = j < N;
     const double v = valid ? nu[j] : nu[0];
     const double cv = c2 * v, kv = PLANCK_C * v * v * v;
     int n0, n1;
-    seg_range(L, w, &n0, &n1);
-    double phi = 1.0, F = 0.0, inv = 0.0;
-    for (int n = n0; n < n1; ++n) {
-        if (((n - n0) & 31) == 0) inv = (n + lane < n1) ? 1.0 / T[n + lane] : 0.0; // 32 layers at once
-        const double invT = __shfl_sync(0xffffffffu, inv, (n - n0) & 31);
-        if (valid) {
+    seg_range(L, w, SEG, &n0, &n1);
+    double phi = 1.0, F = 0.0;
+    if (valid) {
+        for (int n = n0; n < n1; ++n) {
             double e2, e3;
             exp_int23(dtau[(size_t)n * N + j], &e2, &e3);
             const double tr = 2.0 * e3;
-            F += phi * (1.0 - tr) * (kv / expm1(cv * invT));
+            F += phi * (1.0 - tr) * bose(kv, cv * rcp64_any(T[n]));
             phi *= tr;
         }
     }
@@ -244,7 +255,7 @@ __global__ void __launch_bounds__(32 * RT_SEG) emission_kernel(const double* __r
     __syncthreads();
     if (w == 0 && valid) {
         double Ft = 0.0, ph = 1.0;
-        for (int s = 0; s < RT_SEG; ++s) {
+        for (int s = 0; s < SEG; ++s) {
             Ft += ph * segF[s][lane];
             ph *= segP[s][lane];
         }
@@ -256,34 +267,34 @@ __global__ void __launch_bounds__(32 * RT_SEG) emission_kernel(const double* __r
 //   dF0/ddtau_n = Phi_n (F_{n+1} - S_n) dT_n/ddtau_n,  dT/ddtau = -2 E2(dtau),
 //   dF0/dS_n = Phi_n (1 - T_n) (+ Phi_L for the bottom source, n = L-1),
 // where F_{n+1} = upward flux below layer n: F_L = S_B, F_n = T_n F_{n+1} + (1 - T_n) S_n.
-// Three passes over each warp's layer segment: (1) T, E2, S stored and the
+// Three passes over each group's layer segment: (1) T, E2, S stored and the
 // segment's maps F_top = A F_bottom + C and prod T; (2) after chaining the
 // segments, F_{n+1} down the segment; (3) Phi_n along it, g_dtau and the
-// per-layer sums of lambda dF0/dS_n dS_n/dT_n over the block's 32 points.
-__global__ void __launch_bounds__(32 * RT_SEG) emission_adjoint_kernel(
+// per-layer sums of lambda dF0/dS_n dS_n/dT_n over the block's points.
+template <int PTS>
+__global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     const double* __restrict__ g_F0, const double* __restrict__ dtau, const double* __restrict__ T,
     const double* __restrict__ nu, int L, int64_t N, double* __restrict__ g_dtau, double* __restrict__ part,
     double* __restrict__ w_tr, double* __restrict__ w_e2, double* __restrict__ w_S)
 {
-    __shared__ double segA[RT_SEG][32], segC[RT_SEG][32], segFin[RT_SEG][32], segPhi[RT_SEG][32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
+    constexpr int SEG = RT_THREADS / PTS;
+    __shared__ double segA[SEG][PTS], segC[SEG][PTS], segFin[SEG][PTS], segPhi[SEG][PTS];
+    const int lane = threadIdx.x % PTS, w = threadIdx.x / PTS;
+    const int64_t j = (int64_t)blockIdx.x * PTS + lane;
     const bool valid = j < N;
     const double v = valid ? nu[j] : nu[0];
     const double lam = valid ? g_F0[j] : 0.0;
     const double cv = c2 * v, kv = PLANCK_C * v * v * v;
     int n0, n1;
-    seg_range(L, w, &n0, &n1);
+    seg_range(L, w, SEG, &n0, &n1);
     // (1) per-layer factors and the segment's backward map
-    double A = 1.0, Cm = 0.0, inv = 0.0;
-    for (int n = n1 - 1; n >= n0; --n) {
-        if (((n1 - 1 - n) & 31) == 0) inv = (n - lane >= n0) ? 1.0 / T[n - lane] : 0.0; // 32 layers at once
-        const double invT = __shfl_sync(0xffffffffu, inv, (n1 - 1 - n) & 31);
-        if (valid) {
+    double A = 1.0, Cm = 0.0;
+    if (valid) {
+        for (int n = n1 - 1; n >= n0; --n) {
             const size_t i = (size_t)n * N + j;
             double e2, e3;
             exp_int23(dtau[i], &e2, &e3);
-            const double tr = 2.0 * e3, Sn = kv / expm1(cv * invT);
+            const double tr = 2.0 * e3, Sn = bose(kv, cv * rcp64_any(T[n]));
             w_tr[i] = tr;
             w_e2[i] = e2;
             w_S[i] = Sn;
@@ -297,12 +308,12 @@ __global__ void __launch_bounds__(32 * RT_SEG) emission_adjoint_kernel(
     if (w == 0) {
         // flux entering each segment from below, and Phi at each segment's top
         double Fb = valid ? planck_pi(v, T[L - 1]) : 0.0;
-        for (int s = RT_SEG - 1; s >= 0; --s) {
+        for (int s = SEG - 1; s >= 0; --s) {
             segFin[s][lane] = Fb;
             Fb = segA[s][lane] * Fb + segC[s][lane];
         }
         double ph = 1.0;
-        for (int s = 0; s < RT_SEG; ++s) {
+        for (int s = 0; s < SEG; ++s) {
             segPhi[s][lane] = ph;
             ph *= segA[s][lane];
         }
@@ -318,17 +329,17 @@ __global__ void __launch_bounds__(32 * RT_SEG) emission_adjoint_kernel(
             F = tr * F + (1.0 - tr) * w_S[i];
         }
     }
-    // (3) forward along the segment
+    // (3) forward along the segment (as many steps in every group of a warp, for the sums)
     double phi = segPhi[w][lane];
-    const double phiL = segPhi[RT_SEG - 1][lane] * segA[RT_SEG - 1][lane];
+    const double phiL = segPhi[SEG - 1][lane] * segA[SEG - 1][lane];
     const double inv_kv = 1.0 / kv;
-    for (int n = n0; n < n1; ++n) {
-        if (((n - n0) & 31) == 0) inv = (n + lane < n1) ? 1.0 / T[n + lane] : 0.0;
-        const double invT = __shfl_sync(0xffffffffu, inv, (n - n0) & 31);
+    const int most = (L + SEG - 1) / SEG;
+    for (int k = 0; k < most; ++k) {
+        const int n = n0 + k;
         double gT = 0.0;
-        if (valid) {
+        if (valid && n < n1) {
             const size_t i = (size_t)n * N + j;
-            const double tr = w_tr[i], Sn = w_S[i];
+            const double tr = w_tr[i], Sn = w_S[i], invT = rcp64_any(T[n]);
             g_dtau[i] = lam * phi * (g_dtau[i] - Sn) * (-2.0 * w_e2[i]);
             double gS = lam * phi * (1.0 - tr);
             if (n == L - 1) gS += lam * phiL;
@@ -336,8 +347,8 @@ __global__ void __launch_bounds__(32 * RT_SEG) emission_adjoint_kernel(
             // d(pi B)/dT = B (u/T)/(1 - e^-u), and 1/(1 - e^-u) = 1 + 1/(e^u - 1) = 1 + B/kv
             gT = gS * Sn * (cv * invT * invT) * fma(Sn, inv_kv, 1.0);
         }
-        for (int o = 16; o > 0; o >>= 1) gT += __shfl_xor_sync(0xffffffffu, gT, o);
-        if (lane == 0) part[(size_t)n * gridDim.x + blockIdx.x] = gT;
+        for (int o = PTS / 2; o > 0; o >>= 1) gT += __shfl_xor_sync(0xffffffffu, gT, o, PTS);
+        if (lane == 0 && n < n1) part[(size_t)n * gridDim.x + blockIdx.x] = gT;
     }
 }
 
@@ -567,17 +578,25 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
     return launched(1);
 }
 
+// Points a block of the emission kernels takes: see emission_kernel.
+static int emission_points(int64_t N) { return N >= 608 * 32 ? 32 : N >= 608 * 16 ? 16 : 8; }
+
 int rt_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
                 cudaStream_t st)
 {
-    emission_kernel<<<(unsigned)((N + 31) / 32), 32 * RT_SEG, 0, st>>>(dtau, T, nu, L, N, F0);
+    const int pts = emission_points(N);
+    const unsigned nb = (unsigned)((N + pts - 1) / pts);
+    if (pts == 32) emission_kernel<32><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
+    else if (pts == 16) emission_kernel<16><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
+    else emission_kernel<8><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
     return launched(1);
 }
 
 // [L][nb] per-block layer partials, then T_n, E2_n and S_n as [L][N] each
 size_t rt_emission_ws(int32_t L, int64_t N)
 {
-    int64_t nb = (N + 31) / 32;
+    const int pts = emission_points(N);
+    int64_t nb = (N + pts - 1) / pts;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     return al(sizeof(double) * (size_t)L * (size_t)nb) + 3 * al(sizeof(double) * (size_t)L * (size_t)N);
 }
@@ -585,7 +604,8 @@ size_t rt_emission_ws(int32_t L, int64_t N)
 int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
                         int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st)
 {
-    const int64_t nb = (N + 31) / 32;
+    const int pts = emission_points(N);
+    const int64_t nb = (N + pts - 1) / pts;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     char* base = (char*)ws;
     double* part = (double*)base;
@@ -593,8 +613,9 @@ int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T,
     double* w_tr = (double*)(base + al(sizeof(double) * (size_t)L * (size_t)nb));
     double* w_e2 = (double*)((char*)w_tr + LN);
     double* w_S = (double*)((char*)w_e2 + LN);
-    emission_adjoint_kernel<<<(unsigned)nb, 32 * RT_SEG, 0, st>>>(g_F0, dtau, T, nu, L, N, g_dtau, part, w_tr, w_e2,
-                                                                  w_S);
+    auto* kernel = pts == 32 ? emission_adjoint_kernel<32>
+                             : pts == 16 ? emission_adjoint_kernel<16> : emission_adjoint_kernel<8>;
+    kernel<<<(unsigned)nb, RT_THREADS, 0, st>>>(g_F0, dtau, T, nu, L, N, g_dtau, part, w_tr, w_e2, w_S);
     layer_sum_kernel<<<L, RT_THREADS, 0, st>>>(part, (int)nb, L, g_T);
     return launched(2);
 }

@@ -563,10 +563,10 @@ class SpectrumLogL(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, theta, model):
-        th = theta.detach().cpu().double().tolist()
-        o = model.logl_grad_async(th).clone()
-        ctx.save_for_backward(o[1:].to(theta.device, theta.dtype))
-        return o[0:1].to(theta.device, theta.dtype).reshape(())
+        # one copy to theta's device and type holds both (model.out is the next call's too)
+        o = model.logl_grad_async(theta.detach().tolist()).to(theta.device, theta.dtype, copy=True)
+        ctx.save_for_backward(o[1:])
+        return o[0].clone()
 
     @staticmethod
     def backward(ctx, g):
