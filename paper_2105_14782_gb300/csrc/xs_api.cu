@@ -427,7 +427,8 @@ int model_forward_impl(const xs_model* m, const double* theta, double* F0out, ch
                             m->cia_vmr2, m->gravity, m->mu, 1, dtau, st);
         if (r) return r;
     }
-    return xsi::rt_emission(dtau, T, m->nu, m->L, m->N, F0out, st);
+    return xsi::rt_emission(dtau, T, m->nu, m->L, m->N, F0out, st,
+                            (xs_flags & xsi::XS_RUN_KEEP_ADJ) ? ws + p.emws : nullptr);
 }
 
 } // namespace
@@ -476,7 +477,7 @@ int model_adjoint_impl(const xs_model* m, const double* theta, const double* gF,
     double* gTtmp = (double*)(ws + p.gTtmp);
     double* gb = (double*)(ws + p.gb);
     int r;
-    if ((r = xsi::rt_emission_adjoint(gF, dtau, T, m->nu, m->L, m->N, gdtau, gT, ws + p.emws, st))) return r;
+    if ((r = xsi::rt_emission_adjoint(gF, dtau, T, m->nu, m->L, m->N, gdtau, gT, ws + p.emws, st, true))) return r;
     if (m->cia_alpha &&
         (r = xsi::rt_tau_cia_adjoint(gdtau, m->cia_alpha, m->cia_T, m->cia_nT, T, m->P_bar, m->dP_bar, m->L, m->N,
                                      m->cia_vmr1, m->cia_vmr2, m->gravity, m->mu, gT, st)))

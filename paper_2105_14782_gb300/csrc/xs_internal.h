@@ -75,11 +75,12 @@ int rt_tau(const void* const* sigma, int32_t S, const double* vmr, const double*
 int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const double* P, const double* dP,
                    int32_t L, int64_t N, double g, double mu, int prec, const double* g_dtau, double* const* g_sigma,
                    double* g_vmr, cudaStream_t st);
+// keep: the adjoint's workspace, filled for an adjoint of the same call (reuse)
 int rt_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
-                cudaStream_t st);
+                cudaStream_t st, void* keep = nullptr);
 size_t rt_emission_ws(int32_t L, int64_t N);
 int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
-                        int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st);
+                        int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st, bool reuse = false);
 int rt_loglike(const double* F, const double* d, const double* s, int64_t N, double* logL, double* g_F,
                cudaStream_t st);
 // layer temperatures (T may be null) and mixing ratios (vmr may be null)

@@ -225,11 +225,13 @@ __device__ __forceinline__ void seg_range(int L, int w, int segs, int* n0, int* 
     *n1 = (int)(((int64_t)L * (w + 1)) / segs);
 }
 
-template <int PTS>
+// KEEP: the layer's T_n, E2_n and S_n are stored for the adjoint of the same call.
+template <int PTS, bool KEEP>
 __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __restrict__ dtau,
                                                               const double* __restrict__ T,
                                                               const double* __restrict__ nu, int L, int64_t N,
-                                                              double* __restrict__ F0)
+                                                              double* __restrict__ F0, double* __restrict__ w_tr,
+                                                              double* __restrict__ w_e2, double* __restrict__ w_S)
 {
     constexpr int SEG = RT_THREADS / PTS;
     __shared__ double segP[SEG][PTS], segF[SEG][PTS];
@@ -244,9 +246,15 @@ __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __re
     if (valid) {
         for (int n = n0; n < n1; ++n) {
             double e2, e3;
-            exp_int23(dtau[(size_t)n * N + j], &e2, &e3);
-            const double tr = 2.0 * e3;
-            F += phi * (1.0 - tr) * bose(kv, cv * rcp64_any(T[n]));
+            const size_t i = (size_t)n * N + j;
+            exp_int23(dtau[i], &e2, &e3);
+            const double tr = 2.0 * e3, Sn = bose(kv, cv * rcp64_any(T[n]));
+            if (KEEP) {
+                w_tr[i] = tr;
+                w_e2[i] = e2;
+                w_S[i] = Sn;
+            }
+            F += phi * (1.0 - tr) * Sn;
             phi *= tr;
         }
     }
@@ -270,8 +278,9 @@ __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __re
 // Three passes over each group's layer segment: (1) T, E2, S stored and the
 // segment's maps F_top = A F_bottom + C and prod T; (2) after chaining the
 // segments, F_{n+1} down the segment; (3) Phi_n along it, g_dtau and the
-// per-layer sums of lambda dF0/dS_n dS_n/dT_n over the block's points.
-template <int PTS>
+// per-layer sums of lambda dF0/dS_n dS_n/dT_n over the block's points.  REUSE: the
+// factors of (1) are the forward's (KEEP) and only chained.
+template <int PTS, bool REUSE>
 __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     const double* __restrict__ g_F0, const double* __restrict__ dtau, const double* __restrict__ T,
     const double* __restrict__ nu, int L, int64_t N, double* __restrict__ g_dtau, double* __restrict__ part,
@@ -292,12 +301,19 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     if (valid) {
         for (int n = n1 - 1; n >= n0; --n) {
             const size_t i = (size_t)n * N + j;
-            double e2, e3;
-            exp_int23(dtau[i], &e2, &e3);
-            const double tr = 2.0 * e3, Sn = bose(kv, cv * rcp64_any(T[n]));
-            w_tr[i] = tr;
-            w_e2[i] = e2;
-            w_S[i] = Sn;
+            double tr, Sn;
+            if (REUSE) {
+                tr = w_tr[i];
+                Sn = w_S[i];
+            } else {
+                double e2, e3;
+                exp_int23(dtau[i], &e2, &e3);
+                tr = 2.0 * e3;
+                Sn = bose(kv, cv * rcp64_any(T[n]));
+                w_tr[i] = tr;
+                w_e2[i] = e2;
+                w_S[i] = Sn;
+            }
             Cm = tr * Cm + (1.0 - tr) * Sn;
             A *= tr;
         }
@@ -581,42 +597,62 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
 // Points a block of the emission kernels takes: see emission_kernel.
 static int emission_points(int64_t N) { return N >= 608 * 32 ? 32 : N >= 608 * 16 ? 16 : 8; }
 
-int rt_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
-                cudaStream_t st)
-{
-    const int pts = emission_points(N);
-    const unsigned nb = (unsigned)((N + pts - 1) / pts);
-    if (pts == 32) emission_kernel<32><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
-    else if (pts == 16) emission_kernel<16><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
-    else emission_kernel<8><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0);
-    return launched(1);
-}
-
 // [L][nb] per-block layer partials, then T_n, E2_n and S_n as [L][N] each
-size_t rt_emission_ws(int32_t L, int64_t N)
-{
-    const int pts = emission_points(N);
-    int64_t nb = (N + pts - 1) / pts;
-    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    return al(sizeof(double) * (size_t)L * (size_t)nb) + 3 * al(sizeof(double) * (size_t)L * (size_t)N);
-}
-
-int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
-                        int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st)
+struct EmissionWs {
+    double *part, *tr, *e2, *S;
+    size_t bytes;
+};
+static EmissionWs emission_ws(int32_t L, int64_t N, void* ws)
 {
     const int pts = emission_points(N);
     const int64_t nb = (N + pts - 1) / pts;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t part = al(sizeof(double) * (size_t)L * (size_t)nb), LN = al(sizeof(double) * (size_t)L * (size_t)N);
     char* base = (char*)ws;
-    double* part = (double*)base;
-    const size_t LN = al(sizeof(double) * (size_t)L * (size_t)N);
-    double* w_tr = (double*)(base + al(sizeof(double) * (size_t)L * (size_t)nb));
-    double* w_e2 = (double*)((char*)w_tr + LN);
-    double* w_S = (double*)((char*)w_e2 + LN);
-    auto* kernel = pts == 32 ? emission_adjoint_kernel<32>
-                             : pts == 16 ? emission_adjoint_kernel<16> : emission_adjoint_kernel<8>;
-    kernel<<<(unsigned)nb, RT_THREADS, 0, st>>>(g_F0, dtau, T, nu, L, N, g_dtau, part, w_tr, w_e2, w_S);
-    layer_sum_kernel<<<L, RT_THREADS, 0, st>>>(part, (int)nb, L, g_T);
+    return {(double*)base, (double*)(base + part), (double*)(base + part + LN), (double*)(base + part + 2 * LN),
+            part + 3 * LN};
+}
+
+template <int PTS>
+static void launch_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
+                            void* keep, cudaStream_t st)
+{
+    const unsigned nb = (unsigned)((N + PTS - 1) / PTS);
+    const EmissionWs w = emission_ws(L, N, keep);
+    if (keep) emission_kernel<PTS, true><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0, w.tr, w.e2, w.S);
+    else emission_kernel<PTS, false><<<nb, RT_THREADS, 0, st>>>(dtau, T, nu, L, N, F0, nullptr, nullptr, nullptr);
+}
+
+int rt_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
+                cudaStream_t st, void* keep)
+{
+    const int pts = emission_points(N);
+    if (pts == 32) launch_emission<32>(dtau, T, nu, L, N, F0, keep, st);
+    else if (pts == 16) launch_emission<16>(dtau, T, nu, L, N, F0, keep, st);
+    else launch_emission<8>(dtau, T, nu, L, N, F0, keep, st);
+    return launched(1);
+}
+
+size_t rt_emission_ws(int32_t L, int64_t N) { return emission_ws(L, N, nullptr).bytes; }
+
+template <int PTS>
+static void launch_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
+                                    int64_t N, double* g_dtau, const EmissionWs& w, bool reuse, cudaStream_t st)
+{
+    const unsigned nb = (unsigned)((N + PTS - 1) / PTS);
+    auto* k = reuse ? emission_adjoint_kernel<PTS, true> : emission_adjoint_kernel<PTS, false>;
+    k<<<nb, RT_THREADS, 0, st>>>(g_F0, dtau, T, nu, L, N, g_dtau, w.part, w.tr, w.e2, w.S);
+}
+
+int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
+                        int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st, bool reuse)
+{
+    const int pts = emission_points(N);
+    const EmissionWs w = emission_ws(L, N, ws);
+    if (pts == 32) launch_emission_adjoint<32>(g_F0, dtau, T, nu, L, N, g_dtau, w, reuse, st);
+    else if (pts == 16) launch_emission_adjoint<16>(g_F0, dtau, T, nu, L, N, g_dtau, w, reuse, st);
+    else launch_emission_adjoint<8>(g_F0, dtau, T, nu, L, N, g_dtau, w, reuse, st);
+    layer_sum_kernel<<<L, RT_THREADS, 0, st>>>(w.part, (int)((N + pts - 1) / pts), L, g_T);
     return launched(2);
 }
 
