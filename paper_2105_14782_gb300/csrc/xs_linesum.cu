@@ -24,11 +24,18 @@
 // interval's middle (less where the smallest Lorentz width already keeps the poles
 // away), and |z| >= Z0 at every point of the interval.  Measured over a in 1e-4 .. 100
 // and half-widths of 0.01 .. 300 Doppler units against wofz, the interpolation error is
-// below 1.5e-8 of the profile with 10 nodes, kappa = 4.5, Z0 = 6 (FP32) and below 2e-16
-// with 18 nodes, kappa = 5, Z0 >= 8 (FP64, where the forms need |z| >= 10): under the rounding of the evaluations.
+// below 1.6e-8 of the profile with 12 nodes, kappa = 3.3, Z0 = 6 (FP32; 1.9e-8 with 10
+// and kappa = 4.5) and below 2e-16 with 18 nodes, kappa = 5, Z0 >= 8 (FP64, where the
+// forms need |z| >= 10): under the rounding of the evaluations.  At one accuracy more
+// nodes allow a smaller kappa: the far evaluations go as nodes x kappa, the near lines as
+// kappa, but registers, polynomials and node weights as the nodes.  FP32, 100 layers of
+// 220,000 lines forward + gradient: 34.7 ms with 10 nodes (kappa 4.5), 31.6 with 12,
+// 32.1 with 14 (2.7), 31.6 with 16 (2.4); 3,060,000 lines x 4 layers 45.6, 45.2, 47.1,
+// 46.4 ms; FP64, 80 layers of a retrieval 23.7 ms with 18 nodes, 22.9 with 20 (4.0) and
+// 22.4 with 24 (3.1), but one layer 278, 285 and 290 us.
 //
 // What it saves: of the in-cut pairs of 220,000 lines on a 20,000-point grid about 4% are
-// evaluated at a point and the rest at 10 nodes per interval.  The 100-layer forward +
+// evaluated at a point and the rest at the nodes of an interval.  The 100-layer forward +
 // gradient step on them went from 224 to 52 ms, 4 layers of 3,060,000 lines on 100,000
 // points from 564 to 68 ms (every pair evaluated before), 20,000 lines on 20,000 points
 // and 10 layers forward from 1.12 to 0.34 ms.
@@ -48,7 +55,10 @@ namespace xsd {
 
 constexpr int LEAF = 32;       // grid points of a leaf: one per lane
 constexpr int LEVELS = 4;      // leaves and the intervals of 4, 16, 64 leaves
-constexpr int FAR_WARPS = 4;   // neighbouring intervals of one block share most lines
+// Neighbouring intervals of one block share most lines.  Two warps end a block sooner than
+// four, whose registers wait for the longest list: 20,000 lines x 10 layers 217 against
+// 222 us, 100 layers with the gradient 31.6 against 32.1 ms (eight warps: 6% above four).
+constexpr int FAR_WARPS = 2;
 
 // most warps of a leaf kernel's block (choose_leaf_blocks)
 template <class R> struct LeafWarps { static constexpr int v = 4; };
@@ -57,32 +67,36 @@ template <> struct LeafWarps<double> { static constexpr int v = 8; };
 // nodes and far condition per precision
 template <class R> struct Far;
 template <> struct Far<float> {
-    static constexpr int n = 10;
-    static constexpr double kappa = 4.5, Z0 = 6.0;
+    static constexpr int n = 12;
+    static constexpr double kappa = 3.3, Z0 = 6.0;
 };
 template <> struct Far<double> {
     static constexpr int n = 18;
     static constexpr double kappa = 5.0, Z0 = 10.0;
 };
 
-__device__ const ChebTable<10> CHEB10 = make_cheb<10>();
-__device__ const ChebTable<18> CHEB18 = make_cheb<18>();
-template <int n> __device__ __forceinline__ double cheb(int k, int m) { return (n == 10) ? CHEB10.T[k][m] : CHEB18.T[k][m]; }
+template <class R> static __device__ const ChebTable<Far<R>::n> CHEB = make_cheb<Far<R>::n>();
+template <int n> __device__ __forceinline__ double cheb(int k, int m)
+{
+    if constexpr (n == Far<float>::n) return CHEB<float>.T[k][m];
+    else return CHEB<double>.T[k][m];
+}
 struct ChebTableF {
-    float T[10][10];
+    float T[Far<float>::n][Far<float>::n];
 };
 constexpr ChebTableF make_cheb_f()
 {
+    constexpr int n = Far<float>::n;
     ChebTableF r{};
-    const ChebTable<10> c = make_cheb<10>();
-    for (int k = 0; k < 10; ++k)
-        for (int m = 0; m < 10; ++m) r.T[k][m] = (float)c.T[k][m];
+    const ChebTable<n> c = make_cheb<n>();
+    for (int k = 0; k < n; ++k)
+        for (int m = 0; m < n; ++m) r.T[k][m] = (float)c.T[k][m];
     return r;
 }
-__device__ const ChebTableF CHEB10F = make_cheb_f();
+__device__ const ChebTableF CHEB_F = make_cheb_f();
 // in the type of the path
-__device__ __forceinline__ float cheb_r(float, int k, int m) { return CHEB10F.T[k][m]; }
-__device__ __forceinline__ double cheb_r(double, int k, int m) { return CHEB18.T[k][m]; }
+__device__ __forceinline__ float cheb_r(float, int k, int m) { return CHEB_F.T[k][m]; }
+__device__ __forceinline__ double cheb_r(double, int k, int m) { return CHEB<double>.T[k][m]; }
 // the nodes as literals for unrolled loops
 template <int n> struct NodeTable {
     float t[n];
