@@ -414,12 +414,13 @@ def step_bench(dev, stream, atm, prec, steps, warmup, rank, world, dist, e2e_ste
 
 
 def roofline(res, atm, workload, steps, n_sm, clk):
-    """The dominant line-sum kernel against the FP32 pipe: FP32 flops per launch
-    (flops per in-cut triple x the launch's triples) over its mean launch time."""
+    """The dominant line-sum kernels against the FP32 pipe: FP32 flops of a step's
+    launches (flops per in-cut triple x the triples) over their mean time."""
     fwd_ms, fwd_n, adj_ms, adj_n = res["prof"]
     kind = "adj" if adj_ms >= fwd_ms else "fwd"
-    k_ms = (adj_ms if kind == "adj" else fwd_ms) / max(adj_n if kind == "adj" else fwd_n, 1)
-    per_launch = res["triples"] / len(atm.species)  # one launch per species and step, averaged over species
+    groups = max(adj_n if kind == "adj" else fwd_n, 1)  # species with plans of one shape run together
+    k_ms = (adj_ms if kind == "adj" else fwd_ms) / groups
+    per_launch = res["triples"] * steps / groups
     fl = FLOPS_PER_TRIPLE.get(workload)
     measured = bool(fl) and FLOPS_PER_TRIPLE["sources_sha256"] == kernel_sources_sha256()
     fpt = fl[kind] if measured else None
@@ -432,13 +433,13 @@ def roofline(res, atm, workload, steps, n_sm, clk):
     traffic = None
     if TRAFFIC["sources_sha256"] == kernel_sources_sha256() and TRAFFIC.get(workload):
         traffic = TRAFFIC[workload][kind] * len(atm.p_bar)
-    # algorithmic bytes of one launch (averaged over species): per (layer, line) the
-    # records rec1 + rec2 + near range (+ rec3 in the adjoint), per line the cut range
-    # and centre pair, per layer and point the lambda or near-sum read and the output
+    # algorithmic bytes of one group of launches: per (layer, line) the records rec1 +
+    # rec2 (+ rec3 in the adjoint, + the part of 1/beta beyond a float in the forward),
+    # per line the centre pair, per species, layer and point the lambda or sigma
     L, N = len(atm.p_bar), len(atm.nu)
-    nl_avg = sum(sp.n for sp in atm.species) / len(atm.species)
-    rec = 48 if kind == "adj" else 40
-    algo_bytes = nl_avg * (rec * L + 16) + L * N * (8 + (0 if kind == "adj" else 4))
+    rec = 40 if kind == "adj" else 36
+    algo_bytes = (sum(sp.n * (rec * L + 8) for sp in atm.species) +
+                  len(atm.species) * L * N * (8 if kind == "adj" else 4)) * steps / groups
     name = ("up_kernel + far_adjoint_kernel + leaf_adjoint_f32" if kind == "adj" else
             "far_sum_kernel + down_kernel + leaf_kernel_f32")
     return {"bound": "alu", "achieved": achieved, "peak": peak_max, "unit": "TFLOP/s",

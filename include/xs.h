@@ -139,9 +139,8 @@ int xs_compute(const xs_lines* lines, const double* nu, int64_t N, const double*
  * process exits.  Problems whose smallest plan (one layer at a time) needs more
  * than 64 MiB, i.e. xs_workspace_min_bytes(n, N, L, prec) > 64 MiB, are
  * rejected with XS_ETOOBIG before any launch.  That plan holds about n * 68
- * bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records, the
- * near-pair sums (N * 8 bytes, mixed) and split-K partials (up to 64 * N * 8
- * bytes); xs_workspace_min_bytes gives the exact figure.
+ * bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records and the
+ * adjoint's partial sums; xs_workspace_min_bytes gives the exact figure.
  * The first call on each device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call
  * before any stream capture.  All calls on a device share the one array and
@@ -449,10 +448,10 @@ int lines_contribution_filter(const xs_lines* lines, const double* P_bar, const 
 
 /*
  * Diagnostics (no paper counterpart).  xs_profile(1) makes the library record a
- * CUDA event pair around every line-sum kernel launch (forward and adjoint,
- * on the launching stream) until xs_profile(0); xs_profile_read synchronises
- * those events and returns the summed kernel times in ms and the launch counts
- * since profiling was enabled.  xs_launch_count returns how many kernels the
+ * CUDA event pair around the line-sum kernels of every chunk of layers (forward
+ * and adjoint, all species that run together, on the launching stream) until
+ * xs_profile(0); xs_profile_read synchronises those events and returns the summed
+ * times in ms and the event pairs' counts since profiling was enabled.  xs_launch_count returns how many kernels the
  * library has launched since it was loaded (host-side counter, all threads).
  */
 int xs_profile(int enable);

@@ -84,9 +84,9 @@ template <> struct vec4<double> { using type = double4_32a; };
 // Per-precision Faddeeva tier table.
 template <class R> struct Tier;
 template <> struct Tier<float> {
-    // The FP32 path evaluates w only through the wing forms (|z| >= 25, main
-    // kernels), the polynomial in 1/|z|^2 (6 <= |z| < 25) and the series below
-    // |z| = 6 (near kernels, w_series_tab); these are the series' parameters.
+    // The FP32 path evaluates w only through the wing forms (|z| >= 16.5), the
+    // polynomial in 1/|z|^2 (6 <= |z| < 16.5) and the series below |z| = 6
+    // (series_sums); these are the series' parameters.
     static constexpr float z2_series = 64.0f;  // K(a) is precomputed for lines with a^2 below this
     static constexpr float h = 0.7f;           // series step (error ~1e-8 relative)
 };
@@ -244,7 +244,7 @@ __device__ __forceinline__ double exp_negsq(double x)
     return fma(e, -lo, e);
 }
 
-// Per-line table for w_series_tab: d[n + SER_OFF] = 1/(n^2 h^2 + a^2) for n != 0 and 0
+// Per-line table for series_sums: d[n + SER_OFF] = 1/(n^2 h^2 + a^2) for n != 0 and 0
 // for n = 0, n = -SER_OFF .. SER_TAB - 1 - SER_OFF.  The odd row length keeps the lanes
 // that fill 32 rows on different banks.
 constexpr int SER_OFF = 6;   // terms on each side of the peak

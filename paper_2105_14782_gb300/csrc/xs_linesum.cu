@@ -54,7 +54,9 @@
 namespace xsd {
 
 constexpr int LEAF = 32;       // grid points of a leaf: one per lane
-constexpr int LEVELS = 4;      // leaves and the intervals of 4, 16, 64 leaves
+constexpr int TOP_LOG = 6;     // the largest intervals have 64 leaves;
+constexpr int TOP = 1 << TOP_LOG; // an interval has 2 or 4 below it (Tree::shift 1 or 2)
+constexpr int LEVELS = TOP_LOG + 1; // most levels
 // Neighbouring intervals of one block share most lines.  Two warps end a block sooner than
 // four, whose registers wait for the longest list: 20,000 lines x 10 layers 217 against
 // 222 us, 100 layers with the gradient 31.6 against 32.1 ms (eight warps: 6% above four).
@@ -122,6 +124,7 @@ struct Tree {
     const int2* win;    // lines [x, y) with an in-cut point in it (leaves only)
     const int2* pq;     // per layer: lines [x, y) too near for the far form
     int cnt[LEVELS], off[LEVELS], total;
+    int shift, top;     // log2 of the intervals below one; the top level: TOP_LOG / shift
     int on;             // 0: no intervals (small workspaces): every line is near
 };
 
@@ -242,10 +245,11 @@ __global__ void setup_kernel(const __grid_constant__ Batch<R> batch, const doubl
     t -= n_agg;
     if (!tr.on || t >= 4 * (int64_t)tr.total) return;
     const int which = (int)(t & 3), q = (int)(t >> 2);
-    int k = LEVELS - 1;
+    int k = tr.top;
     while (k > 0 && q < tr.off[k]) --k;
-    const int64_t j0 = (int64_t)(q - tr.off[k]) * (LEAF << (2 * k));
-    const int64_t j1 = min64(N, j0 + (LEAF << (2 * k))) - 1;
+    const int points = LEAF << (tr.shift * k);
+    const int64_t j0 = (int64_t)(q - tr.off[k]) * points;
+    const int64_t j1 = min64(N, j0 + points) - 1;
     const double v0 = nu[j0], v1 = nu[j1];
     if (which == 0) {
         const double h = 0.5 * (v1 - v0);
@@ -531,12 +535,13 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi) { return min(max(v,
 
 // The set of interval i of a level, from the top interval above it downwards: near
 // lines are kept out of the parent's far ones.
+template <int shift>
 __device__ __forceinline__ FarSet far_set(const Tree& tr, int level, int i, int nloc)
 {
     FarSet f{};
     bool left = false, right = false; // the interval above has far lines on that side
-    for (int k = LEVELS - 1; k >= level; --k) {
-        const int at = tr.off[k] + (i >> (2 * (k - level)));
+    for (int k = TOP_LOG / shift; k >= level; --k) {
+        const int at = tr.off[k] + (i >> (shift * (k - level)));
         const int2 c = tr.cov[at], s = tr.pq[(size_t)tr.total * nloc + at];
         const int a = c.x, b = max(c.x, c.y);
         f.A = left ? f.a : a;
@@ -551,6 +556,12 @@ __device__ __forceinline__ FarSet far_set(const Tree& tr, int level, int i, int 
         right = f.b > f.q;
     }
     return f;
+}
+
+// both steps unrolled: the loads of a loop of unknown length wait for one another
+__device__ __forceinline__ FarSet far_set(const Tree& tr, int level, int i, int nloc)
+{
+    return tr.shift == 2 ? far_set<2>(tr, level, i, nloc) : far_set<1>(tr, level, i, nloc);
 }
 
 // The lines of an interval that are not its parent's, as one numbering 0 .. total - 1.
@@ -1060,7 +1071,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
 __device__ __forceinline__ bool far_task(const Tree& tr, const FarWork& fw, int* level, int* i, int* part)
 {
     int k = 0;
-    while (k < LEVELS - 1 && (int)blockIdx.x < fw.block0[k]) ++k;
+    while (k < tr.top && (int)blockIdx.x < fw.block0[k]) ++k;
     const int r = blockIdx.x - fw.block0[k];
     *level = k;
     *part = r % fw.parts[k];
@@ -1086,6 +1097,11 @@ __device__ __forceinline__ Lines<R> layer_lines(Lines<R> ln, int64_t nl, int nlo
     if (ln.clo) ln.clo += lay;
     return ln;
 }
+
+// Blocks on an SM that the far adjoint's registers have to leave room for (102 and 128 a
+// thread): unbounded the FP32 one takes 123 and is 17% slower (16 warps an SM, not 20).
+template <class R> struct FarBlocks { static constexpr int v = 10; };
+template <> struct FarBlocks<double> { static constexpr int v = 8; };
 
 template <class R>
 __global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(const __grid_constant__ Batch<R> batch,
@@ -1114,7 +1130,7 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(const __grid_co
 }
 
 template <class R>
-__global__ void __launch_bounds__(32 * FAR_WARPS) far_adjoint_kernel(const __grid_constant__ Batch<R> batch,
+__global__ void __launch_bounds__(32 * FAR_WARPS, FarBlocks<R>::v) far_adjoint_kernel(const __grid_constant__ Batch<R> batch,
                                                                      const double* __restrict__ nu, int layer0,
                                                                      const double* __restrict__ T)
 {
@@ -1204,26 +1220,26 @@ struct LeafPoly<float> {
 };
 
 // Polynomials of the leaves: the node sums of each level plus the polynomial of the
-// interval above, from the top interval down.  A block takes the leaves under one interval
-// of level `root` and repeats the chain of intervals above it: root = 3 (64 leaves, nothing
-// repeated) where that makes enough blocks to fill the chip, smaller subtrees otherwise.
+// interval above, from the top interval down.  A block takes 2^root_log leaves and repeats
+// the chain of intervals above them: root_log = 6 (64 leaves, nothing repeated) where that
+// makes enough blocks to fill the chip, smaller subtrees otherwise.
 template <class R> struct DownRows { static constexpr int v = 64; }; // intervals of a level that a block takes at a time
 template <> struct DownRows<double> { static constexpr int v = 32; };
 template <class R>
 __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const __grid_constant__ Batch<R> batch, int Lc,
-                                                                     int root)
+                                                                     int root_log)
 {
     const Species<R>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
     const FarWork& fw = sp.fw;
-    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
-    __shared__ double v[DownRows<R>::v][n], c[2][TOP / 4][n];
+    constexpr int n = Far<R>::n;
+    __shared__ double v[DownRows<R>::v][n], c[2][TOP / 2][n];
     const int m = threadIdx.x % n, row = threadIdx.x / n, rows = blockDim.x / n;
     const int nloc = blockIdx.y;
-    for (int k = LEVELS - 1; k >= 0; --k) {
-        const int below = max(root - k, 0);
-        const int many = 1 << (2 * below);                                   // intervals of this level
-        const int first = k >= root ? blockIdx.x >> (2 * (k - root)) : blockIdx.x * many;
+    for (int k = tr.top; k >= 0; --k) {
+        const int below = root_log - tr.shift * k;
+        const int many = 1 << max(below, 0); // intervals of this level
+        const int first = below <= 0 ? blockIdx.x >> -below : blockIdx.x * many;
         for (int q0 = 0; q0 < many; q0 += rows) {
             const int q = q0 + row, i = first + q;
             const bool mine = q < many && i < tr.cnt[k];
@@ -1231,9 +1247,9 @@ __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const 
                 double s = 0.0;
                 for (int p = 0; p < fw.parts[k]; ++p)
                     s += sp.sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
-                if (k < LEVELS - 1) {
-                    const Geo g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> 2)];
-                    s += clenshaw<n, double>(c[(k + 1) & 1][q >> 2], in_span(fma(g.h, cheb<n>(1, m), g.mid), gp));
+                if (k < tr.top) {
+                    const Geo g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> tr.shift)];
+                    s += clenshaw<n, double>(c[(k + 1) & 1][q >> tr.shift], in_span(fma(g.h, cheb<n>(1, m), g.mid), gp));
                 }
                 v[row][m] = s;
             }
@@ -1278,7 +1294,7 @@ __device__ __forceinline__ R node_weight(const R* M, int m)
 }
 
 // Node weights of all intervals: per layer and top interval, one warp per leaf takes its
-// points, then the larger intervals take the nodes of the four below (whose weights
+// points, then the larger intervals take the nodes of those below (whose weights
 // reproduce every polynomial of the degree kept).  In the FP32 path in FP32, as lambda
 // itself: the rounding of one leaf's weights is independent of the next one's.
 // weights[layer][interval][n].
@@ -1290,13 +1306,13 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
 {
     const Species<R>& spc = batch.s[blockIdx.z];
     const Tree& tr = spc.tree;
-    constexpr int n = Far<R>::n, TOP = 1 << (2 * (LEVELS - 1));
+    constexpr int n = Far<R>::n;
     __shared__ R M[UP_WARPS][n], w[2][TOP][n];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int nloc = blockIdx.y, top = blockIdx.x;
     const double* g = spc.g_sigma + (size_t)(layer0 + nloc) * N;
-    for (int k = 0; k < LEVELS; ++k) {
-        const int many = 1 << (2 * (LEVELS - 1 - k));
+    for (int k = 0; k <= tr.top; ++k) {
+        const int many = 1 << (tr.shift * (tr.top - k)), below = 1 << tr.shift;
         for (int q = row; q < many; q += UP_WARPS) {
             const int i = top * many + q;
             if (i >= tr.cnt[k]) break;
@@ -1309,12 +1325,12 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
                 if (j < N) add_moments<n, R>((R)(g[j] * lam_scale), (R)in_span(nu[j], sp), s);
             } else {
 #pragma unroll 1
-                for (int r = lane; r < 4 * n; r += 32) {
-                    const int ch = 4 * i + r / n, m = r % n; // child interval and its node
+                for (int r = lane; r < below * n; r += 32) {
+                    const int ch = below * i + r / n, m = r % n; // child interval and its node
                     if (ch >= tr.cnt[k - 1]) break;
                     const Geo gc = tr.geo[tr.off[k - 1] + ch];
                     const R x = (R)in_span(fma(gc.h, cheb<n>(1, m), gc.mid), sp);
-                    add_moments<n, R>(w[(k - 1) & 1][4 * q + r / n][m], x, s);
+                    add_moments<n, R>(w[(k - 1) & 1][below * q + r / n][m], x, s);
                 }
             }
             __syncwarp();
@@ -2073,14 +2089,27 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 // leaf's warp, a few microseconds, about what the three launches of the intervals cost.
 constexpr int64_t TREE_MIN_LINES = 256;
 
+// Density of lines from which an interval has two intervals below it instead of four, in
+// half lines a grid point.  A level's list holds the lines between its far radius and that
+// of the interval above, so halving makes seven levels of a third of the list each instead
+// of four: 2/3 of the far evaluations for 1.5 times the polynomials, node weights and
+// reductions.  FP32, 20,000 points x 20 layers, us with quarters and halves: at one line a
+// point forward 362 and 371, adjoint 498 and 487; at two 615 and 606, 883 and 840; at
+// eight 2016 and 1893, 3126 and 2888.  FP64, 4,096 points x 20 layers, a line every two
+// points 2039 and 1877, 3920 and 3606 (one layer 279 and 286, 483 and 493), one a point
+// 3807 and 3464, 7249 and 6517.  With the choice at run time calls that keep the quarters
+// are up to 1% slower than with four fixed levels (one FP64 layer 268 -> 275 us).
+template <class R> struct DenseLines { static constexpr int64_t v = 4; };
+template <> struct DenseLines<double> { static constexpr int64_t v = 1; };
+
 struct XsPlan {
     int prec, Lc, nchunks, leaf_blocks, leaf_warps, leaf_split;
     Tree tree; // counts and offsets; pointers set at run time
     FarWork fw;
     int far_blocks;
     size_t rows; // node-sum rows of all levels and parts
-    size_t off_jr, off_nuf, off_inv, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq, off_fwd,
-        off_coef, off_wts, off_slots, off_leaf, off_gbl, total;
+    size_t off_jr, off_nuf, off_inv, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq,
+        off_fwd, off_coef, off_wts, off_slots, off_leaf, off_gbl, total;
 };
 
 // Parts of the far lists: enough warps to fill the GPU several times over, each with a
@@ -2093,9 +2122,11 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
     int block = 0;
     size_t row = 0;
     p->fw.slots = 0;
-    for (int k = LEVELS - 1; k >= 0; --k) {
-        const double share = std::min(1.0, 16.0 * (double)(LEAF << (2 * k)) / (double)N);
-        const int64_t est = (k == LEVELS - 1) ? nl : (int64_t)(share * (double)nl);
+    const Tree& tr = p->tree;
+    const double lengths = tr.shift == 2 ? 16.0 : 8.0;
+    for (int k = tr.top; k >= 0; --k) {
+        const double share = std::min(1.0, lengths * (double)(LEAF << (tr.shift * k)) / (double)N);
+        const int64_t est = (k == tr.top) ? nl : (int64_t)(share * (double)nl);
         const int64_t want = (warps + (int64_t)Lc * p->tree.cnt[k] - 1) / ((int64_t)Lc * p->tree.cnt[k]);
         const int parts = (int)std::max<int64_t>(1, std::min(want, est / min_lines));
         p->fw.parts[k] = parts;
@@ -2157,8 +2188,10 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     p.off_gbl = take(sizeof(double) * (size_t)L);
     p.tree.on = tree ? 1 : 0;
     if (tree) {
-        for (int k = 0; k < LEVELS; ++k) {
-            const int64_t pts = (int64_t)LEAF << (2 * k);
+        p.tree.shift = 2 * nl >= (mixed ? DenseLines<float>::v : DenseLines<double>::v) * N ? 1 : 2;
+        p.tree.top = TOP_LOG / p.tree.shift;
+        for (int k = 0; k <= p.tree.top; ++k) {
+            const int64_t pts = (int64_t)LEAF << (p.tree.shift * k);
             p.tree.cnt[k] = (int)((N + pts - 1) / pts);
             p.tree.off[k] = p.tree.total;
             p.tree.total += p.tree.cnt[k];
@@ -2284,8 +2317,9 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
     const double unscale = FAST ? MIXED_UNSCALE : 1.0;
     const unsigned nz = (unsigned)b.n;
     const Tree& tr = p.tree;
-    int setup_blocks = 0, param_blocks = 0, far_blocks = 0;
+    int setup_blocks = 0, param_blocks = 0, far_blocks = 0, intervals = 0;
     for (int m = 0; m < b.n; ++m) {
+        intervals = std::max(intervals, b.s[m].tree.total);
         setup_blocks = std::max(setup_blocks, b.s[m].setup_blocks);
         param_blocks = std::max(param_blocks, b.s[m].param_blocks);
         far_blocks = std::max(far_blocks, b.s[m].far_blocks);
@@ -2311,7 +2345,7 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
             count_launch();
             if (tr.on) {
                 near_range_kernel<R>
-                    <<<dim3(blocks_of(2 * (int64_t)tr.total, 256), (unsigned)lc, nz), 256, 0, st>>>(b, l0);
+                    <<<dim3(blocks_of(2 * (int64_t)intervals, 256), (unsigned)lc, nz), 256, 0, st>>>(b, l0);
                 count_launch();
             }
         }
@@ -2322,10 +2356,11 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
         if (!adjoint) {
             if (tr.on) {
                 far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(b, nu, l0);
-                int root = LEVELS - 1;
-                while (root > 1 && (int64_t)tr.cnt[root] * lc * b.n < 2 * 152) --root;
-                const int rows = std::min(DownRows<R>::v, 1 << (2 * root));
-                down_kernel<R><<<dim3((unsigned)tr.cnt[root], (unsigned)lc, nz), rows * Far<R>::n, 0, st>>>(b, lc, root);
+                int root = TOP_LOG; // log2 of the leaves of a block
+                auto subtrees = [&] { return blocks_of(tr.cnt[0], 1 << root); };
+                while (root > 2 && (int64_t)subtrees() * lc * b.n < 2 * 152) root -= 2;
+                const int rows = std::min(DownRows<R>::v, 1 << root);
+                down_kernel<R><<<dim3(subtrees(), (unsigned)lc, nz), rows * Far<R>::n, 0, st>>>(b, lc, root);
                 count_launch(2);
             }
             if constexpr (FAST)
@@ -2335,8 +2370,8 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                                                                                            p.leaf_split);
         } else {
             if (tr.on) {
-                up_kernel<R><<<dim3((unsigned)tr.cnt[LEVELS - 1], (unsigned)lc, nz), 32 * UP_WARPS, 0, st>>>(b, nu, N, l0,
-                                                                                                            unscale);
+                up_kernel<R><<<dim3(blocks_of(tr.cnt[0], TOP), (unsigned)lc, nz), 32 * UP_WARPS, 0, st>>>(b, nu, N, l0,
+                                                                                                         unscale);
                 far_adjoint_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(b, nu, l0, T);
                 count_launch(2);
             }

@@ -60,7 +60,7 @@ extern "C" int xs_compute_noalloc(const xs_lines* lines, const double* nu, int64
     r = noalloc_scratch(&scratch);
     if (r != XS_OK) return r;
     // Every scratch region the forward pass reads is written earlier in the same
-    // call (cut ranges, per-layer minima, line records, split-K partials), so the
+    // call (cut ranges, per-layer minima, line records), so the
     // previous call's contents never need clearing.
     const xsi::XsJob job{lines, scratch, XS_NOALLOC_SCRATCH_BYTES, sigma, nullptr, nullptr, nullptr};
     return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, false, (cudaStream_t)stream);

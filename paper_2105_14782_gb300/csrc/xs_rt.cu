@@ -590,7 +590,8 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
         sp.p[m] = sigma[m];
         gp.p[m] = g_sigma ? g_sigma[m] : nullptr;
     }
-    tau_adjoint_kernel<<<(unsigned)(RT_CLUSTER * L), RT_THREADS, 0, st>>>(sp, gp, S, vmr, dP, L, N, g, mu, prec == XS_PREC_MIXED, g_dtau, g_vmr);
+    tau_adjoint_kernel<<<(unsigned)(RT_CLUSTER * L), RT_THREADS, 0, st>>>(sp, gp, S, vmr, dP, L, N, g, mu,
+                                                                           prec == XS_PREC_MIXED, g_dtau, g_vmr);
     return launched(1);
 }
 

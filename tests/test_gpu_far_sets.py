@@ -33,7 +33,10 @@ def grid(kind, N, rng):
 
 CASES = [("log", 1, 300, 25.0), ("log", 31, 256, 25.0), ("log", 33, 255, 25.0), ("log", 129, 1000, 3.0),
          ("log", 2049, 3000, 25.0), ("log", 2048, 700, 0.01), ("random", 513, 2000, 2.0), ("gaps", 700, 2000, 4.0),
-         ("log", 8200, 1500, 6.0)]
+         ("log", 8200, 1500, 6.0),
+         # on both sides of the density from which intervals are halved, not quartered
+         ("log", 2049, 2 * 2049 - 1, 2.0), ("log", 2049, 2 * 2049, 2.0), ("log", 2300, 1149, 3.0), ("log", 2300, 1150, 3.0),
+         ("gaps", 700, 6000, 4.0), ("random", 70, 3000, 1.0)]
 P = np.array([1e-3, 0.3, 30.0])
 T = np.array([700.0, 1200.0, 1900.0])
 
