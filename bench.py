@@ -47,30 +47,29 @@ WALL_BUDGET_S = 1600.0
 
 FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM on sm_103a (one FFMA = 2 flops)
 
-# FP32 flops per in-cut triple of the two line-sum kernels, from the SASS
-# instruction counts of one ncu capture per workload (FFMA 2, FADD/FMUL 1, packed
-# FFMA2 4, FADD2/FMUL2 2 flops per thread instruction; MUFU reciprocals not
-# counted), divided by the launch's in-cut triples.  Valid only for the kernel
-# sources they were taken on (the hash); otherwise the bench reports no rate and says so.
+# FP32 flops per in-cut triple of a forward's and an adjoint's line-sum kernels, from the
+# instruction counters of one ncu capture per workload (FFMA 2, FADD/FMUL 1, packed
+# FFMA2 4, FADD2/FMUL2 2 flops per thread instruction; MUFU reciprocals not counted),
+# divided by the in-cut triples (most of which are covered by interval nodes).  Valid
+# only for the kernel sources they were taken on (the hash); otherwise the bench reports
+# no rate and says so.
 FLOPS_PER_TRIPLE = {
-    "sources_sha256": "bcfd701beb7a1f40c608e700fbcde5e1301ffb6eae228c6aed4523b1b23de8d7",
-    "scale": {"fwd": 9.00, "adj": 13.21,
-              "capture": "both species' launches of a 5-layer slice of the 10.2M-line workload (10,000,000 + "
-                         "200,000 lines, 100,000 points): 3.44e13 and 5.05e13 FP32 flops over 3.82e12 triples"},
-    "emission": {"fwd": 9.16, "adj": 13.38,
-                 "capture": "both species' launches of a 20-layer slice of the emission workload (200,000 + 20,000 "
-                            "lines, 20,000 points): 6.05e11 and 8.84e11 FP32 flops over 6.60e10 triples"},
+    "sources_sha256": "3014e98dbf773b6f1bfcea7fae5f82b34265f53effaa55d8d4723987b9013e13",
+    "scale": {"fwd": 0.4646, "adj": 0.8651,
+              "capture": "one step of a 5-layer slice of the 10.2M-line workload (10,000,000 + 200,000 lines, "
+                         "100,000 points): 1.78e+12 and 3.31e+12 FP32 flops over 3.82e+12 triples"},
+    "emission": {"fwd": 0.9448, "adj": 1.6799,
+                 "capture": "one step of a 20-layer slice of the emission workload (200,000 + 20,000 lines, "
+                            "20,000 points): 6.24e+10 and 1.11e+11 FP32 flops over 6.6e+10 triples"},
 }
 
-# DRAM bytes (read + write) per layer of one launch of each line-sum kernel, averaged
-# over the two species' launches, from one ncu capture of the same reduced-layer
-# slices (the traffic is per layer: each layer's records are read once from DRAM
-# when L2 serves the re-reads); null unless the sources still hash to the captured ones.
+# DRAM bytes (read + write) per layer of a forward's and an adjoint's line-sum kernels, both
+# species, from the same captures; null unless the sources still hash to the captured ones.
 TRAFFIC = {
-    "sources_sha256": "bcfd701beb7a1f40c608e700fbcde5e1301ffb6eae228c6aed4523b1b23de8d7",
-    "scale": {"fwd": 2.992e8, "adj": 3.132e8},
-    "emission": {"fwd": 3.04e7, "adj": 5.76e7},
-    "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of both species' launches, 5-layer slice of the "
+    "sources_sha256": "3014e98dbf773b6f1bfcea7fae5f82b34265f53effaa55d8d4723987b9013e13",
+    "scale": {"fwd": 1.068e+10, "adj": 1.497e+10},
+    "emission": {"fwd": 1.713e+07, "adj": 2.059e+07},
+    "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one step's line-sum kernels, 5-layer slice of the "
                "10.2M-line workload and 20-layer slice of the emission workload, scaled to the launch's layers",
 }
 
@@ -432,7 +431,7 @@ def roofline(res, atm, workload, steps, n_sm, clk):
     peak_med = n_sm * FP32_LANES_PER_SM * 2 * sm_med * 1e6 / 1e12
     traffic = None
     if TRAFFIC["sources_sha256"] == kernel_sources_sha256() and TRAFFIC.get(workload):
-        traffic = TRAFFIC[workload][kind] * len(atm.p_bar)
+        traffic = TRAFFIC[workload][kind] * len(atm.p_bar) * steps / groups
     # algorithmic bytes of one group of launches: per (layer, line) the records rec1 +
     # rec2 (+ rec3 in the adjoint, + the part of 1/beta beyond a float in the forward),
     # per line the centre pair, per species, layer and point the lambda or sigma
@@ -446,7 +445,7 @@ def roofline(res, atm, workload, steps, n_sm, clk):
             "frac": achieved / peak_max if measured else None,
             "traffic": traffic, "kernel": name, "kernel_ms_per_launch": k_ms, "triples_per_launch": per_launch,
             "flops_per_triple": fpt,
-            "flops_basis": (f"ncu SASS FP32 instruction counts ({fl['capture']})" if measured else
+            "flops_basis": (f"ncu FP32 instruction counters ({fl['capture']})" if measured else
                             "ncu counts not taken on these sources"),
             "peak_note": f"FP32 pipe: {n_sm} SMs (device) x {FP32_LANES_PER_SM} lanes x 2 flop x {sm_max:.0f} MHz "
                          "(max SM clock); derived, not measured",

@@ -34,11 +34,11 @@
 // 46.4 ms; FP64, 80 layers of a retrieval 23.7 ms with 18 nodes, 22.9 with 20 (4.0) and
 // 22.4 with 24 (3.1), but one layer 278, 285 and 290 us.
 //
-// What it saves: of the in-cut pairs of 220,000 lines on a 20,000-point grid about 4% are
-// evaluated at a point and the rest at the nodes of an interval.  The 100-layer forward +
-// gradient step on them went from 224 to 52 ms, 4 layers of 3,060,000 lines on 100,000
-// points from 564 to 68 ms (every pair evaluated before), 20,000 lines on 20,000 points
-// and 10 layers forward from 1.12 to 0.34 ms.
+// What it saves: of the in-cut pairs of 220,000 lines on a 20,000-point grid about 1% are
+// evaluated at a point and the rest at the nodes of an interval.  With every pair evaluated
+// the 100-layer forward + gradient step on them took 224 ms, now 29.6; 4 layers of
+// 3,060,000 lines on 100,000 points 564 and 44.3 ms; 20,000 lines on 20,000 points and 10
+// layers forward 1.12 and 0.22 ms.
 //
 // Precision (XS_PREC_MIXED): per-line scalars are formed in FP64 and rounded
 // once; line-centre offsets come from per-line float pairs (hi + lo where it
@@ -1130,9 +1130,9 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(const __grid_co
 }
 
 template <class R>
-__global__ void __launch_bounds__(32 * FAR_WARPS, FarBlocks<R>::v) far_adjoint_kernel(const __grid_constant__ Batch<R> batch,
-                                                                     const double* __restrict__ nu, int layer0,
-                                                                     const double* __restrict__ T)
+__global__ void __launch_bounds__(32 * FAR_WARPS, FarBlocks<R>::v)
+    far_adjoint_kernel(const __grid_constant__ Batch<R> batch, const double* __restrict__ nu, int layer0,
+                       const double* __restrict__ T)
 {
     const Species<R>& sp = batch.s[blockIdx.z];
     if ((int)blockIdx.x >= sp.far_blocks) return;
