@@ -76,3 +76,19 @@ def test_adjoint_with_and_without_far_sets(xs, kind, N, n, cut):
     assert np.max(np.abs(out[xs.PREC_FP64, "full"] - ref)) <= 1e-10 * big
     for name in ("full", "small"):
         assert np.max(np.abs(out[xs.PREC_MIXED, name] - ref)) <= 1e-4 * big
+
+
+@pytest.mark.parametrize("n,N", [(650, 6755), (1516, 2472)])
+def test_fp64_nodes_keep_the_precision(xs, n, N):
+    """FP64: far lines at nodes against every line at every point, few lines in narrow
+    intervals over a wide band (where a node's position, rounded to an ulp of nu, would be
+    1e-12 of an interval off): each is within about 1e-14 of the exact sum (the strengths'
+    exponents, the same in both), so 3e-14 of each other."""
+    nu, L = W.grid_lognu(N), 2
+    dl = xs.DeviceLines(W.water_like(n, seed=n))
+    p, t = dev([1e-3, 100.0]), dev([900.0, 1700.0])
+    small = torch.empty(xs.lib().xs_workspace_min_bytes(n, N, L, xs.PREC_FP64), dtype=torch.uint8, device="cuda")
+    a = xs.xs_compute(dl, dev(nu), t, p, 1.0, 25.0, xs.PREC_FP64)
+    b = xs.xs_compute(dl, dev(nu), t, p, 1.0, 25.0, xs.PREC_FP64, workspace=small)
+    m = b > 0
+    assert float(((a - b).abs()[m] / b[m]).max()) < 3e-14
