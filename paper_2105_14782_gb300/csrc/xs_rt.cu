@@ -115,12 +115,31 @@ __device__ __forceinline__ double bose(double a, double u)
     return fma(fma(-q, d, n), y, q);
 }
 
-// pi B(nu, T) = planck_c nu^3/(e^u - 1), u = c2 nu/T
+// pi B(nu, T) = planck_c nu^3/(e^u - 1), u = c2 nu/T.  An error of u grows u-fold in
+// e^u and stands undiminished in the adjoint's F_{n+1} - S_n, so u is formed to half an ulp:
+// the quotient by 1/T gets its residual, with what rounding c2 nu lost, back.  One function
+// for every layer's source and the bottom's, so that the bottom layer, which lies on its own
+// temperature, sees F_L - S_{L-1} = 0 exactly.
 constexpr double PLANCK_C = PI * 2.0 * hP * cL * cL;
-__device__ __forceinline__ double planck_pi(double nu, double T)
-{
-    return bose(PLANCK_C * nu * nu * nu, c2 * nu / T);
-}
+struct Planck {
+    double kv, cv, cl; // planck_c nu^3; c2 nu and its rounding error
+    __device__ __forceinline__ explicit Planck(double v)
+        : kv(PLANCK_C * v * v * v), cv(c2 * v), cl(fma(c2, v, -cv))
+    {
+    }
+    __device__ __forceinline__ double operator()(double T) const
+    {
+        const int e = __double2hiint(T) & 0x7ff00000;
+        double u;
+        if (e < 0x20b00000 || e > 0x5f300000) { // beyond 2^-500..2^500: 0, infinities, NaN
+            u = cv / T;
+        } else {
+            const double y = rcp64(T), q = cv * y;
+            u = fma(fma(-q, T, cv) + cl, y, q);
+        }
+        return bose(kv, u);
+    }
+};
 
 struct SigPtrs {
     const void* p[XS_MAX_SPECIES];
@@ -239,7 +258,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __re
     const int64_t j = (int64_t)blockIdx.x * PTS + lane;
     const bool valid = j < N;
     const double v = valid ? nu[j] : nu[0];
-    const double cv = c2 * v, kv = PLANCK_C * v * v * v;
+    const Planck planck(v);
     int n0, n1;
     seg_range(L, w, SEG, &n0, &n1);
     double phi = 1.0, F = 0.0;
@@ -248,7 +267,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __re
             double e2, e3;
             const size_t i = (size_t)n * N + j;
             exp_int23(dtau[i], &e2, &e3);
-            const double tr = 2.0 * e3, Sn = bose(kv, cv * rcp64_any(T[n]));
+            const double tr = 2.0 * e3, Sn = planck(T[n]);
             if (KEEP) {
                 w_tr[i] = tr;
                 w_e2[i] = e2;
@@ -267,7 +286,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_kernel(const double* __re
             Ft += ph * segF[s][lane];
             ph *= segP[s][lane];
         }
-        F0[j] = Ft + ph * planck_pi(v, T[L - 1]);
+        F0[j] = Ft + ph * planck(T[L - 1]);
     }
 }
 
@@ -293,7 +312,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     const bool valid = j < N;
     const double v = valid ? nu[j] : nu[0];
     const double lam = valid ? g_F0[j] : 0.0;
-    const double cv = c2 * v, kv = PLANCK_C * v * v * v;
+    const Planck planck(v);
     int n0, n1;
     seg_range(L, w, SEG, &n0, &n1);
     // (1) per-layer factors and the segment's backward map
@@ -309,7 +328,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
                 double e2, e3;
                 exp_int23(dtau[i], &e2, &e3);
                 tr = 2.0 * e3;
-                Sn = bose(kv, cv * rcp64_any(T[n]));
+                Sn = planck(T[n]);
                 w_tr[i] = tr;
                 w_e2[i] = e2;
                 w_S[i] = Sn;
@@ -323,7 +342,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     __syncthreads();
     if (w == 0) {
         // flux entering each segment from below, and Phi at each segment's top
-        double Fb = valid ? planck_pi(v, T[L - 1]) : 0.0;
+        double Fb = valid ? planck(T[L - 1]) : 0.0;
         for (int s = SEG - 1; s >= 0; --s) {
             segFin[s][lane] = Fb;
             Fb = segA[s][lane] * Fb + segC[s][lane];
@@ -348,7 +367,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
     // (3) forward along the segment (as many steps in every group of a warp, for the sums)
     double phi = segPhi[w][lane];
     const double phiL = segPhi[SEG - 1][lane] * segA[SEG - 1][lane];
-    const double inv_kv = 1.0 / kv;
+    const double inv_kv = 1.0 / planck.kv;
     const int most = (L + SEG - 1) / SEG;
     for (int k = 0; k < most; ++k) {
         const int n = n0 + k;
@@ -361,7 +380,7 @@ __global__ void __launch_bounds__(RT_THREADS) emission_adjoint_kernel(
             if (n == L - 1) gS += lam * phiL;
             phi *= tr;
             // d(pi B)/dT = B (u/T)/(1 - e^-u), and 1/(1 - e^-u) = 1 + 1/(e^u - 1) = 1 + B/kv
-            gT = gS * Sn * (cv * invT * invT) * fma(Sn, inv_kv, 1.0);
+            gT = gS * Sn * (planck.cv * invT * invT) * fma(Sn, inv_kv, 1.0);
         }
         for (int o = PTS / 2; o > 0; o >>= 1) gT += __shfl_xor_sync(0xffffffffu, gT, o, PTS);
         if (lane == 0 && n < n1) part[(size_t)n * gridDim.x + blockIdx.x] = gT;

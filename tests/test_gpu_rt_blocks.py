@@ -49,3 +49,15 @@ def test_transfer_at_the_block_sizes(N):
     Fn = F.cpu().numpy()
     assert ll.item() == pytest.approx(oracle.loglike(Fn, d, e), rel=1e-13)
     assert np.allclose(gF.cpu().numpy(), (d - Fn) / e ** 2, rtol=1e-14)
+
+
+@pytest.mark.parametrize("L", [1, 5, 40])
+def test_bottom_layer_on_its_own_temperature(L):
+    """The bottom source has the last layer's temperature, so F0 does not depend on that
+    layer's optical depth: its derivative is a difference of equal terms, exactly zero."""
+    from paper_2105_14782_gb300 import xs
+    N = 1003
+    rng = np.random.default_rng(L)
+    dtau, lam = rng.lognormal(-1.0, 2.0, (L, N)), rng.standard_normal(N)
+    gd, _ = xs.emission_spectrum_adjoint(dev(lam), dev(dtau), dev(rng.uniform(400.0, 2000.0, L)), dev(W.grid_lognu(N)))
+    assert torch.all(gd[L - 1] == 0.0)
