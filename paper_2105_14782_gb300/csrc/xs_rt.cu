@@ -119,7 +119,9 @@ __device__ __forceinline__ double bose(double a, double u)
 // e^u and stands undiminished in the adjoint's F_{n+1} - S_n, so u is formed to half an ulp:
 // the quotient by 1/T gets its residual, with what rounding c2 nu lost, back.  One function
 // for every layer's source and the bottom's, so that the bottom layer, which lies on its own
-// temperature, sees F_L - S_{L-1} = 0 exactly.
+// temperature, sees F_L - S_{L-1} = 0 exactly.  Against quadruple precision, 24 layers x 300
+// points, rms of F and g_dtau 3.4e-16 and 3.6e-16; with a rounded product c2 nu (1/T) 4.9e-16
+// and 5.7e-16, with a division 4.5e-16 and 4.6e-16; no difference in time beyond the runs'.
 constexpr double PLANCK_C = PI * 2.0 * hP * cL * cL;
 struct Planck {
     double kv, cv, cl; // planck_c nu^3; c2 nu and its rounding error
