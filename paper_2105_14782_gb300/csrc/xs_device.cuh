@@ -486,8 +486,8 @@ __device__ __forceinline__ void w_series_deriv(double x, double a, double inv_a,
 // ------------------------------------------------------------------ wing polynomials
 //
 // The asymptotic series of Eq. asywofz, truncated after the term k = ASY_K, as a
-// polynomial in u = 1/|z|^2 with per-line coefficients (FP32 near kernels,
-// 6 <= |z| < 25).  Term k is c_k Re(i z^-(2k+1))/sqrt(pi) = c_k Im(z^(2k+1)) u^(2k+1)/sqrt(pi),
+// polynomial in u = 1/|z|^2 with per-line coefficients (FP32, |z| >= 6, a < WIDE_A).
+// Term k is c_k Re(i z^-(2k+1))/sqrt(pi) = c_k Im(z^(2k+1)) u^(2k+1)/sqrt(pi),
 // c_k = (2k-1)!!/2^k.  Writing z^m = x alpha_m + i beta_m with alpha_m, beta_m
 // homogeneous polynomials in r = |z|^2 and a (x^2 = r - a^2), multiplication by
 // z^2 = (r - 2a^2) + 2iax gives
@@ -499,13 +499,16 @@ __device__ __forceinline__ void w_series_deriv(double x, double a, double inv_a,
 // fixed x gives
 //   a H_a = sum_n E_n u^(n+1) - 2 a^2 sum_n (n+1) C_n u^(n+2),  E_n = (1/sqrt(pi)) sum_{k+j=n} (2j+1) c_k q_kj a^(2j+1).
 // With ASY_K = 6 the truncation and FP32 rounding stay below 4e-7 of H for |z| >= 6.
-// To keep every coefficient inside the FP32 range (a up to 25, scaled strengths
-// up to ~1e13) the polynomials are written in v = ASY_S u (v < 1 for |z| >= 6):
+// To keep every coefficient inside the FP32 range (powers up to a^13, a^15 in the adjoint;
+// a < WIDE_A, scaled strengths up to 1e18) the polynomials are written in v = ASY_S u (v < 1 for |z| >= 6):
 // the table holds c_k q_kj / ASY_S^k and a^(2j) enters as (a^2/ASY_S)^j, so that
 // H = u sum_n C'_n v^n with C'_n = C_n / ASY_S^n (a power of two: exact).
 constexpr int ASY_K = 6;
 constexpr int ASY_N = 2 * ASY_K + 1; // powers u^1 .. u^13
 constexpr float ASY_S = 32.0f;
+// Lines from this a on have |z| >= 100 at every point and take the K = 1 wing form where
+// the lines beside them need the polynomial.
+constexpr float WIDE_A = 100.0f;
 
 struct AsyTable {
     float cq[ASY_K + 1][ASY_K + 1]; // c_k q_kj / ASY_S^k (j <= k)

@@ -678,7 +678,9 @@ __device__ __forceinline__ V warp_sum(V v)
 // K = 1 where |z| >= 100 (the K = 2 terms are below 4e-8 there), K = 2 from |z| = 16.5
 // (the first dropped term is 15/(8 |z|^6), below 1e-7), the K = 6 polynomial in
 // 1/|z|^2 (asy_coeffs) from |z| = 6.  A warp takes the cheapest form that all of its
-// 32 lines allow.
+// 32 lines allow, but for lines with a >= WIDE_A among others that need the polynomial: its
+// powers of a leave the FP32 range at a of a few hundred, and a wing form holds for such a
+// line everywhere.
 constexpr float WING1_Z2 = 1.0e4f, WING2_Z2 = 272.25f;
 
 __device__ __forceinline__ void wing2_consts(const float4& p1, float c, float* k2, float* k3, float* k4)
@@ -772,7 +774,7 @@ __device__ __forceinline__ double far_sum(const Lines<float>& ln, const FarList&
             }
         } else {
             const float4 p2 = ln.r2[lc];
-            if (__all_sync(0xffffffffu, z2 >= WING2_Z2)) {
+            if (__all_sync(0xffffffffu, z2 >= WING2_Z2) || p2.y >= WIDE_A) {
                 float a2, a3, a4;
                 wing2_consts(q1, p2.x, &a2, &a3, &a4);
                 const float2 k2 = dup(a2), k3 = dup(a3), k4 = dup(a4);
@@ -909,7 +911,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
             }
         } else {
             const float4 p2 = ln.r2[lc];
-            if (__all_sync(0xffffffffu, z2 >= WING2_Z2)) {
+            if (__all_sync(0xffffffffu, z2 >= WING2_Z2) || p2.y >= WIDE_A) {
                 float r[6];
                 rho_moments<6>(o2, w2, nb, G, r);
                 const float cc = p2.x * p2.x, Q = Al * rcp_fast(cc * cc);
@@ -1593,11 +1595,13 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
                 if (have) {
                     tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
                     tl.r2[lane] = p2;
+                    const bool wide = p2.y >= WIDE_A; // summed below
                     float C[ASY_N];
-                    asy_coeffs(p2.y, p2.z, C);
+                    asy_coeffs(wide ? 0.0f : p2.y, wide ? 0.0f : p2.z, C);
                     store16(tl.hc[lane], C, ASY_N);
                     if (p2.y * p2.y < NEAR_POLY_Z2) series_table(p2.y, tl.sd[lane]);
                 }
+                unsigned wide = __ballot_sync(0xffffffffu, have && p2.y >= WIDE_A);
                 __syncwarp();
                 // the staged lines in ascending order (warp-uniform loop)
                 for (int q = 0; q < cnt; ++q) {
@@ -1622,6 +1626,19 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
                             scaled_pair(dh, dl, c4.x, b.z, &x, &xl);
                             acc = fmaf(c4.z, w_series_re(x, xl, c4.y, b.w, c4.w, tl.sd[q]), acc);
                         }
+                    }
+                }
+                if (wide) {
+                    __syncwarp();
+                    if (have) tl.hc[lane][0] = ln.r1[l];
+                    __syncwarp();
+                    for (; wide; wide &= wide - 1) {
+                        const int q = __ffs(wide) - 1;
+                        const float4 u = tl.hc[q][0], b = tl.nb[q];
+                        const float d = (ohi + b.x) + (olo + b.y);
+                        const bool in = !masked || in_range((int)j, tl.jr[q]);
+                        const float rho = rcp_fast(fmaf(d, d, u.x));
+                        acc = fmaf(in ? rho : 0.0f, fmaf(fmaf(u.w, rho, u.z), rho, u.y), acc);
                     }
                 }
             }
@@ -1771,6 +1788,24 @@ __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
     }
 }
 
+// A line's K = 1 wing forms of f_T and f_b as polynomials in rho (see far_adjoint_sum):
+// hf = {G, f_T's first three coefficients}, {its last, f_b's first two}, hg = {f_b's last two}
+__device__ __forceinline__ void stage_wing1_adj(const float4& p1, float aS, float nn, float hT, float4* hf, float4* hg)
+{
+    const float G = p1.x, Al = p1.y, F1 = p1.z, F2 = p1.w;
+    const float U2 = F1 - 2.0f * G * Al, U4 = -6.0f * G * F2;
+    hf[0] = make_float4(G, Al * (aS + nn), aS * F1 + hT * 2.0f * F1 + nn * U2, (aS + 2.0f * hT + 6.0f * nn) * F2);
+    hf[1] = make_float4(nn * U4, Al, U2, 0.0f);
+    hg[0] = make_float4(6.0f * F2, U4, 0.0f, 0.0f);
+}
+__device__ __forceinline__ void add_wing1_adj(const float4* hf, const float4* hg, float d, bool in, float& aT, float& aB)
+{
+    const float4 t = hf[0], u = hf[1], v = hg[0];
+    const float rho = rcp_fast(fmaf(d, d, t.x)), r = in ? rho : 0.0f;
+    aT = fmaf(r, fmaf(fmaf(fmaf(u.x, rho, t.w), rho, t.z), rho, t.y), aT);
+    aB = fmaf(r, fmaf(fmaf(fmaf(v.y, rho, v.x), rho, u.z), rho, u.y), aB);
+}
+
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(const __grid_constant__ Batch<float> batch,
                                                                             const double* __restrict__ nu, int64_t N,
                                                                             double W, int layer0,
@@ -1869,14 +1904,16 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                     if (have) {
                         tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
                         tl.r2[lane] = p2;
-                            tl.aS[lane] = p3.x;
+                        tl.aS[lane] = p3.x;
                         tl.nn[lane] = p3.y;
+                        const bool wide = p2.y >= WIDE_A; // summed below
                         float F[ASY_N + 1], G[ASY_N + 1];
-                        asy_coeffs_adj(p2.y, p2.z, p3.x, hT, p3.y, F, G);
+                        asy_coeffs_adj(wide ? 0.0f : p2.y, wide ? 0.0f : p2.z, p3.x, hT, p3.y, F, G);
                         store16(tl.hf[lane], F, ASY_N + 1);
                         store16(tl.hg[lane], G, ASY_N + 1);
                         if (p2.y * p2.y < NEAR_POLY_Z2) series_table(p2.y, tl.sd[lane]);
                     }
+                    unsigned wide = __ballot_sync(0xffffffffu, have && p2.y >= WIDE_A);
                     __syncwarp();
                     for (int q = 0; q < cnt; ++q) {
                         const bool in = lf.live && (!masked || in_range((int)j, tl.jr[q]));
@@ -1910,6 +1947,17 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                                 aT += tl.aS[q] * V0 + hT * Db + tl.nn[q] * V2;
                                 aB += V2;
                             }
+                        }
+                    }
+                    if (wide) {
+                        __syncwarp();
+                        if (have) stage_wing1_adj(ln.r1[l], p3.x, p3.y, hT, tl.hf[lane], tl.hg[lane]);
+                        __syncwarp();
+                        for (; wide; wide &= wide - 1) {
+                            const int q = __ffs(wide) - 1;
+                            const float4 b = tl.nb[q];
+                            const float d = (ohi + b.x) + (olo + b.y);
+                            add_wing1_adj(tl.hf[q], tl.hg[q], d, !masked || in_range((int)j, tl.jr[q]), aT, aB);
                         }
                     }
                 }

@@ -1,0 +1,51 @@
+"""Mixed precision where its FP32 forms could leave the range of FP32: lists of very wide
+lines with lines of no width among them, against FP64, sums and adjoints, with the
+tolerances of the other mixed cases (1e-5 of sigma above 1e-6 of a layer's largest, 1e-4 of
+the largest gradient)."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a, dtype=np.float64), device="cuda")
+
+
+def compare(lines, nu, T, P, cut, lam_of, sb=1.0):
+    """lam_of(sigma): dF/dsigma from the FP64 sigma [L][N]."""
+    from paper_2105_14782_gb300 import xs
+    dl = xs.DeviceLines(lines)
+    args = dl, dev(nu), dev(T), dev(P)
+    want = xs.xs_compute(*args, sb, cut, xs.PREC_FP64)
+    lam = lam_of(want)
+    ref = [v.cpu().numpy() for v in xs.xs_compute_adjoint(*args, lam, sb, cut, xs.PREC_FP64)]
+    big = max(np.max(np.abs(ref[0] * T)), abs(ref[1][0]))
+    assert torch.isfinite(want).all() and np.isfinite(big)
+    m = want > 1e-6 * want.amax(dim=1, keepdim=True)
+    small = torch.empty(xs.lib().xs_workspace_min_bytes(dl.n, len(nu), len(T), xs.PREC_MIXED), dtype=torch.uint8,
+                        device="cuda")
+    for ws in (None, small):  # the full plan and the smallest accepted workspace
+        got = xs.xs_compute(*args, sb, cut, xs.PREC_MIXED, workspace=ws).double()
+        assert torch.isfinite(got).all()
+        assert float(((got - want).abs() / want)[m].max()) < 1e-5
+        g_T, g_b = (v.cpu().numpy() for v in xs.xs_compute_adjoint(*args, lam, sb, cut, xs.PREC_MIXED, workspace=ws))
+        assert np.isfinite(g_T).all() and np.isfinite(g_b).all()
+        assert np.max(np.abs(g_T - ref[0]) * T) <= 1e-4 * big and abs(g_b - ref[1])[0] <= 1e-4 * big
+
+
+@pytest.mark.parametrize("nu0,every", [(1000.0, 40), (500.0, 40), (500.0, 7), (200.0, 40)])
+def test_lines_without_width_among_wide_ones(nu0, every):
+    """At 100 bar these lines are 1,700 to 8,500 Doppler widths wide (a); the ones without
+    width need the near forms at the same points."""
+    n, N = 2000, 2000
+    lines = W.water_like(n, seed=int(nu0) + every, nu_min=nu0, nu_max=1.01 * nu0)
+    lines.gamma_ref[:] = 0.1
+    lines.gamma_ref[::every] = 0.0
+    lines.ln_S0[1::every] += np.log(1e3)  # up to 1e-17 cm/molecule
+    rng = np.random.default_rng(every)
+    compare(lines, W.grid_lognu(N, nu0, 1.01 * nu0), np.array([700.0, 1000.0, 1000.0]), np.array([0.1, 30.0, 100.0]),
+            0.003 * nu0, lambda s: (1.0 + 0.5 * dev(rng.uniform(size=(3, N)))) / s.amax(dim=1, keepdim=True))
