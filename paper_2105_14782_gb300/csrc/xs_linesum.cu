@@ -827,26 +827,31 @@ __device__ __forceinline__ double far_sum(const Lines<float>& ln, const FarList&
 //   V0      += Q (3.75 rho^3 - 15 G rho^4 + 12 G^2 rho^5),
 //   D_beta  += Q (15 rho^3 - 60 G rho^4 + 48 G^2 rho^5),
 //   D_gamma += Q (3.75 rho^3 - 67.5 G rho^4 + 180 G^2 rho^5 - 120 G^3 rho^6).
-// A lane first sums Lambda_m rho_m^k over the nodes and then applies its line's
-// coefficients once.
+// A lane first sums Lambda_m v_m^k over the nodes and then applies its line's coefficients
+// once.  v = rho for two moments; for more, v = rho D0 with D0 = 1/rho at the line's nearest
+// point: it lies in 0.2 .. 1, so the powers stay in range whatever the units, where rho goes as
+// 1/nu^2, its sixth power beyond FP32 below 10 cm^-1.  With b = B/D0 = 1/|z|^2 and g = G/D0 <= 1 there, the forms above are
+//   V0      = (Al/D0) (v + 1.5 b v^2 - 2 g b v^3 + b^2 (3.75 v^3 - 15 g v^4 + 12 g^2 v^5))
+// and so on.
 
 template <int K>
 __device__ __forceinline__ void rho_moments(const float2 (&o2)[Far<float>::n / 2], const float2 (&w2)[Far<float>::n / 2],
-                                            float nb, float G, float (&r)[K])
+                                            float nb, float G, float D0, float (&r)[K])
 {
     float2 s[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) s[k] = dup(0.0f);
-    const float2 nb2 = dup(nb), G2 = dup(G);
+    const float2 nb2 = dup(nb), G2 = dup(G), s0 = dup(D0);
 #pragma unroll
     for (int p = 0; p < Far<float>::n / 2; ++p) {
         const float2 d = __fadd2_rn(o2[p], nb2);
-        const float2 rho = rcp2_shared(__ffma2_rn(d, d, G2));
-        float2 t = __fmul2_rn(w2[p], rho);
+        float2 v = rcp2_shared(__ffma2_rn(d, d, G2));
+        if (K > 2) v = __fmul2_rn(v, s0);
+        float2 t = __fmul2_rn(w2[p], v);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             s[k] = __fadd2_rn(s[k], t);
-            if (k + 1 < K) t = __fmul2_rn(t, rho);
+            if (k + 1 < K) t = __fmul2_rn(t, v);
         }
     }
 #pragma unroll
@@ -892,34 +897,36 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
         }
         const float dist = fmaxf(fabsf(nb) - h, 0.0f);
         const float D0 = fmaf(dist, dist, G), z2 = D0 * c2min;
-        const float U2 = F1 - 2.0f * G * Al;
+        const float iD = rcp_fast(D0), A0 = Al * iD, g = G * iD;
         float V0, Db, Dg;
         if (__all_sync(0xffffffffu, z2 >= WING1_Z2)) {
             // the F2 terms are up to 12 a^2/|z|^4 of f_b's leading one
             if (__all_sync(0xffffffffu, 12.0f * G <= 2.0e-8f * z2 * D0)) {
-                float r[2];
-                rho_moments<2>(o2, w2, nb, G, r);
+                float r[2]; // of rho itself: its square stays in range
+                rho_moments<2>(o2, w2, nb, G, D0, r);
                 V0 = fmaf(F1, r[1], Al * r[0]);
                 Db = 2.0f * F1 * r[1];
-                Dg = fmaf(U2, r[1], Al * r[0]);
+                Dg = fmaf(F1 - 2.0f * G * Al, r[1], Al * r[0]);
             } else {
                 float r[4];
-                rho_moments<4>(o2, w2, nb, G, r);
-                V0 = fmaf(F2, r[2], fmaf(F1, r[1], Al * r[0]));
-                Db = 2.0f * fmaf(F2, r[2], F1 * r[1]);
-                Dg = fmaf(-6.0f * G * F2, r[3], fmaf(6.0f * F2, r[2], fmaf(U2, r[1], Al * r[0])));
+                rho_moments<4>(o2, w2, nb, G, D0, r);
+                const float b1 = F1 * iD * iD, b2 = F2 * iD * iD * iD, u2 = b1 - 2.0f * g * A0;
+                V0 = fmaf(b2, r[2], fmaf(b1, r[1], A0 * r[0]));
+                Db = 2.0f * fmaf(b2, r[2], b1 * r[1]);
+                Dg = fmaf(-6.0f * g * b2, r[3], fmaf(6.0f * b2, r[2], fmaf(u2, r[1], A0 * r[0])));
             }
         } else {
             const float4 p2 = ln.r2[lc];
             if (__all_sync(0xffffffffu, z2 >= WING2_Z2) || p2.y >= WIDE_A) {
                 float r[6];
-                rho_moments<6>(o2, w2, nb, G, r);
-                const float cc = p2.x * p2.x, Q = Al * rcp_fast(cc * cc);
-                const float g4 = G * r[3], g5 = G * G * r[4], g6 = G * G * G * r[5];
-                V0 = fmaf(F2, r[2], fmaf(F1, r[1], Al * r[0])) + Q * (3.75f * r[2] - 15.0f * g4 + 12.0f * g5);
-                Db = 2.0f * fmaf(F2, r[2], F1 * r[1]) + Q * (15.0f * r[2] - 60.0f * g4 + 48.0f * g5);
-                Dg = fmaf(-6.0f * G * F2, r[3], fmaf(6.0f * F2, r[2], fmaf(U2, r[1], Al * r[0]))) +
-                     Q * (3.75f * r[2] - 67.5f * g4 + 180.0f * g5 - 120.0f * g6);
+                rho_moments<6>(o2, w2, nb, G, D0, r);
+                const float b = rcp_fast(D0 * (p2.x * p2.x)), g4 = g * r[3], g5 = g * g * r[4], g6 = g * g * g * r[5];
+                const float q0 = fmaf(1.5f, r[1], -2.0f * g * r[2]), q = fmaf(3.75f, r[2], fmaf(-15.0f, g4, 12.0f * g5));
+                V0 = A0 * fmaf(b, fmaf(b, q, q0), r[0]);
+                Db = A0 * b * fmaf(4.0f * b, q, 2.0f * q0);
+                Dg = A0 * fmaf(b, fmaf(b, 3.75f * r[2] - 67.5f * g4 + 180.0f * g5 - 120.0f * g6,
+                                       1.5f * r[1] - 12.0f * g * r[2] + 12.0f * g * g4),
+                               fmaf(-2.0f * g, r[1], r[0]));
             } else {
                 // moments of u v^n, u = 1/|z|^2, v = ASY_S u, against the K = 6 coefficients
                 float2 s[ASY_N + 1];

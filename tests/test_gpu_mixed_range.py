@@ -1,5 +1,5 @@
 """Mixed precision where its FP32 forms could leave the range of FP32: lists of very wide
-lines with lines of no width among them, against FP64, sums and adjoints, with the
+lines with lines of no width among them, low wavenumbers, against FP64, sums and adjoints, with the
 tolerances of the other mixed cases (1e-5 of sigma above 1e-6 of a layer's largest, 1e-4 of
 the largest gradient)."""
 import numpy as np
@@ -49,3 +49,16 @@ def test_lines_without_width_among_wide_ones(nu0, every):
     rng = np.random.default_rng(every)
     compare(lines, W.grid_lognu(N, nu0, 1.01 * nu0), np.array([700.0, 1000.0, 1000.0]), np.array([0.1, 30.0, 100.0]),
             0.003 * nu0, lambda s: (1.0 + 0.5 * dev(rng.uniform(size=(3, N)))) / s.amax(dim=1, keepdim=True))
+
+
+@pytest.mark.parametrize("nu0,T0", [(7.69, 1000.0), (3.84, 500.0), (0.5, 300.0)])
+@pytest.mark.parametrize("weight", [1e20, 1e25])
+def test_low_wavenumbers(nu0, T0, weight):
+    """Doppler widths go as the wavenumber, so 1/distance^2 reaches 1e7 cm^2 at these, its sixth
+    power beyond FP32; weights of dF/dsigma as a well-measured spectrum gives them."""
+    n, N = 1500, 2000
+    lines = W.water_like(n, seed=5, nu_min=0.999 * nu0, nu_max=1.011 * nu0)
+    lines.mass_amu = 28.0
+    rng = np.random.default_rng(3)
+    compare(lines, W.grid_lognu(N, nu0, 1.01 * nu0), np.array([0.8 * T0, T0, T0]), np.array([1e-6, 1e-4, 1e-3]),
+            0.004 * nu0, lambda s: weight * (1.0 + 0.5 * dev(rng.uniform(size=(3, N)))))
