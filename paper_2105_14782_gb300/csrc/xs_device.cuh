@@ -96,6 +96,9 @@ template <> struct Tier<double> {
     static constexpr double z2_mid = 1600.0;   // |z| >= 40 : K = 5
     static constexpr double z2_k7 = 441.0;     // |z| >= 21 : K = 7
     static constexpr double z2_series = 100.0; // |z| >= 10 : K = 12, below: series
+    // Below this a leaf's nearest |z|^2 to a line has the line's series data staged: it and a
+    // point's own |z|^2 round differently (by up to 1e-9 at an ulp of nu).
+    static constexpr double z2_stage = z2_series * (1.0 + 1e-6);
     static constexpr double h = 0.5;           // series step (error ~1e-17)
 };
 

@@ -1745,7 +1745,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
                 });
             } else {
                 if (have) stage_poly64<ASY64_K>(p2.y, p2.z, tl.C[lane]);
-                if (have && z2 < Tier<double>::z2_series) {
+                if (have && z2 < Tier<double>::z2_stage) {
                     tl.ia[lane] = p2.y > 0.0 ? 1.0 / p2.y : 0.0;
                     series_table64(p2.y, tl.sd[lane]);
                 }
@@ -2051,12 +2051,12 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
                     tl.aS[lane] = ln.r3[2 * (size_t)l];
                     tl.nn[lane] = ln.r3[2 * (size_t)l + 1];
                     if (masked) tl.jr[lane] = ln.jr[l];
-                    if (z2 < Tier<double>::z2_series) {
+                    if (z2 < Tier<double>::z2_stage) {
                         tl.ia[lane] = p2.y > 0.0 ? 1.0 / p2.y : 0.0;
                         series_table64(p2.y, tl.sd[lane]);
                     }
                 }
-                unsigned near = __ballot_sync(0xffffffffu, z2 < Tier<double>::z2_series); // lines with series points
+                unsigned near = __ballot_sync(0xffffffffu, z2 < Tier<double>::z2_stage); // lines with series points
                 __syncwarp();
                 const int q = min(lane % NEAR64, cnt - 1), half = lane / NEAR64;
                 const double amp = lane % NEAR64 < cnt ? tl.r2[q].z : 0.0;
