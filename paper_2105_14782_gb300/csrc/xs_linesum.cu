@@ -584,6 +584,8 @@ struct FarList {
 // ------------------------------------------------------------------ packed helpers
 
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 lo2(const float4& v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4& v) { return make_float2(v.z, v.w); }
 // both reciprocals from one: 1/D1 = D2/(D1 D2), 1/D2 = D1/(D1 D2) (about 1.5 ulp); trades
 // a second MUFU op (16 a clock and SM) for FP32 multiplies (128 a clock and SM)
 __device__ __forceinline__ float2 rcp2_shared(float2 v)
@@ -1463,18 +1465,54 @@ constexpr float NEAR_POLY_Z2 = 36.0f;
 
 __device__ __forceinline__ bool in_range(int j, int2 r) { return j >= r.x && j <= r.y; }
 
-// A warp's leaf: its points and its near lines as up to three ranges (the middle one
-// inside every line's cut, the outer ones masked per point).  `split` neighbouring warps
-// of the block share a leaf and take every split-th chunk of its lines.
+// zero for the lines of a group of four that do not reach point j
+__device__ __forceinline__ void mask4(const int2* jr, int j, float2& a, float2& b)
+{
+    a.x = in_range(j, jr[0]) ? a.x : 0.0f;
+    a.y = in_range(j, jr[1]) ? a.y : 0.0f;
+    b.x = in_range(j, jr[2]) ? b.x : 0.0f;
+    b.y = in_range(j, jr[3]) ? b.y : 0.0f;
+}
+
+// A warp's leaf: its points and its near lines as up to five ranges (the first and last masked
+// per point, the others inside every line's cut).  `split` neighbouring warps of the block
+// share a leaf and take every split-th chunk of its lines.
+constexpr int RANGES = 5;
+// |z|^2 from which short forms hold: without far sets the lines nearer than it are a range
+// of their own, so that few chunks mix them with others.  A window of fewer lines than
+// SPLIT_LINES stays one masked range: each range ends in a chunk that is not full (128 lines on
+// 50,000 points x 100 layers 567 us split, 627 not; 64 lines 622 and 480).
+constexpr int SPLIT_LINES = 96;
+
+// first index of v[0], v[stride], .. that holds at least x
+template <class V>
+__device__ __forceinline__ int first_index(const V* v, int stride, int64_t n, V x)
+{
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t m = (lo + hi) >> 1;
+        if (v[stride * m] >= x) hi = m; else lo = m + 1;
+    }
+    return (int)lo;
+}
+// the centres, FP32: relative to the first grid point (no digits are needed here)
+__device__ __forceinline__ const float* near_keys(const Lines<float>& ln) { return (const float*)ln.nuf; }
+__device__ __forceinline__ const double* near_keys(const Lines<double>& ln) { return ln.nu_hat; }
+__device__ __forceinline__ int near_stride(const Lines<float>&) { return 2; }
+__device__ __forceinline__ int near_stride(const Lines<double>&) { return 1; }
+__device__ __forceinline__ float near_key(const Lines<float>&, double mid, double nu0, float r) { return (float)(mid - nu0) + r; }
+__device__ __forceinline__ double near_key(const Lines<double>&, double mid, double, float r) { return mid + r; }
+template <class R> struct ShortForm { static constexpr double z2 = WING2_Z2; };
+template <> struct ShortForm<double> { static constexpr double z2 = Tier<double>::z2_k7; };
 template <class R>
 struct Leaf {
     int64_t jb, jl;
     int lane, i, sub;
     bool any, live; // the leaf has points; the lane has one
-    int s[3], e[3];
+    int s[RANGES], e[RANGES];
     Geo g;
 
-    __device__ void init(const Tree& tr, const double* nu_hat, int64_t nl, const double* nu, int64_t N, double W,
+    __device__ void init(const Tree& tr, const Lines<R>& ln, const float* agg, int64_t nl, const double* nu, int64_t N,
                          int nloc, int split)
     {
         const int w = threadIdx.x >> 5;
@@ -1487,7 +1525,7 @@ struct Leaf {
         g = {0.0, 0.0, 0.0};
         live = any && jb + lane <= jl;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) s[k] = e[k] = 0;
+        for (int k = 0; k < RANGES; ++k) s[k] = e[k] = 0;
         if (!any) return;
         if (tr.on) {
             g = tr.geo[i];
@@ -1495,20 +1533,35 @@ struct Leaf {
             const int2 w = tr.win[i];
             s[0] = w.x;
             e[0] = fs.a;
-            s[1] = fs.p;
-            e[1] = fs.q;
-            s[2] = fs.b;
-            e[2] = w.y;
+            s[2] = fs.p;
+            e[2] = fs.q;
+            s[4] = fs.b;
+            e[4] = w.y;
         } else {
-            int v = 0;
-            if (lane == 0) v = first_line(nu_hat, nl, nu[jb], W, 1);
-            if (lane == 1) v = first_line(nu_hat, nl, nu[jl], W, 0);
-            s[0] = __shfl_sync(0xffffffffu, v, 0);
-            e[0] = __shfl_sync(0xffffffffu, v, 1);
-            g = {0.5 * (nu[jb] + nu[jl]), 0.5 * (nu[jl] - nu[jb]), 0.0};
+            // no far sets: the lines that cover the leaf, around the near ones, and on each
+            // side those cut inside it.  A lane a search, in whole numbers (an FP64 operation
+            // of a warp takes the SM's FP64 pipe for 16 clocks).
+            const double v0 = nu[jb], v1 = nu[jl];
+            g = {0.5 * (v0 + v1), 0.5 * (v1 - v0), 0.0};
+            const int upper = lane == 0 || lane == 3; // jr.y >= jb, jr.x > jl, jr.x > jb, jr.y >= jl
+            const int f = first_index((const int*)ln.jr + upper, 2, nl, (int)(lane & 1 ? jl : jb) + !upper);
+            s[0] = __shfl_sync(0xffffffffu, f, 0);
+            e[4] = __shfl_sync(0xffffffffu, f, 1);
+            if (e[4] - s[0] < SPLIT_LINES) {
+                e[0] = s[4] = e[4];
+            } else {
+                const float a2 = agg[1] * agg[1], z2 = ShortForm<R>::z2;
+                const float r = a2 < z2 ? (float)g.h + sqrtf(z2 - a2) * rcp_fast(agg[0]) : 0.0f;
+                const R v = near_key(ln, g.mid, nu[0], lane & 1 ? r : -r);
+                const int n = first_index(near_keys(ln), near_stride(ln), nl, v);
+                e[0] = s[1] = __shfl_sync(0xffffffffu, f, 3);
+                e[3] = s[4] = max(e[0], __shfl_sync(0xffffffffu, f, 2));
+                e[1] = s[2] = clampi(__shfl_sync(0xffffffffu, n, 0), s[1], e[3]);
+                e[2] = s[3] = clampi(__shfl_sync(0xffffffffu, n, 1), s[2], e[3]);
+            }
         }
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
+        for (int k = 0; k < RANGES; ++k)
             if (!XS_CHECK(s[k] >= 0 && e[k] <= nl)) e[k] = s[k];
     }
 };
@@ -1531,7 +1584,7 @@ __device__ __forceinline__ double split_sum(double v, int split)
 // sigma of one leaf: FP32
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(const __grid_constant__ Batch<float> batch,
                                                                            const double* __restrict__ nu, int64_t N,
-                                                                           double W, int layer0, double unscale,
+                                                                           int layer0, double unscale,
                                                                            int split)
 {
     const Species<float>& sp = batch.s[blockIdx.z];
@@ -1542,7 +1595,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     NearTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<float> lf;
-    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
     const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1553,8 +1606,8 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
     float shi = 0.0f, slo = 0.0f;
 #pragma unroll 1
-    for (int k = 0; k < 3; ++k) {
-        const bool masked = k != 1;
+    for (int k = 0; k < RANGES; ++k) {
+        const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
         for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
             const int l = t0 + lane;
@@ -1575,29 +1628,47 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
             const int cnt = min(32, ce - t0);
             float acc = 0.0f;
             if (__all_sync(0xffffffffu, z2 >= WING2_Z2)) {
-                // no point closer than |z| = 16.5 to any of the lines: wing forms
+                // no point closer than |z| = 16.5 to any of the lines: wing forms, a field of
+                // the 32 lines a row, so that one load fills two packed pairs of lines (some 7
+                // instructions a line and warp, 14 a line at a time)
                 const bool k1only = __all_sync(0xffffffffu, z2 >= WING1_Z2);
-                if (have) {
-                    const float4 p1 = ln.r1[l];
-                    float a2 = 0.f, a3 = 0.f, a4 = 0.f;
-                    if (!k1only) wing2_consts(p1, p2.x, &a2, &a3, &a4);
-                    tl.hc[lane][0] = make_float4(nb, p1.x, p1.y, p1.z);
-                    tl.hc[lane][1] = k1only ? make_float4(p1.w, 0.f, 0.f, nbl) : make_float4(a2, a3, a4, nbl);
+                float* const f = (float*)tl.hc;
+                const float4 p1 = have ? ln.r1[l] : make_float4(1.f, 0.f, 0.f, 0.f);
+                f[lane] = nb;
+                f[32 + lane] = nbl;
+                f[64 + lane] = p1.x;
+                f[96 + lane] = p1.y;
+                f[128 + lane] = p1.z;
+                if (k1only) {
+                    f[160 + lane] = p1.w;
+                } else {
+                    float a2, a3, a4;
+                    wing2_consts(p1, p2.x, &a2, &a3, &a4);
+                    f[160 + lane] = a2;
+                    f[192 + lane] = a3;
+                    f[224 + lane] = a4;
                 }
                 __syncwarp();
-#pragma unroll 2
-                for (int q = 0; q < cnt; ++q) {
-                    const float4 u0 = tl.hc[q][0], u1 = tl.hc[q][1];
-                    const float d = (ohi + u0.x) + (olo + u1.w);
-                    const float rho = rcp_fast(fmaf(d, d, u0.y));
-                    float u;
-                    if (k1only)
-                        u = fmaf(fmaf(u1.x, rho, u0.w), rho, u0.z);
-                    else
-                        u = fmaf(fmaf(fmaf(fmaf(u1.z, rho, u1.y), rho, u1.x), rho, u0.w), rho, u0.z);
-                    const bool in = !masked || in_range((int)j, tl.jr[q]);
-                    acc = fmaf(in ? rho : 0.0f, u, acc);
+                const float4* const r = (const float4*)f;
+                float2 a01 = dup(0.0f), a23 = a01;
+                for (int q = 0; q < (cnt + 3) / 4; ++q) {
+                    const float4 b = r[q], bl = r[8 + q], G = r[16 + q], k0 = r[24 + q], k1 = r[32 + q], k2 = r[40 + q];
+                    const float2 d0 = __fadd2_rn(__fadd2_rn(dup(ohi), lo2(b)), __fadd2_rn(dup(olo), lo2(bl)));
+                    const float2 d1 = __fadd2_rn(__fadd2_rn(dup(ohi), hi2(b)), __fadd2_rn(dup(olo), hi2(bl)));
+                    float2 r0 = rcp2_shared(__ffma2_rn(d0, d0, lo2(G))), r1 = rcp2_shared(__ffma2_rn(d1, d1, hi2(G)));
+                    float2 u0 = lo2(k2), u1 = hi2(k2);
+                    if (!k1only) {
+                        const float4 k3 = r[48 + q], k4 = r[56 + q];
+                        u0 = __ffma2_rn(__ffma2_rn(lo2(k4), r0, lo2(k3)), r0, u0);
+                        u1 = __ffma2_rn(__ffma2_rn(hi2(k4), r1, hi2(k3)), r1, u1);
+                    }
+                    u0 = __ffma2_rn(__ffma2_rn(u0, r0, lo2(k1)), r0, lo2(k0));
+                    u1 = __ffma2_rn(__ffma2_rn(u1, r1, hi2(k1)), r1, hi2(k0));
+                    if (masked) mask4(tl.jr + 4 * q, (int)j, r0, r1);
+                    a01 = __ffma2_rn(r0, u0, a01);
+                    a23 = __ffma2_rn(r1, u1, a23);
                 }
+                acc = (a01.x + a01.y) + (a23.x + a23.y);
             } else {
                 if (have) {
                     tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
@@ -1652,6 +1723,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
             two_sum(shi, slo, acc); // the chunk's FP32 partial into the compensated sum
         }
     }
+    if (!tr.on && split == 1) { // nothing to add; the scale is a power of two
+        if (lf.live) sigma[(size_t)layer * N + j] = (shi + slo) * (float)unscale;
+        return;
+    }
     const double near = split_sum<LeafWarps<float>::v>((double)shi + (double)slo, split);
     if (!lf.live || lf.sub) return;
     // the far lines' part
@@ -1698,7 +1773,7 @@ __device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, dou
 // exponential a term of the series.)
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(const __grid_constant__ Batch<double> batch,
                                                                            const double* __restrict__ nu, int64_t N,
-                                                                           double W, int layer0, double unscale,
+                                                                           int layer0, double unscale,
                                                                            int split)
 {
     const Species<double>& sp = batch.s[blockIdx.z];
@@ -1709,15 +1784,15 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     NearTile64& tl = ((NearTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<double> lf;
-    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
     const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
     const double nuj = nu[j];
     double acc = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < 3; ++k) {
-        const bool masked = k != 1;
+    for (int k = 0; k < RANGES; ++k) {
+        const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
         for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
             const int l = t0 + lane;
@@ -1815,7 +1890,7 @@ __device__ __forceinline__ void add_wing1_adj(const float4* hf, const float4* hg
 
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(const __grid_constant__ Batch<float> batch,
                                                                             const double* __restrict__ nu, int64_t N,
-                                                                            double W, int layer0,
+                                                                            int layer0,
                                                                             const double* __restrict__ T,
                                                                             double lam_scale, int split)
 {
@@ -1828,7 +1903,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<float> lf;
-    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
     if (lf.any) {
         const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
@@ -1837,13 +1912,14 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
         const double lamd = lf.live ? g_sigma[(size_t)layer * N + j] * lam_scale : 0.0;
         const float hT = (float)(0.5 / T[layer]);
         const float lam = (float)lamd;
+        float Th = 0.f, Tl = 0.f, Bh = 0.f, Bl = 0.f; // the chunks' sums as hi + lo floats
         const Span span(lf.g, nu[0]);
         const float rh = span.rh, rl = span.rl;
         const double oj = nuj - lf.g.mid;
         const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
 #pragma unroll 1
-        for (int k = 0; k < 3; ++k) {
-            const bool masked = k != 1;
+        for (int k = 0; k < RANGES; ++k) {
+            const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
             for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
                 const int l = t0 + lane;
@@ -1866,47 +1942,71 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                 const int cnt = min(32, ce - t0);
                 float aT = 0.0f, aB = 0.0f;
                 if (__all_sync(0xffffffffu, z2 >= WING2_Z2)) {
-                    // wing forms, f_T and f_b as polynomials in rho (K = 1 from |z| = 100)
+                    // wing forms, f_T and f_b as polynomials in rho (K = 1 from |z| = 100), rows of
+                    // fields as in the forward kernel
                     const bool k1only = __all_sync(0xffffffffu, z2 >= WING1_Z2);
-                    if (have) {
-                        const float4 p1 = ln.r1[l];
-                        const float G = p1.x, Al = p1.y, F1 = p1.z, F2 = p1.w, aS = p3.x, nn = p3.y;
-                        const float U2 = F1 - 2.0f * G * Al;
-                        float U3 = 6.0f * F2, U4 = -6.0f * G * F2;
-                        float T3 = (aS + 2.0f * hT + 6.0f * nn) * F2, T4 = nn * U4;
-                        if (!k1only) {
-                            const float cc = p2.x * p2.x, Q = Al * rcp_fast(cc * cc);
-                            const float GQ = G * Q, G2Q = G * GQ;
-                            T3 = fmaf(Q, 3.75f * aS + 15.0f * hT + 3.75f * nn, T3);
-                            T4 = fmaf(-GQ, 15.0f * aS + 60.0f * hT + 67.5f * nn, T4);
-                            U3 = fmaf(3.75f, Q, U3);
-                            U4 = fmaf(-67.5f, GQ, U4);
-                            tl.hg[lane][1] = make_float4(G2Q * (12.0f * aS + 48.0f * hT + 180.0f * nn),
-                                                         -120.0f * G * G2Q * nn, 180.0f * G2Q, -120.0f * G * G2Q);
-                        }
-                        tl.hf[lane][0] = make_float4(nb, G, Al * (aS + nn), aS * F1 + hT * 2.0f * F1 + nn * U2);
-                        tl.hf[lane][1] = make_float4(T3, T4, Al, U2);
-                        tl.hg[lane][0] = make_float4(U3, U4, nbl, 0.f);
+                    float* const f = (float*)tl.hf;
+                    const float4 p1 = have ? ln.r1[l] : make_float4(1.f, 0.f, 0.f, 0.f);
+                    const float G = p1.x, Al = p1.y, F1 = p1.z, F2 = p1.w, aS = p3.x, nn = p3.y;
+                    const float U2 = F1 - 2.0f * G * Al;
+                    float U3 = 6.0f * F2, U4 = -6.0f * G * F2;
+                    float T3 = (aS + 2.0f * hT + 6.0f * nn) * F2, T4 = nn * U4;
+                    if (!k1only) {
+                        const float cc = p2.x * p2.x, Q = Al * rcp_fast(cc * cc);
+                        const float GQ = G * Q, G2Q = G * GQ;
+                        T3 = fmaf(Q, 3.75f * aS + 15.0f * hT + 3.75f * nn, T3);
+                        T4 = fmaf(-GQ, 15.0f * aS + 60.0f * hT + 67.5f * nn, T4);
+                        U3 = fmaf(3.75f, Q, U3);
+                        U4 = fmaf(-67.5f, GQ, U4);
+                        f[352 + lane] = G2Q * (12.0f * aS + 48.0f * hT + 180.0f * nn);
+                        f[384 + lane] = -120.0f * G * G2Q * nn;
+                        f[416 + lane] = 180.0f * G2Q;
+                        f[448 + lane] = -120.0f * G * G2Q;
                     }
+                    f[lane] = nb;
+                    f[32 + lane] = nbl;
+                    f[64 + lane] = G;
+                    f[96 + lane] = Al * (aS + nn);
+                    f[128 + lane] = aS * F1 + hT * 2.0f * F1 + nn * U2;
+                    f[160 + lane] = T3;
+                    f[192 + lane] = T4;
+                    f[224 + lane] = Al;
+                    f[256 + lane] = U2;
+                    f[288 + lane] = U3;
+                    f[320 + lane] = U4;
                     __syncwarp();
-#pragma unroll 2
-                    for (int q = 0; q < cnt; ++q) {
-                        const float4 u0 = tl.hf[q][0], u1 = tl.hf[q][1], u2 = tl.hg[q][0];
-                        const float d = (ohi + u0.x) + (olo + u2.z);
-                        const float rho = rcp_fast(fmaf(d, d, u0.y));
-                        float pt = u1.y, pu = u2.y;
+                    const float4* const r = (const float4*)f;
+                    float2 t01 = dup(0.0f), t23 = t01, b01 = t01, b23 = t01;
+                    for (int q = 0; q < (cnt + 3) / 4; ++q) {
+                        const float4 b = r[q], bl = r[8 + q], g = r[16 + q];
+                        const float2 d0 = __fadd2_rn(__fadd2_rn(dup(ohi), lo2(b)), __fadd2_rn(dup(olo), lo2(bl)));
+                        const float2 d1 = __fadd2_rn(__fadd2_rn(dup(ohi), hi2(b)), __fadd2_rn(dup(olo), hi2(bl)));
+                        float2 r0 = rcp2_shared(__ffma2_rn(d0, d0, lo2(g))), r1 = rcp2_shared(__ffma2_rn(d1, d1, hi2(g)));
+                        const float4 t4 = r[48 + q], u4 = r[80 + q];
+                        float2 pt0 = lo2(t4), pt1 = hi2(t4), pu0 = lo2(u4), pu1 = hi2(u4);
                         if (!k1only) {
-                            const float4 u3 = tl.hg[q][1];
-                            pt = fmaf(fmaf(u3.y, rho, u3.x), rho, pt);
-                            pu = fmaf(fmaf(u3.w, rho, u3.z), rho, pu);
+                            const float4 t5 = r[88 + q], t6 = r[96 + q], u5 = r[104 + q], u6 = r[112 + q];
+                            pt0 = __ffma2_rn(__ffma2_rn(lo2(t6), r0, lo2(t5)), r0, pt0);
+                            pt1 = __ffma2_rn(__ffma2_rn(hi2(t6), r1, hi2(t5)), r1, pt1);
+                            pu0 = __ffma2_rn(__ffma2_rn(lo2(u6), r0, lo2(u5)), r0, pu0);
+                            pu1 = __ffma2_rn(__ffma2_rn(hi2(u6), r1, hi2(u5)), r1, pu1);
                         }
-                        pt = fmaf(fmaf(fmaf(pt, rho, u1.x), rho, u0.w), rho, u0.z);
-                        pu = fmaf(fmaf(fmaf(pu, rho, u2.x), rho, u1.w), rho, u1.z);
-                        const bool in = !masked || in_range((int)j, tl.jr[q]);
-                        const float r = in ? rho : 0.0f;
-                        aT = fmaf(r, pt, aT);
-                        aB = fmaf(r, pu, aB);
+#pragma unroll
+                        for (int k = 2; k >= 0; --k) { // the three lower coefficients of each
+                            const float4 t = r[24 + 8 * k + q], u = r[56 + 8 * k + q];
+                            pt0 = __ffma2_rn(pt0, r0, lo2(t));
+                            pt1 = __ffma2_rn(pt1, r1, hi2(t));
+                            pu0 = __ffma2_rn(pu0, r0, lo2(u));
+                            pu1 = __ffma2_rn(pu1, r1, hi2(u));
+                        }
+                        if (masked) mask4(tl.jr + 4 * q, (int)j, r0, r1);
+                        t01 = __ffma2_rn(r0, pt0, t01);
+                        t23 = __ffma2_rn(r1, pt1, t23);
+                        b01 = __ffma2_rn(r0, pu0, b01);
+                        b23 = __ffma2_rn(r1, pu1, b23);
                     }
+                    aT = (t01.x + t01.y) + (t23.x + t23.y);
+                    aB = (b01.x + b01.y) + (b23.x + b23.y);
                 } else {
                     if (have) {
                         tl.nb[lane] = make_float4(nb, nbl, ln.clo[l], p2.y > 0.0f ? rcp_fast(p2.y) : 0.0f);
@@ -1968,10 +2068,12 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                         }
                     }
                 }
-                sT += (double)(lam * aT);
-                sB += (double)(lam * aB);
+                two_sum(Th, Tl, lam * aT);
+                two_sum(Bh, Bl, lam * aB);
             }
         }
+        sT = (double)Th + (double)Tl;
+        sB = (double)Bh + (double)Bl;
     }
     block_pair<LeafWarps<float>::v>(sT, sB, sp.leaf + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
 }
@@ -2009,7 +2111,7 @@ __device__ __forceinline__ void near_adjoint64(const NearAdjTile64& tl, int q, i
 // point a lane.
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(const __grid_constant__ Batch<double> batch,
                                                                             const double* __restrict__ nu, int64_t N,
-                                                                            double W, int layer0,
+                                                                            int layer0,
                                                                             const double* __restrict__ T,
                                                                             double lam_scale, int split)
 {
@@ -2022,7 +2124,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<double> lf;
-    lf.init(tr, sp.ln.nu_hat, nl, nu, N, W, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
     if (lf.any) {
         const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
@@ -2033,8 +2135,8 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
         tl.pos[lane] = nuj;
         tl.lam[lane] = lam;
 #pragma unroll 1
-        for (int k = 0; k < 3; ++k) {
-            const bool masked = k != 1;
+        for (int k = 0; k < RANGES; ++k) {
+            const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
             for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
                 const int l = t0 + lane;
@@ -2146,9 +2248,15 @@ namespace {
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Lists shorter than this are summed point by point: 256 lines are eight chunks of a
-// leaf's warp, a few microseconds, about what the three launches of the intervals cost.
-constexpr int64_t TREE_MIN_LINES = 256;
+// Lists shorter than this are summed point by point.  With the intervals a call pays three
+// more launches, and polynomials and node weights per layer whatever the list's length.  FP32,
+// us without and with them, forward and adjoint: 255 lines on 4,096 points x 20 layers 43 and
+// 64, 60 and 78; on 50,000 x 100 698 and 787, 1084 and 852 (128 lines 502 and 764, 810 and
+// 823).  FP64 pairs cost ten times more: 64 lines on 4,096 points 185 and 118, 339 and 270; x 20
+// layers 312 and 246, 635 and 614; 32 lines 117 and 102, 210 and 246.
+template <class R> struct ShortList { static constexpr int64_t v = 256; };
+template <> struct ShortList<double> { static constexpr int64_t v = 64; };
+int64_t tree_min_lines(int prec) { return prec == XS_PREC_MIXED ? ShortList<float>::v : ShortList<double>::v; }
 
 // Density of lines from which an interval has two intervals below it instead of four, in
 // half lines a grid point.  A level's list holds the lines between its far radius and that
@@ -2287,7 +2395,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
 size_t xs_workspace_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
 {
     if (n_lines < 0 || N <= 0 || L <= 0) return 0;
-    return plan_xs(n_lines, N, L, prec, L, n_lines >= TREE_MIN_LINES).total;
+    return plan_xs(n_lines, N, L, prec, L, n_lines >= tree_min_lines(prec)).total;
 }
 
 size_t xs_workspace_min_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
@@ -2301,7 +2409,7 @@ namespace xsi {
 // The largest chunk of layers whose plan fits, with the intervals if any such fits.
 static int pick_plan(int64_t nl, int64_t N, int32_t L, int prec, size_t ws_bytes, XsPlan* out)
 {
-    for (int tree = nl >= TREE_MIN_LINES ? 1 : 0; tree >= 0; --tree)
+    for (int tree = nl >= tree_min_lines(prec) ? 1 : 0; tree >= 0; --tree)
         for (int Lc = L;; Lc = (Lc + 1) / 2) {
             XsPlan p = plan_xs(nl, N, L, prec, Lc, tree != 0);
             if (p.total <= ws_bytes) {
@@ -2425,9 +2533,9 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, W, l0, unscale, p.leaf_split);
+                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, unscale, p.leaf_split);
             else
-                leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(b, nu, N, W, l0, unscale,
+                leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(b, nu, N, l0, unscale,
                                                                                            p.leaf_split);
         } else {
             if (tr.on) {
@@ -2437,9 +2545,9 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, W, l0, T, unscale, p.leaf_split);
+                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, T, unscale, p.leaf_split);
             else
-                leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(b, nu, N, W, l0, T,
+                leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(b, nu, N, l0, T,
                                                                                               unscale, p.leaf_split);
         }
         prof_end(adjoint ? 1 : 0, st);
