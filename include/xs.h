@@ -101,9 +101,11 @@ int xs_check_sorted(const double* v, int64_t n, int strict, int* flag_dev, xs_st
 int xs_checked_build(void);
 int xs_check_status(int clear);
 
-/* Workspace bytes xs_compute / xs_compute_adjoint need for these sizes.  A
- * workspace down to xs_workspace_min_bytes still works (layers are then done in
- * chunks); sizes in between pick the largest chunk that fits. */
+/* Workspace bytes xs_compute / xs_compute_adjoint need for these sizes, and the
+ * bytes with which they still run well, layers in chunks.  Sizes in between pick the
+ * largest chunk that fits.  Somewhat smaller workspaces are accepted, down to the
+ * per-line records of one layer, but sum every line at every point of its cut;
+ * XS_EINVAL below. */
 size_t xs_workspace_bytes(int64_t n_lines, int64_t N, int32_t L, int prec);
 size_t xs_workspace_min_bytes(int64_t n_lines, int64_t N, int32_t L, int prec);
 
@@ -137,10 +139,10 @@ int xs_compute(const xs_lines* lines, const double* nu, int64_t N, const double*
  * meaning are exactly those of xs_compute; the scratch comes from a fixed 64 MiB
  * device array inside libxs that every GPU loading the library holds until the
  * process exits.  Problems whose smallest plan (one layer at a time) needs more
- * than 64 MiB, i.e. xs_workspace_min_bytes(n, N, L, prec) > 64 MiB, are
- * rejected with XS_ETOOBIG before any launch.  That plan holds about n * 68
- * bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records and the
- * adjoint's partial sums; xs_workspace_min_bytes gives the exact figure.
+ * than 64 MiB are rejected with XS_ETOOBIG before any launch; where
+ * xs_workspace_min_bytes(n, N, L, prec) <= 64 MiB none are.  That plan holds about
+ * n * 92 bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records and
+ * the adjoint's partial sums.
  * The first call on each device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call
  * before any stream capture.  All calls on a device share the one array and

@@ -201,7 +201,7 @@ int xs_compute(const xs_lines* lines, const double* nu, int64_t N, const double*
     int r = check_common(lines, nu, N, T, P_bar, L, broad_scale, wing_cut, prec);
     if (r) return r;
     if (!sigma || !workspace) return XS_EINVAL;
-    if (workspace_bytes < xs_workspace_min_bytes(lines->n, N, L, prec)) return XS_EINVAL;
+    if (workspace_bytes < xsi::xs_least_bytes(lines->n, N, L, prec)) return XS_EINVAL;
     const xsi::XsJob job{lines, workspace, workspace_bytes, sigma, nullptr, nullptr, nullptr};
     return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, false, S(stream));
 }
@@ -214,7 +214,7 @@ int xs_compute_adjoint(const xs_lines* lines, const double* nu, int64_t N, const
     int r = check_common(lines, nu, N, T, P_bar, L, broad_scale, wing_cut, prec);
     if (r) return r;
     if (!g_sigma || !g_T || !g_broad || !workspace) return XS_EINVAL;
-    if (workspace_bytes < xs_workspace_min_bytes(lines->n, N, L, prec)) return XS_EINVAL;
+    if (workspace_bytes < xsi::xs_least_bytes(lines->n, N, L, prec)) return XS_EINVAL;
     const xsi::XsJob job{lines, workspace, workspace_bytes, nullptr, g_sigma, g_T, g_broad};
     return xsi::xs_run(1, &job, nu, N, T, P_bar, L, broad_scale, wing_cut, prec, true, S(stream));
 }

@@ -58,6 +58,9 @@ struct XsJob {
 int xs_run(int n, const XsJob* job, const double* nu, int64_t N, const double* T, const double* P, int32_t L, double sb,
            double W, int prec, bool adjoint, cudaStream_t st, int flags = 0, double* g_T_sum = nullptr);
 
+// the smallest workspace that xs_run takes: a layer at a time, without the intervals
+size_t xs_least_bytes(int64_t n_lines, int64_t N, int32_t L, int prec);
+
 // MODIT forward and adjoint with the composite model's flags (KEEP_ADJ, REUSE as above)
 int modit_forward(const xs_lines* lines, double nu_min, double nu_max, int64_t N, const double* T, const double* P_bar,
                   int32_t L, double broad_scale, int32_t n_gamma, int64_t n_fft, int prec, void* sigma,

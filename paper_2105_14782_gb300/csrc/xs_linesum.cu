@@ -145,7 +145,7 @@ struct Lines {
 struct FarWork {
     int parts[LEVELS], block0[LEVELS]; // block0: first block of the level
     size_t out0[LEVELS];               // first node-sum row of the level (in rows of n)
-    int slot0[LEVELS], slots;          // first adjoint slot of the level, slots per layer
+    int slot0[LEVELS], slots;          // first adjoint slot of the level, slots a layer
 };
 
 // One species of a launch: its lists, workspace arrays and plan.  The line sums of a
@@ -1167,7 +1167,7 @@ __global__ void __launch_bounds__(32 * FAR_WARPS, FarBlocks<R>::v)
                     sp.wts + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
                     (R)(0.5 / T[layer]), sT, sB);
     if ((threadIdx.x & 31) == 0) {
-        const size_t o = (size_t)layer * fw.slots + fw.slot0[k] + (size_t)part * tr.cnt[k] + i;
+        const size_t o = (size_t)nloc * fw.slots + fw.slot0[k] + (size_t)part * tr.cnt[k] + i;
         sp.slots[2 * o] = sT;
         sp.slots[2 * o + 1] = sB;
     }
@@ -1845,7 +1845,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
-// a block's sums of the leaves' (f_T, f_b) to part[layer][block], fixed order
+// a block's sums of the leaves' (f_T, f_b) to part[layer of the chunk][block], fixed order
 template <int warps>
 __device__ __forceinline__ void block_pair(double sT, double sB, double* part)
 {
@@ -2075,7 +2075,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
         sT = (double)Th + (double)Tl;
         sB = (double)Bh + (double)Bl;
     }
-    block_pair<LeafWarps<float>::v>(sT, sB, sp.leaf + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
+    block_pair<LeafWarps<float>::v>(sT, sB, sp.leaf + 2 * ((size_t)nloc * gridDim.x + blockIdx.x));
 }
 
 // Moments over half of the leaf's points (the lane's half) of lambda u^(n+1) for the lane's
@@ -2182,13 +2182,14 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
             }
         }
     }
-    block_pair<LeafWarps<double>::v>(sT, sB, sp.leaf + 2 * ((size_t)layer * gridDim.x + blockIdx.x));
+    block_pair<LeafWarps<double>::v>(sT, sB, sp.leaf + 2 * ((size_t)nloc * gridDim.x + blockIdx.x));
 }
 
 // g_T[n] = sum over the leaf blocks' and the far kernel's partials of layer n (one
-// block per layer, fixed order); gbl[n] the same for the broadening term.
+// block per layer of the chunk, fixed order); gbl[n] the same for the broadening term.
 template <class R>
-__global__ void __launch_bounds__(256) adjoint_reduce_kernel(const __grid_constant__ Batch<R> batch, int leaf_blocks)
+__global__ void __launch_bounds__(256) adjoint_reduce_kernel(const __grid_constant__ Batch<R> batch, int layer0,
+                                                             int leaf_blocks)
 {
     __shared__ double red[2][256];
     const Species<R>& sp = batch.s[blockIdx.z];
@@ -2215,8 +2216,8 @@ __global__ void __launch_bounds__(256) adjoint_reduce_kernel(const __grid_consta
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        sp.g_T[n] = red[0][0];
-        sp.gbl[n] = red[1][0];
+        sp.g_T[layer0 + n] = red[0][0];
+        sp.gbl[layer0 + n] = red[1][0];
     }
 }
 
@@ -2285,7 +2286,7 @@ struct XsPlan {
 // list long enough to pay for its reduction (FP64 evaluations cost about ten times
 // more).  A level's list is estimated from its share of the grid: the lines between
 // its own far radius and its parent's, about 16 interval lengths.
-void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
+void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed, bool compact)
 {
     const int64_t warps = mixed ? 10000 : 8000, min_lines = mixed ? 1024 : 64;
     int block = 0;
@@ -2297,14 +2298,15 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed)
         const double share = std::min(1.0, lengths * (double)(LEAF << (tr.shift * k)) / (double)N);
         const int64_t est = (k == tr.top) ? nl : (int64_t)(share * (double)nl);
         const int64_t want = (warps + (int64_t)Lc * p->tree.cnt[k] - 1) / ((int64_t)Lc * p->tree.cnt[k]);
-        const int parts = (int)std::max<int64_t>(1, std::min(want, est / min_lines));
-        p->fw.parts[k] = parts;
+        int64_t parts = std::max<int64_t>(1, std::min(want, est / min_lines));
+        if (compact) parts = std::min(parts, std::max<int64_t>(1, nl / (512 * (int64_t)p->tree.cnt[k])));
+        p->fw.parts[k] = (int)parts;
         p->fw.block0[k] = block;
         p->fw.out0[k] = row;
         p->fw.slot0[k] = p->fw.slots;
-        block += parts * ((p->tree.cnt[k] + FAR_WARPS - 1) / FAR_WARPS);
+        block += (int)parts * ((p->tree.cnt[k] + FAR_WARPS - 1) / FAR_WARPS);
         row += (size_t)parts * Lc * p->tree.cnt[k];
-        p->fw.slots += parts * p->tree.cnt[k];
+        p->fw.slots += (int)parts * p->tree.cnt[k];
     }
     p->far_blocks = block;
     p->rows = row;
@@ -2330,8 +2332,14 @@ void choose_leaf_blocks(XsPlan* p, int64_t N, int Lc, bool mixed, bool small)
     p->leaf_blocks = (int)((leaves + per - 1) / per);
 }
 
-XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
+// What of the intervals a plan holds: COMPACT has four intervals below each one and splits
+// their lists in as many parts as cost about a byte a line, the least space with which far
+// lines go to the nodes.
+enum Intervals { LEAVES_ONLY, COMPACT, FULL };
+
+XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, Intervals how)
 {
+    const bool tree = how != LEAVES_ONLY;
     XsPlan p{};
     p.prec = prec;
     p.Lc = Lc;
@@ -2357,7 +2365,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     p.off_gbl = take(sizeof(double) * (size_t)L);
     p.tree.on = tree ? 1 : 0;
     if (tree) {
-        p.tree.shift = 2 * nl >= (mixed ? DenseLines<float>::v : DenseLines<double>::v) * N ? 1 : 2;
+        p.tree.shift = how == FULL && 2 * nl >= (mixed ? DenseLines<float>::v : DenseLines<double>::v) * N ? 1 : 2;
         p.tree.top = TOP_LOG / p.tree.shift;
         for (int k = 0; k <= p.tree.top; ++k) {
             const int64_t pts = (int64_t)LEAF << (p.tree.shift * k);
@@ -2365,7 +2373,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
             p.tree.off[k] = p.tree.total;
             p.tree.total += p.tree.cnt[k];
         }
-        split_far(&p, nl, N, Lc, mixed);
+        split_far(&p, nl, N, Lc, mixed, how == COMPACT);
         p.off_geo = take(sizeof(Geo) * (size_t)p.tree.total);
         p.off_cov = take(sizeof(int2) * (size_t)p.tree.total);
         p.off_win = take(sizeof(int2) * (size_t)p.tree.cnt[0]);
@@ -2382,9 +2390,9 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
     off = base;
     if (tree) {
         p.off_wts = take(rs * n * (size_t)Lc * p.tree.total);
-        p.off_slots = take(sizeof(double) * 2 * (size_t)L * p.fw.slots);
+        p.off_slots = take(sizeof(double) * 2 * (size_t)Lc * p.fw.slots);
     }
-    p.off_leaf = take(sizeof(double) * 2 * (size_t)L * p.leaf_blocks);
+    p.off_leaf = take(sizeof(double) * 2 * (size_t)Lc * p.leaf_blocks);
     p.total = std::max(off, fwd_end);
     p.nchunks = (L + Lc - 1) / Lc;
     return p;
@@ -2395,23 +2403,34 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, bool tree)
 size_t xs_workspace_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
 {
     if (n_lines < 0 || N <= 0 || L <= 0) return 0;
-    return plan_xs(n_lines, N, L, prec, L, n_lines >= tree_min_lines(prec)).total;
+    return plan_xs(n_lines, N, L, prec, L, n_lines >= tree_min_lines(prec) ? FULL : LEAVES_ONLY).total;
 }
+
+// Lists of this length and more ask for the intervals in the smallest workspace too: without
+// them 20,000 lines on 20,000 points and 10 layers take 7.6 ms instead of 1.0, 220,000 and 4
+// layers 32.7 ms instead of 1.1.  They cost 8 to 13 bytes a grid point beside the lines' 92 to
+// 96 each; shorter lists would grow by more than they gain.
+constexpr int64_t COMPACT_MIN_LINES = 2048;
 
 size_t xs_workspace_min_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
 {
     if (n_lines < 0 || N <= 0 || L <= 0) return 0;
-    return plan_xs(n_lines, N, L, prec, 1, false).total;
+    return plan_xs(n_lines, N, L, prec, 1, n_lines >= COMPACT_MIN_LINES ? COMPACT : LEAVES_ONLY).total;
 }
 
 namespace xsi {
 
+size_t xs_least_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
+{
+    return plan_xs(n_lines, N, L, prec, 1, LEAVES_ONLY).total;
+}
+
 // The largest chunk of layers whose plan fits, with the intervals if any such fits.
 static int pick_plan(int64_t nl, int64_t N, int32_t L, int prec, size_t ws_bytes, XsPlan* out)
 {
-    for (int tree = nl >= tree_min_lines(prec) ? 1 : 0; tree >= 0; --tree)
+    for (int how = nl >= tree_min_lines(prec) ? FULL : LEAVES_ONLY; how >= LEAVES_ONLY; --how)
         for (int Lc = L;; Lc = (Lc + 1) / 2) {
-            XsPlan p = plan_xs(nl, N, L, prec, Lc, tree != 0);
+            XsPlan p = plan_xs(nl, N, L, prec, Lc, (Intervals)how);
             if (p.total <= ws_bytes) {
                 *out = p;
                 return XS_OK;
@@ -2552,11 +2571,14 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
         }
         prof_end(adjoint ? 1 : 0, st);
         count_launch();
+        if (adjoint) { // the next chunk of layers takes the partials' space
+            adjoint_reduce_kernel<R><<<dim3((unsigned)lc, 1, nz), 256, 0, st>>>(b, l0, p.leaf_blocks);
+            count_launch();
+        }
     }
     if (adjoint) {
-        adjoint_reduce_kernel<R><<<dim3((unsigned)L, 1, nz), 256, 0, st>>>(b, p.leaf_blocks);
         broad_sum_kernel<R><<<1, 32, 0, st>>>(b, L, 1.0 / sb, g_T_sum);
-        count_launch(2);
+        count_launch();
     }
     return (cudaGetLastError() == cudaSuccess) ? XS_OK : XS_ECUDA;
 }

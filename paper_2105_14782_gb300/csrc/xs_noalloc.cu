@@ -55,7 +55,7 @@ extern "C" int xs_compute_noalloc(const xs_lines* lines, const double* nu, int64
     if (r) return r;
     if (!sigma) return XS_EINVAL;
     // the smallest plan (one layer at a time) must fit the fixed array
-    if (xs_workspace_min_bytes(lines->n, N, L, prec) > XS_NOALLOC_SCRATCH_BYTES) return XS_ETOOBIG;
+    if (xsi::xs_least_bytes(lines->n, N, L, prec) > XS_NOALLOC_SCRATCH_BYTES) return XS_ETOOBIG;
     void* scratch = nullptr;
     r = noalloc_scratch(&scratch);
     if (r != XS_OK) return r;
