@@ -171,7 +171,7 @@ struct Species {
     R *rec3, *clo;
     Geo* geo;
     int2 *cov, *win, *pq;
-    double *sums, *coef; // forward: node sums, leaf polynomials
+    double *sums, *coef, *near; // forward: node sums, leaf polynomials, slices' sums
     R* wts;              // adjoint: node weights,
     double *slots, *leaf, *gbl; // and the partials of the far, the leaf and the reduction kernel
     void* sigma;
@@ -1475,8 +1475,8 @@ __device__ __forceinline__ void mask4(const int2* jr, int j, float2& a, float2& 
 }
 
 // A warp's leaf: its points and its near lines as up to five ranges (the first and last masked
-// per point, the others inside every line's cut).  `split` neighbouring warps of the block
-// share a leaf and take every split-th chunk of its lines.
+// per point, the others inside every line's cut).  `split` neighbouring warps of `slices`
+// blocks share a leaf and take its chunks of lines in turn.
 constexpr int RANGES = 5;
 // |z|^2 from which short forms hold: without far sets the lines nearer than it are a range
 // of their own, so that few chunks mix them with others.  A window of fewer lines than
@@ -1507,18 +1507,24 @@ template <> struct ShortForm<double> { static constexpr double z2 = Tier<double>
 template <class R>
 struct Leaf {
     int64_t jb, jl;
-    int lane, i, sub;
+    int lane, i, sub, slice;
     bool any, live; // the leaf has points; the lane has one
     int s[RANGES], e[RANGES];
     Geo g;
 
     __device__ void init(const Tree& tr, const Lines<R>& ln, const float* agg, int64_t nl, const double* nu, int64_t N,
-                         int nloc, int split)
+                         int nloc, int split, int slices)
     {
         const int w = threadIdx.x >> 5;
         lane = threadIdx.x & 31;
-        i = (blockIdx.x * (blockDim.x >> 5) + w) / split;
-        sub = w % split;
+        int block = blockIdx.x;
+        slice = 0;
+        if (slices > 1) {
+            block /= slices;
+            slice = blockIdx.x - block * slices;
+        }
+        i = (block * (int)(blockDim.x >> 5) + w) / split;
+        sub = slice * split + w % split;
         jb = (int64_t)i * LEAF;
         jl = min64(N - 1, jb + LEAF - 1);
         any = jb < N;
@@ -1585,7 +1591,7 @@ __device__ __forceinline__ double split_sum(double v, int split)
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(const __grid_constant__ Batch<float> batch,
                                                                            const double* __restrict__ nu, int64_t N,
                                                                            int layer0, double unscale,
-                                                                           int split)
+                                                                           int split, int slices)
 {
     const Species<float>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1595,7 +1601,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     NearTile& tl = tiles[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<float> lf;
-    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split, slices);
     const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1609,7 +1615,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     for (int k = 0; k < RANGES; ++k) {
         const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
+        for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split * slices) {
             const int l = t0 + lane;
             const bool have = l < ce;
             __syncwarp();
@@ -1723,12 +1729,16 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
             two_sum(shi, slo, acc); // the chunk's FP32 partial into the compensated sum
         }
     }
-    if (!tr.on && split == 1) { // nothing to add; the scale is a power of two
+    if (!tr.on && split * slices == 1) { // nothing to add; the scale is a power of two
         if (lf.live) sigma[(size_t)layer * N + j] = (shi + slo) * (float)unscale;
         return;
     }
     const double near = split_sum<LeafWarps<float>::v>((double)shi + (double)slo, split);
-    if (!lf.live || lf.sub) return;
+    if (!lf.live || lf.sub % split) return;
+    if (slices > 1) {
+        sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = near;
+        return;
+    }
     // the far lines' part
     const double far =
         tr.on ? LeafPoly<float>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
@@ -1774,7 +1784,7 @@ __device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, dou
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(const __grid_constant__ Batch<double> batch,
                                                                            const double* __restrict__ nu, int64_t N,
                                                                            int layer0, double unscale,
-                                                                           int split)
+                                                                           int split, int slices)
 {
     const Species<double>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1784,7 +1794,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     NearTile64& tl = ((NearTile64*)smem64)[threadIdx.x >> 5];
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     Leaf<double> lf;
-    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split, slices);
     const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
     const int lane = lf.lane;
     const int64_t j = min64(lf.jb + lane, N - 1);
@@ -1794,7 +1804,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     for (int k = 0; k < RANGES; ++k) {
         const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
+        for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split * slices) {
             const int l = t0 + lane;
             const bool have = lane < NEAR64 && l < ce;
             __syncwarp();
@@ -1840,9 +1850,31 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
         }
     }
     acc = split_sum<LeafWarps<double>::v>(acc, split);
-    if (!lf.live || lf.sub) return;
+    if (!lf.live || lf.sub % split) return;
+    if (slices > 1) {
+        sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = acc;
+        return;
+    }
     if (tr.on) acc += LeafPoly<double>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
     sigma[(size_t)layer * N + j] = acc * unscale;
+}
+
+// sigma from the slices' sums over the near lines (in order) and the far lines' polynomials
+template <class R>
+__global__ void __launch_bounds__(256) slices_kernel(const __grid_constant__ Batch<R> batch, const double* __restrict__ nu,
+                                                     int64_t N, int layer0, double unscale, int slices)
+{
+    const Species<R>& sp = batch.s[blockIdx.z];
+    const int nloc = blockIdx.y;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= N) return;
+    double s = 0.0;
+    for (int k = 0; k < slices; ++k) s += sp.near[((size_t)k * gridDim.y + nloc) * N + j];
+    if (sp.tree.on) {
+        const int i = (int)(j / LEAF);
+        s += LeafPoly<R>::eval(sp.coef, (size_t)nloc * sp.tree.cnt[0] + i, in_span(nu[j], sp.tree.geo[i]));
+    }
+    ((R*)sp.sigma)[(size_t)(layer0 + nloc) * N + j] = (R)(s * unscale);
 }
 
 // a block's sums of the leaves' (f_T, f_b) to part[layer of the chunk][block], fixed order
@@ -1892,7 +1924,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                                                                             const double* __restrict__ nu, int64_t N,
                                                                             int layer0,
                                                                             const double* __restrict__ T,
-                                                                            double lam_scale, int split)
+                                                                            double lam_scale, int split, int slices)
 {
     const Species<float>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1903,7 +1935,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<float> lf;
-    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split, slices);
     if (lf.any) {
         const Lines<float> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
@@ -1921,7 +1953,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
         for (int k = 0; k < RANGES; ++k) {
             const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split) {
+            for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split * slices) {
                 const int l = t0 + lane;
                 const bool have = l < ce;
                 __syncwarp();
@@ -2113,7 +2145,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
                                                                             const double* __restrict__ nu, int64_t N,
                                                                             int layer0,
                                                                             const double* __restrict__ T,
-                                                                            double lam_scale, int split)
+                                                                            double lam_scale, int split, int slices)
 {
     const Species<double>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -2124,7 +2156,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
     const int nloc = blockIdx.y, layer = layer0 + nloc;
     double sT = 0.0, sB = 0.0;
     Leaf<double> lf;
-    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split);
+    lf.init(tr, sp.ln, sp.agg + 4 * layer, nl, nu, N, nloc, split, slices);
     if (lf.any) {
         const Lines<double> ln = layer_lines(sp.ln, nl, nloc);
         const int lane = lf.lane;
@@ -2138,7 +2170,7 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
         for (int k = 0; k < RANGES; ++k) {
             const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split) {
+            for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split * slices) {
                 const int l = t0 + lane;
                 const bool have = lane < NEAR64 && l < ce;
                 const int cnt = min(NEAR64, ce - t0);
@@ -2273,14 +2305,19 @@ template <class R> struct DenseLines { static constexpr int64_t v = 4; };
 template <> struct DenseLines<double> { static constexpr int64_t v = 1; };
 
 struct XsPlan {
-    int prec, Lc, nchunks, leaf_blocks, leaf_warps, leaf_split;
+    int prec, Lc, nchunks, leaf_blocks, leaf_warps, leaf_split, slices; // leaf_blocks: of all slices
     Tree tree; // counts and offsets; pointers set at run time
     FarWork fw;
     int far_blocks;
     size_t rows; // node-sum rows of all levels and parts
     size_t off_jr, off_nuf, off_inv, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq,
-        off_fwd, off_coef, off_wts, off_slots, off_leaf, off_gbl, total;
+        off_fwd, off_coef, off_near, off_wts, off_slots, off_leaf, off_gbl, total;
 };
+
+// What of the intervals a plan holds: COMPACT has four intervals below each one and splits
+// their lists in as many parts as cost about a byte a line, the least space with which far
+// lines go to the nodes.
+enum Intervals { LEAVES_ONLY, COMPACT, FULL };
 
 // Parts of the far lists: enough warps to fill the GPU several times over, each with a
 // list long enough to pay for its reduction (FP64 evaluations cost about ten times
@@ -2317,11 +2354,12 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed, bool compac
 // smaller blocks, so that the work reaches more SMs (one layer of 4,096 points has 128
 // leaves: in FP64, 16 blocks of 8 leaves took 616 us, 128 blocks with 8 warps on a leaf
 // 125 us; FP32, 32 blocks of 4 leaves 22 us, 128 blocks of one 14 us).
-void choose_leaf_blocks(XsPlan* p, int64_t N, int Lc, bool mixed, bool small)
+void choose_leaf_blocks(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed, Intervals how)
 {
     const int most = mixed ? LeafWarps<float>::v : LeafWarps<double>::v;
     const int64_t leaves = (N + LEAF - 1) / LEAF, all = leaves * Lc;
     const int64_t want = mixed ? 152 * 16 : 152 * 8; // warps
+    const bool small = how == LEAVES_ONLY; // the smallest workspaces hold one partial per full block
     int split = 1;
     while (!small && split < most && all * split < want) split *= 2;
     int warps = most;
@@ -2329,13 +2367,13 @@ void choose_leaf_blocks(XsPlan* p, int64_t N, int Lc, bool mixed, bool small)
     p->leaf_split = split;
     p->leaf_warps = warps;
     const int per = warps / split;
-    p->leaf_blocks = (int)((leaves + per - 1) / per);
+    // and of long lists between blocks as well: 1,000,000 lines at 64 points 60 cm^-1 apart, one
+    // layer, 25.1 -> 1.3 ms (its two leaves ran on two SMs), 60,000 on 2,000 points 235 -> 147 us;
+    // FP64, 6,000 on 500 1312 -> 507 us
+    const int64_t lines = mixed ? 8192 : 512; // of the whole list for each slice
+    p->slices = how == FULL ? (int)std::max<int64_t>(1, std::min<int64_t>({64, want / (all * split), nl / lines})) : 1;
+    p->leaf_blocks = (int)((leaves + per - 1) / per) * p->slices;
 }
-
-// What of the intervals a plan holds: COMPACT has four intervals below each one and splits
-// their lists in as many parts as cost about a byte a line, the least space with which far
-// lines go to the nodes.
-enum Intervals { LEAVES_ONLY, COMPACT, FULL };
 
 XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, Intervals how)
 {
@@ -2353,7 +2391,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, Intervals how
         off += align256(bytes);
         return o;
     };
-    choose_leaf_blocks(&p, N, Lc, mixed, !tree); // the smallest workspaces hold one partial per full block
+    choose_leaf_blocks(&p, nl, N, Lc, mixed, how);
     p.off_jr = take(sizeof(int2) * n1);
     p.off_nuf = take(mixed ? sizeof(float2) * n1 : 0);
     p.off_inv = take(sizeof(double) * n1);
@@ -2386,6 +2424,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, Intervals how
         p.off_coef = take(sizeof(double) * (mixed ? LeafPoly<float>::stride : LeafPoly<double>::stride) * (size_t)Lc *
                           p.tree.cnt[0]);
     }
+    p.off_near = take(p.slices > 1 ? sizeof(double) * p.slices * (size_t)Lc * (size_t)N : 0);
     const size_t fwd_end = off;
     off = base;
     if (tree) {
@@ -2476,6 +2515,7 @@ static Species<R> make_species(const xs_lines* ln, const XsPlan& p, char* ws, in
     s.pq = (int2*)(ws + p.off_pq);
     s.sums = (double*)(ws + p.off_fwd);
     s.coef = (double*)(ws + p.off_coef);
+    s.near = (double*)(ws + p.off_near);
     s.wts = (R*)(ws + p.off_wts);
     s.slots = (double*)(ws + p.off_slots);
     s.leaf = (double*)(ws + p.off_leaf);
@@ -2491,7 +2531,7 @@ static Species<R> make_species(const xs_lines* ln, const XsPlan& p, char* ws, in
 }
 
 // The line sums (or their adjoints) of a batch of species with plans of the same shape
-// (same chunks of layers, same use of the intervals); p: the first one's.
+// (same chunks of layers, same use of the intervals, same slices); p: the first one's.
 template <class R>
 static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64_t N, const double* T, const double* P,
                      int32_t L, double sb, double W, bool adjoint, cudaStream_t st, int flags, double* g_T_sum)
@@ -2552,10 +2592,10 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, unscale, p.leaf_split);
+                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, unscale, p.leaf_split, p.slices);
             else
                 leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(b, nu, N, l0, unscale,
-                                                                                           p.leaf_split);
+                                                                                           p.leaf_split, p.slices);
         } else {
             if (tr.on) {
                 up_kernel<R><<<dim3(blocks_of(tr.cnt[0], TOP), (unsigned)lc, nz), 32 * UP_WARPS, 0, st>>>(b, nu, N, l0,
@@ -2564,10 +2604,14 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, T, unscale, p.leaf_split);
+                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, T, unscale, p.leaf_split, p.slices);
             else
                 leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(b, nu, N, l0, T,
-                                                                                              unscale, p.leaf_split);
+                                                                                              unscale, p.leaf_split, p.slices);
+        }
+        if (!adjoint && p.slices > 1) {
+            slices_kernel<R><<<dim3(blocks_of(N, 256), (unsigned)lc, nz), 256, 0, st>>>(b, nu, N, l0, unscale, p.slices);
+            count_launch();
         }
         prof_end(adjoint ? 1 : 0, st);
         count_launch();
@@ -2603,7 +2647,8 @@ static int run_species(int n, const XsJob* job, const XsPlan* plan, const double
         }
         const int first = m;
         Batch<R> b{};
-        while (m < n && job[m].lines->n > 0 && plan[m].tree.on == plan[first].tree.on && plan[m].Lc == plan[first].Lc) {
+        while (m < n && job[m].lines->n > 0 && plan[m].tree.on == plan[first].tree.on && plan[m].Lc == plan[first].Lc &&
+               plan[m].slices == plan[first].slices) {
             Species<R>& s = b.s[b.n++];
             s = make_species<R>(job[m].lines, plan[m], (char*)job[m].ws, L);
             s.sigma = job[m].sigma;
