@@ -12,6 +12,8 @@
 // and stages the input points, their reciprocals and values once; a pair's logarithm of
 // a ratio near one is then a quotient from the reciprocal and a short polynomial instead of
 // a division and a logarithm.  Several lanes share an output point.
+#include <algorithm>
+
 #include "xs_device.cuh"
 #include "xs_internal.h"
 
@@ -368,7 +370,10 @@ int response_ip_rv(const double* F1, const double* nu, int64_t N, const double* 
 size_t response_workspace_bytes(int64_t N_out)
 {
     if (N_out <= 0) return 0;
-    return al256(sizeof(double) * (size_t)N_out) + al256(sizeof(double) * (size_t)blocks(N_out));
+    // a partial a block; grids of RESP_SHORT points and a little more have fewer blocks than
+    // shorter ones, and a workspace that serves a grid serves every shorter one too
+    const size_t parts = std::max(blocks(N_out), blocks(std::min(N_out, RESP_SHORT - 1)));
+    return al256(sizeof(double) * (size_t)N_out) + al256(sizeof(double) * parts);
 }
 
 int response_rotation_adjoint(const double* g_F1, const double* F0, const double* nu, int64_t N, double vsini,
