@@ -619,15 +619,16 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
 // Points a block of the emission kernels takes: see emission_kernel.
 static int emission_points(int64_t N) { return N >= 608 * 32 ? 32 : N >= 608 * 16 ? 16 : 8; }
 
-// [L][nb] per-block layer partials, then T_n, E2_n and S_n as [L][N] each
+// [L][nb] per-block layer partials, then T_n, E2_n and S_n as [L][N] each.  The partials'
+// space is that of the smallest blocks, so that the size grows with N and a workspace that
+// serves a grid serves every smaller one.
 struct EmissionWs {
     double *part, *tr, *e2, *S;
     size_t bytes;
 };
 static EmissionWs emission_ws(int32_t L, int64_t N, void* ws)
 {
-    const int pts = emission_points(N);
-    const int64_t nb = (N + pts - 1) / pts;
+    const int64_t nb = (N + 7) / 8;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t part = al(sizeof(double) * (size_t)L * (size_t)nb), LN = al(sizeof(double) * (size_t)L * (size_t)N);
     char* base = (char*)ws;
