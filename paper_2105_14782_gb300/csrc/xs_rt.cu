@@ -238,8 +238,7 @@ __global__ void __cluster_dims__(RT_CLUSTER, 1, 1)
 // sectors) and its RT_THREADS/PTS groups of lanes take contiguous segments of the layers:
 // each reduces its segment to (prod T, local sum), and the segments are chained in
 // order.  Bound by FP64 operations (about 70 a point and layer) on the SMs that have
-// blocks: 32 points a block from 608 blocks (four a SM) on, fewer points and shorter
-// segments below (a served request of 20 layers x 2,003 points ran on 63 SMs).
+// blocks: see emission_points.
 __device__ __forceinline__ void seg_range(int L, int w, int segs, int* n0, int* n1)
 {
     *n0 = (int)(((int64_t)L * w) / segs);
@@ -616,8 +615,35 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
     return launched(1);
 }
 
-// Points a block of the emission kernels takes: see emission_kernel.
-static int emission_points(int64_t N) { return N >= 608 * 32 ? 32 : N >= 608 * 16 ? 16 : 8; }
+// Points a block of the emission kernels takes.  A group of lanes of a warp is a segment, so a
+// warp's time is its longest segment's layers, and what counts is the sum of that over a
+// block's warps times the blocks an SM gets: in whole blocks while they are few (below four
+// an SM), on average then.  A few layers leave most segments of the small blocks empty (3
+// layers x 9,000 points 47 us with 8, 12 with 32; 20 x 2,003 23 with 8, 19 with 16); 60 x 3,000
+// take 8 points, for more SMs.
+static int emission_points(int32_t L, int64_t N)
+{
+    constexpr int SMS = 152;
+    int best = 32;
+    double least = 0.0;
+    for (int pts = 32; pts >= 8; pts /= 2) {
+        const int segs = RT_THREADS / pts, group = 32 / pts; // segments of a block and of a warp
+        int layers = 0;
+        for (int w = 0; w < segs; w += group) {
+            int most = 0;
+            for (int g = w; g < w + group; ++g)
+                most = std::max(most, (int)((int64_t)L * (g + 1) / segs - (int64_t)L * g / segs));
+            layers += most;
+        }
+        const int64_t nb = (N + pts - 1) / pts;
+        const double cost = layers * (nb >= 4 * SMS ? (double)nb / SMS : (double)((nb + SMS - 1) / SMS));
+        if (pts == 32 || cost < least) {
+            least = cost;
+            best = pts;
+        }
+    }
+    return best;
+}
 
 // [L][nb] per-block layer partials, then T_n, E2_n and S_n as [L][N] each.  The partials'
 // space is that of the smallest blocks, so that the size grows with N and a workspace that
@@ -649,7 +675,7 @@ static void launch_emission(const double* dtau, const double* T, const double* n
 int rt_emission(const double* dtau, const double* T, const double* nu, int32_t L, int64_t N, double* F0,
                 cudaStream_t st, void* keep)
 {
-    const int pts = emission_points(N);
+    const int pts = emission_points(L, N);
     if (pts == 32) launch_emission<32>(dtau, T, nu, L, N, F0, keep, st);
     else if (pts == 16) launch_emission<16>(dtau, T, nu, L, N, F0, keep, st);
     else launch_emission<8>(dtau, T, nu, L, N, F0, keep, st);
@@ -670,7 +696,7 @@ static void launch_emission_adjoint(const double* g_F0, const double* dtau, cons
 int rt_emission_adjoint(const double* g_F0, const double* dtau, const double* T, const double* nu, int32_t L,
                         int64_t N, double* g_dtau, double* g_T, void* ws, cudaStream_t st, bool reuse)
 {
-    const int pts = emission_points(N);
+    const int pts = emission_points(L, N);
     const EmissionWs w = emission_ws(L, N, ws);
     if (pts == 32) launch_emission_adjoint<32>(g_F0, dtau, T, nu, L, N, g_dtau, w, reuse, st);
     else if (pts == 16) launch_emission_adjoint<16>(g_F0, dtau, T, nu, L, N, g_dtau, w, reuse, st);
