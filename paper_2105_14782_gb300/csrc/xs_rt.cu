@@ -4,6 +4,7 @@
 // these steps read and write [L][N] arrays once or twice and are bound by HBM.
 #include <algorithm>
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "xs_device.cuh"
 #include "xs_internal.h"
@@ -174,50 +175,60 @@ __global__ void tau_kernel(SigPtrs sig, int S, const double* __restrict__ vmr, c
     }
 }
 
-// Sum over a cluster of RT_CLUSTER blocks, fixed order; the result is valid in thread 0
-// of rank 0.  One block cannot draw enough of the chip for a row of 1e4-1e5 points.
+// Sum over a cluster of C blocks, fixed order; the result is valid in thread 0 of rank 0.
+// One block cannot draw enough of the chip for a row of 1e4-1e5 points.
 constexpr int RT_CLUSTER = 8;
+template <int C>
 __device__ __forceinline__ double cluster_sum(double v, double* red, double* slot)
 {
     namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
     red[threadIdx.x] = v;
     __syncthreads();
     for (int s = blockDim.x / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *slot = red[0];
-    cl.sync();
     double t = 0.0;
-    if (threadIdx.x == 0 && cl.block_rank() == 0)
-        for (int b = 0; b < RT_CLUSTER; ++b) t += *cl.map_shared_rank(slot, b);
-    cl.sync(); // the slots are read before they are written again or a block ends
+    if constexpr (C == 1) {
+        t = red[0];
+        __syncthreads(); // read before it is written again
+    } else {
+        cg::cluster_group cl = cg::this_cluster();
+        if (threadIdx.x == 0) *slot = red[0];
+        cl.sync();
+        if (threadIdx.x == 0 && cl.block_rank() == 0)
+            for (int b = 0; b < C; ++b) t += *cl.map_shared_rank(slot, b);
+        cl.sync(); // the slots are read before they are written again or a block ends
+    }
     return t;
 }
 
-// g_sigma[m] = g_dtau col vmr; g_vmr[m][n] = col sum_j g_dtau sigma_m.  A cluster of
+// g_sigma[m] = g_dtau col vmr; g_vmr[m][n] = col sum_j g_dtau sigma_m.  A cluster of C
 // blocks per layer, one pass over the row for all species (one block per layer and a pass
 // per species before: 101 layers x 49,999 points 178 us, 4 layers x 100,000 points 304 us).
-__global__ void __cluster_dims__(RT_CLUSTER, 1, 1)
-    tau_adjoint_kernel(SigPtrs sig, GSigPtrs gsig, int S, const double* __restrict__ vmr,
+// M: the number of species, XS_MAX_SPECIES for any.
+template <int C, int M>
+__global__ void __launch_bounds__(RT_THREADS)
+    tau_adjoint_kernel(SigPtrs sig, GSigPtrs gsig, int species, const double* __restrict__ vmr,
                        const double* __restrict__ dP, int L, int64_t N, double g, double mu, int is_float,
                        const double* __restrict__ g_dtau, double* __restrict__ g_vmr)
 {
     __shared__ double red[RT_THREADS], slot;
-    const int n = blockIdx.x / RT_CLUSTER, rank = blockIdx.x % RT_CLUSTER;
+    const int S = M < XS_MAX_SPECIES ? M : species;
+    const int n = blockIdx.x / C, rank = blockIdx.x % C;
     const double col = dP[n] * 1e6 / (mu * amu * g);
-    double acc[XS_MAX_SPECIES], cv[XS_MAX_SPECIES];
+    double acc[M], cv[M];
 #pragma unroll
-    for (int m = 0; m < XS_MAX_SPECIES; ++m) {
+    for (int m = 0; m < M; ++m) {
         acc[m] = 0.0;
         cv[m] = m < S ? col * vmr[(size_t)m * L + n] : 0.0;
     }
-    for (int64_t j = (int64_t)rank * blockDim.x + threadIdx.x; j < N; j += RT_CLUSTER * blockDim.x) {
+#pragma unroll (M <= 2 ? 4 : 1)
+    for (int64_t j = (int64_t)rank * blockDim.x + threadIdx.x; j < N; j += C * blockDim.x) {
         const size_t i = (size_t)n * N + j;
         const double gd = g_dtau[i];
 #pragma unroll
-        for (int m = 0; m < XS_MAX_SPECIES; ++m) {
+        for (int m = 0; m < M; ++m) {
             if (m >= S) break;
             const double v = is_float ? (double)((const float*)sig.p[m])[i] : ((const double*)sig.p[m])[i];
             acc[m] = fma(gd, v, acc[m]);
@@ -225,9 +236,9 @@ __global__ void __cluster_dims__(RT_CLUSTER, 1, 1)
         }
     }
 #pragma unroll
-    for (int m = 0; m < XS_MAX_SPECIES; ++m) {
+    for (int m = 0; m < M; ++m) {
         if (m >= S) break;
-        const double t = cluster_sum(acc[m], red, &slot);
+        const double t = cluster_sum<C>(acc[m], red, &slot);
         if (threadIdx.x == 0 && rank == 0) g_vmr[(size_t)m * L + n] = col * t;
     }
 }
@@ -417,7 +428,7 @@ __global__ void __cluster_dims__(RT_CLUSTER, 1, 1)
         acc = fma(r, r, acc);
         if (gF) gF[j] = r * is;
     }
-    const double t = cluster_sum(acc, red, &slot);
+    const double t = cluster_sum<RT_CLUSTER>(acc, red, &slot);
     if (threadIdx.x == 0 && blockIdx.x == 0) logL[0] = -0.5 * t;
 }
 
@@ -610,8 +621,36 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
         sp.p[m] = sigma[m];
         gp.p[m] = g_sigma ? g_sigma[m] : nullptr;
     }
-    tau_adjoint_kernel<<<(unsigned)(RT_CLUSTER * L), RT_THREADS, 0, st>>>(sp, gp, S, vmr, dP, L, N, g, mu,
-                                                                           prec == XS_PREC_MIXED, g_dtau, g_vmr);
+    // blocks a layer: up to 8, fewer where the layers alone fill the chip or a block had less
+    // than 1,024 points (a cluster costs more to launch and to join than so short a row: 1,000
+    // layers of 50 points 154 us with 8 blocks, 300 of 9,727 88 us)
+    int c = 1;
+    while (c < RT_CLUSTER && (int64_t)c * L < 256 && 2 * c * 1024 <= N) c *= 2;
+    auto pick = [&](auto M) {
+        constexpr int m = decltype(M)::value;
+        return c == 8   ? tau_adjoint_kernel<8, m>
+               : c == 4 ? tau_adjoint_kernel<4, m>
+               : c == 2 ? tau_adjoint_kernel<2, m>
+                        : tau_adjoint_kernel<1, m>;
+    };
+    auto* k = S == 1   ? pick(std::integral_constant<int, 1>{})
+              : S == 2 ? pick(std::integral_constant<int, 2>{})
+                       : pick(std::integral_constant<int, XS_MAX_SPECIES>{});
+    int threads = RT_THREADS;
+    while (threads > 32 && threads * (int64_t)c * 4 > N) threads /= 2; // four points a thread
+    cudaLaunchAttribute cluster{};
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = (unsigned)c;
+    cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(c * L));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = c > 1 ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, k, sp, gp, (int)S, vmr, dP, (int)L, N, g, mu, (int)(prec == XS_PREC_MIXED), g_dtau, g_vmr) !=
+        cudaSuccess)
+        return XS_ECUDA;
     return launched(1);
 }
 
