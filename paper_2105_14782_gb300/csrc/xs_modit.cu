@@ -265,9 +265,11 @@ __global__ void modit_images_kernel(int64_t M, R* __restrict__ A)
     A[i] = (R)v;
 }
 
-// Frequencies a thread takes, 256 apart: e^(-2 pi gamma'_k f) is advanced from one to the
-// next by a product.
-constexpr int MODIT_STEP = 256;
+// A thread's frequencies lie MODIT_STEP apart: e^(-2 pi gamma'_k f) is advanced from one to
+// the next by a product.  Blocks of 64 threads: with 256, short transforms of a few layers had
+// one to a few blocks, whose FP64 operations waited for one SM's pipe (FP32, 2,000 lines on
+// 1,000 points, one layer 174 -> 131 us; 20,000 x 5 layers with the adjoint 552 -> 441).
+constexpr int MODIT_STEP = 64;
 
 // Y[n][m] = sum_k Z[n][k][m] K_k(m) for m = 0..M/2
 template <class R, int F>
