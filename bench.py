@@ -4,8 +4,8 @@
 One step = one HMC-style forward + gradient of the 100-layer emission model:
 layer temperatures, both species' line-sum cross-sections, optical depth,
 emission solve, Gaussian log-likelihood, and the adjoints of all of them, in the
-mixed precision form (FP32 Voigt and compensated sums, FP64 offsets and
-strengths, FP64 radiative transfer).  The metric counts the Voigt evaluations that the
+mixed precision form (FP32 Voigt and compensated sums, offsets and strength
+exponents formed in FP64 and carried as FP32 pairs, FP64 radiative transfer).  The metric counts the Voigt evaluations that the
 sum stands for: every in-cut (line, grid point, layer) triple once in the forward line
 sum and once in its adjoint.  Triples far from the line are summed through
 interpolation nodes (to below FP32 rounding, csrc/xs_linesum.cu), so they cost less
@@ -733,7 +733,8 @@ def main():
                            WORKLOAD_TEXT[args.workload].replace("100 layers", f"{L} layers"),
                            "step": "forward + gradient (logL and dlogL/dtheta, theta = T0, alpha, 2 log10 VMR, "
                                    "broadening scale)",
-                           "precision": "FP32 Voigt + compensated FP32 sums, FP64 offsets/strengths, FP64 RT"
+                           "precision": "FP32 Voigt + compensated FP32 sums, offsets and strength exponents formed in "
+                                        "FP64 and carried as FP32 pairs, FP64 RT"
                            if prec == xs.PREC_MIXED else "FP64 throughout",
                            "evals_per_step": res["evals_per_step"], "in_cut_triples": res["triples"],
                            "l2": "inputs larger than L2: the per-step line records (tens of GB) are rewritten "

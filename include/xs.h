@@ -44,8 +44,10 @@ typedef enum {
 
 typedef enum {
     XS_PREC_FP64 = 0, /* every step in double precision */
-    XS_PREC_MIXED = 1 /* Voigt evaluation and line sum in FP32 (compensated), line-centre
-                         offsets and strength exponentials in FP64; sigma stored as float */
+    XS_PREC_MIXED = 1 /* Voigt evaluation and line sum in FP32 (compensated); line-centre offsets and
+                         the arguments of the strengths' exponentials formed in FP64 and carried
+                         as FP32 pairs (to 1e-10), the strengths' derivatives, widths and adjoint
+                         weights in FP32; sigma stored as float */
 } xs_prec;
 
 #define XS_MAX_SPECIES 8

@@ -62,3 +62,23 @@ def test_low_wavenumbers(nu0, T0, weight):
     rng = np.random.default_rng(3)
     compare(lines, W.grid_lognu(N, nu0, 1.01 * nu0), np.array([0.8 * T0, T0, T0]), np.array([1e-6, 1e-4, 1e-3]),
             0.004 * nu0, lambda s: weight * (1.0 + 0.5 * dev(rng.uniform(size=(3, N)))))
+
+
+@pytest.mark.parametrize("n,N,L", [(300, 40, 3), (3000, 2500, 5), (20000, 1500, 4)])
+def test_weights_of_mixed_sign(n, N, L):
+    """A fitted spectrum's dF/dsigma has both signs and its sums cancel.  An evaluation is good to
+    1e-6 and the terms of dln sigma/dln T are up to ten times one (E'' c2/T of 5,000 cm^-1), so
+    1e-5 of the sum of |lambda| sigma bounds T g_T and g_b (1e-3 to 1e-1 of what weights of one
+    sign would give)."""
+    from paper_2105_14782_gb300 import xs
+    dl = xs.DeviceLines(W.water_like(n, seed=n))
+    rng = np.random.default_rng(n)
+    nu, P = W.grid_lognu(N), 10.0 ** np.linspace(-3, 2, L)
+    args = dl, dev(nu), dev(1300.0 * P ** 0.1), dev(P)
+    s = xs.xs_compute(*args, 1.1, 25.0, xs.PREC_FP64)
+    lam = dev(rng.standard_normal((L, N))) / s.amax(dim=1, keepdim=True)
+    size = (lam * s).abs().sum(dim=1)
+    want = xs.xs_compute_adjoint(*args, lam, 1.1, 25.0, xs.PREC_FP64)
+    got = xs.xs_compute_adjoint(*args, lam, 1.1, 25.0, xs.PREC_MIXED)
+    assert torch.all((got[0] - want[0]).abs() * args[2] <= 1e-5 * size)
+    assert abs((got[1] - want[1]).item()) <= 1e-5 * float(size.sum())
