@@ -152,6 +152,7 @@ struct FarWork {
     int parts[LEVELS], block0[LEVELS]; // block0: first block of the level
     size_t out0[LEVELS];               // first node-sum row of the level (in rows of n)
     int slot0[LEVELS], slots;          // first adjoint slot of the level, slots a layer
+    size_t rows;                       // node-sum rows of all levels
 };
 
 // One species of a launch: its lists, workspace arrays and plan.  The line sums of a
@@ -535,6 +536,10 @@ __global__ void near_range_kernel(const __grid_constant__ Batch<R> batch, int la
 struct FarSet {
     int a, p, q, b;
     int A, P, Q, B;
+    __device__ __forceinline__ bool in_order(int64_t nl) const
+    {
+        return 0 <= a && a <= A && A <= P && P <= p && p <= q && q <= Q && Q <= B && B <= b && b <= nl;
+    }
 };
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return min(max(v, lo), hi); }
@@ -548,6 +553,7 @@ __device__ __forceinline__ FarSet far_set(const Tree& tr, int level, int i, int 
     bool left = false, right = false; // the interval above has far lines on that side
     for (int k = TOP_LOG / shift; k >= level; --k) {
         const int at = tr.off[k] + (i >> (shift * (k - level)));
+        if (!XS_CHECK(at >= 0 && at < tr.total)) return FarSet{};
         const int2 c = tr.cov[at], s = tr.pq[(size_t)tr.total * nloc + at];
         const int a = c.x, b = max(c.x, c.y);
         f.A = left ? f.a : a;
@@ -1140,12 +1146,12 @@ __global__ void __launch_bounds__(32 * FAR_WARPS) far_sum_kernel(const __grid_co
     const FarList fl(fs);
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
-    if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
+    if (!XS_CHECK(fs.in_order(nl))) t0 = t1 = 0;
     int idx;
     const double s = far_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), sp.agg[4 * (layer0 + nloc)],
                              idx);
     const size_t row = fw.out0[k] + ((size_t)part * gridDim.y + nloc) * tr.cnt[k] + i;
-    if (idx >= 0) sp.sums[row * n + idx] = s;
+    if (idx >= 0 && XS_CHECK(idx < n && row < fw.rows)) sp.sums[row * n + idx] = s;
 }
 
 template <class R>
@@ -1167,15 +1173,17 @@ __global__ void __launch_bounds__(32 * FAR_WARPS, FarBlocks<R>::v)
     const FarList fl(fs);
     int t0, t1;
     part_range(fl.total, part, fw.parts[k], &t0, &t1);
-    if (!XS_CHECK(fs.a >= 0 && fs.b <= nl && fl.total >= 0)) t0 = t1 = 0;
+    if (!XS_CHECK(fs.in_order(nl))) t0 = t1 = 0;
     double sT, sB;
     far_adjoint_sum(ln, fl, t0, t1, Span(tr.geo[tr.off[k] + i], nu[0]), sp.agg[4 * layer],
                     sp.wts + ((size_t)nloc * tr.total + tr.off[k] + i) * n,
                     (R)(0.5 / T[layer]), sT, sB);
     if ((threadIdx.x & 31) == 0) {
         const size_t o = (size_t)nloc * fw.slots + fw.slot0[k] + (size_t)part * tr.cnt[k] + i;
-        sp.slots[2 * o] = sT;
-        sp.slots[2 * o + 1] = sB;
+        if (XS_CHECK(o < (size_t)gridDim.y * fw.slots)) {
+            sp.slots[2 * o] = sT;
+            sp.slots[2 * o + 1] = sB;
+        }
     }
 }
 
@@ -1269,11 +1277,13 @@ __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const 
         const int first = below <= 0 ? blockIdx.x >> -below : blockIdx.x * many;
         for (int q0 = 0; q0 < many; q0 += rows) {
             const int q = q0 + row, i = first + q;
-            const bool mine = q < many && i < tr.cnt[k];
+            const bool mine = q < many && i < tr.cnt[k] && XS_CHECK(i >= 0 && row < DownRows<R>::v && (k == 0 || q < TOP / 2));
             if (mine) {
                 double s = 0.0;
-                for (int p = 0; p < fw.parts[k]; ++p)
-                    s += sp.sums[(fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i) * n + m];
+                for (int p = 0; p < fw.parts[k]; ++p) {
+                    const size_t at = fw.out0[k] + ((size_t)p * Lc + nloc) * tr.cnt[k] + i;
+                    if (XS_CHECK(at < fw.rows)) s += sp.sums[at * n + m];
+                }
                 if (k < tr.top) {
                     const Geo g = tr.geo[tr.off[k] + i], gp = tr.geo[tr.off[k + 1] + (i >> tr.shift)];
                     s += clenshaw<n, double>(c[(k + 1) & 1][q >> tr.shift], node_in_span(g, cheb<n>(1, m), gp));
@@ -1342,7 +1352,7 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
         const int many = 1 << (tr.shift * (tr.top - k)), below = 1 << tr.shift;
         for (int q = row; q < many; q += UP_WARPS) {
             const int i = top * many + q;
-            if (i >= tr.cnt[k]) break;
+            if (i >= tr.cnt[k] || !XS_CHECK(q < TOP)) break;
             const Geo sp = tr.geo[tr.off[k] + i];
             R s[n];
 #pragma unroll
@@ -1363,7 +1373,7 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
             __syncwarp();
             int idx;
             const R v = warp_reduce_scatter(s, idx);
-            if (idx >= 0) M[row][idx] = v;
+            if (idx >= 0 && XS_CHECK(idx < n)) M[row][idx] = v;
             __syncwarp();
             if (lane < n) {
                 const R x = node_weight<n, R>(M[row], lane);
@@ -1742,12 +1752,12 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     const double near = split_sum<LeafWarps<float>::v>((double)shi + (double)slo, split);
     if (!lf.live || lf.sub % split) return;
     if (slices > 1) {
-        sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = near;
+        if (XS_CHECK(lf.slice < slices && j < N)) sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = near;
         return;
     }
     // the far lines' part
     const double far =
-        tr.on ? LeafPoly<float>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
+        tr.on && XS_CHECK(lf.i < tr.cnt[0]) ? LeafPoly<float>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g)) : 0.0;
     sigma[(size_t)layer * N + j] = (float)((far + near) * unscale);
 }
 
@@ -1858,10 +1868,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     acc = split_sum<LeafWarps<double>::v>(acc, split);
     if (!lf.live || lf.sub % split) return;
     if (slices > 1) {
-        sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = acc;
+        if (XS_CHECK(lf.slice < slices && j < N)) sp.near[((size_t)lf.slice * gridDim.y + nloc) * N + j] = acc;
         return;
     }
-    if (tr.on) acc += LeafPoly<double>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
+    if (tr.on && XS_CHECK(lf.i < tr.cnt[0])) acc += LeafPoly<double>::eval(sp.coef, (size_t)nloc * tr.cnt[0] + lf.i, in_span(nuj, lf.g));
     sigma[(size_t)layer * N + j] = acc * unscale;
 }
 
@@ -2315,7 +2325,6 @@ struct XsPlan {
     Tree tree; // counts and offsets; pointers set at run time
     FarWork fw;
     int far_blocks;
-    size_t rows; // node-sum rows of all levels and parts
     size_t off_jr, off_nuf, off_inv, off_agg, off_rec1, off_rec2, off_rec3, off_clo, off_geo, off_cov, off_win, off_pq,
         off_fwd, off_coef, off_near, off_wts, off_slots, off_leaf, off_gbl, total;
 };
@@ -2352,7 +2361,7 @@ void split_far(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed, bool compac
         p->fw.slots += (int)parts * p->tree.cnt[k];
     }
     p->far_blocks = block;
-    p->rows = row;
+    p->fw.rows = row;
 }
 
 // Blocks of the leaf kernels.  With enough leaves, a warp each and full blocks; fewer
@@ -2426,7 +2435,7 @@ XsPlan plan_xs(int64_t nl, int64_t N, int32_t L, int prec, int Lc, Intervals how
     // the forward's node sums and polynomials; the adjoint's weights and partials reuse the space
     const size_t base = off;
     if (tree) {
-        p.off_fwd = take(sizeof(double) * n * p.rows);
+        p.off_fwd = take(sizeof(double) * n * p.fw.rows);
         p.off_coef = take(sizeof(double) * (mixed ? LeafPoly<float>::stride : LeafPoly<double>::stride) * (size_t)Lc *
                           p.tree.cnt[0]);
     }
