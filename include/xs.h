@@ -143,7 +143,7 @@ int xs_compute(const xs_lines* lines, const double* nu, int64_t N, const double*
  * process exits.  Problems whose smallest plan (one layer at a time) needs more
  * than 64 MiB are rejected with XS_ETOOBIG before any launch; where
  * xs_workspace_min_bytes(n, N, L, prec) <= 64 MiB none are.  That plan holds about
- * n * 92 bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records and
+ * n * 68 bytes (XS_PREC_MIXED) or n * 96 bytes (XS_PREC_FP64) of per-line records and
  * the adjoint's partial sums.
  * The first call on each device looks up the array's device address
  * (cudaGetSymbolAddress, with that device current); make that first call

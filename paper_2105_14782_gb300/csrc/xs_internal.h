@@ -9,6 +9,9 @@
 
 namespace xsi {
 
+// streaming multiprocessors of a GB300, for the splits that fill the chip
+constexpr int SMS = 152;
+
 // NVTX range named after the library call, around its host-side work and
 // launches; costs a few nanoseconds and records nothing unless a profiler
 // (nsys, ncu's NVTX filters) is attached

@@ -2373,12 +2373,12 @@ void choose_leaf_blocks(XsPlan* p, int64_t nl, int64_t N, int Lc, bool mixed, In
 {
     const int most = mixed ? LeafWarps<float>::v : LeafWarps<double>::v;
     const int64_t leaves = (N + LEAF - 1) / LEAF, all = leaves * Lc;
-    const int64_t want = mixed ? 152 * 16 : 152 * 8; // warps
+    const int64_t want = mixed ? xsi::SMS * 16 : xsi::SMS * 8; // warps
     const bool small = how == LEAVES_ONLY; // the smallest workspaces hold one partial per full block
     int split = 1;
     while (!small && split < most && all * split < want) split *= 2;
     int warps = most;
-    while (!small && warps > split && all * split / warps < 2 * 152) warps /= 2;
+    while (!small && warps > split && all * split / warps < 2 * xsi::SMS) warps /= 2;
     p->leaf_split = split;
     p->leaf_warps = warps;
     const int per = warps / split;
@@ -2462,7 +2462,7 @@ size_t xs_workspace_bytes(int64_t n_lines, int64_t N, int32_t L, int prec)
 
 // Lists of this length and more ask for the intervals in the smallest workspace too: without
 // them 20,000 lines on 20,000 points and 10 layers take 7.6 ms instead of 1.0, 220,000 and 4
-// layers 32.7 ms instead of 1.1.  They cost 8 to 13 bytes a grid point beside the lines' 92 to
+// layers 32.7 ms instead of 1.1.  They cost 8 to 13 bytes a grid point beside the lines' 68 to
 // 96 each; shorter lists would grow by more than they gain.
 constexpr int64_t COMPACT_MIN_LINES = 2048;
 
@@ -2601,7 +2601,7 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 far_sum_kernel<R><<<fgrid, 32 * FAR_WARPS, 0, st>>>(b, nu, l0);
                 int root = TOP_LOG; // log2 of the leaves of a block
                 auto subtrees = [&] { return blocks_of(tr.cnt[0], 1 << root); };
-                while (root > 2 && (int64_t)subtrees() * lc * b.n < 2 * 152) root -= 2;
+                while (root > 2 && (int64_t)subtrees() * lc * b.n < 2 * SMS) root -= 2;
                 const int rows = std::min(DownRows<R>::v, 1 << root);
                 down_kernel<R><<<dim3(subtrees(), (unsigned)lc, nz), rows * Far<R>::n, 0, st>>>(b, lc, root);
                 count_launch(2);

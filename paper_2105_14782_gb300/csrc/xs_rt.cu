@@ -1,7 +1,8 @@
 // Layer optical depth (Eq. dtau_line), the pure-absorption emission solve of
 // Sec. 3 (Eqs. rerr, rerr_tq, trans, sourcepla) with its adjoint, the Gaussian
-// log-likelihood and the power-law temperature profile.  All double precision:
-// these steps read and write [L][N] arrays once or twice and are bound by HBM.
+// log-likelihood and the power-law temperature profile.  All double precision: the emission
+// solve and its adjoint are bound by the FP64 pipe, the optical depth and the likelihood by
+// memory or, on short rows, by latency.
 #include <algorithm>
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -622,10 +623,11 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
         gp.p[m] = g_sigma ? g_sigma[m] : nullptr;
     }
     // blocks a layer: up to 8, fewer where the layers alone fill the chip or a block had less
-    // than 1,024 points (a cluster costs more to launch and to join than so short a row: 1,000
-    // layers of 50 points 154 us with 8 blocks, 300 of 9,727 88 us)
+    // than 1,024 points (4,096 from 128 layers on): a cluster costs more to launch and to join
+    // than so short a row (1,000 layers of 50 points 154 us with 8 blocks, 300 of 9,727 88 us)
+    const int64_t points = L < 128 ? 1024 : 4096;
     int c = 1;
-    while (c < RT_CLUSTER && (int64_t)c * L < 256 && 2 * c * 1024 <= N) c *= 2;
+    while (c < RT_CLUSTER && (int64_t)c * L < 256 && 2 * c * points <= N) c *= 2;
     auto pick = [&](auto M) {
         constexpr int m = decltype(M)::value;
         return c == 8   ? tau_adjoint_kernel<8, m>
@@ -662,7 +664,6 @@ int rt_tau_adjoint(const void* const* sigma, int32_t S, const double* vmr, const
 // take 8 points, for more SMs.
 static int emission_points(int32_t L, int64_t N)
 {
-    constexpr int SMS = 152;
     int best = 32;
     double least = 0.0;
     for (int pts = 32; pts >= 8; pts /= 2) {
