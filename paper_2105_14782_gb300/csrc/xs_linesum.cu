@@ -1607,7 +1607,7 @@ __device__ __forceinline__ double split_sum(double v, int split)
 __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(const __grid_constant__ Batch<float> batch,
                                                                            const double* __restrict__ nu, int64_t N,
                                                                            int layer0, double unscale,
-                                                                           int split, int slices)
+                                                                           int split, int slices, int stride)
 {
     const Species<float>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1628,10 +1628,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_kernel_f32(cons
     const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
     float shi = 0.0f, slo = 0.0f;
 #pragma unroll 1
-    for (int k = 0; k < RANGES; ++k) {
+    for (int k = 0; k < RANGES; k += tr.on ? 2 : 1) { // without 1 and 3 where there are far sets
         const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split * slices) {
+        for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += stride) {
             const int l = t0 + lane;
             const bool have = l < ce;
             __syncwarp();
@@ -1800,7 +1800,7 @@ __device__ __forceinline__ double near_poly64(const NearTile64& tl, int cnt, dou
 __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(const __grid_constant__ Batch<double> batch,
                                                                            const double* __restrict__ nu, int64_t N,
                                                                            int layer0, double unscale,
-                                                                           int split, int slices)
+                                                                           int split, int slices, int stride)
 {
     const Species<double>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1817,10 +1817,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_kernel_f64(con
     const double nuj = nu[j];
     double acc = 0.0;
 #pragma unroll 1
-    for (int k = 0; k < RANGES; ++k) {
+    for (int k = 0; k < RANGES; k += tr.on ? 2 : 1) { // without 1 and 3 where there are far sets
         const bool masked = k == 0 || k == RANGES - 1;
         const int ce = lf.e[k];
-        for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split * slices) {
+        for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += stride) {
             const int l = t0 + lane;
             const bool have = lane < NEAR64 && l < ce;
             __syncwarp();
@@ -1940,7 +1940,8 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
                                                                             const double* __restrict__ nu, int64_t N,
                                                                             int layer0,
                                                                             const double* __restrict__ T,
-                                                                            double lam_scale, int split, int slices)
+                                                                            double lam_scale, int split, int slices,
+                                                                            int stride)
 {
     const Species<float>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -1966,10 +1967,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<float>::v) leaf_adjoint_f32(con
         const double oj = nuj - lf.g.mid;
         const float ohi = (float)oj, olo = (float)(oj - (double)ohi), h = (float)lf.g.h;
 #pragma unroll 1
-        for (int k = 0; k < RANGES; ++k) {
+        for (int k = 0; k < RANGES; k += tr.on ? 2 : 1) { // without 1 and 3 where there are far sets
             const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += 32 * split * slices) {
+            for (int t0 = lf.s[k] + 32 * lf.sub; t0 < ce; t0 += stride) {
                 const int l = t0 + lane;
                 const bool have = l < ce;
                 __syncwarp();
@@ -2161,7 +2162,8 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
                                                                             const double* __restrict__ nu, int64_t N,
                                                                             int layer0,
                                                                             const double* __restrict__ T,
-                                                                            double lam_scale, int split, int slices)
+                                                                            double lam_scale, int split, int slices,
+                                                                            int stride)
 {
     const Species<double>& sp = batch.s[blockIdx.z];
     const Tree& tr = sp.tree;
@@ -2183,10 +2185,10 @@ __global__ void __launch_bounds__(32 * LeafWarps<double>::v) leaf_adjoint_f64(co
         tl.pos[lane] = nuj;
         tl.lam[lane] = lam;
 #pragma unroll 1
-        for (int k = 0; k < RANGES; ++k) {
+        for (int k = 0; k < RANGES; k += tr.on ? 2 : 1) { // without 1 and 3 where there are far sets
             const bool masked = k == 0 || k == RANGES - 1;
             const int ce = lf.e[k];
-            for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += NEAR64 * split * slices) {
+            for (int t0 = lf.s[k] + NEAR64 * lf.sub; t0 < ce; t0 += stride) {
                 const int l = t0 + lane;
                 const bool have = lane < NEAR64 && l < ce;
                 const int cnt = min(NEAR64, ce - t0);
@@ -2595,6 +2597,7 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
         const dim3 lgrid((unsigned)p.leaf_blocks, (unsigned)lc, nz);
         const dim3 fgrid((unsigned)far_blocks, (unsigned)lc, nz);
         const int lthreads = 32 * p.leaf_warps;
+        const int stride = (FAST ? 32 : NEAR64) * p.leaf_split * p.slices; // lines from a warp's chunk to its next
         prof_begin(adjoint ? 1 : 0, st);
         if (!adjoint) {
             if (tr.on) {
@@ -2607,10 +2610,10 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, unscale, p.leaf_split, p.slices);
+                leaf_kernel_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, unscale, p.leaf_split, p.slices, stride);
             else
                 leaf_kernel_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearTile64), st>>>(b, nu, N, l0, unscale,
-                                                                                           p.leaf_split, p.slices);
+                                                                                           p.leaf_split, p.slices, stride);
         } else {
             if (tr.on) {
                 up_kernel<R><<<dim3(blocks_of(tr.cnt[0], TOP), (unsigned)lc, nz), 32 * UP_WARPS, 0, st>>>(b, nu, N, l0,
@@ -2619,10 +2622,10 @@ static int run_batch(const Batch<R>& b, const XsPlan& p, const double* nu, int64
                 count_launch(2);
             }
             if constexpr (FAST)
-                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, T, unscale, p.leaf_split, p.slices);
+                leaf_adjoint_f32<<<lgrid, lthreads, 0, st>>>(b, nu, N, l0, T, unscale, p.leaf_split, p.slices, stride);
             else
                 leaf_adjoint_f64<<<lgrid, lthreads, p.leaf_warps * sizeof(NearAdjTile64), st>>>(b, nu, N, l0, T,
-                                                                                              unscale, p.leaf_split, p.slices);
+                                                                                              unscale, p.leaf_split, p.slices, stride);
         }
         if (!adjoint && p.slices > 1) {
             slices_kernel<R><<<dim3(blocks_of(N, 256), (unsigned)lc, nz), 256, 0, st>>>(b, nu, N, l0, unscale, p.slices);
