@@ -911,7 +911,6 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
         }
         const float dist = fmaxf(fabsf(nb) - h, 0.0f);
         const float D0 = fmaf(dist, dist, G), z2 = D0 * c2min;
-        const float iD = rcp_fast(D0), A0 = Al * iD, g = G * iD;
         float V0, Db, Dg;
         if (__all_sync(0xffffffffu, z2 >= WING1_Z2)) {
             // the F2 terms are up to 12 a^2/|z|^4 of f_b's leading one
@@ -924,6 +923,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
             } else {
                 float r[4];
                 rho_moments<4>(o2, w2, nb, G, D0, r);
+                const float iD = rcp_fast(D0), A0 = Al * iD, g = G * iD;
                 const float b1 = F1 * iD * iD, b2 = F2 * iD * iD * iD, u2 = b1 - 2.0f * g * A0;
                 V0 = fmaf(b2, r[2], fmaf(b1, r[1], A0 * r[0]));
                 Db = 2.0f * fmaf(b2, r[2], b1 * r[1]);
@@ -934,6 +934,7 @@ __device__ __forceinline__ void far_adjoint_sum(const Lines<float>& ln, const Fa
             if (__all_sync(0xffffffffu, z2 >= WING2_Z2) || p2.y >= WIDE_A) {
                 float r[6];
                 rho_moments<6>(o2, w2, nb, G, D0, r);
+                const float iD = rcp_fast(D0), A0 = Al * iD, g = G * iD;
                 const float b = rcp_fast(D0 * (p2.x * p2.x)), g4 = g * r[3], g5 = g * g * r[4], g6 = g * g * g * r[5];
                 const float q0 = fmaf(1.5f, r[1], -2.0f * g * r[2]), q = fmaf(3.75f, r[2], fmaf(-15.0f, g4, 12.0f * g5));
                 V0 = A0 * fmaf(b, fmaf(b, q, q0), r[0]);
