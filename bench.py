@@ -54,21 +54,21 @@ FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM on sm_103a (one FFMA = 2 flops)
 # only for the kernel sources they were taken on (the hash); otherwise the bench reports
 # no rate and says so.
 FLOPS_PER_TRIPLE = {
-    "sources_sha256": "0fc70c285cbccde8e0bc8996aebe98508327cfa43f9bb7c578420d03f6ac6ab3",
-    "scale": {"fwd": 0.4646, "adj": 0.8651,
+    "sources_sha256": "a1cfbc091fe5be510eb8f4315092095be43c2e18a9ac1121c6b61c2fe45ac1e8",
+    "scale": {"fwd": 0.4645, "adj": 0.8713,
               "capture": "one step of a 5-layer slice of the 10.2M-line workload (10,000,000 + 200,000 lines, "
-                         "100,000 points): 1.78e+12 and 3.31e+12 FP32 flops over 3.82e+12 triples"},
-    "emission": {"fwd": 0.9448, "adj": 1.6799,
+                         "100,000 points): 1.78e+12 and 3.33e+12 FP32 flops over 3.82e+12 triples"},
+    "emission": {"fwd": 0.9441, "adj": 1.6998,
                  "capture": "one step of a 20-layer slice of the emission workload (200,000 + 20,000 lines, "
-                            "20,000 points): 6.24e+10 and 1.11e+11 FP32 flops over 6.6e+10 triples"},
+                            "20,000 points): 6.24e+10 and 1.12e+11 FP32 flops over 6.6e+10 triples"},
 }
 
 # DRAM bytes (read + write) per layer of a forward's and an adjoint's line-sum kernels, both
 # species, from the same captures; null unless the sources still hash to the captured ones.
 TRAFFIC = {
-    "sources_sha256": "0fc70c285cbccde8e0bc8996aebe98508327cfa43f9bb7c578420d03f6ac6ab3",
-    "scale": {"fwd": 1.068e+10, "adj": 1.497e+10},
-    "emission": {"fwd": 1.713e+07, "adj": 2.059e+07},
+    "sources_sha256": "a1cfbc091fe5be510eb8f4315092095be43c2e18a9ac1121c6b61c2fe45ac1e8",
+    "scale": {"fwd": 1.076e+10, "adj": 1.512e+10},
+    "emission": {"fwd": 1.752e+07, "adj": 2.116e+07},
     "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one step's line-sum kernels, 5-layer slice of the "
                "10.2M-line workload and 20-layer slice of the emission workload, scaled to the launch's layers",
 }
@@ -480,7 +480,7 @@ def serving(dev, budget_s):
     fin, wall = serve.closed_loop(sched, chains=256, offered_rate=200.0, duration_s=15.0, cancel_at_end=True)
     closed = serve.summarize(fin, wall)
     closed.update(chains=256, offered_req_per_s=200.0, window_s=15.0,
-                  note="saturated: 200 req/s offered against a capacity of a few req/s; its latencies are queueing "
+                  note="saturated: 200 req/s offered far above capacity; its latencies are queueing "
                        "under overload, not a sustained p99")
     cap = closed["evals_per_s"] / mean_ev
     slo = 4.0
