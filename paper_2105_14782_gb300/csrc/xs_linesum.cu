@@ -44,7 +44,8 @@
 // offsets (then carried as float pairs), node sums, the intervals' polynomials and a leaf
 // polynomial's constant term.  FP32 pairs: the strength's exponential and its products (to
 // 1e-10, rounded once), running sums (TwoSum).  FP32: widths, stimulated emission, dlnS/dT, Voigt
-// values, the leaf polynomials' other coefficients, the adjoint's lambda and node weights.
+// values, the leaf polynomials' other coefficients, the adjoint's lambda and, summed as pairs, the
+// node weights.
 // Measured against XS_PREC_FP64 over lists of 1,000 to 200,000 lines and 1e-6 to 1e3 bar, the
 // relative rms error of sigma is 5.7e-8 to 1.13e-7 (5.8e-8 to 7e-6 when every pair was evaluated
 // at its point), that of g_T with weights of mixed sign 1e-9 to 2.2e-8 of what weights of one
@@ -1304,48 +1305,92 @@ __global__ void __launch_bounds__(DownRows<R>::v * Far<R>::n) down_kernel(const 
     }
 }
 
-// moments sum w T_k(x) of a weight at x, added to s
-template <int n, class R>
-__device__ __forceinline__ void add_moments(R w, R x, R (&s)[n])
+// A weight's products and sums on the way up: FP64, or float pairs in the FP32 path.  In plain
+// FP32 the roundings of the levels add up to three times that of lambda itself: g_b of weights
+// of mixed sign at 4 to 100 cm^-1 is off by 3.2e-9 to 3.5e-9 of what weights of one sign give,
+// 0.7e-9 to 1.9e-9 with pairs (1.1e-9 to 3.1e-9 with every line evaluated at every point).  One
+// layer's adjoint takes 80 us in plain FP32, 84 with pairs, 119 with FP64; 220,000 lines x 20
+// layers 3.71, 3.72 and 3.82 ms.
+template <class R> struct UpSum { using type = double; };
+template <> struct UpSum<float> { using type = Pair; };
+__device__ __forceinline__ Pair times(const Pair& w, float t)
 {
-    R a = w, b = w * x;
-    const R x2 = x + x;
+    const float p = w.hi * t;
+    return {p, fmaf(w.lo, t, fmaf(w.hi, t, -p))};
+}
+__device__ __forceinline__ double times(double w, double t) { return w * t; }
+__device__ __forceinline__ Pair up_weight(double v, float) { return {(float)v, 0.0f}; }
+__device__ __forceinline__ double up_weight(double v, double) { return v; }
+__device__ __forceinline__ float rounded(const Pair& v) { return v.hi + v.lo; }
+__device__ __forceinline__ double rounded(double v) { return v; }
+
+// moments sum w T_k(x) of a weight at x, added to s
+template <int n>
+__device__ __forceinline__ void add_moments(double w, double x, double (&s)[n])
+{
+    double a = w, b = w * x;
+    const double x2 = x + x;
     s[0] += a;
     s[1] += b;
 #pragma unroll
     for (int k = 2; k < n; ++k) {
-        const R t = x2 * b - a;
+        const double t = x2 * b - a;
         s[k] += t;
+        a = b;
+        b = t;
+    }
+}
+template <int n>
+__device__ __forceinline__ void add_moments(const Pair& w, float x, Pair (&s)[n])
+{
+    float a = 1.0f, b = x;
+    const float x2 = x + x;
+    s[0] = add(s[0], w);
+#pragma unroll
+    for (int k = 1; k < n; ++k) {
+        s[k] = add(s[k], times(w, b));
+        const float t = fmaf(x2, b, -a);
         a = b;
         b = t;
     }
 }
 
 // node weight m from the moments M: sum_k (1 or 2)/n M_k T_k(t_m)
-template <int n, class R>
-__device__ __forceinline__ R node_weight(const R* M, int m)
+template <int n>
+__device__ __forceinline__ double node_weight(const double* M, int m)
 {
-    R s = R(0.5) * M[0];
+    double s = 0.5 * M[0];
 #pragma unroll
-    for (int k = 1; k < n; ++k) s += M[k] * cheb_r(R(0), k, m);
-    return s * R(2.0 / n);
+    for (int k = 1; k < n; ++k) s += M[k] * cheb_r(0.0, k, m);
+    return s * (2.0 / n);
+}
+template <int n>
+__device__ __forceinline__ Pair node_weight(const Pair* M, int m)
+{
+    Pair s = {0.5f * M[0].hi, 0.5f * M[0].lo};
+#pragma unroll
+    for (int k = 1; k < n; ++k) s = add(s, times(M[k], cheb_r(0.0f, k, m)));
+    constexpr float c = (float)(2.0 / n), cl = (float)(2.0 / n - (double)c);
+    Pair r = times(s, c);
+    r.lo = fmaf(s.hi, cl, r.lo);
+    return r;
 }
 
 // Node weights of all intervals: per layer and top interval, one warp per leaf takes its
 // points, then the larger intervals take the nodes of those below (whose weights
-// reproduce every polynomial of the degree kept).  In the FP32 path in FP32, as lambda
-// itself: the rounding of one leaf's weights is independent of the next one's.
-// weights[layer][interval][n].
+// reproduce every polynomial of the degree kept).  In the FP32 path lambda is rounded once and
+// the sums are float pairs (UpSum); the weights are stored in FP32.  weights[layer][interval][n].
 constexpr int UP_WARPS = 16;
 template <class R>
 __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant__ Batch<R> batch,
                                                            const double* __restrict__ nu, int64_t N, int layer0,
                                                            double lam_scale)
 {
+    using A = typename UpSum<R>::type;
     const Species<R>& spc = batch.s[blockIdx.z];
     const Tree& tr = spc.tree;
     constexpr int n = Far<R>::n;
-    __shared__ R M[UP_WARPS][n], w[2][TOP][n];
+    __shared__ A M[UP_WARPS][n], w[2][TOP][n];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     const int nloc = blockIdx.y, top = blockIdx.x;
     const double* g = spc.g_sigma + (size_t)(layer0 + nloc) * N;
@@ -1355,31 +1400,30 @@ __global__ void __launch_bounds__(32 * UP_WARPS) up_kernel(const __grid_constant
             const int i = top * many + q;
             if (i >= tr.cnt[k] || !XS_CHECK(q < TOP)) break;
             const Geo sp = tr.geo[tr.off[k] + i];
-            R s[n];
+            A s[n];
 #pragma unroll
-            for (int m = 0; m < n; ++m) s[m] = R(0);
+            for (int m = 0; m < n; ++m) s[m] = A{};
             if (k == 0) {
                 const int64_t j = (int64_t)i * LEAF + lane;
-                if (j < N) add_moments<n, R>((R)(g[j] * lam_scale), (R)in_span(nu[j], sp), s);
+                if (j < N) add_moments<n>(up_weight(g[j] * lam_scale, R(0)), (R)in_span(nu[j], sp), s);
             } else {
 #pragma unroll 1
                 for (int r = lane; r < below * n; r += 32) {
                     const int ch = below * i + r / n, m = r % n; // child interval and its node
                     if (ch >= tr.cnt[k - 1]) break;
                     const Geo gc = tr.geo[tr.off[k - 1] + ch];
-                    const R x = (R)node_in_span(gc, cheb<n>(1, m), sp);
-                    add_moments<n, R>(w[(k - 1) & 1][below * q + r / n][m], x, s);
+                    add_moments<n>(w[(k - 1) & 1][below * q + r / n][m], (R)node_in_span(gc, cheb<n>(1, m), sp), s);
                 }
             }
             __syncwarp();
             int idx;
-            const R v = warp_reduce_scatter(s, idx);
+            const A v = warp_reduce_scatter(s, idx);
             if (idx >= 0 && XS_CHECK(idx < n)) M[row][idx] = v;
             __syncwarp();
             if (lane < n) {
-                const R x = node_weight<n, R>(M[row], lane);
+                const A x = node_weight<n>(M[row], lane);
                 w[k & 1][q][lane] = x;
-                spc.wts[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = x;
+                spc.wts[((size_t)nloc * tr.total + tr.off[k] + i) * n + lane] = rounded(x);
             }
             __syncwarp();
         }
