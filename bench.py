@@ -54,21 +54,21 @@ FP32_LANES_PER_SM = 128  # FP32 FMA lanes per SM on sm_103a (one FFMA = 2 flops)
 # only for the kernel sources they were taken on (the hash); otherwise the bench reports
 # no rate and says so.
 FLOPS_PER_TRIPLE = {
-    "sources_sha256": "a1cfbc091fe5be510eb8f4315092095be43c2e18a9ac1121c6b61c2fe45ac1e8",
-    "scale": {"fwd": 0.4645, "adj": 0.8713,
+    "sources_sha256": "5c607c8f2d6dde5806338f84abb47dedc660847548e292ddef02ffd22a1ad3bb",
+    "scale": {"fwd": 0.4645, "adj": 0.8714,
               "capture": "one step of a 5-layer slice of the 10.2M-line workload (10,000,000 + 200,000 lines, "
                          "100,000 points): 1.78e+12 and 3.33e+12 FP32 flops over 3.82e+12 triples"},
-    "emission": {"fwd": 0.9441, "adj": 1.6998,
+    "emission": {"fwd": 0.9441, "adj": 1.7052,
                  "capture": "one step of a 20-layer slice of the emission workload (200,000 + 20,000 lines, "
-                            "20,000 points): 6.24e+10 and 1.12e+11 FP32 flops over 6.6e+10 triples"},
+                            "20,000 points): 6.24e+10 and 1.13e+11 FP32 flops over 6.6e+10 triples"},
 }
 
 # DRAM bytes (read + write) per layer of a forward's and an adjoint's line-sum kernels, both
 # species, from the same captures; null unless the sources still hash to the captured ones.
 TRAFFIC = {
-    "sources_sha256": "a1cfbc091fe5be510eb8f4315092095be43c2e18a9ac1121c6b61c2fe45ac1e8",
-    "scale": {"fwd": 1.076e+10, "adj": 1.512e+10},
-    "emission": {"fwd": 1.752e+07, "adj": 2.116e+07},
+    "sources_sha256": "5c607c8f2d6dde5806338f84abb47dedc660847548e292ddef02ffd22a1ad3bb",
+    "scale": {"fwd": 1.074e+10, "adj": 1.510e+10},
+    "emission": {"fwd": 1.749e+07, "adj": 2.106e+07},
     "capture": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one step's line-sum kernels, 5-layer slice of the "
                "10.2M-line workload and 20-layer slice of the emission workload, scaled to the launch's layers",
 }
